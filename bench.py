@@ -36,8 +36,8 @@ def workload_config(world):
     """The `config` object of the JSON line, the same for both arms."""
     w = WORKLOAD
     return {"workload": w["workload"], "grid": [w["n1"], w["n2"]], "kmax": w["kmax"],
-            "l2": "inputs larger than L2: each step streams its 235 MB working set (state 33.5 MB, "
-                  "uv 134 MB, gk 67 MB) through the 129 MB L2; flushed once before the timed steps",
+            "l2": "inputs larger than L2: each step streams its 185 MB working set (state 33.5 MB, "
+                  "uv 101 MB, gk 50 MB) through the 129 MB L2; flushed once before the timed steps",
             "parallelism": f"replicas{world}"}
 FLUSH_BYTES = 512 * 1024 * 1024
 
@@ -54,12 +54,22 @@ def _peaks():
 PASS_NAMES = ("A", "B", "C", "CA")
 
 
-def pass_bytes(n1, n2, K1, K2, esz):
+def step_points(K, least=12):
+    """Points a side of the step's alias-free transforms: the least 3 * 2^a
+    that holds 3 K + 1 (a product of two fields of K harmonics then folds
+    onto none of the retained ones)."""
+    n = least
+    while n < 3 * K + 1:
+        n *= 2
+    return n
+
+
+def pass_bytes(K1, K2, esz):
     """Algorithmic HBM bytes of passes A, B, C and of the fused CA (pass C
     followed by the next step's pass A, which then reads no state): each
     array read or written once."""
     box = (2 * K1 + 1) * (K2 + 1) * esz
-    col = n1 * (K2 + 1) * esz
+    col = step_points(K1) * (K2 + 1) * esz
     return [box + 2 * col, 2 * col + col, col + 2 * box, col + 2 * box + 2 * col]
 
 
@@ -233,7 +243,7 @@ def measure_batched(flame, inputs, nflames=256, steps=500, plain_steps=20):
     for f in fl:
         f.sync_status()
     pts_step = sum(n1 * n2 for n1, n2 in grids)
-    bytes_step = sum(sum(pass_bytes(n1, n2, f.K1, f.K2, 8)) for (n1, n2), f in zip(grids, fl))
+    bytes_step = sum(sum(pass_bytes(f.K1, f.K2, 8)[:3]) for f in fl)
     for f in fl:
         f.close()
     rate = pts_step * steps / (t_batch * 1e-3)
@@ -246,23 +256,25 @@ def measure_batched(flame, inputs, nflames=256, steps=500, plain_steps=20):
             "effective_gbs": gbs, "frac_of_hbm": gbs / peak, "peak_kind": kind}
 
 
-def passB_model_flops(n1, n2):
-    """Model flops of one pass B launch (the row pass): per row, two
-    half-length inverse complex FFTs (even and odd grid points) and one
-    forward, 5 M log2 M each (M = N2/2), the odd points' pre-twiddle (6 M),
-    g = u^2 + v^2 (3 per grid point: 6 M) and the real post-processing
-    (10 per kept output, about 5 M)."""
+def passB_model_flops(K1, K2):
+    """Model flops of one pass B launch (the row pass) on the alias-free grid:
+    per row, two half-length inverse complex FFTs (even and odd grid points)
+    and one forward, 5 M log2 M each (M = half a row), the odd points'
+    pre-twiddle (6 M), g = u^2 + v^2 (3 per grid point: 6 M) and the real
+    post-processing (10 per kept output, about 5 M)."""
     import math
-    m = n2 // 2
-    return n1 * (15.0 * m * math.log2(m) + 17.0 * m)
+    m = step_points(K2, 24) // 2
+    return step_points(K1) * (15.0 * m * math.log2(m) + 17.0 * m)
 
 
-def step_model_flops(n1, n2):
-    """Model flops of one step per grid point: three real 2-D transforms
-    (two inverse, one forward) at 2.5 N log2 N each (N = N1 N2) and about 5
-    pointwise flops (the product, the linear operator and the update)."""
+def step_model_flops(K1, K2):
+    """Model flops of one step: three real 2-D transforms on the alias-free
+    grid (two inverse, one forward) at 2.5 N log2 N each (N its points) and
+    about 5 pointwise flops a point (the product, the linear operator and the
+    update)."""
     import math
-    return 7.5 * math.log2(n1 * n2) + 5.0
+    n = step_points(K1) * step_points(K2, 24)
+    return n * (7.5 * math.log2(n) + 5.0)
 
 
 def measure_trajectory(flame, inputs, n1, n2, prec, kmax, nsteps, fp64_peak=None):
@@ -280,15 +292,17 @@ def measure_trajectory(flame, inputs, n1, n2, prec, kmax, nsteps, fp64_peak=None
     ms = min(_ev_time(lambda: f.step(st, m, t, nsteps), s) for _ in range(3))
     f.sync_status()
     esz = 16 if prec == "fp64" else 8
-    bytes_step = sum(pass_bytes(n1, n2, f.K1, f.K2, esz)[:3])
+    K1, K2 = f.K1, f.K2
+    bytes_step = sum(pass_bytes(K1, K2, esz)[:3])
     f.close()
     out = {"workload": f"trajectory-{n1}x{n2}-{prec}-{nsteps}steps", "steps": nsteps,
            "value": n1 * n2 * nsteps / (ms * 1e-3), "unit": "points/s", "ms_per_step": ms / nsteps,
            "effective_gbs": bytes_step / (ms * 1e-3 / nsteps) / 1e9,
            "note": "graph-captured steps; the working set is L2-resident"}
     if prec == "fp64" and fp64_peak:
-        fl_rate = step_model_flops(n1, n2) * n1 * n2 / (ms * 1e-3 / nsteps)
-        out.update({"model_flops_per_point": step_model_flops(n1, n2), "achieved_gflops": fl_rate / 1e9,
+        fl_step = step_model_flops(K1, K2)
+        fl_rate = fl_step / (ms * 1e-3 / nsteps)
+        out.update({"model_flops_per_point": fl_step / (n1 * n2), "achieved_gflops": fl_rate / 1e9,
                     "fp64_peak_gflops": fp64_peak / 1e9, "peak_kind": "measured (flame_fma_peak)",
                     "frac_of_fp64_peak": fl_rate / fp64_peak})
     return out
@@ -342,7 +356,7 @@ def run_ours(args):
     flush = torch.empty(FLUSH_BYTES, dtype=torch.uint8, device="cuda")
     stream = torch.cuda.current_stream()
     esz = 8 if w["prec"] == "fp32" else 16
-    pbytes = pass_bytes(n1, n2, f.K1, f.K2, esz)
+    pbytes = pass_bytes(f.K1, f.K2, esz)
 
     # Steps run back to back, pass by pass, exactly as flame_step enqueues
     # them: A, then (B, CA) for every step but the last and B, C for the last
@@ -455,10 +469,10 @@ def run_ours(args):
     roof_alu = None
     if PASS_NAMES[dom] == "B":
         fp32_peak = flame.flame_fma_peak("fp32")
-        ach = passB_model_flops(n1, n2) / (avg[dom] * 1e-3) / 1e12
+        ach = passB_model_flops(f.K1, f.K2) / (avg[dom] * 1e-3) / 1e12
         roof_alu = {"bound": "alu", "kernel": "passB", "achieved": ach, "peak": fp32_peak / 1e12,
                     "peak_kind": "measured (flame_fma_peak, scalar FP32 FMA)", "unit": "TFLOP/s",
-                    "frac": ach / (fp32_peak / 1e12), "model_flops": passB_model_flops(n1, n2)}
+                    "frac": ach / (fp32_peak / 1e12), "model_flops": passB_model_flops(f.K1, f.K2)}
     if not args.no_extras:
         batched = measure_batched(flame, inputs)
         adjoint = measure_adjoint(flame, inputs)
@@ -524,7 +538,7 @@ def run_suite(args):
         ms = _ev_time(lambda: f.step(st, m, t, nsteps), s)
         f.sync_status()
         esz = 16 if prec == "fp64" else 8
-        gbs = sum(pass_bytes(n1, n2, f.K1, f.K2, esz)[:3]) / (ms * 1e-3 / nsteps) / 1e9  # passes A, B, C
+        gbs = sum(pass_bytes(f.K1, f.K2, esz)[:3]) / (ms * 1e-3 / nsteps) / 1e9  # passes A, B, C
         print(json.dumps({"suite": f"trajectory-{n1}x{n2}-{prec}", "steps": nsteps, "ms_per_step": ms / nsteps,
                           "points_per_s": n1 * n2 * nsteps / (ms * 1e-3), "effective_gbs": gbs,
                           "note": "graph-captured; L2-resident" if n1 * n2 <= 2 ** 21 else "graph-captured"}),
@@ -616,8 +630,9 @@ def run_suite(args):
 # descriptors, and the translation units that instantiate them.  Host code
 # (flame_api.cu) and kernels off the step (adjoint, FP64, Heun, FFT pair)
 # are not in it.
-STEP_SOURCES = ("fft_engine.cuh", "flame_kernels.cuh", "flame_ops.cuh", "flame_internal.h",
-                "flame_f32_a.cu", "flame_f32_b.cu", "flame_f32_c.cu")
+STEP_SOURCES = ("fft_engine.cuh", "line3.cuh", "flame_kernels.cuh", "flame_step.cuh", "flame_step_ops.cuh",
+                "flame_launch.cuh", "flame_internal.h", "flame_step_f32_a.cu", "flame_step_f32_b.cu",
+                "flame_step_f32_c.cu")
 
 
 def kernel_sources_sha256():

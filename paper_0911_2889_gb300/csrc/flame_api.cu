@@ -22,6 +22,7 @@
 #include "flame.h"
 #include "flame_internal.h"
 #include "fft_engine.cuh"
+#include "line3.cuh"
 
 using flame::FlameDesc;
 using flame::Ops;
@@ -119,13 +120,13 @@ bool flame::encode_gk_map(CUtensorMap *map, void *gk, int n1, int ldk) {
                   CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-bool flame::encode_uv_map(CUtensorMap *map, void *uv, int n1, int ldk) {
+bool flame::encode_uv_map(CUtensorMap *map, void *uv, int n1, int ldk, int box_pairs) {
     const auto encode = tensor_map_encoder();
     if (!encode || !map || !uv || n1 < 2 || (n1 & 1) || ldk < 1) return false;
     // uv as floats: (8 floats of a row pair) x k2 (32-byte stride) x row pair
     const cuuint64_t dims[3] = {8, (cuuint64_t)ldk, (cuuint64_t)(n1 / 2)};
     const cuuint64_t strides[2] = {32, (cuuint64_t)ldk * 32};
-    const cuuint32_t box[3] = {8, 1, (cuuint32_t)flame::uv_box_pairs(n1)};
+    const cuuint32_t box[3] = {8, 1, (cuuint32_t)box_pairs};
     const cuuint32_t estr[3] = {1, 1, 1};
     return encode(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, uv, dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
                   CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_NONE,
@@ -151,11 +152,14 @@ struct GraphEntry {
 
 struct flame_ctx {
     flame_params p;  // resolved
-    StepArgs sa;
+    StepArgs sa;      // the public grid (transforms, area, adjoint)
+    StepArgs ss;      // the step's alias-free grid
     int logn1, logm;
     int device;
     size_t csz;       // bytes of one complex element
-    void *tw1, *twm;  // twiddle tables
+    void *tabs;       // one allocation: the tables, rowsum, dscal and status below
+    void *tw1, *twm;  // twiddle tables of the public grid's lines
+    void *tw1s, *twms;  // ... and of the step grid's
     void *uv, *gk;    // step workspaces
     void *spec;       // c2r workspace, N1 x (N2/2 + 1)
     void *aw;         // area / adjoint workspace, N1 x ldk pairs
@@ -171,7 +175,7 @@ struct flame_ctx {
     // eviction does not wait for the device
     std::vector<cudaGraphExec_t> retired;
     // ensemble state (owned by the first handle of a batch call): the
-    // descriptors, then the flames' uv maps and gk maps (FP32)
+    // descriptors
     void *batch_desc = nullptr;
     size_t batch_cap = 0;
     void *batch_host = nullptr;  // pinned staging of the descriptors' upload
@@ -200,7 +204,8 @@ struct flame_ctx {
     int var_a_bat = 0, var_b_bat = 0;
     // tensor map of uv for the tensor-store variant of pass A (FP32)
     CUtensorMap uv_map, gk_map;  // tensor maps of uv and gk for the tensor-store variants (FP32)
-    bool has_uv_map = false, has_gk_map = false;
+    CUtensorMap uv_map_full;  // uv of the public grid (steps that record the area)
+    bool has_uv_map = false, has_gk_map = false, has_uv_map_full = false;
     const CUtensorMap *map() const { return has_uv_map ? &uv_map : nullptr; }
     const CUtensorMap *gmap() const { return has_gk_map ? &gk_map : nullptr; }
     // multi-step runs fuse pass C of each step with pass A of the next
@@ -230,6 +235,8 @@ template <class R> flame_status alloc_tables(flame_ctx *h) {
     using C = typename Ops<R>::C;
     CUDA_TRY(Ops<R>::init_twiddles(static_cast<C *>(h->tw1), h->logn1, h->cap));
     CUDA_TRY(Ops<R>::init_twiddles(static_cast<C *>(h->twm), h->logm, h->cap));
+    CUDA_TRY(Ops<R>::init_twiddles3(static_cast<C *>(h->tw1s), h->ss.la, h->cap));
+    CUDA_TRY(Ops<R>::init_twiddles3(static_cast<C *>(h->twms), h->ss.lb, h->cap));
     return FLAME_OK;
 }
 
@@ -244,16 +251,12 @@ void free_ctx(flame_ctx *h) {
     if (h->batch_up) cudaEventDestroy(h->batch_up);
     for (cudaStream_t q : h->batch_streams) cudaStreamDestroy(q);
     for (cudaEvent_t ev : h->batch_events) cudaEventDestroy(ev);
-    cudaFree(h->tw1);
-    cudaFree(h->twm);
+    cudaFree(h->tabs);
     cudaFree(h->uv);
     cudaFree(h->gk);
     cudaFree(h->spec);
     cudaFree(h->aw);
-    cudaFree(h->rowsum);
     cudaFree(h->adj);
-    cudaFree(h->dscal);
-    cudaFree(h->status);
     cudaFree(h->io);
     for (auto e : h->io_ev) cudaEventDestroy(e);
     if (h->cpy) cudaStreamDestroy(h->cpy);
@@ -264,12 +267,12 @@ void free_ctx(flame_ctx *h) {
 FlameDesc make_desc(flame_ctx *h, void *state, double *mean, double *t) {
     FlameDesc d;
     memset(&d, 0, sizeof d);  // descriptors are compared bytewise
-    d.a = h->sa;
+    d.a = h->ss;
     d.state = state;
     d.uv = h->uv;
     d.gk = h->gk;
-    d.tw1 = h->tw1;
-    d.twm = h->twm;
+    d.tw1 = h->tw1s;
+    d.twm = h->twms;
     d.t_in = t;
     d.coef = h->dscal + 8;
     d.mean = mean;
@@ -293,51 +296,9 @@ bool first_stage(int stage) {
     return stage == flame::kStageEuler || stage == flame::kStageHeun1 || stage == flame::kStageIF1;
 }
 
-// A recorded step with the surface area: pass B's area variant sums the
-// area of the rows it transforms (rec_area = 1); where that variant does not
-// fit in shared memory (FP64 rows of 8192 points) the separate area kernels
-// compute it first, into handle scratch (rec_area = 2).
-cudaError_t enqueue_step_area(flame_ctx *h, FlameDesc d, cudaStream_t s) {
+// One evaluation of the right-hand side and its stage, on the step grid.
+cudaError_t enqueue_passes(flame_ctx *h, const FlameDesc &d, cudaStream_t s) {
     cudaError_t e;
-    d.rec_area = 1;
-    d.arow = h->rowsum;
-    const bool f64 = h->p.prec == FLAME_FP64;
-    if ((e = f64 ? Ops<double>::passA(d, s, h->var_a) : Ops<float>::passA(d, s, h->var_a, h->map())) != cudaSuccess)
-        return e;
-    e = f64 ? Ops<double>::passB_area(d, s) : Ops<float>::passB_area(d, s);
-    if (e == cudaErrorNotSupported) {
-        cudaGetLastError();
-        flame::AdjDesc ad;
-        memset(&ad, 0, sizeof ad);
-        ad.a = h->sa;
-        ad.state = d.state;
-        ad.mean = d.mean;
-        ad.t = d.t_in;
-        ad.uv = h->uv;
-        ad.gk = h->gk;
-        ad.aw = h->aw;
-        ad.rowsum = h->rowsum;
-        ad.area = h->dscal + 6;
-        ad.dmean = h->dscal + 3;
-        ad.tw1 = h->tw1;
-        ad.twm = h->twm;
-        // the area kernels use the step's workspaces: run them, then the
-        // step's passes from the start
-        if ((e = f64 ? Ops<double>::area(ad, s) : Ops<float>::area(ad, s)) != cudaSuccess) return e;
-        d.rec_area = 2;
-        d.aval = h->dscal + 6;
-        if ((e = f64 ? Ops<double>::passA(d, s, h->var_a) : Ops<float>::passA(d, s, h->var_a, h->map())) !=
-            cudaSuccess)
-            return e;
-        e = f64 ? Ops<double>::passB(d, s, h->var_b) : Ops<float>::passB(d, s, h->var_b, h->gmap());
-    }
-    if (e != cudaSuccess) return e;
-    return f64 ? Ops<double>::passC(d, s) : Ops<float>::passC(d, s);
-}
-
-cudaError_t enqueue_step(flame_ctx *h, const FlameDesc &d, cudaStream_t s) {
-    cudaError_t e;
-    if (d.rec && h->rec_area && first_stage(d.stage)) return enqueue_step_area(h, d, s);
     if (h->p.prec == FLAME_FP64) {
         {
             FLAME_RANGE("flame pass A");
@@ -362,6 +323,57 @@ cudaError_t enqueue_step(flame_ctx *h, const FlameDesc &d, cudaStream_t s) {
     return Ops<float>::passC(d, s);
 }
 
+// A recorded step with the surface area, whose sum is over the public grid's
+// points: the step runs there, and its row pass sums the area of the rows it
+// transforms (rec_area = 1); where that pass does not fit in shared memory
+// (FP64 rows of 8192 points) the separate area kernels compute it first, into
+// handle scratch (rec_area = 2), and the step runs on its own grid.
+cudaError_t enqueue_step_area(flame_ctx *h, const FlameDesc &ds, cudaStream_t s) {
+    cudaError_t e;
+    FlameDesc d = ds;
+    d.a = h->sa;
+    d.tw1 = h->tw1;
+    d.twm = h->twm;
+    d.rec_area = 1;
+    d.arow = h->rowsum;
+    const bool f64 = h->p.prec == FLAME_FP64;
+    const CUtensorMap *um = h->has_uv_map_full ? &h->uv_map_full : nullptr;
+    if ((e = f64 ? Ops<double>::passA_full(d, s, false, nullptr) : Ops<float>::passA_full(d, s, false, um)) != cudaSuccess)
+        return e;
+    e = f64 ? Ops<double>::passB_area(d, s) : Ops<float>::passB_area(d, s);
+    if (e == cudaErrorNotSupported) {
+        cudaGetLastError();
+        flame::AdjDesc ad;
+        memset(&ad, 0, sizeof ad);
+        ad.a = h->sa;
+        ad.state = d.state;
+        ad.mean = d.mean;
+        ad.t = d.t_in;
+        ad.uv = h->uv;
+        ad.gk = h->gk;
+        ad.aw = h->aw;
+        ad.rowsum = h->rowsum;
+        ad.area = h->dscal + 6;
+        ad.dmean = h->dscal + 3;
+        ad.tw1 = h->tw1;
+        ad.twm = h->twm;
+        // the area kernels use the step's workspaces: run them, then the
+        // step's passes from the start
+        if ((e = f64 ? Ops<double>::area(ad, s) : Ops<float>::area(ad, s)) != cudaSuccess) return e;
+        d = ds;
+        d.rec_area = 2;
+        d.aval = h->dscal + 6;
+        return enqueue_passes(h, d, s);
+    }
+    if (e != cudaSuccess) return e;
+    return f64 ? Ops<double>::passC_full(d, s) : Ops<float>::passC_full(d, s);
+}
+
+cudaError_t enqueue_step(flame_ctx *h, const FlameDesc &d, cudaStream_t s) {
+    if (d.rec && h->rec_area && first_stage(d.stage)) return enqueue_step_area(h, d, s);
+    return enqueue_passes(h, d, s);
+}
+
 // The pass C stages of one step of a scheme.
 int scheme_stages(int scheme, int *stages) {
     if (scheme == kSchemeHeun) {
@@ -382,24 +394,18 @@ int scheme_stages(int scheme, int *stages) {
 // (passes A and B) and a pass C that applies the stage's update.  With
 // fusion, pass C of each stage runs fused with pass A of the next:
 // A, (B, CA) x (stages - 1), B, C.  Same arithmetic as separate passes.
+// (Steps that record the area run on the public grid: they are not fused.)
 cudaError_t enqueue_scheme(flame_ctx *h, FlameDesc d, int scheme, int n, cudaStream_t s) {
     int st[2];
     const int ns = scheme_stages(scheme, st);
     const int total = ns * n;
     cudaError_t e = cudaSuccess;
-    if (h->fuse && total > 1) {
+    if (h->fuse && total > 1 && !(d.rec && h->rec_area)) {
         e = Ops<float>::passA(d, s, h->var_a, h->map());
         for (int i = 0; i < total && e == cudaSuccess; ++i) {
             d.stage = st[i % ns];
-            FlameDesc dc = d;
-            if (d.rec && h->rec_area && first_stage(d.stage)) {
-                dc.rec_area = 1;
-                dc.arow = h->rowsum;
-                e = Ops<float>::passB_area(dc, s);
-            } else {
-                e = Ops<float>::passB(d, s, h->var_b, h->gmap());
-            }
-            if (e == cudaSuccess) e = i + 1 < total ? Ops<float>::passCA(dc, s, h->map()) : Ops<float>::passC(dc, s);
+            e = Ops<float>::passB(d, s, h->var_b, h->gmap());
+            if (e == cudaSuccess) e = i + 1 < total ? Ops<float>::passCA(d, s, h->map()) : Ops<float>::passC(d, s);
         }
         return e;
     }
@@ -443,8 +449,8 @@ void setup_l2_window(flame_ctx *h, size_t state_bytes) {
 }
 
 // ---------------------------------------------------------------- autotuner
-// For FP32 grids with compile-time kernels (N1, N2/2 in 256..4096) the
-// alternative shapes of passes A and B are timed once per (grid, K,
+// For FP32 grids with two-line kernels (lines of 192 points and more) the
+// alternatives of passes A and B are timed once per (grid, K,
 // precision, device) on scratch buffers, and the fastest is kept for the
 // process.  FLAME_AUTOTUNE=0 keeps the default shapes.
 using TuneKey = std::tuple<int, int, int, int, int, int>;
@@ -458,7 +464,7 @@ std::mutex g_tune_mu;
 // two-line stand-ins of the one-line variants (for the grouped launches when
 // only the single-flame choice is known)
 int two_line_a(int v) { return v == flame::kVariantOneLine ? flame::kVariantDirect : v; }
-int two_line_b(int v) { return v == flame::kVariantOneLineB ? flame::kVariantDefault : v; }
+int two_line_b(int v) { return v == flame::kVariantOneLineB ? flame::kVariantDirectB : v; }
 
 // Autotuner cache file (FLAME_TUNE_CACHE=path): a flat JSON object mapping
 // "<GPU name>|<N1>x<N2>|<K1>,<K2>|<precision>" to [pass A variant, pass B
@@ -554,8 +560,7 @@ bool fuse_allowed(const flame_ctx *h) {
     if (env && strcmp(env, "0") == 0) return false;
     // (not with the one-line column passes: the fused pass is a two-line
     // kernel, and fused and separate steps must give the same bits)
-    return h->p.prec == FLAME_FP32_MIXED && h->has_uv_map && h->logn1 >= 8 && h->logn1 <= 12 &&
-           h->var_a != flame::kVariantOneLine;
+    return h->p.prec == FLAME_FP32_MIXED && h->has_uv_map && h->var_a != flame::kVariantOneLine;
 }
 
 flame_status autotune(flame_ctx *h) {
@@ -564,16 +569,8 @@ flame_status autotune(flame_ctx *h) {
     if (force) {
         int va = 0, vb = 0;
         if (sscanf(force, "%d,%d", &va, &vb) == 2) {
-            h->var_a = va == 4   ? flame::kVariantOneLine
-                       : va == 3 ? flame::kVariantTma
-                       : va == 2 ? flame::kVariantRadix8A
-                       : va      ? flame::kVariantDirect
-                                 : flame::kVariantDefault;
-            h->var_b = vb == 4   ? flame::kVariantWarpB
-                       : vb == 3 ? flame::kVariantOneLineB
-                       : vb == 2 ? flame::kVariantTmaB
-                       : vb      ? flame::kVariantRadix8
-                                 : flame::kVariantDefault;
+            h->var_a = va >= 0 && va <= 4 ? va : flame::kVariantDirect;
+            h->var_b = vb >= 0 && vb <= 4 ? vb : flame::kVariantDirectB;
             h->var_a_bat = h->var_a;  // forced: the grouped launches take them too
             h->var_b_bat = h->var_b;
             h->fuse = fuse_allowed(h);
@@ -585,8 +582,7 @@ flame_status autotune(flame_ctx *h) {
         h->fuse = fuse_allowed(h);
         return FLAME_OK;
     }
-    if (h->p.prec != FLAME_FP32_MIXED || h->logn1 < 8 || h->logn1 > 12 || h->logm < 8 || h->logm > 12)
-        return FLAME_OK;
+    if (h->p.prec != FLAME_FP32_MIXED || h->ss.la < 6 || h->ss.lb < 6) return FLAME_OK;
     const TuneKey key{h->p.n_theta, h->p.n_phi, h->p.K1, h->p.K2, (int)h->p.prec, h->device};
     {
         std::lock_guard<std::mutex> lk(g_tune_mu);
@@ -611,13 +607,6 @@ flame_status autotune(flame_ctx *h) {
             h->var_b = it->second.b;
             h->var_a_bat = it->second.a_bat;
             h->var_b_bat = it->second.b_bat;
-            // a variant the handle cannot run (no tensor map) falls back to the default shape
-            if (h->var_a == flame::kVariantTma && !h->has_uv_map) h->var_a = flame::kVariantDefault;
-            if (h->var_b == flame::kVariantTmaB && !h->has_gk_map) h->var_b = flame::kVariantDefault;
-            if (h->var_a_bat == flame::kVariantTma && !h->has_uv_map) h->var_a_bat = flame::kVariantDefault;
-            if (h->var_b_bat == flame::kVariantTmaB && !h->has_gk_map) h->var_b_bat = flame::kVariantDefault;
-            if (h->var_b == flame::kVariantWarpB && !h->has_gk_map) h->var_b = flame::kVariantDefault;
-            if (h->var_b_bat == flame::kVariantWarpB && !h->has_gk_map) h->var_b_bat = flame::kVariantDefault;
             h->fuse = it->second.fuse != 0 && fuse_allowed(h);
             g_tune[key] = TuneChoice{h->var_a, h->var_b, h->fuse ? 1 : 0, h->var_a_bat, h->var_b_bat};
             return FLAME_OK;
@@ -672,43 +661,31 @@ flame_status autotune(flame_ctx *h) {
     };
     // pass A variants are timed with their pass C (the one-line pass A
     // brings the one-line pass C)
-    const int avars[5] = {flame::kVariantDefault, flame::kVariantDirect, flame::kVariantRadix8A, flame::kVariantTma,
-                          flame::kVariantOneLine};
-    const int bvars[5] = {flame::kVariantDefault, flame::kVariantRadix8, flame::kVariantTmaB, flame::kVariantOneLineB,
-                          flame::kVariantWarpB};
-    float best_a = 1e30f, best_b = 1e30f, best_a2 = 1e30f, best_b2 = 1e30f;
+    const int avars[3] = {flame::kVariantDirect, flame::kVariantTma, flame::kVariantOneLine};
+    const int bvars[3] = {flame::kVariantDirectB, flame::kVariantTmaB, flame::kVariantOneLineB};
+    float best_a = 1e30f, best_b = 1e30f;
     for (int v : avars) {
         if (v == flame::kVariantTma && !h->has_uv_map) continue;
-        if (v == flame::kVariantOneLine && h->logn1 > 11) continue;
+        if (v == flame::kVariantOneLine && h->ss.la > 9) continue;
         float ms = 0;
         if (e == cudaSuccess) e = time_it(2, v, &ms);
         if (e == cudaSuccess && ms < best_a) {
             best_a = ms;
             h->var_a = v;
         }
-        if (e == cudaSuccess && v != flame::kVariantOneLine && ms < best_a2) {
-            best_a2 = ms;
-            h->var_a_bat = v;
-        }
     }
+    // the grouped launches write by direct stores, two lines per thread
+    h->var_a_bat = flame::kVariantDirect;
+    h->var_b_bat = flame::kVariantDirectB;
     d.onec = h->var_a == flame::kVariantOneLine;
     for (int v : bvars) {
         if (v == flame::kVariantTmaB && !h->has_gk_map) continue;
-        if (v == flame::kVariantOneLineB && h->logm > 11) continue;
-        if (v == flame::kVariantWarpB && (h->logm != 12 || !h->has_gk_map)) continue;
+        if (v == flame::kVariantOneLineB && h->ss.lb > 9) continue;
         float ms = 0;
         if (e == cudaSuccess) e = time_it(1, v, &ms);
-        // the warp-local variant measures level with variant 2 (within the
-        // timing noise): it is taken only when clearly faster, so that the
-        // choice does not flip from run to run
-        if (v == flame::kVariantWarpB) ms *= 1.02f;
         if (e == cudaSuccess && ms < best_b) {
             best_b = ms;
             h->var_b = v;
-        }
-        if (e == cudaSuccess && v != flame::kVariantOneLineB && ms < best_b2) {
-            best_b2 = ms;
-            h->var_b_bat = v;
         }
     }
     // Fused or separate column passes: each way, 4 steps captured as one CUDA
@@ -899,6 +876,13 @@ flame_status flame_create(const flame_params *params, flame_t *out) {
     a.t0 = p.t0;
     a.dt = p.dt;
     a.flags = p.flags;
+    h->ss = a;
+    h->ss.la = flame::step_exponent(p.K1);
+    h->ss.lb = flame::step_exponent(p.K2) - 1;
+    if (h->ss.lb < flame::kMinA) h->ss.lb = flame::kMinA;
+    h->ss.n1 = 3 << h->ss.la;
+    h->ss.n2 = 6 << h->ss.lb;
+    h->ss.logn1 = h->ss.logm = 0;
 
     auto dev_alloc = [&](void **ptr, size_t bytes) -> bool {
         return cudaMalloc(ptr, bytes) == cudaSuccess;
@@ -909,17 +893,32 @@ flame_status flame_create(const flame_params *params, flame_t *out) {
         return fail(FLAME_ECUDA, "cudaGetDevice: %s", cudaGetErrorString(ge));
     }
     const size_t n1 = p.n_theta, ldk = a.ldk, m1 = p.n_phi / 2 + 1;
-    bool ok = dev_alloc(&h->tw1, flame::tw_alloc_len(h->logn1) * h->csz) &&
-              dev_alloc(&h->twm, flame::tw_alloc_len(h->logm) * h->csz) &&
-              dev_alloc(&h->uv, n1 * ldk * 2 * h->csz) && dev_alloc(&h->gk, n1 * ((ldk + 1) & ~(size_t)1) * h->csz) &&
-              dev_alloc(&h->spec, n1 * m1 * h->csz) && dev_alloc(&h->aw, n1 * ldk * 2 * h->csz) &&
-              dev_alloc((void **)&h->rowsum, n1 * sizeof(double)) && dev_alloc((void **)&h->dscal, 16 * sizeof(double)) &&
-              dev_alloc((void **)&h->status, flame::kStatusWords * sizeof(int));
+    size_t tabs = 0;
+    auto place = [&](size_t bytes) {
+        const size_t at = tabs;
+        tabs += (bytes + 255) & ~(size_t)255;
+        return at;
+    };
+    const size_t o_tw1 = place(flame::tw_alloc_len(h->logn1) * h->csz), o_twm = place(flame::tw_alloc_len(h->logm) * h->csz),
+                 o_tw1s = place(flame::tw3_len_of(h->ss.la) * h->csz), o_twms = place(flame::tw3_len_of(h->ss.lb) * h->csz),
+                 o_rowsum = place(n1 * sizeof(double)), o_dscal = place(24 * sizeof(double)),
+                 o_status = place(flame::kStatusWords * sizeof(int));
+    bool ok = dev_alloc(&h->tabs, tabs) && dev_alloc(&h->uv, n1 * ldk * 2 * h->csz) &&
+              dev_alloc(&h->gk, n1 * ((ldk + 1) & ~(size_t)1) * h->csz) && dev_alloc(&h->spec, n1 * m1 * h->csz) &&
+              dev_alloc(&h->aw, n1 * ldk * 2 * h->csz);
     if (!ok) {
         cudaGetLastError();
         free_ctx(h);
         return fail(FLAME_ENOMEM, "flame_create: device allocation failed");
     }
+    char *tb = static_cast<char *>(h->tabs);
+    h->tw1 = tb + o_tw1;
+    h->twm = tb + o_twm;
+    h->tw1s = tb + o_tw1s;
+    h->twms = tb + o_twms;
+    h->rowsum = reinterpret_cast<double *>(tb + o_rowsum);
+    h->dscal = reinterpret_cast<double *>(tb + o_dscal);
+    h->status = reinterpret_cast<int *>(tb + o_status);
     cudaError_t e = cudaStreamCreateWithFlags(&h->cap, cudaStreamNonBlocking);
     if (e != cudaSuccess) {
         h->cap = nullptr;
@@ -929,16 +928,18 @@ flame_status flame_create(const flame_params *params, flame_t *out) {
     flame_status st = p.prec == FLAME_FP64 ? alloc_tables<double>(h) : alloc_tables<float>(h);
     if (st == FLAME_OK) {
         e = cudaMemsetAsync(h->status, 0, flame::kStatusWords * sizeof(int), h->cap);
-        if (e == cudaSuccess) e = cudaMemsetAsync(h->dscal, 0, 16 * sizeof(double), h->cap);
+        if (e == cudaSuccess) e = cudaMemsetAsync(h->dscal, 0, 24 * sizeof(double), h->cap);
         if (e == cudaSuccess) e = cudaStreamSynchronize(h->cap);
         if (e != cudaSuccess) st = fail(FLAME_ECUDA, "flame_create: %s", cudaGetErrorString(e));
     }
     if (st == FLAME_OK)
         setup_l2_window(h, (2 * (size_t)p.K1 + 1) * ldk * h->csz);
+    if (st == FLAME_OK && p.prec == FLAME_FP32_MIXED && h->ss.la >= 6)
+        h->has_uv_map = flame::encode_uv_map(&h->uv_map, h->uv, h->ss.n1, (int)ldk, flame::uv3_box_pairs(h->ss.n1));
+    if (st == FLAME_OK && p.prec == FLAME_FP32_MIXED && h->ss.lb >= 6)
+        h->has_gk_map = flame::encode_gk_map(&h->gk_map, h->gk, h->ss.n1, (int)ldk);
     if (st == FLAME_OK && p.prec == FLAME_FP32_MIXED && h->logn1 >= 8 && h->logn1 <= 12)
-        h->has_uv_map = flame::encode_uv_map(&h->uv_map, h->uv, (int)n1, (int)ldk);
-    if (st == FLAME_OK && p.prec == FLAME_FP32_MIXED && h->logm >= 8 && h->logm <= 12)
-        h->has_gk_map = flame::encode_gk_map(&h->gk_map, h->gk, (int)n1, (int)ldk);
+        h->has_uv_map_full = flame::encode_uv_map(&h->uv_map_full, h->uv, (int)n1, (int)ldk, flame::uv_box_pairs((int)n1));
     if (st == FLAME_OK) st = autotune(h);
     if (st != FLAME_OK) {
         free_ctx(h);
@@ -1100,12 +1101,12 @@ flame_status flame_step_host(flame_t h, void *host_state, double *host_mean, dou
     double *dm = reinterpret_cast<double *>(dstate + boxb), *dtm = dm + 1;
     char *hstate = static_cast<char *>(host_state);
     const bool f64 = h->p.prec == FLAME_FP64;
-    int colsA = 1, quantA = 1, pairsC = 1;
-    if (f64) Ops<double>::tiles(h->sa, h->var_a, &colsA, &quantA, &pairsC);
-    else Ops<float>::tiles(h->sa, h->var_a, &colsA, &quantA, &pairsC);
-    const int tilesA = (int)((ncol + colsA - 1) / colsA), unitsA = (tilesA + quantA - 1) / quantA;
+    int colsA = 1, pairsC = 1;
+    if (f64) Ops<double>::tiles(h->ss, h->var_a, &colsA, &pairsC);
+    else Ops<float>::tiles(h->ss, h->var_a, &colsA, &pairsC);
+    const int tilesA = (int)((ncol + colsA - 1) / colsA);
     const int tilesC = (int)((((ncol + 1) / 2) + pairsC - 1) / pairsC);
-    const int KA = std::min(kChunks, unitsA), KC = std::min(kChunks, tilesC);
+    const int KA = std::min(kChunks, tilesA), KC = std::min(kChunks, tilesC);
     FlameDesc d = make_desc(h, dstate, dm, dtm);
     auto passA = [&](const FlameDesc &x) {
         return f64 ? Ops<double>::passA(x, s, h->var_a) : Ops<float>::passA(x, s, h->var_a, h->map());
@@ -1121,8 +1122,7 @@ flame_status flame_step_host(flame_t h, void *host_state, double *host_mean, dou
     CUDA_TRY(cudaMemcpyAsync(dtm, host_t, sizeof(double), cudaMemcpyHostToDevice, h->cpy));
     // state in by column chunks, pass A of the first step on each as it lands
     for (int i = 0; i < KA; ++i) {
-        const int u0 = (int)((long)unitsA * i / KA), u1 = (int)((long)unitsA * (i + 1) / KA);
-        const int a0 = u0 * quantA, a1 = std::min(u1 * quantA, tilesA + quantA - 1);
+        const int a0 = (int)((long)tilesA * i / KA), a1 = (int)((long)tilesA * (i + 1) / KA);
         const size_t c0 = (size_t)a0 * colsA, c1 = std::min((size_t)a1 * colsA, ncol);
         if (c1 > c0)
             CUDA_TRY(cudaMemcpyAsync(dstate + c0 * colb, hstate + c0 * colb, (c1 - c0) * colb, cudaMemcpyHostToDevice,
@@ -1237,33 +1237,15 @@ flame_status flame_step_batch(const flame_t *hs, void *const *states, double *co
         class_handle.push_back(first[kv.first]);
         flat.insert(flat.end(), kv.second.begin(), kv.second.end());
     }
-    // Per-flame tensor maps for the tensor-store variants, in the order of
-    // flat; with FLAME_BATCH_TMA=1 a class uses them when every flame of it
-    // has both maps.  Off by default: on the ensemble's grids (256x512 ..
-    // 1024x2048) the grouped direct-store kernels measured faster (1.48e11
-    // against 1.44e11 grid-point updates/s for 256 uneven flames).
-    std::vector<CUtensorMap> maps(2 * flat.size());
-    std::vector<bool> class_maps;
-    const char *bt = getenv("FLAME_BATCH_TMA");
-    const bool batch_tma = bt && strcmp(bt, "1") == 0;
-    {
-        size_t i = 0;
-        for (auto &kv : classes) {
-            bool all = true;
-            for (size_t j = 0; j < kv.second.size(); ++j, ++i) {
-                const flame_ctx *hf = nullptr;
-                for (int q = 0; q < nflames && !hf; ++q)
-                    if (states[q] == flat[i].state) hf = hs[q];
-                all = all && hf && hf->has_uv_map && hf->has_gk_map;
-                if (hf && hf->has_uv_map) maps[i] = hf->uv_map;
-                if (hf && hf->has_gk_map) maps[flat.size() + i] = hf->gk_map;
-            }
-            class_maps.push_back(all && batch_tma);
-        }
+    // classes with a flame that needs the general epilogue of pass C
+    std::vector<bool> class_gen;
+    for (const auto &rg : ranges) {
+        bool gen = false;
+        for (size_t i = rg.first; i < rg.first + rg.second; ++i)
+            gen = gen || flat[i].forcing || flat[i].forcing0 != 0.0 || flat[i].rec;
+        class_gen.push_back(gen);
     }
-    const size_t dbytes = flat.size() * sizeof(FlameDesc);
-    const size_t mofs = (dbytes + 127) & ~(size_t)127;  // maps: 64-byte aligned
-    const size_t bytes = mofs + maps.size() * sizeof(CUtensorMap);
+    const size_t dbytes = flat.size() * sizeof(FlameDesc), bytes = dbytes;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     const bool same = h0->batch_key.size() == flat.size() && memcmp(h0->batch_key.data(), flat.data(), dbytes) == 0;
     if (!same) {
@@ -1304,13 +1286,11 @@ flame_status flame_step_batch(const flame_t *hs, void *const *states, double *co
         if (!h0->batch_up) CUDA_TRY(cudaEventCreateWithFlags(&h0->batch_up, cudaEventDisableTiming));
         char *hb = static_cast<char *>(h0->batch_host);
         memcpy(hb, flat.data(), dbytes);
-        memcpy(hb + mofs, maps.data(), maps.size() * sizeof(CUtensorMap));
         CUDA_TRY(cudaMemcpyAsync(h0->batch_desc, hb, bytes, cudaMemcpyHostToDevice, s));
         CUDA_TRY(cudaEventRecord(h0->batch_up, s));
         h0->batch_key = flat;
     }
     const FlameDesc *dev = static_cast<const FlameDesc *>(h0->batch_desc);
-    const CUtensorMap *dmaps = reinterpret_cast<const CUtensorMap *>(static_cast<char *>(h0->batch_desc) + mofs);
     // FLAME_BATCH_VARIANTS=a,b: the grouped launches use these pass A and B
     // variants (in flame_tuning's numbering) instead of the variants the
     // autotuner chose for a single flame of the class's grid
@@ -1329,16 +1309,15 @@ flame_status flame_step_batch(const flame_t *hs, void *const *states, double *co
         const FlameDesc *d = dev + rg.first;
         const int nf = (int)rg.second;
         const flame_ctx *hc = class_handle[ci];
-        const CUtensorMap *um = class_maps[ci] ? dmaps + rg.first : nullptr;
-        const CUtensorMap *gm = class_maps[ci] ? dmaps + flat.size() + rg.first : nullptr;
         const int va = force_a >= 0 ? force_a : hc->var_a_bat, vb = force_b >= 0 ? force_b : hc->var_b_bat;
+        const bool onec = va == flame::kVariantOneLine, gen = class_gen[ci];
         if (h0->p.prec == FLAME_FP64)
             return pass == 0 ? Ops<double>::passA_batch(d, nf, a, q, va)
                  : pass == 1 ? Ops<double>::passB_batch(d, nf, a, q, vb)
-                             : Ops<double>::passC_batch(d, nf, a, q);
-        return pass == 0 ? Ops<float>::passA_batch(d, nf, a, q, va, um)
-             : pass == 1 ? Ops<float>::passB_batch(d, nf, a, q, vb, gm)
-                         : Ops<float>::passC_batch(d, nf, a, q, va == flame::kVariantOneLine);
+                             : Ops<double>::passC_batch(d, nf, a, q, onec, gen);
+        return pass == 0 ? Ops<float>::passA_batch(d, nf, a, q, va)
+             : pass == 1 ? Ops<float>::passB_batch(d, nf, a, q, vb)
+                         : Ops<float>::passC_batch(d, nf, a, q, onec, gen);
     };
     // n steps of every flame.  In one stream: per step and pass, one grouped
     // launch per size class.  With FLAME_BATCH_STREAMS=1 the capture forks

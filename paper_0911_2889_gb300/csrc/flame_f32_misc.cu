@@ -10,7 +10,6 @@ template cudaError_t Ops<float>::cols(const float2 *, float2 *, int, int, int, i
 template cudaError_t Ops<float>::box_from_spec(const float2 *, float2 *, double *, int, int, int, int, cudaStream_t, int *);
 template Geom Ops<float>::geom_cols(int, int, int);
 template Geom Ops<float>::geom_rows(int, int, int);
-template void Ops<float>::tiles(const StepArgs &, int, int *, int *, int *);
 
 #ifdef FLAME_DEBUG_BOUNDS
 static __global__ void k_bounds_probe(int *status, int i, int n) {

@@ -22,7 +22,7 @@ constexpr int kStatusWords = 4;
 // flame_sync_status with the failing index).
 enum BoundsSite : int {
     kSiteAState = 1,    // pass A: state column entry
-    kSiteAUv = 2,       // pass A: (U, V) store (direct and cluster write-outs)
+    kSiteAUv = 2,       // pass A: row spectra store
     kSiteATma = 3,      // pass A: tensor-store coordinates (column, row pair)
     kSiteBUv = 4,       // pass B: row-pair (U, V) load
     kSiteBGk = 5,       // pass B: G store (direct write-out)
@@ -59,21 +59,24 @@ constexpr int kStageHeun2 = 2;
 constexpr int kStageIF1 = 3;
 constexpr int kStageIF2 = 4;
 
-// Kernel variants chosen by the autotuner (0 = default shape).
-constexpr int kVariantDefault = 0;
-constexpr int kVariantDirect = 1;   // pass A: direct stores (no cluster write-out)
-constexpr int kVariantRadix8 = 1;   // pass B: 8 points per thread, 512-thread CTAs
-constexpr int kVariantRadix8A = 2;  // pass A: 8 points per thread, cluster write-out
-constexpr int kVariantTma = 3;      // pass A: column written by tensor stores (FP32)
-constexpr int kVariantTmaB = 2;     // pass B: row pair written by tensor stores (FP32)
-constexpr int kVariantOneLine = 4;  // pass A (and with it pass C): one line per thread group (FP32, 2^8..2^11)
-constexpr int kVariantOneLineB = 3; // pass B: one line per thread group (FP32, 2^8..2^11)
-constexpr int kVariantWarpB = 4;    // pass B: 4096-point rows with warp-local exchanges, tensor-store write-out (FP32)
+// Kernel variants of the step's passes, chosen by the autotuner for FP32
+// lines of 192 points and more (two lines per thread unless said otherwise).
+// The numbers are flame_tuning's; the others of 0 .. 4 are accepted where a
+// saved or forced choice holds them and run the direct-store kernels (pass A
+// 0, 2; pass B 1) or the tensor-store one (pass B 4).
+constexpr int kVariantDirect = 1;   // pass A: direct stores
+constexpr int kVariantTma = 3;      // pass A: column written by tensor stores
+constexpr int kVariantOneLine = 4;  // pass A (and with it pass C): one line per thread (N1 <= 2048)
+constexpr int kVariantDirectB = 0;  // pass B: direct stores
+constexpr int kVariantTmaB = 2;     // pass B: row pair written by tensor stores
+constexpr int kVariantOneLineB = 3; // pass B: one line per thread (N2 <= 4096)
+constexpr int kVariantTmaB4 = 4;    // pass B: as kVariantTmaB
 
 // Plain-old-data arguments of the step kernels.
 struct StepArgs {
     int n1, n2;        // grid
-    int logn1, logm;   // log2 N1, log2 (N2/2)
+    int logn1, logm;   // log2 N1, log2 (N2/2) (public grid)
+    int la, lb;        // N1 = 3 * 2^la, N2/2 = 3 * 2^lb (the step's alias-free grid)
     int K1, K2;        // retained harmonics
     int ldk;           // row length of the compact box and workspaces (K2+1)
     double s1, s2;     // kappa = (s1 k1, s2 k2)
@@ -94,15 +97,15 @@ struct L2Window {
 struct FlameDesc {
     StepArgs a;
     void *state;            // compact box (in place)
-    void *uv;               // N1 x ldk x (U, V) workspace
+    void *uv;               // N1 x ldk pairs: the row spectra at +-k2 (public grid: (U, V))
     void *gk;               // N1 x ldk workspace
     const void *tw1;        // twiddles of length N1
     const void *twm;        // twiddles of length N2/2 (+ real table)
     const double *t_in;     // caller's t (read by pass B)
-    // the step's coefficients, derived from t once by pass B (block 0) and
-    // read by pass C: [0] t_n, [1] c = 1/(2 r0^2), then from byte 16 the
-    // kernel-precision CoefR (1/r0^2, gamma/(2 r0), c/(N1 N2), dt); 48 bytes,
-    // 16-byte aligned (handle scratch)
+    // the step's coefficients, derived from t once by pass B and read by pass
+    // C: [0] t_n, [1] c = 1/(2 r0^2), then from byte 16 the kernel-precision
+    // CoefR (1/r0^2, gamma/(2 r0), c/(N1 N2), dt, ia, ib), [8] n,
+    // [9] 1/(N1 N2); 80 bytes, 16-byte aligned (handle scratch)
     double *coef;
     double *mean;           // caller's mean mode
     double *t_out;          // caller's t (written by pass C)
@@ -124,9 +127,10 @@ struct FlameDesc {
     // right-hand side), and a NaN area slot; written by the first stage
     double *rec;
     int rec_cap;
-    // area in the record: 0 = none (NaN), 1 = summed by pass C from the
-    // per-row-pair sums arow[N1/2] that the area variant of pass B writes,
-    // 2 = the scalar *aval computed by the separate area kernels
+    // area in the record of a step on the public grid: 0 = none (NaN), 1 =
+    // summed by pass C from the per-row-pair sums arow[N1/2] of passB_area, 2
+    // = the scalar *aval computed by the separate area kernels (which a step
+    // on the alias-free grid records too)
     int rec_area;
     double *arow;
     const double *aval;
@@ -186,36 +190,30 @@ template <class R> struct Ops {
     // retained modes of an r2c spectrum -> compact box + FP64 mean
     static cudaError_t box_from_spec(const C *spec, C *state, double *mean, int n1, int n2, int K1, int K2,
                                      cudaStream_t s, int *status = nullptr);
-    // One step pass for one flame (desc by value) or for nflames flames of
-    // the same grid (descs: device array of nflames entries, shape from a).
-    // variant: kVariantDefault, or a tuned alternative (pass A: kVariantDirect
-    // = no cluster write-out, kVariantTma = tensor-store write-out through
-    // uv_map, a map of d.uv made by encode_uv_map; pass B: kVariantRadix8 = 8
-    // points per thread)
-    static cudaError_t passA(const FlameDesc &d, cudaStream_t s, int variant = 0,
-                             const CUtensorMap *uv_map = nullptr);
-    static cudaError_t passB(const FlameDesc &d, cudaStream_t s, int variant = 0,
-                             const CUtensorMap *gk_map = nullptr);
+    // One step pass on the alias-free grid for one flame (desc by value) or
+    // for n flames of the same grid (descs: device array, shape from a).
+    // variant: kVariant*; the maps (encode_uv_map, encode_gk_map of d.uv, d.gk)
+    // are needed by the tensor-store variants only.
+    static cudaError_t init_twiddles3(C *tab, int a, cudaStream_t s);
+    static cudaError_t passA(const FlameDesc &d, cudaStream_t s, int variant = 0, const CUtensorMap *uv_map = nullptr);
+    static cudaError_t passB(const FlameDesc &d, cudaStream_t s, int variant = 0, const CUtensorMap *gk_map = nullptr);
     static cudaError_t passC(const FlameDesc &d, cudaStream_t s);
-    // Pass B that also sums the surface area of its rows (area variant,
-    // arow[pair]); cudaErrorNotSupported when its shared memory exceeds the
-    // device's limit.
-    static cudaError_t passB_area(const FlameDesc &d, cudaStream_t s);
-    // Pass C of one step fused with pass A of the next (FP32, 256 <= N1 <=
-    // 4096, uv written through uv_map); cudaErrorNotSupported otherwise.
+    // Pass C of one step fused with pass A of the next (FP32, columns of 192
+    // points and more, uv written through uv_map); cudaErrorNotSupported otherwise.
     static cudaError_t passCA(const FlameDesc &d, cudaStream_t s, const CUtensorMap *uv_map);
-    // maps (nullable): per-flame tensor maps in device memory (uv maps for
-    // pass A, gk maps for pass B) for the tensor-store variants
-    static cudaError_t passA_batch(const FlameDesc *descs, int nflames, const StepArgs &a, cudaStream_t s,
-                                   int variant = 0, const CUtensorMap *maps = nullptr);
-    static cudaError_t passB_batch(const FlameDesc *descs, int nflames, const StepArgs &a, cudaStream_t s,
-                                   int variant = 0, const CUtensorMap *maps = nullptr);
-    static cudaError_t passC_batch(const FlameDesc *descs, int nflames, const StepArgs &a, cudaStream_t s,
-                                   bool one_line = false);
-    // Tiles (CTAs) of passes A and C: columns per pass-A tile, the tile
-    // multiple a partial pass-A launch must use (clusters), column pairs per
-    // pass-C tile
-    static void tiles(const StepArgs &a, int variant, int *colsA, int *quantA, int *pairsC);
+    static cudaError_t passA_batch(const FlameDesc *descs, int n, const StepArgs &a, cudaStream_t s, int variant);
+    static cudaError_t passB_batch(const FlameDesc *descs, int n, const StepArgs &a, cudaStream_t s, int variant);
+    // gen: some flame needs the general epilogue (forcing, record)
+    static cudaError_t passC_batch(const FlameDesc *descs, int n, const StepArgs &a, cudaStream_t s, bool one_line, bool gen);
+    // Columns per tile of pass A, column pairs per tile of pass C (tiles = CTAs)
+    static void tiles(const StepArgs &a, int variant, int *colsA, int *pairsC);
+    // A step on the public grid that also sums the surface area of its rows
+    // (arow[pair]); passB_area: cudaErrorNotSupported when its shared memory
+    // exceeds the device's limit.  pairs: two lines per thread whatever the
+    // column length (the adjoint step).
+    static cudaError_t passA_full(const FlameDesc &d, cudaStream_t s, bool pairs, const CUtensorMap *uv_map);
+    static cudaError_t passB_area(const FlameDesc &d, cudaStream_t s);
+    static cudaError_t passC_full(const FlameDesc &d, cudaStream_t s);
     // geometry used by the step passes (for the autotuner and the tests)
     static Geom geom_cols(int logn, int nlines, int groups_hint);
     static Geom geom_rows(int logm, int nlines, int groups_hint);
@@ -226,17 +224,19 @@ template <class R> struct Ops {
     static cudaError_t adj_step(const AdjDesc &d, cudaStream_t s);
 };
 
-// Row pairs per tensor store of the uv write-out of pass A (<= 256).
+// Row pairs per tensor store of the uv write-out of pass A (<= 256): on the
+// public grid, and on the alias-free one (n1 = 3 * 2^a; a divisor of n1 / 2).
 __host__ __device__ constexpr int uv_box_pairs(int n1) { return n1 / 2 < 256 ? n1 / 2 : 256; }
+__host__ __device__ constexpr int uv3_box_pairs(int n1) { return n1 / 2 <= 256 ? n1 / 2 : 192; }
 
 // Column pairs per tensor store of the gk write-out of pass B (<= 256).
 __host__ __device__ constexpr int gk_box_pairs(int ldk) { return (ldk + 1) / 2 < 256 ? (ldk + 1) / 2 : 256; }
 
 // Tensor map of an FP32 uv workspace (n1 rows, ldk columns) for the
 // tensor-store write-out of pass A: dimensions (8 floats of a row pair, k2,
-// row pair), box (8, 1, uv_box_pairs(n1)).  False when the CUDA driver has no
+// row pair), box (8, 1, box_pairs).  False when the CUDA driver has no
 // tensor-map encoder or rejects the map (the variant is then not offered).
-bool encode_uv_map(CUtensorMap *map, void *uv, int n1, int ldk);
+bool encode_uv_map(CUtensorMap *map, void *uv, int n1, int ldk, int box_pairs);
 // Tensor map of an FP32 gk workspace (n1 rows, ldk columns, the column count
 // rounded up to even) for the tensor-store write-out of pass B: dimensions
 // (8 floats of a row pair and column pair, row pair, column pair), box

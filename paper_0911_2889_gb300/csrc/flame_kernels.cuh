@@ -17,7 +17,6 @@
 // transform goes through shared memory.
 #pragma once
 
-#include <cooperative_groups.h>
 #include <cuda.h>  // CUtensorMap
 
 #include "fft_engine.cuh"
@@ -173,7 +172,10 @@ __global__ void k_box_from_spec(const CplxT<R> *__restrict__ spec, CplxT<R> *__r
 // ----------------------------------------------------------------------------
 // Twiddle table generation (FP64 sincospi, rounded once)
 // ----------------------------------------------------------------------------
-template <class R> __global__ void k_twiddles(CplxT<R> *tab, int logN, int LE) {
+// grid.y = 3: the radix-16, radix-8 and radix-4 tables (tw_alloc_len entries in all)
+template <class R> __global__ void k_twiddles(CplxT<R> *tab, int logN) {
+    const int LE = 4 - blockIdx.y;
+    for (int l = 4; l > LE; --l) tab += tw_table_len(logN, l);
     const int N = 1 << logN, E = 1 << LE;
     const int len = tw_table_len(logN, LE);
     const int fin = tw_final_offset(logN, LE);
@@ -376,29 +378,10 @@ __device__ __forceinline__ void tma_store_3d(const CUtensorMap *tm, const void *
                  "r"(sa), "r"(x), "r"(y), "r"(z)
                  : "memory");
 }
-// A tensor map read from global memory (one per flame of an ensemble) is
-// made visible to the tensor-map proxy before its first use.
-__device__ __forceinline__ void tensormap_acquire(const CUtensorMap *tm) {
-    asm volatile("fence.proxy.tensormap::generic.acquire.gpu [%0], 128;" ::"l"(reinterpret_cast<unsigned long long>(tm))
-                 : "memory");
-}
 __device__ __forceinline__ void bulk_commit_and_wait_read() {
     asm volatile("cp.async.bulk.commit_group;" ::: "memory");
     asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
 }
-
-// Compile-time CTA shape of the FP32 step kernels (LOG > 0): G line groups of
-// T = 2^LOG / 16 threads, and, for pass A, clusters of CL CTAs (CL G = 8
-// columns) that write their transposed output cooperatively through
-// distributed shared memory, one 128-byte line per row.
-template <int LOG> struct Shape {
-    static constexpr int T = (1 << LOG) >> 4;
-    static constexpr int G = T >= 256 ? 1 : 256 / T;
-    static constexpr int CL = (LOG > 0 && G <= 8) ? 8 / G : 1;
-};
-template <> struct Shape<0> {
-    static constexpr int T = 0, G = 0, CL = 1;
-};
 
 // E points per thread: 16 (runtime-length kernels, FP64) or 8 (compile-time
 // FP32 kernels: 512-thread CTAs at 64 registers, two CTAs per SM).
@@ -475,19 +458,6 @@ template <class C> struct RealTw {
     }
 };
 
-// CTA shape of the compile-time kernels with E points per thread: G line
-// groups of T = 2^LOG / E threads (256 threads for E = 16, 512 for E = 8) and
-// clusters of CL CTAs holding 8 line groups (pass A's write-out).
-template <int LOG, int E> struct ShapeE {
-    static constexpr int T = (1 << LOG) / E;
-    static constexpr int THREADS = E == 16 ? 256 : 512;
-    static constexpr int G = T >= THREADS ? 1 : THREADS / T;
-    static constexpr int CL = (G <= 8) ? 8 / G : 1;
-};
-template <int E> struct ShapeE<0, E> {  // runtime-length kernels: no clusters
-    static constexpr int T = 0, THREADS = 256, G = 0, CL = 1;
-};
-
 // Memory layouts (the state's is also documented in include/flame.h):
 //   state  column-major compact box: element (k1, k2) at k2 * ld1 + (k1 + K1),
 //          ld1 = 2 K1 + 1
@@ -505,13 +475,14 @@ template <int E> struct ShapeE<0, E> {  // runtime-length kernels: no clusters
 // r = 4..11 of the first pass are always zero and are dropped at compile
 // time).  Writes uv[j1][k2] = (U, V) with U = synthesis of a, V = i s2 k2 x
 // synthesis of b.
-template <class R, int LOG, int E, bool CLU = true, bool TMA = false, bool GMAP = false>
+template <class R, int LOG, bool TMA = false>
 __device__ __forceinline__ void passA_body(const FlameDesc &d, int tile, int ntiles, int pf,
                                            const CUtensorMap *tm = nullptr) {
     griddep_wait();
     griddep_launch();
     using V = typename VecOf<R>::type;
     using C = CplxT<R>;
+    constexpr int E = 16;
     extern __shared__ __align__(16) unsigned char smraw[];
     const StepArgs &a = d.a;
     const C *__restrict__ state = static_cast<const C *>(d.state);
@@ -528,9 +499,6 @@ __device__ __forceinline__ void passA_body(const FlameDesc &d, int tile, int nti
     const bool valid = k2 <= a.K2;
     V *base = reinterpret_cast<V *>(smraw) + (size_t)g * 2 * plane_len_e<E>(N1);
     auto sm = make_planes_e<E>(base, N1);
-    constexpr bool STW = false;  // pass A's twiddles stay in L1 (measured faster)
-    C *stw = reinterpret_cast<C *>(reinterpret_cast<V *>(smraw) + (size_t)G * 2 * plane_len_e<E>(N1));
-    if constexpr (STW) TwShared<C>::template fill<(STW ? LOG : 8)>(stw, tw1);  // synced by the transform
     const R s1 = scale1<R>(a), s2k2 = scale2<R>(a) * (R)k2;
     const C *col = state + (size_t)k2 * ld1 + a.K1;  // col[k1], k1 = -K1..K1
     // band rows: r < E/4 (k1 = n <= K1) and r >= 3E/4 (k1 = n - N1 >= -K1);
@@ -552,52 +520,8 @@ __device__ __forceinline__ void passA_body(const FlameDesc &d, int tile, int nti
             }
         }
     }
-    if constexpr (STW) {
-        __syncthreads();
-        fft_line_s<1, (STW ? LOG : 8)>(x, t, sm, tw1, stw);
-    } else {
-        fft_line_e<1, LOG, E>(x, a.logn1, t, sm, tw1);
-    }
-    constexpr int CL = CLU ? ShapeE<LOG, E>::CL : 1;
-    if constexpr (CL > 1 && std::is_same<R, float>::value) {
-        // Park (U, V) of this column at its natural row index, then the CL
-        // CTAs of the cluster (CL G adjacent columns) write rows: CTA q takes
-        // rows [q N1/CL, (q+1) N1/CL), consecutive threads consecutive columns
-        // of one row (CL G x 16 bytes = 128 contiguous bytes per row).
-        namespace cg = cooperative_groups;
-        cg::cluster_group cluster = cg::this_cluster();
-        constexpr int GG = ShapeE<LOG, E>::G, NC = CL * GG, NN = 1 << LOG, ROWS = NN / CL;
-        constexpr int NT = ShapeE<LOG, E>::THREADS;
-        float4 *park = reinterpret_cast<float4 *>(base);
-        __syncthreads();
-#pragma unroll
-        for (int r = 0; r < E; ++r) {
-            const int n = t + r * T;
-            C U = lane0<R>(x[r]);
-            C Vb = lane1<R>(x[r]);
-            park[spad(n)] = make_float4(U.x, U.y, -s2k2 * Vb.y, s2k2 * Vb.x);
-        }
-        cluster.sync();
-        const int q = (int)cluster.block_rank();
-        const int col0 = (tile / CL) * NC;
-        static_assert((ROWS * NC) % NT == 0, "threads per CTA");
-        // element e: row parity e % 2, column (e / 2) % NC, row pair e / (2 NC);
-        // consecutive threads cover one row pair's NC columns x 2 rows
-        // (NC x 32 contiguous bytes of the interleaved uv)
-#pragma unroll
-        for (int i = 0; i < ROWS * NC / NT; ++i) {
-            const int e = (int)threadIdx.x + NT * i;
-            const int c = (e >> 1) % NC, n = q * ROWS + 2 * (e / (2 * NC)) + (e & 1);
-            const int kc = col0 + c;
-            const float4 *rb = cluster.map_shared_rank(
-                reinterpret_cast<const float4 *>(reinterpret_cast<V *>(smraw) + (size_t)(c % GG) * 2 * plane_len_e<E>(NN)),
-                c / GG);
-            const float4 v = rb[spad(n)];
-            if (kc <= a.K2 && FLAME_IN(d.status, uv_index(n, kc, a.ldk) + 1, uv_len(a), kSiteAUv))
-                *reinterpret_cast<float4 *>(uv + uv_index(n, kc, a.ldk)) = v;
-        }
-        cluster.sync();
-    } else if constexpr (TMA && std::is_same<R, float>::value && LOG > 0) {
+    fft_line<1, LOG>(x, a.logn1, t, sm, tw1);
+    if constexpr (TMA && std::is_same<R, float>::value && LOG > 0) {
         // Park (U, V) of this column at row n (16 bytes per row: the order of
         // a column of the interleaved uv, row pair by row pair), then the
         // first thread of the group writes the column with tensor stores of
@@ -628,7 +552,6 @@ __device__ __forceinline__ void passA_body(const FlameDesc &d, int tile, int nti
         }
         if (aligned && t == 0 && valid) {
             constexpr int BP = uv_box_pairs(1 << LOG);
-            if constexpr (GMAP) tensormap_acquire(tm);
 #pragma unroll 1
             for (int p0 = 0; p0 < (N1 >> 1); p0 += BP)
                 if (FLAME_IN(d.status, k2, a.ldk, kSiteATma) && FLAME_IN(d.status, p0, a.n1 >> 1, kSiteATma))
@@ -654,7 +577,7 @@ __device__ __forceinline__ void passA_body(const FlameDesc &d, int tile, int nti
 //   ia = 1/t_n - 1/t_{n+1} = d/(t_n t_{n+1}),  ib = (gamma/2) ln(1 + d/t_n),
 // with d = t_{n+1} - t_n (exact in FP64), written without cancellation.
 struct Coef {
-    double tn, a, b, c;  // a = 1/r0^2, b = gamma/(2 r0), c = 1/(2 r0^2)
+    double n, tn, a, b, c;  // step index n; a = 1/r0^2, b = gamma/(2 r0), c = 1/(2 r0^2)
     double ia, ib;       // integrating-factor exponent coefficients
 };
 // (ia, ib are derived only for the integrating-factor stage: the FP64 log
@@ -663,6 +586,7 @@ __device__ __forceinline__ Coef step_coef(const StepArgs &s, double t, bool if_s
     long n = __double2ll_rn((t - s.t0) / s.dt);
     double tn = s.t0 + (double)n * s.dt;
     Coef k;
+    k.n = (double)n;
     k.tn = tn;
     k.a = 1.0 / (tn * tn);
     k.b = s.gamma / (2.0 * tn);
@@ -690,14 +614,17 @@ template <class R> __device__ __forceinline__ CoefR<R> coef_r(const Coef &cf, co
     const double inv = 1.0 / ((double)s.n1 * (double)s.n2);
     return CoefR<R>{(R)cf.a, (R)cf.b, (R)(cf.c * inv), (R)s.dt, (R)cf.ia, (R)cf.ib};
 }
-// Layout of FlameDesc::coef: t_n, c, then CoefR<R> from byte 16 (64 bytes
-// in all for FP64).
+// Layout of FlameDesc::coef: t_n, c, then CoefR<R> from byte 16 (48 bytes for
+// FP64), then the step index n and 1 / (N1 N2) (what the mean mode's update
+// needs, so that it divides nothing).
 template <class R> __device__ __forceinline__ void store_coef(double *coef, const StepArgs &s, double t,
                                                               bool if_stage) {
     const Coef cf = step_coef(s, t, if_stage);
     coef[0] = cf.tn;
     coef[1] = cf.c;
     *reinterpret_cast<CoefR<R> *>(coef + 2) = coef_r<R>(cf, s);
+    coef[8] = cf.n;
+    coef[9] = 1.0 / ((double)s.n1 * (double)s.n2);
 }
 template <class R> __device__ __forceinline__ CoefR<R> load_coef(const double *coef) {
     return *reinterpret_cast<const CoefR<R> *>(coef + 2);
@@ -729,9 +656,8 @@ template <class F> __device__ __forceinline__ F group_sum(F v, int T, F *scratch
     return s;
 }
 
-template <class R, int LOG, int E, bool TMA = false, bool GMAP = false, bool AREA = false, bool WL = false>
-__device__ __forceinline__ void passB_body(const FlameDesc &d, int tile, int ntiles, int pf,
-                                           const CUtensorMap *tm = nullptr) {
+template <class R, int LOG, int E>
+__device__ __forceinline__ void passB_area_body(const FlameDesc &d, int tile) {
     griddep_wait();
     griddep_launch();
     using V = typename VecOf<R>::type;
@@ -743,21 +669,15 @@ __device__ __forceinline__ void passB_body(const FlameDesc &d, int tile, int nti
     const C *__restrict__ twm = static_cast<const C *>(d.twm);
     const int M = LOG > 0 ? (1 << LOG) : (1 << a.logm), T = M / E;
     const int g = threadIdx.x / T, t = threadIdx.x % T, G = blockDim.x / T;
-    if (threadIdx.x == 0 && pf > 0 && tile + pf < ntiles) {
-        const int p0 = (tile + pf) * G, np = min(G, (a.n1 >> 1) - p0);
-        if (np > 0) l2_prefetch(uv + 2 * (size_t)(2 * p0) * a.ldk, (size_t)np * 2 * a.ldk * 2 * sizeof(C));
-    }
     const int pair = tile * G + g;
     const bool valid = pair < (a.n1 >> 1);
     // per group: the exchange buffer, then M entries of C (sizeof(C) ==
-    // sizeof(V) in both precisions); the area variant adds the synthesis of
-    // Phi on the two rows (M two-line points) and its own staging of row 2p
-    // (M/2 (U, V) entries)
-    const int gstride = 2 * plane_len_e<E>(M) + M + (AREA ? 3 * M : 0);
+    // sizeof(V) in both precisions), the synthesis of Phi on the two rows (M
+    // two-line points) and the staging of row 2p (M/2 (U, V) entries)
+    const int gstride = 2 * plane_len_e<E>(M) + 4 * M;
     V *base = reinterpret_cast<V *>(smraw) + (size_t)g * gstride;
     auto sm = make_planes_e<E>(base, M);  // (E = 8 pads one slot every 8: st_raw/ld_raw)
     const C *P = twm + tw_real_offset(a.logm);  // exp(+2 pi i k/N2), k < M
-    if (tile == 0 && threadIdx.x == 0) store_coef<R>(d.coef, a, *d.t_in, d.stage == kStageIF1);
     constexpr bool STW = kSharedTw<R, LOG, E>;
     constexpr int LS = STW ? LOG : 8;
     C *stw = reinterpret_cast<C *>(reinterpret_cast<V *>(smraw) + (size_t)G * gstride);
@@ -771,15 +691,9 @@ __device__ __forceinline__ void passB_body(const FlameDesc &d, int tile, int nti
         if constexpr (STW) return Pt(k);
         else return __ldg(P + k);
     };
-    // WL: 4096-point rows with the warp-local exchanges of line_fft4096_wl;
-    // the inverse transforms take natural order and leave the points in
-    // digit-swapped order, which the pointwise |z|^2 and the forward
-    // transform (digit-swapped in, natural out) take as they are
-    static_assert(!WL || (STW && LOG == 12 && !AREA), "warp-local exchanges: FP32 4096-point rows");
     auto fft = [&](auto dirc, CV<V>(&x)[E]) {
         constexpr int DIR = decltype(dirc)::value;
-        if constexpr (WL) line_fft4096_wl<DIR, (DIR > 0)>(x, t, sm, TwShared<C>{stw, stw + 240});
-        else if constexpr (STW) fft_line_s<DIR, LS>(x, t, sm, twm, stw);
+        if constexpr (STW) fft_line_s<DIR, LS>(x, t, sm, twm, stw);
         else fft_line_e<DIR, LOG, E>(x, a.logm, t, sm, twm);
     };
 
@@ -794,10 +708,8 @@ __device__ __forceinline__ void passB_body(const FlameDesc &d, int tile, int nti
     // (M entries per group) while row 2p+1 is transformed; row 2p+1's stays
     // in registers.
     C *h_first = reinterpret_cast<C *>(base + 2 * plane_len_e<E>(M));
-    CV<V> *phi_park = reinterpret_cast<CV<V> *>(base + 2 * plane_len_e<E>(M) + M);  // area variant
-    UV<R> *stage0 = AREA ? reinterpret_cast<UV<R> *>(base + 2 * plane_len_e<E>(M) + 3 * M)
-                         : reinterpret_cast<UV<R> *>(base),
-          *stage1 = reinterpret_cast<UV<R> *>(h_first);
+    CV<V> *phi_park = reinterpret_cast<CV<V> *>(base + 2 * plane_len_e<E>(M) + M);
+    UV<R> *stage0 = reinterpret_cast<UV<R> *>(base + 2 * plane_len_e<E>(M) + 3 * M), *stage1 = reinterpret_cast<UV<R> *>(h_first);
     const int half = M >> 1;
     UV<R> e0[E / 2];
     {
@@ -847,7 +759,7 @@ __device__ __forceinline__ void passB_body(const FlameDesc &d, int tile, int nti
         });
     };
     CV<V> x[E];
-    // Area variant: Phi on rows 2p, 2p+1 (without the mean mode), as the
+    // Phi on rows 2p, 2p+1 (without the mean mode), as the
     // inverse row transform of S[k] = P_2p[k] + i P_2p+1[k], P the column
     // synthesis of Phi: for k2 >= 1, P = V / (i s2 k2) (pass A wrote V =
     // i s2 k2 P); for k2 = 0, P(j1) = 2 Re sum_{k1 = 1..K1} Phi_{k1,0}
@@ -855,7 +767,7 @@ __device__ __forceinline__ void passB_body(const FlameDesc &d, int tile, int nti
     __shared__ R ared[32];
     R apart = 0;  // this thread's share of the rows' area sums
     R rr = 0;     // r0 + Phi_0
-    if constexpr (AREA) {
+    {
         rr = (R)(*d.t_in + *d.mean);
         const C *st0 = static_cast<const C *>(d.state) + a.K1;  // column k2 = 0, index k1
         const C *t1r = static_cast<const C *>(d.tw1) + tw_real_offset(a.logn1);  // exp(2 pi i k / 2 N1), k < N1
@@ -901,14 +813,12 @@ __device__ __forceinline__ void passB_body(const FlameDesc &d, int tile, int nti
     // one row (q = 0, 1 the lanes), phi from the parked synthesis (re: row 2p,
     // im: row 2p+1)
     auto area_terms = [&](const V(&gv)[E], bool second) {
-        if constexpr (AREA) {
 #pragma unroll
-            for (int r = 0; r < E; ++r) {
-                const CV<V> ph = phi_park[t + r * T];
-                const V pv = second ? ph.im : ph.re;
-                const R R0 = rr + pv.x, R1 = rr + pv.y;
-                apart += R0 * sqrt_r(fma_rn(R0, R0, gv[r].x)) + R1 * sqrt_r(fma_rn(R1, R1, gv[r].y));
-            }
+        for (int r = 0; r < E; ++r) {
+            const CV<V> ph = phi_park[t + r * T];
+            const V pv = second ? ph.im : ph.re;
+            const R R0 = rr + pv.x, R1 = rr + pv.y;
+            apart += R0 * sqrt_r(fma_rn(R0, R0, gv[r].x)) + R1 * sqrt_r(fma_rn(R1, R1, gv[r].y));
         }
     };
     build(std::true_type{}, stage0, x);
@@ -922,7 +832,7 @@ __device__ __forceinline__ void passB_body(const FlameDesc &d, int tile, int nti
 #pragma unroll
     for (int r = 0; r < E; ++r) h_first[t + r * T] = C{sq0[r].x, sq0[r].y};
     fft(std::integral_constant<int, 1>{}, x);
-    if constexpr (AREA) {
+    {
         V sq1[E];
 #pragma unroll
         for (int r = 0; r < E; ++r) sq1[r] = vfma(x[r].re, x[r].re, vmul(x[r].im, x[r].im));
@@ -944,14 +854,6 @@ __device__ __forceinline__ void passB_body(const FlameDesc &d, int tile, int nti
     for (int r = E / 2; r < E; ++r) sm.st_raw(spad_e<E>(t + r * T), x[r]);
     if (t == 0) sm.st_raw(0, x[0]);
     __syncthreads();
-    // Tensor-store write-out (FP32, compile-time lengths): G of the row pair
-    // is staged in the h region (free again: the forward transform has read
-    // it) in the order of the column-pair interleaved gk, complex index
-    // 4 (k/2) + k%2 for row 2p and + 2 for row 2p+1, and the first thread of
-    // the group writes it with tensor stores of gk_box_pairs(ldk) column
-    // pairs.  Other cases store directly.
-    constexpr bool kTma = TMA && std::is_same<R, float>::value && LOG > 0;
-    const bool staged = kTma && (__cvta_generic_to_shared(smraw) & 127) == 0;
     static_for<0, E / 2>([&](auto rc) {
         constexpr int r = decltype(rc)::value;
         const int k = t + r * T;
@@ -962,29 +864,13 @@ __device__ __forceinline__ void passB_body(const FlameDesc &d, int tile, int nti
             CV<V> Ev{vmul(vadd(h.re, hc.re), vbc(hf)), vmul(vsub(h.im, hc.im), vbc(hf))};
             CV<V> Ov{vmul(vadd(h.im, hc.im), vbc(hf)), vmul(vsub(hc.re, h.re), vbc(hf))};
             CV<V> Y = cadd(Ev, cmul_s(Ov, w.x, -w.y));
-            C *dst = staged ? h_first + 4 * (k >> 1) + (k & 1)
-                            : gk + gk_index(2 * pair, k, a.n1);  // row 2p+1 two slots further
-            if (staged || FLAME_IN(d.status, gk_index(2 * pair, k, a.n1) + 2, gk_len(a), kSiteBGk)) {
+            C *dst = gk + gk_index(2 * pair, k, a.n1);  // row 2p+1 two slots further
+            if (FLAME_IN(d.status, gk_index(2 * pair, k, a.n1) + 2, gk_len(a), kSiteBGk)) {
                 dst[0] = lane0<R>(Y);
                 dst[2] = lane1<R>(Y);
             }
         }
     });
-    if constexpr (kTma) {
-        if (staged) {
-            fence_async_smem();
-            __syncthreads();
-            if (t == 0 && valid) {
-                const int nq = (a.ldk + 1) >> 1, BQ = gk_box_pairs(a.ldk);
-                if constexpr (GMAP) tensormap_acquire(tm);
-#pragma unroll 1
-                for (int q0 = 0; q0 < nq; q0 += BQ)
-                    if (FLAME_IN(d.status, pair, a.n1 >> 1, kSiteBTma) && FLAME_IN(d.status, q0, (gk_len(a) / a.n1) >> 1, kSiteBTma))
-                        tma_store_3d(tm, h_first + 4 * q0, 0, pair, q0);
-                bulk_commit_and_wait_read();
-            }
-        }
-    }
 }
 
 // Explicitly rounded scalar arithmetic: the update of pass C is compiled in
@@ -1085,88 +971,104 @@ __device__ __forceinline__ void update_entry(const FlameDesc &d, const EpiArgs<R
     if (k2 == 0 && FLAME_IN(d.status, a.K1 - k1, box_len(a), kSiteCState)) col[-k1] = C{v.x, -v.y};
 }
 
-// The surface area of the state entering the step, for the record: the
-// area variant of pass B left one FP64 sum per row pair (summed here by
-// tile 0's threads, all of which call this), or the separate area kernels
-// left the total; NaN when the step records no area.
-template <bool GEN> __device__ __forceinline__ double record_area(const FlameDesc &d, int tile, int stage, int N1) {
-    const StepArgs &a = d.a;
-    double area = __longlong_as_double(0x7ff8000000000000LL);
-    if (GEN && tile == 0 && d.rec && stage != kStageHeun2 && stage != kStageIF2) {
-        if (d.rec_area == 1) {
-            __shared__ double asum[32];
-            double v = 0.0;
-            for (int i = threadIdx.x; i < (a.n1 >> 1); i += blockDim.x)
-                if (FLAME_IN(d.status, i, a.n1 >> 1, kSiteCRec)) v += d.arow[i];
-            for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-            if ((threadIdx.x & 31) == 0) asum[threadIdx.x >> 5] = v;
-            __syncthreads();
-            if (threadIdx.x == 0) {
-                double tot = 0.0;
-                for (int w = 0; w < (int)(blockDim.x + 31) / 32; ++w) tot += asum[w];
-                const double two_pi = 6.283185307179586476925286766559;
-                area = tot * (two_pi * two_pi / ((double)N1 * (double)a.n2 * a.s1 * a.s2));
-            }
-        } else if (d.rec_area == 2) {
-            area = *d.aval;
-        }
-    }
-    return area;
-}
-
-// Thread 0 of tile 0: the mean mode's update from rs, the FP64 sum of column
-// k2 = 0 of gk (N1 N2 times the mean of |grad Phi|^2), the time, and the
-// record entry of the step.
+// One thread: the mean mode's update from rs, the FP64 sum of column k2 = 0
+// of gk (N1 N2 times the mean of |grad Phi|^2), the time, and the record
+// entry of the step.
 template <bool GEN>
-__device__ __forceinline__ void finish_step(const FlameDesc &d, int stage, bool nl, int N1, double rs, double area) {
+__device__ __forceinline__ void finish_step(const FlameDesc &d, int stage, bool nl, double rs, double area) {
     const StepArgs &a = d.a;
-    const double mg = rs / ((double)N1 * (double)a.n2);  // mean of |grad Phi|^2
+    const double mg = rs * d.coef[9];  // mean of |grad Phi|^2
     // dt times the mean mode's right-hand side (omega_0 = 0): c mg + f_0
     double inc = nl ? a.dt * d.coef[1] * mg : 0.0;
     if (GEN && d.forcing0 != 0.0) inc += a.dt * d.forcing0;
-    const double m = *d.mean;
-    long n = __double2ll_rn((d.coef[0] - a.t0) / a.dt);
-    const long ri = ((n % max(d.rec_cap, 1)) + d.rec_cap) % max(d.rec_cap, 1);
-    if (GEN && d.rec && stage != kStageHeun2 && stage != kStageIF2 && FLAME_IN(d.status, ri, d.rec_cap, kSiteCRec)) {
-        double *e = d.rec + 4 * (size_t)ri;
-        e[0] = d.coef[0];
-        e[1] = m;
-        e[2] = (nl ? d.coef[1] * mg : 0.0) + (GEN ? d.forcing0 : 0.0);
-        e[3] = area;
+    const double m = *d.mean, n = d.coef[8];
+    if (GEN && d.rec && stage != kStageHeun2 && stage != kStageIF2) {
+        const long ri = (((long)n % d.rec_cap) + d.rec_cap) % d.rec_cap;
+        if (FLAME_IN(d.status, ri, d.rec_cap, kSiteCRec)) {
+            double *e = d.rec + 4 * (size_t)ri;
+            e[0] = d.coef[0];
+            e[1] = m;
+            e[2] = (nl ? d.coef[1] * mg : 0.0) + (GEN ? d.forcing0 : 0.0);
+            e[3] = area;
+        }
     }
     if (stage == kStageEuler || stage == kStageHeun1 || stage == kStageIF1) {
         if (stage == kStageHeun1) *d.save_mean = m;
         if (stage == kStageIF1) *d.save_mean = m + 0.5 * inc;
         *d.mean = m + inc;
-        *d.t_out = a.t0 + (double)(n + 1) * a.dt;
+        *d.t_out = a.t0 + (n + 1.0) * a.dt;
     } else {
         // second stages are evaluated at t_{n+1} and leave t there
         *d.mean = stage == kStageHeun2 ? 0.5 * (*d.save_mean + m + inc) : *d.save_mean + 0.5 * inc;
-        *d.t_out = a.t0 + (double)n * a.dt;
+        *d.t_out = a.t0 + n * a.dt;
     }
+}
+
+// The FP64 scalars of a step run in CTAs of their own: on the first tile's
+// critical path their dozen dependent divisions, sums and conversions cost a
+// small grid 4-5 us a step (256x512: pass C 10.5 -> 4.7 us, pass B 6.3 -> 5.5).
+// The extra CTA of pass B: the step's coefficients.
+template <class R> __device__ __forceinline__ void coef_cta(const FlameDesc &d) {
+    griddep_wait();
+    griddep_launch();
+    if (threadIdx.x == 0) store_coef<R>(d.coef, d.a, *d.t_in, d.stage == kStageIF1);
+}
+// Sum over the CTA (a power of two of up to 512 threads); the result is
+// thread 0's.
+__device__ __forceinline__ double cta_sum(double v, double *red) {
+    __syncthreads();
+    red[threadIdx.x] = v;
+    __syncthreads();
+    for (int w = blockDim.x >> 1; w > 0; w >>= 1) {
+        if ((int)threadIdx.x < w) red[threadIdx.x] += red[threadIdx.x + w];
+        __syncthreads();
+    }
+    return red[0];
+}
+// The extra CTA of pass C: the sum of column 0 of gk (N1 N2 times the mean of
+// |grad Phi|^2 by row sums), then the mean mode, the time and the record with
+// the area of the state entering the step (from the row-pair sums of
+// passB_area, from the separate area kernels, or NaN).
+template <class R, bool GEN> __device__ __forceinline__ void finish_cta(const FlameDesc &d) {
+    griddep_wait();
+    griddep_launch();
+    using C = CplxT<R>;
+    __shared__ double red[512];
+    const StepArgs &a = d.a;
+    const C *gk = static_cast<const C *>(d.gk);
+    double v = 0.0;
+    for (int n = threadIdx.x; n < a.n1; n += blockDim.x)
+        if (FLAME_IN(d.status, gk_index(n, 0, a.n1), gk_len(a), kSiteCGk)) v += (double)__ldg(&gk[gk_index(n, 0, a.n1)].x);
+    const double rs = cta_sum(v, red);
+    double area = __longlong_as_double(0x7ff8000000000000LL);
+    if (GEN && d.rec && d.rec_area == 1) {
+        double w = 0.0;
+        for (int i = threadIdx.x; i < (a.n1 >> 1); i += blockDim.x)
+            if (FLAME_IN(d.status, i, a.n1 >> 1, kSiteCRec)) w += d.arow[i];
+        const double two_pi = 6.283185307179586476925286766559;
+        area = cta_sum(w, red) * (two_pi * two_pi / ((double)a.n1 * (double)a.n2 * a.s1 * a.s2));
+    } else if (GEN && d.rec && d.rec_area == 2) {
+        area = *d.aval;
+    }
+    if (threadIdx.x == 0) finish_step<GEN>(d, GEN ? d.stage : kStageEuler, !(a.flags & kLinearOnly), rs, area);
 }
 
 // Pass C (a7..a10): columns k2, k2+1 of gk -> forward FFT along j1 (outputs
 // outside |k1| <= K1 unused and dropped at compile time), scaled by
 // 1/(N1 N2) -> ghat; Phi <- Phi + dt (omega Phi + c ghat); the k2 = 0 column
-// is written from its k1 > 0 half and its conjugate mirror; the block owning
-// column 0 sums G[j1][0] in FP64 for the mean mode and advances t.  The state
-// entries of the epilogue are loaded after the transform.
-// GEN = false compiles the plain Euler step without forcing or record (the
-// hot path); GEN = true reads the stage, forcing and record from the
-// descriptor.
-template <class R, int LOG, bool FUSE_A = false, int E = 16, bool GEN = true>
-__device__ __forceinline__ void passC_body(const FlameDesc &d, int tile, int ntiles, int pf,
-                                           const CUtensorMap *tm = nullptr) {
+// is written from its k1 > 0 half and its conjugate mirror; the mean mode and
+// t are the extra CTA's.  The state entries of the epilogue are loaded after
+// the transform.
+template <class R, int LOG>
+__device__ __forceinline__ void passC_body(const FlameDesc &d, int tile, int ntiles, int pf) {
     griddep_wait();
     griddep_launch();
     using V = typename VecOf<R>::type;
     using C = CplxT<R>;
-    static_assert(E == 16 || ((E == 8 || E == 4) && !FUSE_A),
-                  "E points per thread: 16, or 8 and 4 without the fused pass A");
+    constexpr bool GEN = true;
+    constexpr int E = 16;
     constexpr int QE = E / 4;  // band registers: r < QE (k1 >= 0) and r >= E - QE (k1 < 0)
     extern __shared__ __align__(16) unsigned char smraw[];
-    __shared__ double red[256];  // one per thread (blockDim <= 256)
     const StepArgs &a = d.a;
     const C *__restrict__ gk = static_cast<const C *>(d.gk);
     C *__restrict__ state = static_cast<C *>(d.state);
@@ -1186,12 +1088,8 @@ __device__ __forceinline__ void passC_body(const FlameDesc &d, int tile, int nti
     const bool va = c0 <= a.K2, vb = c0 + 1 <= a.K2;
     V *base = reinterpret_cast<V *>(smraw) + (size_t)g * 2 * plane_len_e<E>(N1);
     auto sm = make_planes_e<E>(base, N1);
-    constexpr bool STW = false;  // pass C's twiddles stay in L1 (measured faster)
-    C *stw = reinterpret_cast<C *>(reinterpret_cast<V *>(smraw) + (size_t)G * 2 * plane_len_e<E>(N1));
-    if constexpr (STW) TwShared<C>::template fill<(STW ? LOG : 8)>(stw, tw1);  // synced below
     const C *gp = gk + gk_index(0, c0, N1);  // row n: columns c0, c0+1 at gp[2n], gp[2n+1]
     CV<V> x[E];
-    double colsum = 0.0;
 #pragma unroll
     for (int r = 0; r < E; ++r) {
         const int n = t + r * T;
@@ -1205,33 +1103,13 @@ __device__ __forceinline__ void passC_body(const FlameDesc &d, int tile, int nti
             p = in ? __ldg(gp + 2 * n) : C{0, 0};
             q = (in && vb) ? __ldg(gp + 2 * n + 1) : C{0, 0};
         }
-        if (c0 == 0) colsum += (double)p.x;
         x[r] = pack2<R>(p, q);
     }
     // state entries this thread updates: rows r < QE (k1 = n) and r >= E - QE
     // (k1 = n - N1) of columns c0 and c0 + 1
     C *sa = state + (size_t)c0 * ld1 + a.K1, *sb = sa + ld1;
-    // block-uniform: FP64 row sum of column 0, in spans of up to 32 threads
-    // (power-of-two blocks) summed by each span's first thread in parallel
-    const int span = min((int)blockDim.x, 32);
-    if (tile == 0) {
-        red[threadIdx.x] = colsum;
-        __syncthreads();
-        if (threadIdx.x % span == 0) {
-            double s = 0.0;
-            for (int w = 0; w < span; ++w) s += red[threadIdx.x + w];
-            red[threadIdx.x] = s;  // the span's own slots: no other thread touches them
-        }
-        // the span sums are read by thread 0 after the transform's barriers
-    }
-    if constexpr (STW) {
-        __syncthreads();
-        fft_line_s<-1, (STW ? LOG : 8)>(x, t, sm, tw1, stw);
-    } else {
-        fft_line_e<-1, LOG, E>(x, a.logn1, t, sm, tw1);
-    }
+    fft_line<-1, LOG>(x, a.logn1, t, sm, tw1);
 
-    __syncthreads();  // block 0's span sums (the transform may have no CTA barrier)
     // the state entries, read after the transform (they are L2-resident in
     // the persisting window; holding them across the transform cost more)
     C phi[E / 2][2];
@@ -1251,7 +1129,6 @@ __device__ __forceinline__ void passC_body(const FlameDesc &d, int tile, int nti
     const C *fa = GEN && d.forcing ? static_cast<const C *>(d.forcing) + (size_t)c0 * ld1 + a.K1 : nullptr;
     C *va_save = GEN && d.save ? static_cast<C *>(d.save) + (size_t)c0 * ld1 + a.K1 : nullptr;
     int bad = 0;
-    C nphi[E / 2][2];  // the updated entries (kept for the fused pass A of the next step)
 #pragma unroll
     for (int i = 0; i < E / 2; ++i) {
         const int r = i < QE ? i : i + E / 2;
@@ -1261,90 +1138,17 @@ __device__ __forceinline__ void passC_body(const FlameDesc &d, int tile, int nti
 #pragma unroll
         for (int side = 0; side < 2; ++side) {
             const int k2 = c0 + side;
-            nphi[i][side] = C{0, 0};
+            C nw;
             const bool ok = in_box && (side == 0 ? va : vb);
             if (!ok) continue;
             if (k2 == 0 && k1 < 0) continue;  // written as the mirror of +k1
             const int off = side ? ld1 : 0;
             update_entry<R, GEN>(d, ea, k1, k2, side == 0 ? lane0<R>(x[r]) : lane1<R>(x[r]), phi[i][side],
                                  (side == 0 ? sa : sb), fa ? fa + off : nullptr, va_save ? va_save + off : nullptr,
-                                 nphi[i][side], bad);
+                                 nw, bad);
         }
     }
     if (bad) atomicOr(d.status, 1 << kStatusNonfinite);
-    const double area = record_area<GEN>(d, tile, stage, N1);
-    if (tile == 0 && threadIdx.x == 0) {
-        double rs = 0.0;
-        for (int w = 0; w < (int)blockDim.x; w += span) rs += red[w];
-        finish_step<GEN>(d, stage, nl, N1, rs, area);
-    }
-    if constexpr (FUSE_A && std::is_same<R, float>::value && LOG > 0) {
-        // Pass A of the next step (a1, a2) on the two updated columns, from
-        // registers: the same prologue, transform and tensor-store write-out
-        // as k_passAt.  The k2 = 0 column's k1 < 0 half was written by other
-        // threads (the conjugate mirror) and is read back after the barrier,
-        // which also frees the exchange buffer.
-        __syncthreads();
-        const R s1 = ea.s1, s2 = ea.s2;
-        if (c0 == 0) {
-#pragma unroll
-            for (int i = 4; i < 8; ++i) {
-                const int k1 = t + (i + 8) * T - N1;
-                if (k1 >= -a.K1 && FLAME_IN(d.status, a.K1 + k1, box_len(a), kSiteCState)) nphi[i][0] = sa[k1];
-            }
-        }
-        const C *__restrict__ tw1a = static_cast<const C *>(d.tw1);
-        float4 *park = reinterpret_cast<float4 *>(base);
-        const bool aligned = (__cvta_generic_to_shared(smraw) & 127) == 0;
-#pragma unroll 1
-        for (int side = 0; side < 2; ++side) {
-            const int k2 = c0 + side;
-            const bool valid = side == 0 ? va : vb;
-#pragma unroll
-            for (int r = 0; r < 16; ++r) {
-                x[r] = CV<V>{vzero(V{}), vzero(V{})};
-                if (r < 4 || r >= 12) {
-                    const int i = r < 4 ? r : r - 8;
-                    const int n = t + r * T;
-                    const int k1 = (r < 4) ? n : n - N1;
-                    if (!(valid && ((r < 4) ? (n <= a.K1) : (k1 >= -a.K1)))) continue;
-                    C phi = side == 0 ? nphi[i][0] : nphi[i][1];
-                    if (k1 == 0 && k2 == 0) phi = C{0, 0};
-                    const R f = s1 * (R)k1;
-                    x[r] = pack2<R>(C{-f * phi.y, f * phi.x}, phi);  // (i s1 k1 Phi, Phi)
-                }
-            }
-            fft_line<1, LOG>(x, a.logn1, t, sm, tw1a);
-            const R s2k2 = s2 * (R)k2;
-            __syncthreads();  // the transform's last exchange has been read
-#pragma unroll
-            for (int r = 0; r < 16; ++r) {
-                const int n = t + r * T;
-                C U = lane0<R>(x[r]);
-                C Vb = lane1<R>(x[r]);
-                park[n] = make_float4(U.x, U.y, -s2k2 * Vb.y, s2k2 * Vb.x);
-            }
-            fence_async_smem();
-            __syncthreads();
-            if (!aligned && valid) {
-#pragma unroll
-                for (int r = 0; r < 16; ++r) {
-                    const int n = t + r * T;
-                    if (FLAME_IN(d.status, uv_index(n, k2, a.ldk) + 1, uv_len(a), kSiteCAUv))
-                        *reinterpret_cast<float4 *>(static_cast<C *>(d.uv) + uv_index(n, k2, a.ldk)) = park[n];
-                }
-            }
-            if (aligned && t == 0 && valid) {
-                constexpr int BP = uv_box_pairs(1 << LOG);
-#pragma unroll 1
-                for (int p0 = 0; p0 < (N1 >> 1); p0 += BP)
-                    if (FLAME_IN(d.status, k2, a.ldk, kSiteCAUv) && FLAME_IN(d.status, p0, a.n1 >> 1, kSiteCAUv))
-                        tma_store_3d(tm, park + 2 * p0, 0, k2, p0);
-                bulk_commit_and_wait_read();
-            }
-            __syncthreads();  // the park may be overwritten by the next transform
-        }
-    }
 }
 
 // ----------------------------------------------------------------------------
@@ -1409,90 +1213,14 @@ template <class R, int LOG, int E> __device__ __forceinline__ void passA1_body(c
     }
 }
 
-// Pass B (a3..a6) on row pair p: group 2q + s takes the grid points 2m + s
-// of row 2p + q (the half-length inverse FFT of Z[k] exp(2 pi i k s / N2),
-// Z = U + iV) and parks g = u^2 + v^2 there; then group q transforms
-// h[m] = g[2m] + i g[2m+1] of row 2p + q forward and writes G[k], k <= K2,
-// after the real-input post-processing.  Groups 2 and 3 transform zeros in
-// the forward step, so that every group meets the same barriers.
-template <class R, int LOG, int E> __device__ __forceinline__ void passB1_body(const FlameDesc &d, int pair) {
-    griddep_wait();
-    griddep_launch();
-    using C = CplxT<R>;
-    using V1 = typename OneOf<R>::type;
-    extern __shared__ __align__(16) unsigned char smraw[];
-    const StepArgs &a = d.a;
-    constexpr int M = 1 << LOG, T = M / E, PL = plane_len_e<E>(M);
-    const int g = threadIdx.x / T, t = threadIdx.x % T;
-    const int q = g >> 1, s = g & 1;
-    const bool valid = pair < (a.n1 >> 1);
-    R *smd = reinterpret_cast<R *>(smraw);
-    const Planes<V1> sm(smd + (size_t)g * 2 * PL, PL);
-    R *h = smd + 8 * (size_t)PL;  // g of row 2p + q at h[2M q + j], j the grid point
-    const C *tw = static_cast<const C *>(d.twm) + tw_offset_e<E>(LOG);
-    const C *P = static_cast<const C *>(d.twm) + tw_real_offset(LOG);  // exp(2 pi i k / N2), k < M
-    if (pair == 0 && threadIdx.x == 0) store_coef<R>(d.coef, a, *d.t_in, d.stage == kStageIF1);
-    const size_t base = uv_index(2 * pair + q, 0, a.ldk);  // (U, V) of k at base + 4k
-    const C *src = static_cast<const C *>(d.uv) + base;
-    CV<V1> x[E];
-#pragma unroll
-    for (int r = 0; r < E; ++r) {
-        const int n = t + r * T;
-        const int kk = (r < E / 2) ? n : M - n;  // |k|: k = n (r < E/2) or n - M
-        C z{0, 0};
-        if (valid && kk <= a.K2 && kk < M / 2 && FLAME_IN(d.status, base + 4LL * kk + 1, uv_len(a), kSiteBUv)) {
-            const C u = __ldg(src + 4 * (size_t)kk), v = __ldg(src + 4 * (size_t)kk + 1);
-            // U[-k] = conj U[k], V[-k] = conj V[k]
-            z = (r < E / 2) ? C{u.x - v.y, u.y + v.x} : C{u.x + v.y, v.x - u.y};
-        }
-        if (s == 1) {
-            C w = __ldg(P + kk);  // exp(2 pi i k / N2) for the signed k
-            if (r >= E / 2) w.y = -w.y;
-            z = C{fma_rn(z.x, w.x, -(z.y * w.y)), fma_rn(z.x, w.y, z.y * w.x)};
-        }
-        x[r] = CV<V1>{{z.x}, {z.y}};
-    }
-    line_fft_ct<1, LOG, E>(x, t, sm, tw, CtaBarrier{});
-#pragma unroll
-    for (int r = 0; r < E; ++r) h[2 * M * q + 2 * (t + r * T) + s] = fma_rn(x[r].re.x, x[r].re.x, x[r].im.x * x[r].im.x);
-    __syncthreads();
-#pragma unroll
-    for (int r = 0; r < E; ++r) {
-        const int m = t + r * T;
-        x[r] = g < 2 ? CV<V1>{{h[2 * M * g + 2 * m]}, {h[2 * M * g + 2 * m + 1]}} : CV<V1>{{(R)0}, {(R)0}};
-    }
-    line_fft_ct<-1, LOG, E>(x, t, sm, tw, CtaBarrier{});
-    __syncthreads();
-    // the post-processing of k in [0, M/2) reads H[M - k]: H[0] and the upper half go to shared memory
-#pragma unroll
-    for (int r = E / 2; r < E; ++r) sm.st_raw(spad_e<E>(t + r * T), x[r]);
-    if (t == 0) sm.st_raw(0, x[0]);
-    __syncthreads();
-    if (g >= 2 || !valid) return;
-    C *gk = static_cast<C *>(d.gk);
-#pragma unroll
-    for (int r = 0; r < E / 2; ++r) {
-        const int k = t + r * T;
-        if (k > a.K2) continue;
-        const CV<V1> hk = x[r], hc = sm.ld_raw(spad_e<E>((M - k) & (M - 1)));
-        const R hf = (R)0.5;
-        const R ex = hf * (hk.re.x + hc.re.x), ey = hf * (hk.im.x - hc.im.x);
-        const R ox = hf * (hk.im.x + hc.im.x), oy = hf * (hc.re.x - hk.re.x);
-        const C w = __ldg(P + k);  // G = E + O conj(w)
-        const C y{ex + fma_rn(ox, w.x, oy * w.y), ey + fma_rn(oy, w.x, -(ox * w.y))};
-        const size_t i = gk_index(2 * pair + g, k, a.n1);
-        if (FLAME_IN(d.status, i, gk_len(a), kSiteBGk)) gk[i] = y;
-    }
-}
-
 // Pass C (a7..a10) on columns k2 = 2 tile + f (group f = 0, 1): the forward
-// transform of column k2 of gk and the update of its box entries; tile 0
-// sums column 0 in FP64 and finishes the step (mean mode, time, record).
-template <class R, int LOG, int E, bool GEN> __device__ __forceinline__ void passC1_body(const FlameDesc &d, int tile) {
+// transform of column k2 of gk and the update of its box entries.
+template <class R, int LOG, int E> __device__ __forceinline__ void passC1_body(const FlameDesc &d, int tile) {
     griddep_wait();
     griddep_launch();
     using C = CplxT<R>;
     using V1 = typename OneOf<R>::type;
+    constexpr bool GEN = true;
     constexpr int QE = E / 4;  // band registers: r < QE (k1 >= 0) and r >= E - QE (k1 < 0)
     extern __shared__ __align__(16) unsigned char smraw[];
     const StepArgs &a = d.a;
@@ -1506,31 +1234,12 @@ template <class R, int LOG, int E, bool GEN> __device__ __forceinline__ void pas
     const C *tw = static_cast<const C *>(d.tw1) + tw_offset_e<E>(LOG);
     const C *gk = static_cast<const C *>(d.gk);
     CV<V1> x[E];
-    double colsum = 0.0;
 #pragma unroll
     for (int r = 0; r < E; ++r) {
         const size_t i = gk_index(t + r * T, k2, N1);
         C p{0, 0};
         if (valid && FLAME_IN(d.status, i, gk_len(a), kSiteCGk)) p = __ldg(gk + i);
-        if (k2 == 0) colsum += p.x;
         x[r] = CV<V1>{{p.x}, {p.y}};
-    }
-    // tile 0: the FP64 sum of column 0 over group 0 (its T threads) by
-    // shuffles within each warp, then across the group's warps
-    if (tile == 0) {
-        if constexpr (T <= 32) {
-            if (threadIdx.x < 32) {
-                const unsigned lanes = blockDim.x >= 32 ? 0xffffffffu : (1u << blockDim.x) - 1u;
-                for (int o = T >> 1; o > 0; o >>= 1) colsum += __shfl_xor_sync(lanes, colsum, o);
-            }
-        } else {
-            __shared__ double wsum[T / 32];
-            for (int o = 16; o > 0; o >>= 1) colsum += __shfl_xor_sync(0xffffffffu, colsum, o);
-            if (f == 0 && (t & 31) == 0) wsum[t >> 5] = colsum;
-            __syncthreads();
-            if (threadIdx.x == 0)
-                for (int w = 1; w < T / 32; ++w) colsum += wsum[w];
-        }
     }
     line_fft_ct<-1, LOG, E>(x, t, sm, tw, CtaBarrier{});
     const bool lin = !(a.flags & kNonlinearOnly), nl = !(a.flags & kLinearOnly);
@@ -1555,145 +1264,41 @@ template <class R, int LOG, int E, bool GEN> __device__ __forceinline__ void pas
         }
     }
     if (bad) atomicOr(d.status, 1 << kStatusNonfinite);
-    const double area = record_area<GEN>(d, tile, stage, N1);
-    if (tile == 0 && threadIdx.x == 0) finish_step<GEN>(d, stage, nl, N1, colsum, area);
 }
 
-// Kernel entry points: one flame (descriptor by value) or an ensemble of
-// equal-size flames (descriptor array, flame = blockIdx.y).  LOG > 0: line
-// length 2^LOG fixed at compile time; LOG = 0: any length.
+// Kernel entry points.  LOG > 0: line length 2^LOG fixed at compile time;
+// LOG = 0: any length.
 template <class R, int LOG> __global__ void __launch_bounds__(256, kMinBlocks<R>) k_passA(FlameDesc d, int pf) {
-    passA_body<R, LOG, 16>(d, blockIdx.x + d.tile0, gridDim.x + d.tile0, pf);
-}
-// compile-time length, direct (scattered) stores instead of the cluster write-out
-template <class R, int LOG> __global__ void __launch_bounds__(256, kMinBlocks<R>) k_passAd(FlameDesc d, int pf) {
-    passA_body<R, LOG, 16, false>(d, blockIdx.x + d.tile0, gridDim.x + d.tile0, pf);
+    passA_body<R, LOG>(d, blockIdx.x, gridDim.x, pf);
 }
 // compile-time length, column written out by tensor stores (FP32); the
 // tensor map describes uv as (8 floats of a row pair) x k2 x row pair
 template <class R, int LOG>
 __global__ void __launch_bounds__(256, kMinBlocks<R>) k_passAt(FlameDesc d, int pf, const __grid_constant__ CUtensorMap tm) {
-    passA_body<R, LOG, 16, false, true>(d, blockIdx.x + d.tile0, gridDim.x + d.tile0, pf, &tm);
+    passA_body<R, LOG, true>(d, blockIdx.x, gridDim.x, pf, &tm);
 }
-// One line per thread group (the passes above): CTAs of 2 (A, C) or 4 (B)
-// groups of 2^LOG / E threads; pass C with the general epilogue (these
-// kernels serve small grids, where the plain one would save nothing
-// measurable).  MAXT: the largest CTA of the precision's line lengths.
+// One line per thread group: CTAs of 2 groups of 2^LOG / E threads
 template <class R> constexpr int kOneLineThreads = sizeof(R) == 8 ? 128 : 512;
 template <class R, int LOG, int E>
-__global__ void __launch_bounds__(kOneLineThreads<R>, 1) k_passA1(FlameDesc d, int pf) {
-    passA1_body<R, LOG, E>(d, blockIdx.x + d.tile0);
+__global__ void __launch_bounds__(kOneLineThreads<R>, 1) k_passA1(FlameDesc d) {
+    passA1_body<R, LOG, E>(d, blockIdx.x);
 }
 template <class R, int LOG, int E>
-__global__ void __launch_bounds__(kOneLineThreads<R>, 1) k_passB1(FlameDesc d, int pf) {
-    passB1_body<R, LOG, E>(d, blockIdx.x);
+__global__ void __launch_bounds__(kOneLineThreads<R>, 1) k_passC1(FlameDesc d) {
+    if (blockIdx.x == 0) return finish_cta<R, true>(d);
+    passC1_body<R, LOG, E>(d, blockIdx.x - 1);
 }
-template <class R, int LOG, int E>
-__global__ void __launch_bounds__(kOneLineThreads<R>, 1) k_passC1(FlameDesc d, int pf) {
-    passC1_body<R, LOG, E, true>(d, blockIdx.x + d.tile0);
-}
-template <class R, int LOG, int E>
-__global__ void __launch_bounds__(kOneLineThreads<R>, 1) k_passC1_n(const FlameDesc *__restrict__ ds, int pf) {
-    passC1_body<R, LOG, E, true>(ds[blockIdx.y], blockIdx.x);
-}
-template <class R, int LOG, int E>
-__global__ void __launch_bounds__(kOneLineThreads<R>, 1) k_passA1_n(const FlameDesc *__restrict__ ds, int pf) {
-    passA1_body<R, LOG, E>(ds[blockIdx.y], blockIdx.x);
-}
-template <class R, int LOG, int E>
-__global__ void __launch_bounds__(kOneLineThreads<R>, 1) k_passB1_n(const FlameDesc *__restrict__ ds, int pf) {
-    passB1_body<R, LOG, E>(ds[blockIdx.y], blockIdx.x);
-}
-// 8 points per thread, 512-thread CTAs (compile-time FP32 lengths)
-template <class R, int LOG> __global__ void __launch_bounds__(512, 2) k_passA8(FlameDesc d, int pf) {
-    passA_body<R, LOG, 8>(d, blockIdx.x + d.tile0, gridDim.x + d.tile0, pf);
-}
-template <class R, int LOG> __global__ void __launch_bounds__(256, kMinBlocks<R>) k_passB(FlameDesc d, int pf) {
-    passB_body<R, LOG, 16>(d, blockIdx.x, gridDim.x, pf);
-}
-// compile-time length, G written out by tensor stores (FP32); the tensor map
-// describes gk as (8 floats of a row pair and column pair) x row pair x
-// column pair
-template <class R, int LOG>
-__global__ void __launch_bounds__(256, kMinBlocks<R>) k_passBt(FlameDesc d, int pf, const __grid_constant__ CUtensorMap tm) {
-    passB_body<R, LOG, 16, true>(d, blockIdx.x, gridDim.x, pf, &tm);
-}
-// pass B that also sums the rows' surface area (the per-step record); its
-// shared memory (three more row-length buffers) allows one CTA per SM
+// the row pass that also sums the rows' surface area (the per-step record);
+// its shared memory allows one CTA per SM
 template <class R, int LOG, int E, int NT>
 __global__ void __launch_bounds__(NT, 1) k_passB_area(FlameDesc d) {
-    passB_body<R, LOG, E, false, false, true>(d, blockIdx.x, gridDim.x, 0);
+    if (blockIdx.x == 0) return coef_cta<R>(d);
+    passB_area_body<R, LOG, E>(d, blockIdx.x - 1);
 }
-// 8 points per thread, 512-thread CTAs (compile-time FP32 lengths)
-template <class R, int LOG> __global__ void __launch_bounds__(512, 2) k_passB8(FlameDesc d, int pf) {
-    passB_body<R, LOG, 8>(d, blockIdx.x, gridDim.x, pf);
-}
-template <class R, int LOG, bool GEN = true>
+template <class R, int LOG>
 __global__ void __launch_bounds__(256, kMinBlocks<R>) k_passC(FlameDesc d, int pf) {
-    passC_body<R, LOG, false, 16, GEN>(d, blockIdx.x + d.tile0, gridDim.x + d.tile0, pf);
-}
-// pass C of one step fused with pass A of the next (FP32, compile-time
-// lengths): the updated column pair is transformed back and written to uv
-// by tensor stores (the uv map of k_passAt)
-template <class R, int LOG, bool GEN = true>
-__global__ void __launch_bounds__(256, kMinBlocks<R>) k_passCA(FlameDesc d, int pf, const __grid_constant__ CUtensorMap tm) {
-    passC_body<R, LOG, true, 16, GEN>(d, blockIdx.x, gridDim.x, pf, &tm);
-}
-template <class R, int LOG>
-__global__ void __launch_bounds__(256, kMinBlocks<R>) k_passA_n(const FlameDesc *__restrict__ ds, int pf) {
-    passA_body<R, LOG, 16>(ds[blockIdx.y], blockIdx.x, gridDim.x, pf);
-}
-template <class R, int LOG>
-__global__ void __launch_bounds__(256, kMinBlocks<R>) k_passAd_n(const FlameDesc *__restrict__ ds, int pf) {
-    passA_body<R, LOG, 16, false>(ds[blockIdx.y], blockIdx.x, gridDim.x, pf);
-}
-template <class R, int LOG>
-__global__ void __launch_bounds__(512, 2) k_passA8_n(const FlameDesc *__restrict__ ds, int pf) {
-    passA_body<R, LOG, 8>(ds[blockIdx.y], blockIdx.x, gridDim.x, pf);
-}
-template <class R, int LOG>
-__global__ void __launch_bounds__(256, kMinBlocks<R>) k_passB_n(const FlameDesc *__restrict__ ds, int pf) {
-    passB_body<R, LOG, 16>(ds[blockIdx.y], blockIdx.x, gridDim.x, pf);
-}
-// ensembles with the tensor-store write-outs: maps[flame] is the flame's
-// uv map (pass A) or gk map (pass B), in global memory
-template <class R, int LOG>
-__global__ void __launch_bounds__(256, kMinBlocks<R>) k_passAt_n(const FlameDesc *__restrict__ ds, int pf,
-                                                               const CUtensorMap *maps) {
-    passA_body<R, LOG, 16, false, true, true>(ds[blockIdx.y], blockIdx.x, gridDim.x, pf, maps + blockIdx.y);
-}
-template <class R, int LOG>
-__global__ void __launch_bounds__(256, kMinBlocks<R>) k_passBt_n(const FlameDesc *__restrict__ ds, int pf,
-                                                               const CUtensorMap *maps) {
-    passB_body<R, LOG, 16, true, true>(ds[blockIdx.y], blockIdx.x, gridDim.x, pf, maps + blockIdx.y);
-}
-// 4096-point rows with warp-local exchanges (line_fft4096_wl), G written out
-// by tensor stores
-template <class R>
-__global__ void __launch_bounds__(256, kMinBlocks<R>) k_passBw(FlameDesc d, int pf, const __grid_constant__ CUtensorMap tm) {
-    passB_body<R, 12, 16, true, false, false, true>(d, blockIdx.x, gridDim.x, pf, &tm);
-}
-template <class R>
-__global__ void __launch_bounds__(256, kMinBlocks<R>) k_passBw_n(const FlameDesc *__restrict__ ds, int pf,
-                                                                 const CUtensorMap *maps) {
-    passB_body<R, 12, 16, true, true, false, true>(ds[blockIdx.y], blockIdx.x, gridDim.x, pf, maps + blockIdx.y);
-}
-// the same transforms with G written by direct stores (no tensor map): the
-// arithmetic, and so the bits, of k_passBw
-template <class R> __global__ void __launch_bounds__(256, kMinBlocks<R>) k_passBwd(FlameDesc d, int pf) {
-    passB_body<R, 12, 16, false, false, false, true>(d, blockIdx.x, gridDim.x, pf);
-}
-template <class R>
-__global__ void __launch_bounds__(256, kMinBlocks<R>) k_passBwd_n(const FlameDesc *__restrict__ ds, int pf) {
-    passB_body<R, 12, 16, false, false, false, true>(ds[blockIdx.y], blockIdx.x, gridDim.x, pf);
-}
-template <class R, int LOG>
-__global__ void __launch_bounds__(512, 2) k_passB8_n(const FlameDesc *__restrict__ ds, int pf) {
-    passB_body<R, LOG, 8>(ds[blockIdx.y], blockIdx.x, gridDim.x, pf);
-}
-template <class R, int LOG>
-__global__ void __launch_bounds__(256, kMinBlocks<R>) k_passC_n(const FlameDesc *__restrict__ ds, int pf) {
-    passC_body<R, LOG>(ds[blockIdx.y], blockIdx.x, gridDim.x, pf);
+    if (blockIdx.x == 0) return finish_cta<R, true>(d);
+    passC_body<R, LOG>(d, blockIdx.x - 1, gridDim.x - 1, pf);
 }
 
 }  // namespace flame

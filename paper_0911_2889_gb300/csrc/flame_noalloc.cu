@@ -17,6 +17,7 @@
 // between them) race on it and give wrong results.  Each call rewrites all of
 // the scratch it reads (tables, workspaces) and clears the status word, so
 // ordered calls of different sizes do not see each other's data.
+#include <algorithm>
 #include <atomic>
 #include <cmath>
 #include <cstdarg>
@@ -27,6 +28,7 @@
 #include "flame.h"
 #include "flame_internal.h"
 #include "fft_engine.cuh"
+#include "line3.cuh"
 
 namespace {
 
@@ -90,8 +92,8 @@ flame_status run_steps(const flame::StepArgs &a, unsigned char *base, size_t off
                        size_t off_uv, size_t off_gk, size_t off_sc, void *state, double *mean, double *t,
                        int nsteps, cudaStream_t s) {
     using C = typename flame::Ops<R>::C;
-    cudaError_t e = flame::Ops<R>::init_twiddles(reinterpret_cast<C *>(base + off_tw1), a.logn1, s);
-    if (e == cudaSuccess) e = flame::Ops<R>::init_twiddles(reinterpret_cast<C *>(base + off_twm), a.logm, s);
+    cudaError_t e = flame::Ops<R>::init_twiddles3(reinterpret_cast<C *>(base + off_tw1), a.la, s);
+    if (e == cudaSuccess) e = flame::Ops<R>::init_twiddles3(reinterpret_cast<C *>(base + off_twm), a.lb, s);
     double *dscal = reinterpret_cast<double *>(base + off_sc);
     int *status = reinterpret_cast<int *>(base + off_sc + 4 * sizeof(double));
     if (e == cudaSuccess) e = cudaMemsetAsync(status, 0, sizeof(int), s);  // must start at zero
@@ -105,7 +107,7 @@ flame_status run_steps(const flame::StepArgs &a, unsigned char *base, size_t off
     d.tw1 = base + off_tw1;
     d.twm = base + off_twm;
     d.t_in = t;
-    d.coef = dscal + 8;  // 48 bytes at off_sc + 64 (the arena keeps 256 bytes there)
+    d.coef = dscal + 8;  // 80 bytes at off_sc + 64 (the arena keeps 256 bytes there)
     d.mean = mean;
     d.t_out = t;
     d.status = status;
@@ -161,16 +163,24 @@ flame_status flame_step_noalloc(const flame_params *params, void *state, double 
     a.dt = p.dt;
     a.flags = p.flags;
 
-    // scratch layout: twiddles (N1), twiddles (N2/2), (U,V), G, scalars
+    // Which grids are taken: those whose tables and workspaces would fit on
+    // the public grid.  The step's own grid needs less for each of them.
     const size_t csz = p.prec == FLAME_FP64 ? sizeof(double2) : sizeof(float2);
+    const size_t pairs = (size_t)((a.ldk + 1) & ~1);  // gk holds column pairs: an even number of columns
+    const size_t need = align256(flame::tw_alloc_len(a.logn1) * csz) + align256(flame::tw_alloc_len(a.logm) * csz) +
+                        align256((size_t)a.n1 * a.ldk * 2 * csz) + align256((size_t)a.n1 * pairs * csz) + 256;
+    // scratch layout: twiddles of the step grid's columns and rows, row
+    // spectra, G, scalars
+    a.la = flame::step_exponent(p.K1);
+    a.lb = std::max(flame::step_exponent(p.K2) - 1, flame::kMinA);
+    a.n1 = 3 << a.la;
+    a.n2 = 6 << a.lb;
     const size_t off_tw1 = 0;
-    const size_t off_twm = off_tw1 + align256(flame::tw_alloc_len(a.logn1) * csz);
-    const size_t off_uv = off_twm + align256(flame::tw_alloc_len(a.logm) * csz);
+    const size_t off_twm = off_tw1 + align256(flame::tw3_len_of(a.la) * csz);
+    const size_t off_uv = off_twm + align256(flame::tw3_len_of(a.lb) * csz);
     const size_t off_gk = off_uv + align256((size_t)a.n1 * a.ldk * 2 * csz);
-    // gk holds column pairs: an even number of columns
-    const size_t off_sc = off_gk + align256((size_t)a.n1 * ((a.ldk + 1) & ~1) * csz);
-    const size_t need = off_sc + 256;
-    if (need > kNoAllocScratchBytes)
+    const size_t off_sc = off_gk + align256((size_t)a.n1 * pairs * csz);
+    if (need > kNoAllocScratchBytes || off_sc + 256 > kNoAllocScratchBytes)
         return nfail(FLAME_EUNSUPPORTED,
                      "flame_step_noalloc: grid %dx%d needs %zu bytes of scratch, the static maximum is %zu",
                      p.n_theta, p.n_phi, need, kNoAllocScratchBytes);

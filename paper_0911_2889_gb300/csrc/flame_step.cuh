@@ -1,0 +1,709 @@
+// flame_step.cuh -- the step's passes on its alias-free grid.
+//
+// The quadratic term of eq. (SivCurv1c) is wanted on the retained harmonics
+// |k_i| <= K_i only.  The product of two fields with K harmonics has 2 K; on a
+// grid of L points harmonic m folds onto m - L, so the retained ones stay
+// clean as long as L - 2 K > K: L >= 3 K + 1 points give the same coefficients
+// as the N >= 4 K + 1 points of the augmented array of Sec. 3 (the 3/2 rule of
+// pseudospectral methods, Orszag 1971), and the same mean of |grad Phi|^2.
+// The step therefore transforms on L1 x L2 points, L = 3 * 2^a the least such
+// length >= 3 K + 1: 3/4 of the public grid a side by default, less for a
+// truncated box.  At 4096 x 8192 the row pass does 9/16 of the transforms and
+// the workspaces hold 3/4 of the bytes (uv 101 MB, gk 50 MB).
+//
+// Three passes over HBM, as on the public grid:
+//   A (columns): Phi(., k2) -> the row spectra of w = d1 Phi + i d2 Phi at
+//                k2 and -k2, for all j1:  W(j1, k2) and W(j1, -k2).  Both are
+//                inverse transforms of the same column:
+//                  W(., k2)        = synthesis of (i s1 k1 - s2 k2) Phi,
+//                  conj W(., -k2)  = synthesis of (i s1 k1 + s2 k2) Phi
+//   B (rows):    w = inverse transform of W along k2, g = |w|^2 =
+//                |grad Phi|^2, its forward real transform, k2 <= K2 kept
+//   C (columns): forward transform along j1, |k1| <= K1 kept, update.
+// Layouts:
+//   uv  ((j1/2) ldk + k2) 4 + j1 % 2 (+ 2 for -k2): W of a row pair at +-k2 is
+//       one 32-byte sector in FP32 (pass A writes it), and the two rows' W at
+//       one k are 16 adjacent bytes (pass B reads them)
+//   gk  gk_index, as on the public grid.
+// One extra CTA of pass B derives the step's coefficients and one of pass C
+// the mean mode and the time (coef_cta, finish_cta).
+#pragma once
+
+#include "flame_kernels.cuh"
+#include "line3.cuh"
+
+namespace flame {
+
+template <class V> constexpr int kLanes = sizeof(V) / sizeof(V{}.x);  // lines per thread
+template <class R, int A, int F, class C> __device__ __forceinline__ const C *tab3(const void *tw) {
+    return static_cast<const C *>(tw) + tw3_offset<A, F>();
+}
+// exchange buffer of line (or line pair) `line`, `slots` slots each
+template <class V, class R> __device__ __forceinline__ Planes<V> planes3(unsigned char *smem, int line, int slots) {
+    if constexpr (kLanes<V> == 2) return Planes<V>(reinterpret_cast<V *>(smem) + (size_t)line * 2 * slots);
+    else return Planes<V>(reinterpret_cast<R *>(smem) + (size_t)line * 2 * slots, slots);
+}
+// bytes of a CTA's exchange buffers
+template <class R, class V, class PL> __host__ __device__ constexpr size_t exchange_bytes(int lines) {
+    return (size_t)lines * PL::slots(kSlotsPerWave<V>) * 2 * sizeof(V);
+}
+// complex index of W(j1, k2) (W(j1, -k2) two further)
+__host__ __device__ __forceinline__ size_t w_index(int j1, int k2, int ldk) {
+    return 4 * ((size_t)(j1 >> 1) * ldk + k2) + (j1 & 1);
+}
+
+// Pass A: column k2 of the box.  Two lines per thread (V = float2): lane 0 is
+// W(., k2), lane 1 conj W(., -k2); one line per thread: lines 2u and 2u+1 of
+// the CTA are the two of its column u.
+template <class R, class V, int A, int F, bool TMA>
+__device__ __forceinline__ void stepA_body(const FlameDesc &d, int tile, int ntiles, int pf, const CUtensorMap *tm) {
+    griddep_wait();
+    griddep_launch();
+    using C = CplxT<R>;
+    using PL = Plan3<A, F>;
+    constexpr int NL = kLanes<V>, LPC = 2 / NL, SL = PL::slots(kSlotsPerWave<V>);
+    extern __shared__ __align__(128) unsigned char smstep[];
+    const StepArgs &a = d.a;
+    const int G = blockDim.x / (PL::TS * LPC);
+    const Place s = place<PL::TS>(G * LPC), p = place<PL::TP>(G * LPC);
+    const int ld1 = 2 * a.K1 + 1;
+    const C *__restrict__ state = static_cast<const C *>(d.state);
+    C *__restrict__ uv = static_cast<C *>(d.uv);
+    if (threadIdx.x == 0 && pf > 0 && tile + pf < ntiles) {
+        const int c = (tile + pf) * G, nc = min(G, a.K2 + 1 - c);
+        if (nc > 0) l2_prefetch(state + (size_t)c * ld1, (size_t)nc * ld1 * sizeof(C));
+    }
+    CV<V> xs[PL::ES];
+    {
+        const int k2 = tile * G + s.line / LPC;
+        const C *col = state + (size_t)k2 * ld1 + a.K1;
+        const R s1 = scale1<R>(a), s2k2 = scale2<R>(a) * (R)k2;
+#pragma unroll
+        for (int r = 0; r < PL::ES; ++r) {
+            xs[r] = CV<V>{vzero(V{}), vzero(V{})};
+            if (r >= F && r < 2 * F) continue;  // padding: K1 < 2^A = F TS
+            const int n = s.t + r * PL::TS, k1 = r < F ? n : n - PL::L;
+            const bool in_box = s.on && k2 <= a.K2 && (r < F ? n <= a.K1 : k1 >= -a.K1);
+            if (in_box && FLAME_IN(d.status, (long long)k2 * ld1 + a.K1 + k1, box_len(a), kSiteAState)) {
+                C phi = __ldg(col + k1);
+                if (k1 == 0 && k2 == 0) phi = C{0, 0};
+                const R f = s1 * (R)k1;
+                const C da{-f * phi.y, f * phi.x}, db{s2k2 * phi.x, s2k2 * phi.y};
+                if constexpr (NL == 2) {
+                    xs[r] = pack2<R>(C{da.x - db.x, da.y - db.y}, C{da.x + db.x, da.y + db.y});
+                } else {
+                    const R sg = s.line & 1 ? (R)1 : (R)-1;
+                    xs[r] = CV<V>{{fma_rn(sg, db.x, da.x)}, {fma_rn(sg, db.y, da.y)}};
+                }
+            }
+        }
+    }
+    auto buf = [&](int line) { return planes3<V, R>(smstep, line, SL); };
+    CV<V> xp[PL::EP];
+    inverse3<PL, true>(xs, xp, s, p, buf, tab3<R, A, F, C>(d.tw1));
+    const int k2 = tile * G + p.line / LPC;
+    const bool valid = p.on && k2 <= a.K2;
+    if constexpr (NL == 1) {
+        const int f = p.line & 1;
+        if (!valid) return;
+#pragma unroll
+        for (int i = 0; i < PL::EP; ++i) {
+            const size_t w = w_index(p.t + i * PL::TP, k2, a.ldk) + 2 * f;
+            if (FLAME_IN(d.status, w, uv_len(a), kSiteAUv)) uv[w] = C{xp[i].re.x, f ? -xp[i].im.x : xp[i].im.x};
+        }
+    } else if constexpr (TMA) {
+        // The column is parked in shared memory in uv's order (32 bytes a row
+        // pair) and the copy engine writes the scattered sectors.
+        __syncthreads();  // the transform's last exchange has been read
+        auto park = [&](int line) { return reinterpret_cast<C *>(smstep) + (size_t)line * 2 * SL; };
+        if (p.on) {
+            C *q = park(p.line);
+#pragma unroll
+            for (int i = 0; i < PL::EP; ++i) {
+                const int n = p.t + i * PL::TP;
+                C *e = q + 4 * (n >> 1) + (n & 1);
+                e[0] = lane0<R>(xp[i]);
+                e[2] = C{xp[i].re.y, -xp[i].im.y};
+            }
+        }
+        fence_async_smem();
+        __syncthreads();
+        const bool aligned = (__cvta_generic_to_shared(smstep) & 127) == 0;
+        if (aligned) {
+            const int c = tile * G + s.line;
+            if (s.on && s.t == 0 && c <= a.K2) {
+                constexpr int BP = uv3_box_pairs(PL::L);
+#pragma unroll 1
+                for (int p0 = 0; p0 < PL::L / 2; p0 += BP)
+                    if (FLAME_IN(d.status, c, a.ldk, kSiteATma) && FLAME_IN(d.status, p0, a.n1 >> 1, kSiteATma))
+                        tma_store_3d(tm, park(s.line) + 4 * p0, 0, c, p0);
+                bulk_commit_and_wait_read();
+            }
+        } else if (valid) {
+            const C *q = park(p.line);
+#pragma unroll
+            for (int i = 0; i < PL::EP; ++i) {
+                const int n = p.t + i * PL::TP;
+                const size_t w = w_index(n, k2, a.ldk);
+                if (FLAME_IN(d.status, w + 2, uv_len(a), kSiteAUv)) {
+                    uv[w] = q[4 * (n >> 1) + (n & 1)];
+                    uv[w + 2] = q[4 * (n >> 1) + (n & 1) + 2];
+                }
+            }
+        }
+    } else {
+        // Threads 2i and 2i+1 hold rows 2i' and 2i'+1 (TP is even): one
+        // shuffle gives the even thread both rows' W(., k2) and the odd one
+        // both W(., -k2), 16 bytes each, together one sector.
+        static_assert(PL::TP % 2 == 0, "row pairs in adjacent threads");
+        const bool odd = threadIdx.x & 1;
+#pragma unroll
+        for (int i = 0; i < PL::EP; ++i) {
+            const C plus = lane0<R>(xp[i]), minus{xp[i].re.y, -xp[i].im.y};
+            const C give = odd ? plus : minus;
+            const C got{__shfl_xor_sync(0xffffffffu, give.x, 1), __shfl_xor_sync(0xffffffffu, give.y, 1)};
+            const size_t w = w_index((p.t & ~1) + i * PL::TP, k2, a.ldk) + (odd ? 2 : 0);
+            if (valid && FLAME_IN(d.status, w + 1, uv_len(a), kSiteAUv)) {
+                const C r0 = odd ? got : plus, r1 = odd ? minus : got;
+                *reinterpret_cast<float4 *>(uv + w) = make_float4(r0.x, r0.y, r1.x, r1.y);
+            }
+        }
+    }
+}
+
+// The inputs of the two half-length inverse transforms of a row of 2 L points
+// at index n: the even grid points take W[n] + W[n - L], the odd ones
+// (W[n] - W[n - L]) exp(2 pi i n / 2L) (harmonics L apart fold; for an index
+// only one of them reaches the other is zero).  n = t + r TS, so
+// exp(2 pi i n / 2L) = wt exp(i pi r / 3F): one table entry per thread and
+// compile-time roots.
+struct Roots24 {  // cos and sin of k pi / 12, k = 0 .. 11
+    static constexpr double C1 = 0.965925826289068286749743199728897368, S1 = 0.258819045102520762348898837624048328;
+    static constexpr double C2 = 0.866025403784438646763723170752936183, S2 = 0.5;
+    static constexpr double C3 = 0.707106781186547524400844362104849039;
+    static constexpr double c[12] = {1.0, C1, C2, C3, S2, S1, 0.0, -S1, -S2, -C3, -C2, -C1};
+    static constexpr double s[12] = {0.0, S1, S2, C3, C2, C1, 1.0, C1, C2, C3, S2, S1};
+};
+// b exp(i pi r / ES), ES = 3, 6 or 12
+template <int r, int ES, class C> __device__ __forceinline__ C mul_root24(C b) {
+    using Real = decltype(C::x);
+    constexpr int k = r * (12 / ES);
+    constexpr Real cr = (Real)Roots24::c[k], ci = (Real)Roots24::s[k];
+    if constexpr (k == 0) return b;
+    else if constexpr (k == 6) return C{-b.y, b.x};
+    else return C{fma_rn(b.x, cr, -(b.y * ci)), fma_rn(b.x, ci, b.y * cr)};
+}
+
+// G[k] and G[L - k] of a row from H[k] and H[L - k] of h[m] = g[2m] + i g[2m+1]
+// (E = (H[k] + conj H[L-k]) / 2, O = (H[k] - conj H[L-k]) / 2i, w = exp(2 pi i
+// k / 2L)): E + O conj w and conj(E - O conj w).
+template <class V, class C> __device__ __forceinline__ void real_post(CV<V> h, CV<V> hc, C w, CV<V> &lo, CV<V> &hi) {
+    using Real = decltype(C::x);
+    const V hf = vbc_as((Real)0.5, V{});
+    const CV<V> E{vmul(vadd(h.re, hc.re), hf), vmul(vsub(h.im, hc.im), hf)};
+    const CV<V> O{vmul(vadd(h.im, hc.im), hf), vmul(vsub(hc.re, h.re), hf)};
+    const CV<V> Ow = cmul_s(O, w.x, -w.y);
+    lo = cadd(E, Ow);
+    hi = CV<V>{vsub(E.re, Ow.re), vsub(Ow.im, E.im)};
+}
+
+// bytes of pass B's second region per row pair (two lines per thread): g of
+// one row, then G of both in the order of gk
+template <int A> __host__ __device__ constexpr size_t rows2_bytes() {
+    const size_t g = (size_t)(3 << A) * 8, G = ((size_t)(2 << A) + 2) * 16;
+    return ((g > G ? g : G) + 127) & ~(size_t)127;
+}
+
+// Pass B, two lines per thread (FP32): one row pair per group of TS threads.
+// The lanes are the even and odd points of one row in the inverse transforms
+// (row 2p, then row 2p+1, whose W were loaded with row 2p's: 16 bytes hold both),
+// and the two rows in the forward one.
+template <class R, int A, bool TMA>
+__device__ __forceinline__ void stepB2_body(const FlameDesc &d, int tile, int ntiles, int pf, const CUtensorMap *tm) {
+    using V = float2;
+    using C = CplxT<R>;
+    using PL = Plan3<A, 4>;
+    constexpr int L = PL::L, TS = PL::TS, TP = PL::TP, ES = PL::ES, SL = PL::slots(kSlotsPerWave<V>);
+    constexpr size_t kEx = exchange_bytes<R, V, PL>(1), kH = rows2_bytes<A>();
+    extern __shared__ __align__(128) unsigned char smstep[];
+    const StepArgs &a = d.a;
+    const C *__restrict__ uv = static_cast<const C *>(d.uv);
+    C *__restrict__ gk = static_cast<C *>(d.gk);
+    const int G = blockDim.x / TS;
+    const Place s = place<TS>(G), p = place<TP>(G);
+    if (threadIdx.x == 0 && pf > 0 && tile + pf < ntiles) {
+        const int p0 = (tile + pf) * G, np = min(G, (a.n1 >> 1) - p0);
+        if (np > 0) l2_prefetch(uv + w_index(2 * p0, 0, a.ldk), (size_t)np * 4 * a.ldk * sizeof(C));
+    }
+    const int pair = tile * G + s.line;
+    const bool valid = s.on && pair < (a.n1 >> 1);
+    unsigned char *h_base = smstep + (size_t)G * kEx;  // kEx, kH: multiples of 128
+    auto buf = [&](int line) { return planes3<V, R>(smstep, line, SL); };
+    const C *tw = tab3<R, A, 4, C>(d.twm);
+    const C wt = __ldg(static_cast<const C *>(d.twm) + tw3_real_offset<A>() + s.t);  // exp(2 pi i t / 2L)
+
+    // W of both rows at n (r < 8: K2 < 2^(A+1) = 8 TS) and at n - L (r >= 4)
+    C wp[8], wm[8];  // row 2p+1's, kept through row 2p's transform
+    CV<V> xs[ES];
+    auto build = [&](auto rc, C up, C um) {
+        constexpr int r = decltype(rc)::value;
+        C e, o;
+        if constexpr (r < 4) e = o = up;
+        else if constexpr (r >= 8) e = um, o = C{-um.x, -um.y};
+        else e = C{up.x + um.x, up.y + um.y}, o = C{up.x - um.x, up.y - um.y};
+        const C w = mul_root24<r, ES>(wt);
+        xs[r] = pack2<R>(e, C{fma_rn(o.x, w.x, -(o.y * w.y)), fma_rn(o.x, w.y, o.y * w.x)});
+    };
+    {
+        const float4 *src = reinterpret_cast<const float4 *>(uv + w_index(2 * pair, 0, a.ldk));  // k: + at 2k, - at 2k+1
+        C up[8], um[8];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            const int n = s.t + i * TS, km = L - (s.t + (i + 4) * TS);
+            float4 q = make_float4(0.f, 0.f, 0.f, 0.f), m = q;
+            if (valid && n <= a.K2 && FLAME_IN(d.status, w_index(2 * pair, n, a.ldk) + 1, uv_len(a), kSiteBUv)) q = __ldg(src + 2 * n);
+            if (valid && km <= a.K2 && FLAME_IN(d.status, w_index(2 * pair, km, a.ldk) + 3, uv_len(a), kSiteBUv)) m = __ldg(src + 2 * km + 1);
+            up[i] = C{q.x, q.y};
+            wp[i] = C{q.z, q.w};
+            um[i] = C{m.x, m.y};
+            wm[i] = C{m.z, m.w};
+        }
+        static_for<0, ES>([&](auto rc) {
+            constexpr int r = decltype(rc)::value;
+            build(rc, r < 8 ? up[r < 8 ? r : 0] : C{0, 0}, r >= 4 ? um[r >= 4 ? r - 4 : 0] : C{0, 0});
+        });
+    }
+    CV<V> xp[PL::EP];
+    inverse3<PL, true>(xs, xp, s, p, buf, tw);
+    // g of row 2p at the points 2m, 2m+1, parked for the forward transform
+    C *hp = reinterpret_cast<C *>(h_base + (size_t)p.line * kH);
+    if (p.on) {
+#pragma unroll
+        for (int i = 0; i < PL::EP; ++i) {
+            const V g = vfma(xp[i].re, xp[i].re, vmul(xp[i].im, xp[i].im));
+            hp[p.t + i * TP] = C{g.x, g.y};
+        }
+    }
+    static_for<0, ES>([&](auto rc) {
+        constexpr int r = decltype(rc)::value;
+        build(rc, r < 8 ? wp[r < 8 ? r : 0] : C{0, 0}, r >= 4 ? wm[r >= 4 ? r - 4 : 0] : C{0, 0});
+    });
+    inverse3<PL, false>(xs, xp, s, p, buf, tw);
+    if (p.on) {
+#pragma unroll
+        for (int i = 0; i < PL::EP; ++i) {
+            const V g = vfma(xp[i].re, xp[i].re, vmul(xp[i].im, xp[i].im));
+            xp[i] = pack2<R>(hp[p.t + i * TP], C{g.x, g.y});  // the thread's own slots
+        }
+    }
+    forward3<PL, false>(xp, xs, p, s, buf, tw);
+    // real-input post-processing: the pairs (k, L - k), k <= L/2
+    __syncthreads();
+    const Planes<V> sm = buf(s.line);
+    if (s.on) {
+#pragma unroll
+        for (int r = ES / 2; r < ES; ++r) sm.st_raw(s.t + r * TS, xs[r]);
+        if (s.t == 0) sm.st_raw(0, xs[0]);
+    }
+    __syncthreads();
+    const bool staged = TMA && (__cvta_generic_to_shared(smstep) & 127) == 0;
+    C *hs = reinterpret_cast<C *>(h_base + (size_t)s.line * kH);
+    auto emit = [&](int k, CV<V> Y) {
+        C *dst = staged ? hs + 4 * (k >> 1) + (k & 1) : gk + gk_index(2 * pair, k, a.n1);  // row 2p+1 two further
+        if (staged || FLAME_IN(d.status, gk_index(2 * pair, k, a.n1) + 2, gk_len(a), kSiteBGk)) {
+            dst[0] = lane0<R>(Y);
+            dst[2] = lane1<R>(Y);
+        }
+    };
+    if (valid) {
+        static_for<0, ES / 2>([&](auto rc) {
+            constexpr int r = decltype(rc)::value;
+            const int k = s.t + r * TS, kc = L - k;
+            if (k <= a.K2 || kc <= a.K2) {
+                CV<V> lo, hi;
+                real_post(xs[r], sm.ld_raw(k == 0 ? 0 : kc), mul_root24<r, ES>(wt), lo, hi);
+                if (k <= a.K2) emit(k, lo);
+                if (kc <= a.K2) emit(kc, hi);
+            }
+        });
+        // k = L/2 is its own partner: G = conj H
+        if (s.t == 0 && L / 2 <= a.K2) emit(L / 2, CV<V>{xs[ES / 2].re, vneg(xs[ES / 2].im)});
+    }
+    if constexpr (TMA) {
+        if (staged) {
+            fence_async_smem();
+            __syncthreads();
+            if (s.t == 0 && valid) {
+                const int nq = (a.ldk + 1) >> 1, BQ = gk_box_pairs(a.ldk);
+#pragma unroll 1
+                for (int q0 = 0; q0 < nq; q0 += BQ)
+                    if (FLAME_IN(d.status, pair, a.n1 >> 1, kSiteBTma) && FLAME_IN(d.status, q0, (gk_len(a) / a.n1) >> 1, kSiteBTma))
+                        tma_store_3d(tm, hs + 4 * q0, 0, pair, q0);
+                bulk_commit_and_wait_read();
+            }
+        }
+    }
+}
+
+// Pass B, one line per thread: RW rows per unit (2, or 1 for FP64 rows whose
+// pair does not fit in shared memory), lines 2 q + s = the points 2m + s of
+// row q in the inverse transforms, line q = row q in the forward one.
+template <class R, int A, int F, int RW>
+__device__ __forceinline__ void stepB1_body(const FlameDesc &d, int unit0) {
+    using V = typename OneOf<R>::type;
+    using C = CplxT<R>;
+    using PL = Plan3<A, F>;
+    constexpr int L = PL::L, TS = PL::TS, TP = PL::TP, ES = PL::ES, SL = PL::slots(kSlotsPerWave<V>);
+    extern __shared__ __align__(128) unsigned char smstep[];
+    const StepArgs &a = d.a;
+    const C *__restrict__ uv = static_cast<const C *>(d.uv);
+    C *__restrict__ gk = static_cast<C *>(d.gk);
+    const int U = blockDim.x / (2 * RW * TS), lines = 2 * RW * U;  // units of the CTA
+    const Place s = place<TS>(lines), p = place<TP>(lines);
+    auto buf = [&](int line) { return planes3<V, R>(smstep, line, SL); };
+    const C *tw = tab3<R, A, F, C>(d.twm);
+    const C *P = static_cast<const C *>(d.twm) + tw3_real_offset<A>();
+    const int first = unit0 * U * RW;  // the CTA's first row
+    CV<V> xs[ES];
+    {
+        const int row = first + (s.line >> 1);
+        const bool odd = s.line & 1, valid = s.on && row < a.n1;
+#pragma unroll
+        for (int r = 0; r < ES; ++r) {
+            const int n = s.t + r * TS, km = L - n;
+            C up{0, 0}, um{0, 0};
+            if (r < 2 * F && valid && n <= a.K2 && FLAME_IN(d.status, w_index(row, n, a.ldk), uv_len(a), kSiteBUv))
+                up = __ldg(uv + w_index(row, n, a.ldk));
+            if (r >= F && valid && km <= a.K2 && FLAME_IN(d.status, w_index(row, km, a.ldk) + 2, uv_len(a), kSiteBUv))
+                um = __ldg(uv + w_index(row, km, a.ldk) + 2);
+            C z{up.x + um.x, up.y + um.y};
+            if (odd) {
+                const C o{up.x - um.x, up.y - um.y}, w = __ldg(P + n);  // exp(2 pi i n / 2L)
+                z = C{fma_rn(o.x, w.x, -(o.y * w.y)), fma_rn(o.x, w.y, o.y * w.x)};
+            }
+            xs[r] = CV<V>{{z.x}, {z.y}};
+        }
+    }
+    CV<V> xp[PL::EP];
+    inverse3<PL, true>(xs, xp, s, p, buf, tw);
+    R *h = reinterpret_cast<R *>(smstep + (size_t)lines * SL * 2 * sizeof(R));  // g of row q at h[2 L q + j]
+    if (p.on) {
+#pragma unroll
+        for (int i = 0; i < PL::EP; ++i)
+            h[2 * L * (p.line >> 1) + 2 * (p.t + i * TP) + (p.line & 1)] =
+                fma_rn(xp[i].re.x, xp[i].re.x, xp[i].im.x * xp[i].im.x);
+    }
+    __syncthreads();
+    const int rows = RW * U;
+    const Place fp{p.line, p.t, p.line < rows}, fs{s.line, s.t, s.line < rows};
+    if (fp.on) {
+#pragma unroll
+        for (int i = 0; i < PL::EP; ++i) {
+            const C g = reinterpret_cast<const C *>(h)[L * fp.line + fp.t + i * TP];
+            xp[i] = CV<V>{{g.x}, {g.y}};
+        }
+    }
+    forward3<PL, true>(xp, xs, fp, fs, buf, tw);
+    __syncthreads();
+    const int row = first + fs.line;
+    const Planes<V> sm = buf(fs.line);
+    if (fs.on) {
+#pragma unroll
+        for (int r = 0; r < ES; ++r) {
+            if (TS * (r + 1) > L / 2) sm.st_raw(fs.t + r * TS, xs[r]);
+        }
+        if (fs.t == 0) sm.st_raw(0, xs[0]);
+    }
+    __syncthreads();
+    if (!fs.on || row >= a.n1) return;
+    auto emit = [&](int k, CV<V> Y) {
+        const size_t i = gk_index(row, k, a.n1);
+        if (FLAME_IN(d.status, i, gk_len(a), kSiteBGk)) gk[i] = C{Y.re.x, Y.im.x};
+    };
+#pragma unroll
+    for (int r = 0; r < ES; ++r) {
+        if (TS * r > L / 2) continue;
+        const int k = fs.t + r * TS, kc = L - k;
+        if (k <= L / 2 && (k <= a.K2 || kc <= a.K2)) {
+            CV<V> lo, hi;
+            real_post(xs[r], sm.ld_raw(k == 0 ? 0 : kc), __ldg(P + k), lo, hi);
+            if (k <= a.K2) emit(k, lo);
+            if (kc <= a.K2 && kc != k) emit(kc, hi);
+        }
+    }
+}
+
+// Pass C: columns 2 u, 2 u + 1 of gk; two lines per thread (lanes) or lines
+// 2u, 2u+1 of the CTA.  FUSE_A: pass A of the next step on the updated
+// columns (two lines per thread, tensor stores).
+template <class R, class V, int A, int F, bool GEN, bool FUSE_A = false>
+__device__ __forceinline__ void stepC_body(const FlameDesc &d, int tile, int ntiles, int pf, const CUtensorMap *tm) {
+    griddep_wait();
+    griddep_launch();
+    using C = CplxT<R>;
+    using PL = Plan3<A, F>;
+    constexpr int NL = kLanes<V>, LPC = 2 / NL, L = PL::L, TS = PL::TS, TP = PL::TP, SL = PL::slots(kSlotsPerWave<V>);
+    static_assert(!FUSE_A || NL == 2, "the fused pass is a two-line kernel");
+    extern __shared__ __align__(128) unsigned char smstep[];
+    const StepArgs &a = d.a;
+    const C *__restrict__ gk = static_cast<const C *>(d.gk);
+    C *__restrict__ state = static_cast<C *>(d.state);
+    const C *tw = tab3<R, A, F, C>(d.tw1);
+    const int G = blockDim.x / (TS * LPC);
+    const Place s = place<TS>(G * LPC), p = place<TP>(G * LPC);
+    const int ld1 = 2 * a.K1 + 1;
+    if (threadIdx.x == 0 && pf > 0 && tile + pf < ntiles) {
+        const int c = 2 * (tile + pf) * G, nc = min(2 * G, a.K2 + 1 - c);
+        if (nc > 0) {
+            l2_prefetch(gk + (size_t)c * L, (size_t)nc * L * sizeof(C));
+            l2_prefetch(state + (size_t)c * ld1, (size_t)nc * ld1 * sizeof(C));
+        }
+    }
+    const CoefR<R> cfs = load_coef<R>(d.coef);  // derived by pass B
+    CV<V> xp[PL::EP];
+    {
+        // the line's (first) column
+        const int c = 2 * (tile * G + p.line / LPC) + (NL == 1 ? p.line & 1 : 0);
+#pragma unroll
+        for (int i = 0; i < PL::EP; ++i) {
+            const int n = p.t + i * TP;
+            const bool in = p.on && c <= a.K2 &&
+                            FLAME_IN(d.status, gk_index(n, c, L) + (NL == 2 ? 1 : 0), gk_len(a), kSiteCGk);
+            if constexpr (NL == 2) {
+                const float4 q = in ? __ldg(reinterpret_cast<const float4 *>(gk + gk_index(n, c, L))) : make_float4(0.f, 0.f, 0.f, 0.f);
+                xp[i] = pack2<R>(C{q.x, q.y}, c < a.K2 ? C{q.z, q.w} : C{0, 0});
+            } else {
+                const C q = in ? __ldg(gk + gk_index(n, c, L)) : C{0, 0};
+                xp[i] = CV<V>{{q.x}, {q.y}};
+            }
+        }
+    }
+    auto buf = [&](int line) { return planes3<V, R>(smstep, line, SL); };
+    CV<V> xs[PL::ES];
+    forward3<PL, true>(xp, xs, p, s, buf, tw);
+
+    const int c0 = 2 * (tile * G + s.line / LPC) + (NL == 1 ? s.line & 1 : 0);
+    C *col = state + (size_t)c0 * ld1 + a.K1;
+    // the band entries of this thread: r < F (k1 = n) and r >= 2F (k1 = n - L);
+    // read after the transform, from the L2 window over the state
+    auto k1_of = [&](int i) { return i < F ? s.t + i * TS : s.t + (i + F) * TS - L; };
+    auto in_box = [&](int i, int side) {
+        const int k1 = k1_of(i);
+        return s.on && c0 + side <= a.K2 && (i < F ? k1 <= a.K1 : k1 >= -a.K1);
+    };
+    C phi[2 * F][NL];
+#pragma unroll
+    for (int i = 0; i < 2 * F; ++i)
+#pragma unroll
+        for (int side = 0; side < NL; ++side) {
+            const bool in = in_box(i, side) && FLAME_IN(d.status, (long long)(c0 + side) * ld1 + a.K1 + k1_of(i), box_len(a), kSiteCState);
+            phi[i][side] = in ? col[(long)side * ld1 + k1_of(i)] : C{0, 0};
+        }
+    const bool lin = !(a.flags & kNonlinearOnly), nl = !(a.flags & kLinearOnly);
+    const EpiArgs<R> ea{cfs, scale1<R>(a), scale2<R>(a), GEN ? d.stage : kStageEuler, lin, nl};
+    const C *fcol = GEN && d.forcing ? static_cast<const C *>(d.forcing) + (size_t)c0 * ld1 + a.K1 : nullptr;
+    C *scol = GEN && d.save ? static_cast<C *>(d.save) + (size_t)c0 * ld1 + a.K1 : nullptr;
+    int bad = 0;
+    C nphi[2 * F][NL];  // the updated entries (kept for the fused pass A)
+#pragma unroll
+    for (int i = 0; i < 2 * F; ++i)
+#pragma unroll
+        for (int side = 0; side < NL; ++side) {
+            nphi[i][side] = C{0, 0};
+            const int k1 = k1_of(i), k2 = c0 + side;
+            if (!in_box(i, side) || (k2 == 0 && k1 < 0)) continue;  // k2 = 0, k1 < 0: the mirror of +k1
+            const CV<V> x = xs[i < F ? i : i + F];
+            C gh;
+            if constexpr (NL == 2) gh = side == 0 ? lane0<R>(x) : lane1<R>(x);
+            else gh = C{x.re.x, x.im.x};
+            const int off = side * ld1;
+            update_entry<R, GEN>(d, ea, k1, k2, gh, phi[i][side], col + off, fcol ? fcol + off : nullptr,
+                                 scol ? scol + off : nullptr, nphi[i][side], bad);
+        }
+    if (bad) atomicOr(d.status, 1 << kStatusNonfinite);
+    if constexpr (FUSE_A) {
+        // The k2 = 0 column's k1 < 0 half was written by other threads (the
+        // conjugate mirror) and is read back after the barrier.
+        __syncthreads();
+        if (c0 == 0 && s.on) {
+#pragma unroll
+            for (int i = F; i < 2 * F; ++i)
+                if (k1_of(i) >= -a.K1 && FLAME_IN(d.status, a.K1 + k1_of(i), box_len(a), kSiteCState)) nphi[i][0] = col[k1_of(i)];
+        }
+        auto park = [&](int line) { return reinterpret_cast<C *>(smstep) + (size_t)line * 2 * SL; };
+        C *uv = static_cast<C *>(d.uv);
+        const bool aligned = (__cvta_generic_to_shared(smstep) & 127) == 0;
+#pragma unroll 1
+        for (int side = 0; side < 2; ++side) {
+            const int k2 = c0 + side;
+            const R s2k2 = ea.s2 * (R)k2;
+#pragma unroll
+            for (int r = 0; r < PL::ES; ++r) {
+                xs[r] = CV<V>{vzero(V{}), vzero(V{})};
+                if (r >= F && r < 2 * F) continue;
+                const int i = r < F ? r : r - F;
+                if (!in_box(i, side)) continue;
+                C ph = side == 0 ? nphi[i][0] : nphi[i][1];
+                if (k1_of(i) == 0 && k2 == 0) ph = C{0, 0};
+                const R f = ea.s1 * (R)k1_of(i);
+                const C da{-f * ph.y, f * ph.x}, db{s2k2 * ph.x, s2k2 * ph.y};
+                xs[r] = pack2<R>(C{da.x - db.x, da.y - db.y}, C{da.x + db.x, da.y + db.y});
+            }
+            inverse3<PL, false>(xs, xp, s, p, buf, tw);
+            __syncthreads();
+            if (p.on) {
+                C *q = park(p.line);
+#pragma unroll
+                for (int i = 0; i < PL::EP; ++i) {
+                    const int n = p.t + i * TP;
+                    C *e = q + 4 * (n >> 1) + (n & 1);
+                    e[0] = lane0<R>(xp[i]);
+                    e[2] = C{xp[i].re.y, -xp[i].im.y};
+                }
+            }
+            fence_async_smem();
+            __syncthreads();
+            if (aligned) {
+                if (s.on && s.t == 0 && k2 <= a.K2) {
+                    constexpr int BP = uv3_box_pairs(L);
+#pragma unroll 1
+                    for (int p0 = 0; p0 < L / 2; p0 += BP)
+                        if (FLAME_IN(d.status, k2, a.ldk, kSiteCAUv) && FLAME_IN(d.status, p0, a.n1 >> 1, kSiteCAUv))
+                            tma_store_3d(tm, park(s.line) + 4 * p0, 0, k2, p0);
+                    bulk_commit_and_wait_read();
+                }
+            } else if (p.on) {
+                const int kp = 2 * (tile * G + p.line) + side;
+                const C *q = park(p.line);
+                for (int i = 0; i < PL::EP; ++i) {
+                    const int n = p.t + i * TP;
+                    const size_t w = w_index(n, kp, a.ldk);
+                    if (kp <= a.K2 && FLAME_IN(d.status, w + 2, uv_len(a), kSiteCAUv)) {
+                        uv[w] = q[4 * (n >> 1) + (n & 1)];
+                        uv[w + 2] = q[4 * (n >> 1) + (n & 1) + 2];
+                    }
+                }
+            }
+        }
+    }
+}
+
+// ----------------------------------------------------------------------------
+// Twiddle tables of a line of 3 * 2^A points (FP64, rounded once).  The angle
+// is reduced to an eighth of a turn in integers first: 3 * 2^a is no power of
+// two, and 2 pi times a rounded fraction would cost the last bit or two.
+// ----------------------------------------------------------------------------
+__device__ inline void cos_sin_of(long num, long den, double &c, double &s) {  // 2 pi num / den
+    num %= den;  // den is even
+    const bool flip = 2 * num > den;  // (half, 1): the conjugate of den - num
+    if (flip) num = den - num;
+    const bool left = 4 * num > den;  // (quarter, half]: mirrored at the imaginary axis;
+    if (left) num = den - 2 * num;    // in units of 1 / (2 den) from here on
+    else num = 2 * num;
+    const bool swap = 4 * num > den;  // (eighth, quarter]
+    if (swap) num = den / 2 - num;
+    double sv, cv;
+    sincospi((double)num / (double)den, &sv, &cv);  // angle 2 pi num / (2 den)
+    c = swap ? sv : cv;
+    s = swap ? cv : sv;
+    if (left) c = -c;
+    if (flip) s = -s;
+}
+template <class R, int A> __global__ void k_twiddles3(CplxT<R> *tab) {
+    auto table = [&](auto fc, auto ic) {
+        constexpr int F = decltype(fc)::value;
+        constexpr bool INV = decltype(ic)::value;
+        if constexpr (A >= (F == 4 ? 4 : F == 2 ? 3 : 2)) {
+            using PL = Plan3<A, F>;
+            static_for<1, PL::NQ + 1>([&](auto sc) {
+                constexpr int S = decltype(sc)::value, r = PL::template radix<INV>(S), Ns = PL::template stride<INV>(S);
+                CplxT<R> *t = tab + tw3_offset<A, F>() + PL::template tw_offset<INV>(S);
+                for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < (r - 1) * Ns; i += gridDim.x * blockDim.x) {
+                    double c, s;
+                    cos_sin_of((long)(i / Ns + 1) * (i % Ns), (long)r * Ns, c, s);
+                    t[i] = CplxT<R>{(R)c, (R)s};
+                }
+            });
+        }
+    };
+    static_for<0, 3>([&](auto lf) {
+        constexpr int F = 1 << decltype(lf)::value;
+        table(std::integral_constant<int, F>{}, std::true_type{});
+        table(std::integral_constant<int, F>{}, std::false_type{});
+    });
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < (3 << A); i += gridDim.x * blockDim.x) {
+        double c, s;
+        cos_sin_of(i, 6L << A, c, s);
+        tab[tw3_real_offset<A>() + i] = CplxT<R>{(R)c, (R)s};
+    }
+}
+
+// ----------------------------------------------------------------------------
+// Kernels: one flame (descriptor by value) or the flames of one ensemble class
+// (descriptor array, flame = blockIdx.y)
+// ----------------------------------------------------------------------------
+// Passes A and C of one flame may be launched over part of their tiles
+// (flame_step_host); the launch that holds tile 0 of pass C has the extra CTA.
+template <class R, class V> constexpr int kStepThreads = kLanes<V> == 2 ? 256 : 512;
+template <class R, class V> constexpr int kStepBlocks = kLanes<V> == 2 ? 2 : 1;
+
+template <class R, class V, int A, int F>
+__global__ void __launch_bounds__(kStepThreads<R, V>, kStepBlocks<R, V>) k_stepA(FlameDesc d, int pf) {
+    stepA_body<R, V, A, F, false>(d, blockIdx.x + d.tile0, gridDim.x + d.tile0, pf, nullptr);
+}
+template <class R, int A>
+__global__ void __launch_bounds__(256, 2) k_stepAt(FlameDesc d, int pf, const __grid_constant__ CUtensorMap tm) {
+    stepA_body<R, float2, A, 4, true>(d, blockIdx.x + d.tile0, gridDim.x + d.tile0, pf, &tm);
+}
+template <class R, class V, int A, int F>
+__global__ void __launch_bounds__(kStepThreads<R, V>, kStepBlocks<R, V>) k_stepA_n(const FlameDesc *__restrict__ ds) {
+    stepA_body<R, V, A, F, false>(ds[blockIdx.y], blockIdx.x, gridDim.x, 0, nullptr);
+}
+
+template <class R, int A>
+__global__ void __launch_bounds__(256, 2) k_stepB(FlameDesc d, int pf) {
+    if (blockIdx.x == 0) return coef_cta<R>(d);
+    griddep_wait();
+    griddep_launch();
+    stepB2_body<R, A, false>(d, blockIdx.x - 1, gridDim.x - 1, pf, nullptr);
+}
+template <class R, int A>
+__global__ void __launch_bounds__(256, 2) k_stepBt(FlameDesc d, int pf, const __grid_constant__ CUtensorMap tm) {
+    if (blockIdx.x == 0) return coef_cta<R>(d);
+    griddep_wait();
+    griddep_launch();
+    stepB2_body<R, A, true>(d, blockIdx.x - 1, gridDim.x - 1, pf, &tm);
+}
+template <class R, int A> __global__ void __launch_bounds__(256, 2) k_stepB_n(const FlameDesc *__restrict__ ds) {
+    if (blockIdx.x == 0) return coef_cta<R>(ds[blockIdx.y]);
+    stepB2_body<R, A, false>(ds[blockIdx.y], blockIdx.x - 1, gridDim.x - 1, 0, nullptr);
+}
+template <class R, int A, int F, int RW> __global__ void __launch_bounds__(512, 1) k_stepB1(FlameDesc d) {
+    if (blockIdx.x == 0) return coef_cta<R>(d);
+    griddep_wait();
+    griddep_launch();
+    stepB1_body<R, A, F, RW>(d, blockIdx.x - 1);
+}
+template <class R, int A, int F, int RW> __global__ void __launch_bounds__(512, 1) k_stepB1_n(const FlameDesc *__restrict__ ds) {
+    if (blockIdx.x == 0) return coef_cta<R>(ds[blockIdx.y]);
+    stepB1_body<R, A, F, RW>(ds[blockIdx.y], blockIdx.x - 1);
+}
+
+template <class R, class V, int A, int F, bool GEN>
+__global__ void __launch_bounds__(kStepThreads<R, V>, kStepBlocks<R, V>) k_stepC(FlameDesc d, int pf) {
+    const int extra = d.tile0 == 0 ? 1 : 0;
+    if (extra && blockIdx.x == 0) return finish_cta<R, GEN>(d);
+    stepC_body<R, V, A, F, GEN>(d, blockIdx.x - extra + d.tile0, gridDim.x - extra + d.tile0, pf, nullptr);
+}
+template <class R, class V, int A, int F, bool GEN>
+__global__ void __launch_bounds__(kStepThreads<R, V>, kStepBlocks<R, V>) k_stepC_n(const FlameDesc *__restrict__ ds) {
+    if (blockIdx.x == 0) return finish_cta<R, GEN>(ds[blockIdx.y]);
+    stepC_body<R, V, A, F, GEN>(ds[blockIdx.y], blockIdx.x - 1, gridDim.x - 1, 0, nullptr);
+}
+template <class R, int A, bool GEN>
+__global__ void __launch_bounds__(256, 2) k_stepCA(FlameDesc d, int pf, const __grid_constant__ CUtensorMap tm) {
+    if (blockIdx.x == 0) return finish_cta<R, GEN>(d);
+    stepC_body<R, float2, A, 4, GEN, true>(d, blockIdx.x - 1, gridDim.x - 1, pf, &tm);
+}
+
+}  // namespace flame
