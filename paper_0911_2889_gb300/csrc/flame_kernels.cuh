@@ -1028,8 +1028,9 @@ __device__ __forceinline__ double cta_sum(double v, double *red) {
 // The extra CTA of pass C: the sum of column 0 of gk (N1 N2 times the mean of
 // |grad Phi|^2 by row sums), then the mean mode, the time and the record with
 // the area of the state entering the step (from the row-pair sums of
-// passB_area, from the separate area kernels, or NaN).
-template <class R, bool GEN> __device__ __forceinline__ void finish_cta(const FlameDesc &d) {
+// passB_area, from the separate area kernels, or NaN).  STEP: gk in the
+// layout of the step's grid (flame_step.cuh).
+template <class R, bool GEN, bool STEP = false> __device__ __forceinline__ void finish_cta(const FlameDesc &d) {
     griddep_wait();
     griddep_launch();
     using C = CplxT<R>;
@@ -1037,8 +1038,10 @@ template <class R, bool GEN> __device__ __forceinline__ void finish_cta(const Fl
     const StepArgs &a = d.a;
     const C *gk = static_cast<const C *>(d.gk);
     double v = 0.0;
-    for (int n = threadIdx.x; n < a.n1; n += blockDim.x)
-        if (FLAME_IN(d.status, gk_index(n, 0, a.n1), gk_len(a), kSiteCGk)) v += (double)__ldg(&gk[gk_index(n, 0, a.n1)].x);
+    for (int n = threadIdx.x; n < a.n1; n += blockDim.x) {
+        const size_t i = STEP ? 4 * (size_t)(n >> 1) + (n & 1) : gk_index(n, 0, a.n1);  // row n of column 0
+        if (FLAME_IN(d.status, i, gk_len(a), kSiteCGk)) v += (double)__ldg(&gk[i].x);
+    }
     const double rs = cta_sum(v, red);
     double area = __longlong_as_double(0x7ff8000000000000LL);
     if (GEN && d.rec && d.rec_area == 1) {

@@ -21,10 +21,13 @@
 //                |grad Phi|^2, its forward real transform, k2 <= K2 kept
 //   C (columns): forward transform along j1, |k1| <= K1 kept, update.
 // Layouts:
-//   uv  ((j1/2) ldk + k2) 4 + j1 % 2 (+ 2 for -k2): W of a row pair at +-k2 is
-//       one 32-byte sector in FP32 (pass A writes it), and the two rows' W at
-//       one k are 16 adjacent bytes (pass B reads them)
-//   gk  gk_index, as on the public grid.
+//   uv  per (row pair, k2): W of both rows at k2, then at -k2.  FP32: (re, re,
+//       im, im) of rows 2p, 2p+1, 16 bytes a sign, the two-line form pass B
+//       works in; FP64: (re, im) of row 2p, then of row 2p+1.  Pass A writes
+//       whole 32-byte sectors and a row pair is one contiguous block.  (With
+//       +k2 and -k2 in planes of their own pass A's tensor stores wrote half
+//       sectors: 4096x8192 40 -> 81 us.)
+//   gk  g_index
 // One extra CTA of pass B derives the step's coefficients and one of pass C
 // the mean mode and the time (coef_cta, finish_cta).
 #pragma once
@@ -47,9 +50,45 @@ template <class V, class R> __device__ __forceinline__ Planes<V> planes3(unsigne
 template <class R, class V, class PL> __host__ __device__ constexpr size_t exchange_bytes(int lines) {
     return (size_t)lines * PL::slots(kSlotsPerWave<V>) * 2 * sizeof(V);
 }
-// complex index of W(j1, k2) (W(j1, -k2) two further)
-__host__ __device__ __forceinline__ size_t w_index(int j1, int k2, int ldk) {
-    return 4 * ((size_t)(j1 >> 1) * ldk + k2) + (j1 & 1);
+// Complex index of the (row pair, k2) entry that holds row j1: 4 complex
+// numbers, two per sign.  FP32: -k2 comes first where k2 / 4 is odd, so that the
+// 16-byte reads of one sign at 8 consecutive k2 in pass B's shared memory meet
+// no bank twice.
+template <class R> __host__ __device__ __forceinline__ int w_half(int k2, bool minus) {
+    return sizeof(R) == 4 ? (int)minus ^ ((k2 >> 2) & 1) : (int)minus;
+}
+__host__ __device__ __forceinline__ size_t w_index(int j1, int k2, int ldk) { return 4 * ((size_t)(j1 >> 1) * ldk + k2); }
+// Complex index of G(j1, k2) in gk: per (column pair, row pair) rows 2p, 2p+1
+// of column 2q, then of 2q+1.  A column pair is contiguous (pass C), a row
+// pair's sector too (pass B, which parks both rows of a column at once).
+__host__ __device__ __forceinline__ size_t g_index(int j1, int k2, int n1) {
+    return 2 * (size_t)(k2 >> 1) * n1 + 4 * (j1 >> 1) + 2 * (k2 & 1) + (j1 & 1);
+}
+// W(j1, +-k2) one at a time
+template <class R> __device__ __forceinline__ void st_w(CplxT<R> *uv, int j1, int k2, int ldk, bool minus, CplxT<R> v) {
+    CplxT<R> *e = uv + w_index(j1, k2, ldk) + 2 * w_half<R>(k2, minus);
+    if constexpr (std::is_same<R, float>::value) {
+        R *f = reinterpret_cast<R *>(e) + (j1 & 1);
+        f[0] = v.x;
+        f[2] = v.y;
+    } else e[j1 & 1] = v;
+}
+template <class R> __device__ __forceinline__ CplxT<R> ld_w(const CplxT<R> *uv, int j1, int k2, int ldk, bool minus) {
+    const CplxT<R> *e = uv + w_index(j1, k2, ldk) + 2 * w_half<R>(k2, minus);
+    if constexpr (std::is_same<R, float>::value) {
+        const R *f = reinterpret_cast<const R *>(e) + (j1 & 1);
+        return CplxT<R>{__ldg(f), __ldg(f + 2)};
+    } else return __ldg(e + (j1 & 1));
+}
+// Two lines per thread: lane 0 of x is W(n, k2), lane 1 conj W(n, -k2), rows
+// 2i and 2i+1 in adjacent threads (TP is even).  One shuffle gives the even
+// thread both rows at k2 and the odd one both at -k2, as uv holds them.
+__device__ __forceinline__ float4 w_pair(CV<float2> x, bool odd) {
+    const float2 plus = make_float2(x.re.x, x.im.x), minus = make_float2(x.re.y, -x.im.y);
+    const float2 give = odd ? plus : minus;
+    const float2 got = make_float2(__shfl_xor_sync(0xffffffffu, give.x, 1), __shfl_xor_sync(0xffffffffu, give.y, 1));
+    const float2 r0 = odd ? got : plus, r1 = odd ? minus : got;
+    return make_float4(r0.x, r1.x, r0.y, r1.y);
 }
 
 // Pass A: column k2 of the box.  Two lines per thread (V = float2): lane 0 is
@@ -65,7 +104,8 @@ __device__ __forceinline__ void stepA_body(const FlameDesc &d, int tile, int nti
     extern __shared__ __align__(128) unsigned char smstep[];
     const StepArgs &a = d.a;
     const int G = blockDim.x / (PL::TS * LPC);
-    const Place s = place<PL::TS>(G * LPC), p = place<PL::TP>(G * LPC);
+    // (two lines per thread: CTAs are whole lines)
+    const Place s = NL == 2 ? place_all<PL::TS>() : place<PL::TS>(G * LPC), p = place<PL::TP>(G * LPC);
     const int ld1 = 2 * a.K1 + 1;
     const C *__restrict__ state = static_cast<const C *>(d.state);
     C *__restrict__ uv = static_cast<C *>(d.uv);
@@ -100,7 +140,7 @@ __device__ __forceinline__ void stepA_body(const FlameDesc &d, int tile, int nti
     }
     auto buf = [&](int line) { return planes3<V, R>(smstep, line, SL); };
     CV<V> xp[PL::EP];
-    inverse3<PL, true>(xs, xp, s, p, buf, tab3<R, A, F, C>(d.tw1));
+    inverse3<PL>(xs, xp, s, p, buf, tab3<R, A, F, C>(d.tw1));
     const int k2 = tile * G + p.line / LPC;
     const bool valid = p.on && k2 <= a.K2;
     if constexpr (NL == 1) {
@@ -108,23 +148,21 @@ __device__ __forceinline__ void stepA_body(const FlameDesc &d, int tile, int nti
         if (!valid) return;
 #pragma unroll
         for (int i = 0; i < PL::EP; ++i) {
-            const size_t w = w_index(p.t + i * PL::TP, k2, a.ldk) + 2 * f;
-            if (FLAME_IN(d.status, w, uv_len(a), kSiteAUv)) uv[w] = C{xp[i].re.x, f ? -xp[i].im.x : xp[i].im.x};
+            const int n = p.t + i * PL::TP;
+            if (FLAME_IN(d.status, w_index(n, k2, a.ldk) + 3, uv_len(a), kSiteAUv))
+                st_w<R>(uv, n, k2, a.ldk, f, C{xp[i].re.x, f ? -xp[i].im.x : xp[i].im.x});
         }
     } else if constexpr (TMA) {
         // The column is parked in shared memory in uv's order (32 bytes a row
         // pair) and the copy engine writes the scattered sectors.
         __syncthreads();  // the transform's last exchange has been read
-        auto park = [&](int line) { return reinterpret_cast<C *>(smstep) + (size_t)line * 2 * SL; };
-        if (p.on) {
-            C *q = park(p.line);
+        static_assert(PL::TP % 2 == 0, "row pairs in adjacent threads");
+        auto park = [&](int line) { return reinterpret_cast<float4 *>(smstep) + (size_t)line * SL; };
+        const bool odd = threadIdx.x & 1;
 #pragma unroll
-            for (int i = 0; i < PL::EP; ++i) {
-                const int n = p.t + i * PL::TP;
-                C *e = q + 4 * (n >> 1) + (n & 1);
-                e[0] = lane0<R>(xp[i]);
-                e[2] = C{xp[i].re.y, -xp[i].im.y};
-            }
+        for (int i = 0; i < PL::EP; ++i) {
+            const float4 w = w_pair(xp[i], odd);
+            if (p.on) park(p.line)[((p.t + i * PL::TP) & ~1) + w_half<R>(k2, odd)] = w;
         }
         fence_async_smem();
         __syncthreads();
@@ -136,37 +174,26 @@ __device__ __forceinline__ void stepA_body(const FlameDesc &d, int tile, int nti
 #pragma unroll 1
                 for (int p0 = 0; p0 < PL::L / 2; p0 += BP)
                     if (FLAME_IN(d.status, c, a.ldk, kSiteATma) && FLAME_IN(d.status, p0, a.n1 >> 1, kSiteATma))
-                        tma_store_3d(tm, park(s.line) + 4 * p0, 0, c, p0);
+                        tma_store_3d(tm, park(s.line) + 2 * p0, 0, c, p0);
                 bulk_commit_and_wait_read();
             }
         } else if (valid) {
-            const C *q = park(p.line);
+            const float4 *q = park(p.line);
 #pragma unroll
             for (int i = 0; i < PL::EP; ++i) {
                 const int n = p.t + i * PL::TP;
-                const size_t w = w_index(n, k2, a.ldk);
-                if (FLAME_IN(d.status, w + 2, uv_len(a), kSiteAUv)) {
-                    uv[w] = q[4 * (n >> 1) + (n & 1)];
-                    uv[w + 2] = q[4 * (n >> 1) + (n & 1) + 2];
-                }
+                const size_t w = w_index(n, k2, a.ldk) + 2 * (n & 1);  // the halves as parked
+                if (FLAME_IN(d.status, w + 1, uv_len(a), kSiteAUv)) *reinterpret_cast<float4 *>(uv + w) = q[n];
             }
         }
     } else {
-        // Threads 2i and 2i+1 hold rows 2i' and 2i'+1 (TP is even): one
-        // shuffle gives the even thread both rows' W(., k2) and the odd one
-        // both W(., -k2), 16 bytes each, together one sector.
         static_assert(PL::TP % 2 == 0, "row pairs in adjacent threads");
         const bool odd = threadIdx.x & 1;
 #pragma unroll
         for (int i = 0; i < PL::EP; ++i) {
-            const C plus = lane0<R>(xp[i]), minus{xp[i].re.y, -xp[i].im.y};
-            const C give = odd ? plus : minus;
-            const C got{__shfl_xor_sync(0xffffffffu, give.x, 1), __shfl_xor_sync(0xffffffffu, give.y, 1)};
-            const size_t w = w_index((p.t & ~1) + i * PL::TP, k2, a.ldk) + (odd ? 2 : 0);
-            if (valid && FLAME_IN(d.status, w + 1, uv_len(a), kSiteAUv)) {
-                const C r0 = odd ? got : plus, r1 = odd ? minus : got;
-                *reinterpret_cast<float4 *>(uv + w) = make_float4(r0.x, r0.y, r1.x, r1.y);
-            }
+            const float4 v = w_pair(xp[i], odd);
+            const size_t w = w_index(p.t + i * PL::TP, k2, a.ldk) + 2 * w_half<R>(k2, odd);
+            if (valid && FLAME_IN(d.status, w + 1, uv_len(a), kSiteAUv)) *reinterpret_cast<float4 *>(uv + w) = v;
         }
     }
 }
@@ -207,113 +234,145 @@ template <class V, class C> __device__ __forceinline__ void real_post(CV<V> h, C
     hi = CV<V>{vsub(E.re, Ow.re), vsub(Ow.im, E.im)};
 }
 
-// bytes of pass B's second region per row pair (two lines per thread): g of
-// one row, then G of both in the order of gk
-template <int A> __host__ __device__ constexpr size_t rows2_bytes() {
-    const size_t g = (size_t)(3 << A) * 8, G = ((size_t)(2 << A) + 2) * 16;
-    return ((g > G ? g : G) + 127) & ~(size_t)127;
+// Bulk copy of a block (16-byte aligned, a multiple of 16 bytes) from global
+// to shared memory by one thread, and the wait of all threads for it on the
+// mbarrier `bar`, which the copying thread initialises: a CTA barrier has to
+// come between.  The wait is bounded; if it runs out, the status says so.
+__device__ __forceinline__ void bulk_load(void *dst, const void *src, unsigned bytes, unsigned long long *bar) {
+    const unsigned sb = (unsigned)__cvta_generic_to_shared(bar), sd = (unsigned)__cvta_generic_to_shared(dst);
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(sb) : "memory");
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(sb), "r"(bytes) : "memory");
+    if (bytes)
+        asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(sd),
+                     "l"(reinterpret_cast<unsigned long long>(src)), "r"(bytes), "r"(sb)
+                     : "memory");
+}
+__device__ __forceinline__ void bulk_wait(unsigned long long *bar, int *status) {
+    const unsigned sb = (unsigned)__cvta_generic_to_shared(bar);
+    unsigned done = 0;
+#pragma unroll 1
+    for (int i = 0; i < (1 << 20) && !done; ++i)
+        asm volatile("{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], 0;\n\tselp.u32 %0, 1, 0, p;\n\t}"
+                     : "=r"(done) : "r"(sb) : "memory");
+    if (!done) atomicOr(status, 1 << kStatusTimeout);
 }
 
-// Pass B, two lines per thread (FP32): one row pair per group of TS threads.
-// The lanes are the even and odd points of one row in the inverse transforms
-// (row 2p, then row 2p+1, whose W were loaded with row 2p's: 16 bytes hold both),
-// and the two rows in the forward one.
+// Pass B, two lines per thread (FP32): one row pair per group of TS threads,
+// the lanes its two rows.  The even and the odd points are two inverse
+// transforms with an exchange buffer each, whose first passes run together as
+// the row pair's W come out of shared memory; the even buffer then takes g at
+// the even points, the odd one the forward transform of g, and the even one G
+// on its way out (32 bytes of gk per column and row pair: 2/3 of a buffer).
+// Bound by shared memory: of its ~8500 wavefronts a 3072-point row pair the six
+// exchanges are 4600; two CTAs of 256 threads per SM.
 template <class R, int A, bool TMA>
 __device__ __forceinline__ void stepB2_body(const FlameDesc &d, int tile, int ntiles, int pf, const CUtensorMap *tm) {
     using V = float2;
     using C = CplxT<R>;
     using PL = Plan3<A, 4>;
     constexpr int L = PL::L, TS = PL::TS, TP = PL::TP, ES = PL::ES, SL = PL::slots(kSlotsPerWave<V>);
-    constexpr size_t kEx = exchange_bytes<R, V, PL>(1), kH = rows2_bytes<A>();
     extern __shared__ __align__(128) unsigned char smstep[];
     const StepArgs &a = d.a;
     const C *__restrict__ uv = static_cast<const C *>(d.uv);
     C *__restrict__ gk = static_cast<C *>(d.gk);
     const int G = blockDim.x / TS;
-    const Place s = place<TS>(G), p = place<TP>(G);
+    const Place s = place_all<TS>(), p = place<TP>(G);
     if (threadIdx.x == 0 && pf > 0 && tile + pf < ntiles) {
         const int p0 = (tile + pf) * G, np = min(G, (a.n1 >> 1) - p0);
         if (np > 0) l2_prefetch(uv + w_index(2 * p0, 0, a.ldk), (size_t)np * 4 * a.ldk * sizeof(C));
     }
     const int pair = tile * G + s.line;
     const bool valid = s.on && pair < (a.n1 >> 1);
-    unsigned char *h_base = smstep + (size_t)G * kEx;  // kEx, kH: multiples of 128
-    auto buf = [&](int line) { return planes3<V, R>(smstep, line, SL); };
+    // The CTA's row pairs (one contiguous block) come in by one bulk copy, into
+    // the exchange buffers, which nothing uses yet.
+    __shared__ __align__(8) unsigned long long loaded;
+    if (threadIdx.x == 0) {
+        const int np = min(G, (a.n1 >> 1) - tile * G);
+        const size_t first = w_index(2 * tile * G, 0, a.ldk), len = (size_t)np * 4 * a.ldk;
+        if (FLAME_IN(d.status, first + len - 1, uv_len(a), kSiteBUv)) bulk_load(smstep, uv + first, (unsigned)(len * sizeof(C)), &loaded);
+        else bulk_load(smstep, uv, 0, &loaded);
+    }
+    auto even = [&](int line) { return planes3<V, R>(smstep, line, SL); };
+    auto odd = [&](int line) { return planes3<V, R>(smstep, G + line, SL); };
     const C *tw = tab3<R, A, 4, C>(d.twm);
     const C wt = __ldg(static_cast<const C *>(d.twm) + tw3_real_offset<A>() + s.t);  // exp(2 pi i t / 2L)
+    __syncthreads();  // the barrier's initialisation
+    bulk_wait(&loaded, d.status);
 
-    // W of both rows at n (r < 8: K2 < 2^(A+1) = 8 TS) and at n - L (r >= 4)
-    C wp[8], wm[8];  // row 2p+1's, kept through row 2p's transform
     CV<V> xs[ES];
-    auto build = [&](auto rc, C up, C um) {
-        constexpr int r = decltype(rc)::value;
-        C e, o;
-        if constexpr (r < 4) e = o = up;
-        else if constexpr (r >= 8) e = um, o = C{-um.x, -um.y};
-        else e = C{up.x + um.x, up.y + um.y}, o = C{up.x - um.x, up.y - um.y};
-        const C w = mul_root24<r, ES>(wt);
-        xs[r] = pack2<R>(e, C{fma_rn(o.x, w.x, -(o.y * w.y)), fma_rn(o.x, w.y, o.y * w.x)});
-    };
     {
-        const float4 *src = reinterpret_cast<const float4 *>(uv + w_index(2 * pair, 0, a.ldk));  // k: + at 2k, - at 2k+1
-        C up[8], um[8];
+        // W at n = t + i TS (i < 8: K2 < 2^(A+1) = 8 TS) and at n - L (n = t + (i + 4) TS), both rows
+        const float4 *src = reinterpret_cast<const float4 *>(smstep) + (size_t)s.line * 2 * a.ldk;  // two per k
+        CV<V> up[8], um[8];
 #pragma unroll
         for (int i = 0; i < 8; ++i) {
             const int n = s.t + i * TS, km = L - (s.t + (i + 4) * TS);
             float4 q = make_float4(0.f, 0.f, 0.f, 0.f), m = q;
-            if (valid && n <= a.K2 && FLAME_IN(d.status, w_index(2 * pair, n, a.ldk) + 1, uv_len(a), kSiteBUv)) q = __ldg(src + 2 * n);
-            if (valid && km <= a.K2 && FLAME_IN(d.status, w_index(2 * pair, km, a.ldk) + 3, uv_len(a), kSiteBUv)) m = __ldg(src + 2 * km + 1);
-            up[i] = C{q.x, q.y};
-            wp[i] = C{q.z, q.w};
-            um[i] = C{m.x, m.y};
-            wm[i] = C{m.z, m.w};
+            if (valid && n <= a.K2) q = src[2 * n + w_half<R>(n, false)];
+            if (valid && km <= a.K2) m = src[2 * km + w_half<R>(km, true)];
+            up[i] = CV<V>{make_float2(q.x, q.y), make_float2(q.z, q.w)};
+            um[i] = CV<V>{make_float2(m.x, m.y), make_float2(m.z, m.w)};
         }
+        __syncthreads();  // the block has been read
+        CV<V> xo[ES];
         static_for<0, ES>([&](auto rc) {
             constexpr int r = decltype(rc)::value;
-            build(rc, r < 8 ? up[r < 8 ? r : 0] : C{0, 0}, r >= 4 ? um[r >= 4 ? r - 4 : 0] : C{0, 0});
+            constexpr int ip = r < 8 ? r : 0, im = r >= 4 ? r - 4 : 0;
+            if constexpr (r < 4) xs[r] = xo[r] = up[ip];
+            else if constexpr (r >= 8) xs[r] = um[im], xo[r] = CV<V>{vneg(um[im].re), vneg(um[im].im)};
+            else xs[r] = cadd(up[ip], um[im]), xo[r] = csub(up[ip], um[im]);
         });
+        inverse3_first<PL>(xs, s, even, tw);
+        static_for<0, ES>([&](auto rc) {
+            constexpr int r = decltype(rc)::value;
+            const C w = mul_root24<r, ES>(wt);
+            xo[r] = cmul_s(xo[r], w.x, w.y);
+        });
+        inverse3_first<PL>(xo, s, odd, tw);
     }
-    CV<V> xp[PL::EP];
-    inverse3<PL, true>(xs, xp, s, p, buf, tw);
-    // g of row 2p at the points 2m, 2m+1, parked for the forward transform
-    C *hp = reinterpret_cast<C *>(h_base + (size_t)p.line * kH);
-    if (p.on) {
+    __syncthreads();
+    V g[PL::EP];  // |w|^2 at the even, then at the odd points of both rows
+    V *hp = reinterpret_cast<V *>(even(p.line).p) + p.t;
+#pragma unroll 1
+    for (int parity = 0;; ++parity) {
+        // (the loop's addresses are to be formed in it: formed before it they spill)
+        Place q = p;
+        asm volatile("" : "+r"(q.line), "+r"(q.t), "+l"(tw));
+        CV<V> xp[PL::EP];
+        inverse3_rest<PL>(xp, q, [&](int line) { return planes3<V, R>(smstep, parity * G + line, SL); }, tw);
 #pragma unroll
-        for (int i = 0; i < PL::EP; ++i) {
-            const V g = vfma(xp[i].re, xp[i].re, vmul(xp[i].im, xp[i].im));
-            hp[p.t + i * TP] = C{g.x, g.y};
+        for (int i = 0; i < PL::EP; ++i) g[i] = vfma(xp[i].re, xp[i].re, vmul(xp[i].im, xp[i].im));
+        if (parity == 1) break;
+        __syncthreads();  // the even buffers have been read
+        if (p.on) {
+#pragma unroll
+            for (int i = 0; i < PL::EP; ++i) hp[i * TP] = g[i];
         }
     }
-    static_for<0, ES>([&](auto rc) {
-        constexpr int r = decltype(rc)::value;
-        build(rc, r < 8 ? wp[r < 8 ? r : 0] : C{0, 0}, r >= 4 ? wm[r >= 4 ? r - 4 : 0] : C{0, 0});
-    });
-    inverse3<PL, false>(xs, xp, s, p, buf, tw);
+    // h[m] = g[2m] + i g[2m+1] of both rows
+    CV<V> xp[PL::EP], hk[ES];
     if (p.on) {
 #pragma unroll
-        for (int i = 0; i < PL::EP; ++i) {
-            const V g = vfma(xp[i].re, xp[i].re, vmul(xp[i].im, xp[i].im));
-            xp[i] = pack2<R>(hp[p.t + i * TP], C{g.x, g.y});  // the thread's own slots
-        }
+        for (int i = 0; i < PL::EP; ++i) xp[i] = CV<V>{hp[i * TP], g[i]};  // the thread's own slots
     }
-    forward3<PL, false>(xp, xs, p, s, buf, tw);
+    forward3<PL, false>(xp, hk, p, s, odd, tw);
     // real-input post-processing: the pairs (k, L - k), k <= L/2
     __syncthreads();
-    const Planes<V> sm = buf(s.line);
+    const Planes<V> sm = odd(s.line);
     if (s.on) {
 #pragma unroll
-        for (int r = ES / 2; r < ES; ++r) sm.st_raw(s.t + r * TS, xs[r]);
-        if (s.t == 0) sm.st_raw(0, xs[0]);
+        for (int r = ES / 2; r < ES; ++r) sm.st_raw(s.t + r * TS, hk[r]);
+        if (s.t == 0) sm.st_raw(0, hk[0]);
     }
     __syncthreads();
     const bool staged = TMA && (__cvta_generic_to_shared(smstep) & 127) == 0;
-    C *hs = reinterpret_cast<C *>(h_base + (size_t)s.line * kH);
+    float4 *hs = even(s.line).p;  // g has been read
     auto emit = [&](int k, CV<V> Y) {
-        C *dst = staged ? hs + 4 * (k >> 1) + (k & 1) : gk + gk_index(2 * pair, k, a.n1);  // row 2p+1 two further
-        if (staged || FLAME_IN(d.status, gk_index(2 * pair, k, a.n1) + 2, gk_len(a), kSiteBGk)) {
-            dst[0] = lane0<R>(Y);
-            dst[2] = lane1<R>(Y);
-        }
+        const float4 v = make_float4(Y.re.x, Y.im.x, Y.re.y, Y.im.y);  // rows 2p, 2p+1
+        if (staged) hs[k] = v;
+        else if (FLAME_IN(d.status, g_index(2 * pair, k, a.n1) + 1, gk_len(a), kSiteBGk))
+            *reinterpret_cast<float4 *>(gk + g_index(2 * pair, k, a.n1)) = v;
     };
     if (valid) {
         static_for<0, ES / 2>([&](auto rc) {
@@ -321,13 +380,13 @@ __device__ __forceinline__ void stepB2_body(const FlameDesc &d, int tile, int nt
             const int k = s.t + r * TS, kc = L - k;
             if (k <= a.K2 || kc <= a.K2) {
                 CV<V> lo, hi;
-                real_post(xs[r], sm.ld_raw(k == 0 ? 0 : kc), mul_root24<r, ES>(wt), lo, hi);
+                real_post(hk[r], sm.ld_raw(k == 0 ? 0 : kc), mul_root24<r, ES>(wt), lo, hi);
                 if (k <= a.K2) emit(k, lo);
                 if (kc <= a.K2) emit(kc, hi);
             }
         });
         // k = L/2 is its own partner: G = conj H
-        if (s.t == 0 && L / 2 <= a.K2) emit(L / 2, CV<V>{xs[ES / 2].re, vneg(xs[ES / 2].im)});
+        if (s.t == 0 && L / 2 <= a.K2) emit(L / 2, CV<V>{hk[ES / 2].re, vneg(hk[ES / 2].im)});
     }
     if constexpr (TMA) {
         if (staged) {
@@ -338,7 +397,7 @@ __device__ __forceinline__ void stepB2_body(const FlameDesc &d, int tile, int nt
 #pragma unroll 1
                 for (int q0 = 0; q0 < nq; q0 += BQ)
                     if (FLAME_IN(d.status, pair, a.n1 >> 1, kSiteBTma) && FLAME_IN(d.status, q0, (gk_len(a) / a.n1) >> 1, kSiteBTma))
-                        tma_store_3d(tm, hs + 4 * q0, 0, pair, q0);
+                        tma_store_3d(tm, hs + 2 * q0, 0, pair, q0);
                 bulk_commit_and_wait_read();
             }
         }
@@ -372,10 +431,10 @@ __device__ __forceinline__ void stepB1_body(const FlameDesc &d, int unit0) {
         for (int r = 0; r < ES; ++r) {
             const int n = s.t + r * TS, km = L - n;
             C up{0, 0}, um{0, 0};
-            if (r < 2 * F && valid && n <= a.K2 && FLAME_IN(d.status, w_index(row, n, a.ldk), uv_len(a), kSiteBUv))
-                up = __ldg(uv + w_index(row, n, a.ldk));
-            if (r >= F && valid && km <= a.K2 && FLAME_IN(d.status, w_index(row, km, a.ldk) + 2, uv_len(a), kSiteBUv))
-                um = __ldg(uv + w_index(row, km, a.ldk) + 2);
+            if (r < 2 * F && valid && n <= a.K2 && FLAME_IN(d.status, w_index(row, n, a.ldk) + 3, uv_len(a), kSiteBUv))
+                up = ld_w<R>(uv, row, n, a.ldk, false);
+            if (r >= F && valid && km <= a.K2 && FLAME_IN(d.status, w_index(row, km, a.ldk) + 3, uv_len(a), kSiteBUv))
+                um = ld_w<R>(uv, row, km, a.ldk, true);
             C z{up.x + um.x, up.y + um.y};
             if (odd) {
                 const C o{up.x - um.x, up.y - um.y}, w = __ldg(P + n);  // exp(2 pi i n / 2L)
@@ -385,7 +444,7 @@ __device__ __forceinline__ void stepB1_body(const FlameDesc &d, int unit0) {
         }
     }
     CV<V> xp[PL::EP];
-    inverse3<PL, true>(xs, xp, s, p, buf, tw);
+    inverse3<PL>(xs, xp, s, p, buf, tw);
     R *h = reinterpret_cast<R *>(smstep + (size_t)lines * SL * 2 * sizeof(R));  // g of row q at h[2 L q + j]
     if (p.on) {
 #pragma unroll
@@ -417,7 +476,7 @@ __device__ __forceinline__ void stepB1_body(const FlameDesc &d, int unit0) {
     __syncthreads();
     if (!fs.on || row >= a.n1) return;
     auto emit = [&](int k, CV<V> Y) {
-        const size_t i = gk_index(row, k, a.n1);
+        const size_t i = g_index(row, k, a.n1);
         if (FLAME_IN(d.status, i, gk_len(a), kSiteBGk)) gk[i] = C{Y.re.x, Y.im.x};
     };
 #pragma unroll
@@ -450,7 +509,7 @@ __device__ __forceinline__ void stepC_body(const FlameDesc &d, int tile, int nti
     C *__restrict__ state = static_cast<C *>(d.state);
     const C *tw = tab3<R, A, F, C>(d.tw1);
     const int G = blockDim.x / (TS * LPC);
-    const Place s = place<TS>(G * LPC), p = place<TP>(G * LPC);
+    const Place s = NL == 2 ? place_all<TS>() : place<TS>(G * LPC), p = place<TP>(G * LPC);
     const int ld1 = 2 * a.K1 + 1;
     if (threadIdx.x == 0 && pf > 0 && tile + pf < ntiles) {
         const int c = 2 * (tile + pf) * G, nc = min(2 * G, a.K2 + 1 - c);
@@ -467,15 +526,11 @@ __device__ __forceinline__ void stepC_body(const FlameDesc &d, int tile, int nti
 #pragma unroll
         for (int i = 0; i < PL::EP; ++i) {
             const int n = p.t + i * TP;
-            const bool in = p.on && c <= a.K2 &&
-                            FLAME_IN(d.status, gk_index(n, c, L) + (NL == 2 ? 1 : 0), gk_len(a), kSiteCGk);
-            if constexpr (NL == 2) {
-                const float4 q = in ? __ldg(reinterpret_cast<const float4 *>(gk + gk_index(n, c, L))) : make_float4(0.f, 0.f, 0.f, 0.f);
-                xp[i] = pack2<R>(C{q.x, q.y}, c < a.K2 ? C{q.z, q.w} : C{0, 0});
-            } else {
-                const C q = in ? __ldg(gk + gk_index(n, c, L)) : C{0, 0};
-                xp[i] = CV<V>{{q.x}, {q.y}};
-            }
+            const bool in = p.on && c <= a.K2 && FLAME_IN(d.status, g_index(n, c, L) + (NL == 2 ? 2 : 0), gk_len(a), kSiteCGk);
+            const C *q = gk + g_index(n, c, L);
+            const C q0 = in ? __ldg(q) : C{0, 0};
+            if constexpr (NL == 2) xp[i] = pack2<R>(q0, in && c < a.K2 ? __ldg(q + 2) : C{0, 0});
+            else xp[i] = CV<V>{{q0.x}, {q0.y}};
         }
     }
     auto buf = [&](int line) { return planes3<V, R>(smstep, line, SL); };
@@ -530,7 +585,8 @@ __device__ __forceinline__ void stepC_body(const FlameDesc &d, int tile, int nti
             for (int i = F; i < 2 * F; ++i)
                 if (k1_of(i) >= -a.K1 && FLAME_IN(d.status, a.K1 + k1_of(i), box_len(a), kSiteCState)) nphi[i][0] = col[k1_of(i)];
         }
-        auto park = [&](int line) { return reinterpret_cast<C *>(smstep) + (size_t)line * 2 * SL; };
+        auto park = [&](int line) { return reinterpret_cast<float4 *>(smstep) + (size_t)line * SL; };
+        const bool odd = threadIdx.x & 1;
         C *uv = static_cast<C *>(d.uv);
         const bool aligned = (__cvta_generic_to_shared(smstep) & 127) == 0;
 #pragma unroll 1
@@ -549,17 +605,13 @@ __device__ __forceinline__ void stepC_body(const FlameDesc &d, int tile, int nti
                 const C da{-f * ph.y, f * ph.x}, db{s2k2 * ph.x, s2k2 * ph.y};
                 xs[r] = pack2<R>(C{da.x - db.x, da.y - db.y}, C{da.x + db.x, da.y + db.y});
             }
-            inverse3<PL, false>(xs, xp, s, p, buf, tw);
             __syncthreads();
-            if (p.on) {
-                C *q = park(p.line);
+            inverse3<PL>(xs, xp, s, p, buf, tw);
+            __syncthreads();
 #pragma unroll
-                for (int i = 0; i < PL::EP; ++i) {
-                    const int n = p.t + i * TP;
-                    C *e = q + 4 * (n >> 1) + (n & 1);
-                    e[0] = lane0<R>(xp[i]);
-                    e[2] = C{xp[i].re.y, -xp[i].im.y};
-                }
+            for (int i = 0; i < PL::EP; ++i) {
+                const float4 w = w_pair(xp[i], odd);
+                if (p.on) park(p.line)[((p.t + i * TP) & ~1) + w_half<R>(k2, odd)] = w;
             }
             fence_async_smem();
             __syncthreads();
@@ -569,19 +621,16 @@ __device__ __forceinline__ void stepC_body(const FlameDesc &d, int tile, int nti
 #pragma unroll 1
                     for (int p0 = 0; p0 < L / 2; p0 += BP)
                         if (FLAME_IN(d.status, k2, a.ldk, kSiteCAUv) && FLAME_IN(d.status, p0, a.n1 >> 1, kSiteCAUv))
-                            tma_store_3d(tm, park(s.line) + 4 * p0, 0, k2, p0);
+                            tma_store_3d(tm, park(s.line) + 2 * p0, 0, k2, p0);
                     bulk_commit_and_wait_read();
                 }
             } else if (p.on) {
                 const int kp = 2 * (tile * G + p.line) + side;
-                const C *q = park(p.line);
+                const float4 *q = park(p.line);
                 for (int i = 0; i < PL::EP; ++i) {
                     const int n = p.t + i * TP;
-                    const size_t w = w_index(n, kp, a.ldk);
-                    if (kp <= a.K2 && FLAME_IN(d.status, w + 2, uv_len(a), kSiteCAUv)) {
-                        uv[w] = q[4 * (n >> 1) + (n & 1)];
-                        uv[w + 2] = q[4 * (n >> 1) + (n & 1) + 2];
-                    }
+                    const size_t w = w_index(n, kp, a.ldk) + 2 * (n & 1);
+                    if (kp <= a.K2 && FLAME_IN(d.status, w + 1, uv_len(a), kSiteCAUv)) *reinterpret_cast<float4 *>(uv + w) = q[n];
                 }
             }
         }
@@ -644,11 +693,16 @@ template <class R, int A> __global__ void k_twiddles3(CplxT<R> *tab) {
 // ----------------------------------------------------------------------------
 // Passes A and C of one flame may be launched over part of their tiles
 // (flame_step_host); the launch that holds tile 0 of pass C has the extra CTA.
-template <class R, class V> constexpr int kStepThreads = kLanes<V> == 2 ? 256 : 512;
-template <class R, class V> constexpr int kStepBlocks = kLanes<V> == 2 ? 2 : 1;
+// Threads of a CTA, and CTAs per SM to allot registers for: 128 registers for
+// two lines of 16 points a thread; one line of EP points takes about 4 EP
+// (FP32) or 8 EP (FP64) less than 64 besides.
+template <class R, class V, int A, int F, int LINES> constexpr int kStepThreads =
+    kLanes<V> == 2 ? 256 : (LINES * Plan3<A, F>::TS > 32 ? LINES * Plan3<A, F>::TS : 32);
+template <class R, class V, int A, int F, int LINES> constexpr int kStepBlocks =
+    kLanes<V> == 2 ? 2 : (sizeof(R) == 8 ? (F == 4 ? 512 : F == 2 ? 640 : 1024) : 1024) / kStepThreads<R, V, A, F, LINES>;
 
 template <class R, class V, int A, int F>
-__global__ void __launch_bounds__(kStepThreads<R, V>, kStepBlocks<R, V>) k_stepA(FlameDesc d, int pf) {
+__global__ void __launch_bounds__(kStepThreads<R, V, A, F, 2>, kStepBlocks<R, V, A, F, 2>) k_stepA(FlameDesc d, int pf) {
     stepA_body<R, V, A, F, false>(d, blockIdx.x + d.tile0, gridDim.x + d.tile0, pf, nullptr);
 }
 template <class R, int A>
@@ -656,7 +710,7 @@ __global__ void __launch_bounds__(256, 2) k_stepAt(FlameDesc d, int pf, const __
     stepA_body<R, float2, A, 4, true>(d, blockIdx.x + d.tile0, gridDim.x + d.tile0, pf, &tm);
 }
 template <class R, class V, int A, int F>
-__global__ void __launch_bounds__(kStepThreads<R, V>, kStepBlocks<R, V>) k_stepA_n(const FlameDesc *__restrict__ ds) {
+__global__ void __launch_bounds__(kStepThreads<R, V, A, F, 2>, kStepBlocks<R, V, A, F, 2>) k_stepA_n(const FlameDesc *__restrict__ ds) {
     stepA_body<R, V, A, F, false>(ds[blockIdx.y], blockIdx.x, gridDim.x, 0, nullptr);
 }
 
@@ -678,31 +732,35 @@ template <class R, int A> __global__ void __launch_bounds__(256, 2) k_stepB_n(co
     if (blockIdx.x == 0) return coef_cta<R>(ds[blockIdx.y]);
     stepB2_body<R, A, false>(ds[blockIdx.y], blockIdx.x - 1, gridDim.x - 1, 0, nullptr);
 }
-template <class R, int A, int F, int RW> __global__ void __launch_bounds__(512, 1) k_stepB1(FlameDesc d) {
+template <class R, int A, int F, int RW>
+__global__ void __launch_bounds__(kStepThreads<R, typename OneOf<R>::type, A, F, 2 * RW>, kStepBlocks<R, typename OneOf<R>::type, A, F, 2 * RW>)
+ k_stepB1(FlameDesc d) {
     if (blockIdx.x == 0) return coef_cta<R>(d);
     griddep_wait();
     griddep_launch();
     stepB1_body<R, A, F, RW>(d, blockIdx.x - 1);
 }
-template <class R, int A, int F, int RW> __global__ void __launch_bounds__(512, 1) k_stepB1_n(const FlameDesc *__restrict__ ds) {
+template <class R, int A, int F, int RW>
+__global__ void __launch_bounds__(kStepThreads<R, typename OneOf<R>::type, A, F, 2 * RW>, kStepBlocks<R, typename OneOf<R>::type, A, F, 2 * RW>)
+ k_stepB1_n(const FlameDesc *__restrict__ ds) {
     if (blockIdx.x == 0) return coef_cta<R>(ds[blockIdx.y]);
     stepB1_body<R, A, F, RW>(ds[blockIdx.y], blockIdx.x - 1);
 }
 
 template <class R, class V, int A, int F, bool GEN>
-__global__ void __launch_bounds__(kStepThreads<R, V>, kStepBlocks<R, V>) k_stepC(FlameDesc d, int pf) {
+__global__ void __launch_bounds__(kStepThreads<R, V, A, F, 2>, kStepBlocks<R, V, A, F, 2>) k_stepC(FlameDesc d, int pf) {
     const int extra = d.tile0 == 0 ? 1 : 0;
-    if (extra && blockIdx.x == 0) return finish_cta<R, GEN>(d);
+    if (extra && blockIdx.x == 0) return finish_cta<R, GEN, true>(d);
     stepC_body<R, V, A, F, GEN>(d, blockIdx.x - extra + d.tile0, gridDim.x - extra + d.tile0, pf, nullptr);
 }
 template <class R, class V, int A, int F, bool GEN>
-__global__ void __launch_bounds__(kStepThreads<R, V>, kStepBlocks<R, V>) k_stepC_n(const FlameDesc *__restrict__ ds) {
-    if (blockIdx.x == 0) return finish_cta<R, GEN>(ds[blockIdx.y]);
+__global__ void __launch_bounds__(kStepThreads<R, V, A, F, 2>, kStepBlocks<R, V, A, F, 2>) k_stepC_n(const FlameDesc *__restrict__ ds) {
+    if (blockIdx.x == 0) return finish_cta<R, GEN, true>(ds[blockIdx.y]);
     stepC_body<R, V, A, F, GEN>(ds[blockIdx.y], blockIdx.x - 1, gridDim.x - 1, 0, nullptr);
 }
 template <class R, int A, bool GEN>
 __global__ void __launch_bounds__(256, 2) k_stepCA(FlameDesc d, int pf, const __grid_constant__ CUtensorMap tm) {
-    if (blockIdx.x == 0) return finish_cta<R, GEN>(d);
+    if (blockIdx.x == 0) return finish_cta<R, GEN, true>(d);
     stepC_body<R, float2, A, 4, GEN, true>(d, blockIdx.x - 1, gridDim.x - 1, pf, &tm);
 }
 

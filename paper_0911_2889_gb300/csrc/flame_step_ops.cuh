@@ -61,6 +61,8 @@ static Geom geom_two_line(int a, int nlines, size_t per_line) {
     return Geom{G * T, (nlines + G - 1) / G, ((G * per_line + 127) & ~(size_t)127)};
 }
 template <int A> static size_t pair_bytes() { return exchange_bytes<float, float2, Plan3<A, 4>>(1); }
+// pass B's two-line CTA: two exchange buffers per row pair
+template <int A> static Geom geom_b2(int npairs) { return geom_two_line(A, npairs, 2 * pair_bytes<A>()); }
 // CTA of a one-line kernel: units of `lines` lines, as many as fill a warp
 template <class R, int A, int F> static Geom geom_one_line(int units, int lines, size_t extra) {
     using PL = Plan3<A, F>;
@@ -148,8 +150,8 @@ cudaError_t Ops<R>::passB(const FlameDesc &d, cudaStream_t s, int variant, const
     }
     if constexpr (sizeof(R) == 4) with_two_line(d.a.lb, [&](auto ac) {
         constexpr int A = decltype(ac)::value;
-        const Geom g = geom_two_line(A, d.a.n1 / 2, pair_bytes<A>() + rows2_bytes<A>());
-        if (variant == kVariantTmaB && gk_map) {
+        const Geom g = geom_b2<A>(d.a.n1 / 2);
+        if ((variant == kVariantTmaB || variant == kVariantTmaB4) && gk_map) {
             const int pf = resident_ctas((const void *)k_stepBt<R, A>, g);
             err = launch_s(none, k_stepBt<R, A>, dim3(g.blocks + 1), g.threads, g.smem, s, d, pf, *gk_map);
         } else {
@@ -172,7 +174,7 @@ cudaError_t Ops<R>::passB_batch(const FlameDesc *ds, int n, const StepArgs &a, c
     }
     if constexpr (sizeof(R) == 4) with_two_line(a.lb, [&](auto ac) {
         constexpr int A = decltype(ac)::value;
-        const Geom g = geom_two_line(A, n * (a.n1 / 2), pair_bytes<A>() + rows2_bytes<A>());
+        const Geom g = geom_b2<A>(n * (a.n1 / 2));
         const int G = g.threads >> (A - 2);
         err = launch_k(k_stepB_n<R, A>, dim3((a.n1 / 2 + G - 1) / G + 1, n), g.threads, g.smem, s, ds);
     });

@@ -171,6 +171,12 @@ inline int step_exponent(int K) {
 // ----------------------------------------------------------------------------
 // Passes
 // ----------------------------------------------------------------------------
+// FP32, lines of 3 * 2^8 points and more, last pass: w^q for q = 4a + b is the
+// product w^(4a) w^b of two table entries, 6 loads for radix 16 instead of 15
+// (a 3072-point line's last pass reads 9 KB of its table instead of 23).  One
+// more rounding of half an ulp; FP64, bound by its arithmetic, loads them all.
+template <class C, class PL> constexpr bool kTwiddleProducts = sizeof(C) == 8 && PL::A >= 8;
+
 // Pass S on a thread's E points x[i] = element t + i T (T = L / E): B = E / r
 // butterflies j = t + b T, twiddles, DFTs.
 template <class PL, int DIR, bool INV, int S, int E, class V, class C>
@@ -184,10 +190,23 @@ __device__ __forceinline__ void butterflies(CV<V> (&x)[E], int t, const C *__res
         if constexpr (Ns > 1) {
             const int j = t + b * T, m = Ns >= PL::L / r ? j : j % Ns;
             const C *w0 = tw + PL::template tw_offset<INV>(S) + m;
+            if constexpr (kTwiddleProducts<C, PL> && S == PL::NQ && r >= 8) {
+                C lo[4], hi = C{1, 0};  // w^1 .. w^3, w^(4a)
 #pragma unroll
-            for (int q = 1; q < r; ++q) {
-                const C w = __ldg(w0 + (q - 1) * Ns);
-                y[q] = cmul_s(y[q], w.x, DIR > 0 ? w.y : -w.y);
+                for (int q = 1; q < 4; ++q) lo[q] = __ldg(w0 + (q - 1) * Ns);
+#pragma unroll
+                for (int q = 1; q < r; ++q) {
+                    if (q % 4 == 0) hi = __ldg(w0 + (q - 1) * Ns);
+                    const C l = lo[q % 4];
+                    const C w = q < 4 ? l : q % 4 == 0 ? hi : C{hi.x * l.x - hi.y * l.y, hi.x * l.y + hi.y * l.x};
+                    y[q] = cmul_s(y[q], w.x, DIR > 0 ? w.y : -w.y);
+                }
+            } else {
+#pragma unroll
+                for (int q = 1; q < r; ++q) {
+                    const C w = __ldg(w0 + (q - 1) * Ns);
+                    y[q] = cmul_s(y[q], w.x, DIR > 0 ? w.y : -w.y);
+                }
             }
         }
         if constexpr (r % 3 == 0) dft_3f<r / 3, DIR>(y);
@@ -240,16 +259,23 @@ template <int T> __device__ __forceinline__ Place place(int lines) {
     return {line, (int)threadIdx.x % T, line < lines};
 }
 
+// ... where the CTA is `lines` lines of TS threads exactly
+template <int T> __device__ __forceinline__ Place place_all() { return {(int)threadIdx.x / T, (int)threadIdx.x % T, true}; }
+
 // Inverse transform (sign +): spectral layout xs in, physical layout xp out.
-// buf(line) is the line's exchange buffer.  FRESH: nothing reads the buffers
-// any more when the call begins.  All threads of the CTA call it.
-template <class PL, bool FRESH, class V, class C, class Buf>
-__device__ __forceinline__ void inverse3(CV<V> (&xs)[PL::ES], CV<V> (&xp)[PL::EP], Place s, Place p, Buf buf,
-                                         const C *__restrict__ tw) {
-    if (s.on) butterflies<PL, 1, true, 0>(xs, s.t, tw);
-    if constexpr (!FRESH) __syncthreads();
-    if (s.on) put<PL, true, 0>(xs, s.t, buf(s.line));
-    __syncthreads();
+// buf(line) is the line's exchange buffer; all threads of the CTA take part in
+// the barriers.  First the pass at the spectral end, stored to the buffers;
+// after a barrier, the rest.  Nothing may read the buffers any more when the
+// first begins.
+template <class PL, class V, class C, class Buf>
+__device__ __forceinline__ void inverse3_first(CV<V> (&xs)[PL::ES], Place s, Buf buf, const C *__restrict__ tw) {
+    if (s.on) {
+        butterflies<PL, 1, true, 0>(xs, s.t, tw);
+        put<PL, true, 0>(xs, s.t, buf(s.line));
+    }
+}
+template <class PL, class V, class C, class Buf>
+__device__ __forceinline__ void inverse3_rest(CV<V> (&xp)[PL::EP], Place p, Buf buf, const C *__restrict__ tw) {
     if (p.on) {
         get<PL, true, 0>(xp, p.t, buf(p.line));
         butterflies<PL, 1, true, 1>(xp, p.t, tw);
@@ -265,8 +291,16 @@ __device__ __forceinline__ void inverse3(CV<V> (&xs)[PL::ES], CV<V> (&xp)[PL::EP
         }
     });
 }
+template <class PL, class V, class C, class Buf>
+__device__ __forceinline__ void inverse3(CV<V> (&xs)[PL::ES], CV<V> (&xp)[PL::EP], Place s, Place p, Buf buf,
+                                         const C *__restrict__ tw) {
+    inverse3_first<PL>(xs, s, buf, tw);
+    __syncthreads();
+    inverse3_rest<PL>(xp, p, buf, tw);
+}
 
 // Forward transform (sign -): physical layout xp in, spectral layout xs out.
+// FRESH: nothing reads the buffers any more when the call begins.
 template <class PL, bool FRESH, class V, class C, class Buf>
 __device__ __forceinline__ void forward3(CV<V> (&xp)[PL::EP], CV<V> (&xs)[PL::ES], Place p, Place s, Buf buf,
                                          const C *__restrict__ tw) {
