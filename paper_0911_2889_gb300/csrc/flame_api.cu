@@ -160,6 +160,7 @@ struct flame_ctx {
     void *tabs;       // one allocation: the tables, rowsum, dscal and status below
     void *tw1, *twm;  // twiddle tables of the public grid's lines
     void *tw1s, *twms;  // ... and of the step grid's
+    void *kap;        // |kappa| of every box entry (FP64), else null
     void *uv, *gk;    // step workspaces
     void *spec;       // c2r workspace, N1 x (N2/2 + 1)
     void *aw;         // area / adjoint workspace, N1 x ldk pairs
@@ -237,6 +238,7 @@ template <class R> flame_status alloc_tables(flame_ctx *h) {
     CUDA_TRY(Ops<R>::init_twiddles(static_cast<C *>(h->twm), h->logm, h->cap));
     CUDA_TRY(Ops<R>::init_twiddles3(static_cast<C *>(h->tw1s), h->ss.la, h->cap));
     CUDA_TRY(Ops<R>::init_twiddles3(static_cast<C *>(h->twms), h->ss.lb, h->cap));
+    if constexpr (sizeof(R) == 8) CUDA_TRY(Ops<R>::init_kappa(static_cast<R *>(h->kap), h->ss, h->cap));
     return FLAME_OK;
 }
 
@@ -273,6 +275,7 @@ FlameDesc make_desc(flame_ctx *h, void *state, double *mean, double *t) {
     d.gk = h->gk;
     d.tw1 = h->tw1s;
     d.twm = h->twms;
+    d.kap = h->kap;
     d.t_in = t;
     d.coef = h->dscal + 8;
     d.mean = mean;
@@ -633,96 +636,76 @@ flame_status autotune(flame_ctx *h) {
     if (e == cudaSuccess) e = cudaEventCreate(&e0);
     if (e == cudaSuccess) e = cudaEventCreate(&e1);
     FlameDesc d = make_desc(h, st, sc, sc + 1);
-    // pass 0: A, 1: B, 2: C then A (variant, with its pass C), 3: C fused with A
-    auto time_it = [&](int pass, int variant, float *ms) -> cudaError_t {
-        cudaError_t r = cudaSuccess;
-        float total = 0.f;
+    // One way to run a step: 4 steps captured as a CUDA graph (the form in
+    // which flame_step runs them), the best of 3 replays after a warm-up.
+    // (Timed pass by pass, with events between the launches, the choice missed
+    // the overlap of one pass's tail with the next one's ramp: the fused
+    // column pass at 4096 x 8192, one-line rows at 1024 x 2048.)
+    auto time_steps = [&](int va, int vb, bool fuse, float *ms) -> cudaError_t {
+        h->var_a = va;
+        h->var_b = vb;
+        h->fuse = fuse;
+        d.onec = va == flame::kVariantOneLine;
+        cudaGraph_t graph = nullptr;
+        cudaGraphExec_t exec = nullptr;
+        cudaError_t r = cudaStreamBeginCapture(h->cap, cudaStreamCaptureModeThreadLocal);
+        if (r == cudaSuccess) {
+            const cudaError_t le = enqueue_scheme(h, d, kSchemeEuler, 4, h->cap);
+            r = cudaStreamEndCapture(h->cap, &graph);
+            if (r == cudaSuccess) r = le;
+        }
+        if (r == cudaSuccess) r = cudaGraphInstantiate(&exec, graph, 0);
         for (int rep = 0; rep < 4 && r == cudaSuccess; ++rep) {
             r = cudaEventRecord(e0, h->cap);
-            if (r == cudaSuccess) {
-                if (pass == 0) r = Ops<float>::passA(d, h->cap, variant, h->map());
-                else if (pass == 1) r = Ops<float>::passB(d, h->cap, variant, h->gmap());
-                else if (pass == 2) {
-                    d.onec = variant == flame::kVariantOneLine;
-                    r = Ops<float>::passC(d, h->cap);
-                    if (r == cudaSuccess) r = Ops<float>::passA(d, h->cap, variant, h->map());
-                } else {
-                    r = Ops<float>::passCA(d, h->cap, h->map());
-                }
-            }
+            if (r == cudaSuccess) r = cudaGraphLaunch(exec, h->cap);
             if (r == cudaSuccess) r = cudaEventRecord(e1, h->cap);
             if (r == cudaSuccess) r = cudaEventSynchronize(e1);
             float t = 0.f;
             if (r == cudaSuccess) r = cudaEventElapsedTime(&t, e0, e1);
-            if (rep > 0) total += t;  // the first run is the warm-up
+            if (rep > 0) *ms = std::min(*ms, t);  // the first replay is the warm-up
         }
-        *ms = total / 3.f;
+        if (exec) cudaGraphExecDestroy(exec);
+        if (graph) cudaGraphDestroy(graph);
         return r;
     };
-    // pass A variants are timed with their pass C (the one-line pass A
-    // brings the one-line pass C)
-    const int avars[3] = {flame::kVariantDirect, flame::kVariantTma, flame::kVariantOneLine};
-    const int bvars[3] = {flame::kVariantDirectB, flame::kVariantTmaB, flame::kVariantOneLineB};
-    float best_a = 1e30f, best_b = 1e30f;
-    for (int v : avars) {
-        if (v == flame::kVariantTma && !h->has_uv_map) continue;
-        if (v == flame::kVariantOneLine && h->ss.la > 9) continue;
-        float ms = 0;
-        if (e == cudaSuccess) e = time_it(2, v, &ms);
-        if (e == cudaSuccess && ms < best_a) {
-            best_a = ms;
-            h->var_a = v;
+    // two lines per thread with tensor or direct stores, one line per thread
+    // in the column passes, the row pass or both; then the fused column pass
+    const int ways[5][2] = {{flame::kVariantTma, flame::kVariantTmaB},
+                            {flame::kVariantDirect, flame::kVariantDirectB},
+                            {flame::kVariantOneLine, flame::kVariantOneLineB},
+                            {flame::kVariantOneLine, flame::kVariantTmaB},
+                            {flame::kVariantTma, flame::kVariantOneLineB}};
+    float best = 1e30f;
+    TuneChoice c{flame::kVariantDirect, flame::kVariantDirectB, 0, flame::kVariantDirect, flame::kVariantDirectB};
+    for (const auto &w : ways) {
+        const bool tma = w[0] == flame::kVariantTma || w[1] == flame::kVariantTmaB;
+        if (tma && !(h->has_uv_map && h->has_gk_map)) continue;
+        if (w[0] == flame::kVariantOneLine && h->ss.la > 9) continue;
+        if (w[1] == flame::kVariantOneLineB && h->ss.lb > 9) continue;
+        float ms = 1e30f;
+        if (e == cudaSuccess) e = time_steps(w[0], w[1], false, &ms);
+        if (e == cudaSuccess && ms < best) {
+            best = ms;
+            c.a = w[0];
+            c.b = w[1];
         }
     }
+    h->var_a = c.a;
+    if (e == cudaSuccess && fuse_allowed(h)) {
+        float ms = 1e30f;
+        e = time_steps(c.a, c.b, true, &ms);
+        c.fuse = e == cudaSuccess && ms < best;
+    }
+    h->var_a = c.a;
+    h->var_b = c.b;
+    h->fuse = c.fuse != 0;
     // the grouped launches write by direct stores, two lines per thread
-    h->var_a_bat = flame::kVariantDirect;
-    h->var_b_bat = flame::kVariantDirectB;
-    d.onec = h->var_a == flame::kVariantOneLine;
-    for (int v : bvars) {
-        if (v == flame::kVariantTmaB && !h->has_gk_map) continue;
-        if (v == flame::kVariantOneLineB && h->ss.lb > 9) continue;
-        float ms = 0;
-        if (e == cudaSuccess) e = time_it(1, v, &ms);
-        if (e == cudaSuccess && ms < best_b) {
-            best_b = ms;
-            h->var_b = v;
-        }
-    }
-    // Fused or separate column passes: each way, 4 steps captured as one CUDA
-    // graph (as flame_step runs them) and replayed; the faster is kept.
-    // (Timed launch by launch, with events between the kernels, the fused
-    // pass looked faster at 4096 x 8192; as a graph the separate passes are.)
-    if (fuse_allowed(h) && e == cudaSuccess) {
-        float ms[2] = {0.f, 0.f};
-        for (int way = 0; way < 2 && e == cudaSuccess; ++way) {
-            h->fuse = way == 1;
-            cudaGraph_t graph = nullptr;
-            cudaGraphExec_t exec = nullptr;
-            e = cudaStreamBeginCapture(h->cap, cudaStreamCaptureModeThreadLocal);
-            if (e == cudaSuccess) {
-                const cudaError_t le = enqueue_scheme(h, d, kSchemeEuler, 4, h->cap);
-                e = cudaStreamEndCapture(h->cap, &graph);
-                if (e == cudaSuccess) e = le;
-            }
-            if (e == cudaSuccess) e = cudaGraphInstantiate(&exec, graph, 0);
-            for (int rep = 0; rep < 4 && e == cudaSuccess; ++rep) {
-                e = cudaEventRecord(e0, h->cap);
-                if (e == cudaSuccess) e = cudaGraphLaunch(exec, h->cap);
-                if (e == cudaSuccess) e = cudaEventRecord(e1, h->cap);
-                if (e == cudaSuccess) e = cudaEventSynchronize(e1);
-                float t = 0.f;
-                if (e == cudaSuccess) e = cudaEventElapsedTime(&t, e0, e1);
-                if (rep > 0) ms[way] += t;  // the first replay is the warm-up
-            }
-            if (exec) cudaGraphExecDestroy(exec);
-            if (graph) cudaGraphDestroy(graph);
-        }
-        h->fuse = e == cudaSuccess && ms[1] < ms[0];
-    }
+    h->var_a_bat = c.a_bat;
+    h->var_b_bat = c.b_bat;
     cleanup();
     if (e != cudaSuccess) return fail(FLAME_ECUDA, "autotune: %s", cudaGetErrorString(e));
     std::lock_guard<std::mutex> lk(g_tune_mu);
-    g_tune[key] = TuneChoice{h->var_a, h->var_b, h->fuse ? 1 : 0, h->var_a_bat, h->var_b_bat};
+    g_tune[key] = c;
     if (!fkey.empty()) {
         auto m = read_tune_file(cache_path);
         m[fkey] = g_tune[key];
@@ -901,7 +884,7 @@ flame_status flame_create(const flame_params *params, flame_t *out) {
     };
     const size_t o_tw1 = place(flame::tw_alloc_len(h->logn1) * h->csz), o_twm = place(flame::tw_alloc_len(h->logm) * h->csz),
                  o_tw1s = place(flame::tw3_len_of(h->ss.la) * h->csz), o_twms = place(flame::tw3_len_of(h->ss.lb) * h->csz),
-                 o_rowsum = place(n1 * sizeof(double)), o_dscal = place(24 * sizeof(double)),
+                 o_kap = place(p.prec == FLAME_FP64 ? (2 * (size_t)p.K1 + 1) * ldk * sizeof(double) : 0), o_rowsum = place(n1 * sizeof(double)), o_dscal = place(24 * sizeof(double)),
                  o_status = place(flame::kStatusWords * sizeof(int));
     bool ok = dev_alloc(&h->tabs, tabs) && dev_alloc(&h->uv, n1 * ldk * 2 * h->csz) &&
               dev_alloc(&h->gk, n1 * ((ldk + 1) & ~(size_t)1) * h->csz) && dev_alloc(&h->spec, n1 * m1 * h->csz) &&
@@ -916,6 +899,7 @@ flame_status flame_create(const flame_params *params, flame_t *out) {
     h->twm = tb + o_twm;
     h->tw1s = tb + o_tw1s;
     h->twms = tb + o_twms;
+    h->kap = p.prec == FLAME_FP64 ? tb + o_kap : nullptr;
     h->rowsum = reinterpret_cast<double *>(tb + o_rowsum);
     h->dscal = reinterpret_cast<double *>(tb + o_dscal);
     h->status = reinterpret_cast<int *>(tb + o_status);

@@ -101,6 +101,7 @@ struct FlameDesc {
     void *gk;               // N1 x ldk workspace
     const void *tw1;        // twiddles of length N1
     const void *twm;        // twiddles of length N2/2 (+ real table)
+    const void *kap;        // |kappa| of every box entry (FP64 handles) or null: pass C forms it
     const double *t_in;     // caller's t (read by pass B)
     // the step's coefficients, derived from t once by pass B and read by pass
     // C: [0] t_n, [1] c = 1/(2 r0^2), then from byte 16 the kernel-precision
@@ -195,6 +196,7 @@ template <class R> struct Ops {
     // variant: kVariant*; the maps (encode_uv_map, encode_gk_map of d.uv, d.gk)
     // are needed by the tensor-store variants only.
     static cudaError_t init_twiddles3(C *tab, int a, cudaStream_t s);
+    static cudaError_t init_kappa(R *kap, const StepArgs &a, cudaStream_t s);
     static cudaError_t passA(const FlameDesc &d, cudaStream_t s, int variant = 0, const CUtensorMap *uv_map = nullptr);
     static cudaError_t passB(const FlameDesc &d, cudaStream_t s, int variant = 0, const CUtensorMap *gk_map = nullptr);
     static cudaError_t passC(const FlameDesc &d, cudaStream_t s);

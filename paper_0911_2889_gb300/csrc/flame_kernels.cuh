@@ -169,6 +169,25 @@ __global__ void k_box_from_spec(const CplxT<R> *__restrict__ spec, CplxT<R> *__r
     }
 }
 
+// |kappa| = sqrt((s1 k1)^2 + (s2 k2)^2) for (k1, k2) != 0.  FP32: x times the
+// hardware reciprocal square root (within a few ulp, far inside the FP32
+// path's per-step tolerance); FP64: the correctly rounded square root.
+template <class R> __device__ __forceinline__ R kappa_norm(R s1k1, R s2k2) {
+    if constexpr (std::is_same<R, float>::value) {
+        const float x = fmaf(s1k1, s1k1, s2k2 * s2k2);
+        return x * rsqrtf(x);
+    } else {
+        return sqrt(fma(s1k1, s1k1, s2k2 * s2k2));
+    }
+}
+
+// |kappa| of every box entry, the table of FlameDesc::kap
+template <class R> __global__ void k_kappa(R *kap, StepArgs a) {
+    const int ld1 = 2 * a.K1 + 1;
+    for (long i = blockIdx.x * (long)blockDim.x + threadIdx.x; i < (long)ld1 * a.ldk; i += (long)gridDim.x * blockDim.x)
+        kap[i] = kappa_norm<R>(scale1<R>(a) * (R)((int)(i % ld1) - a.K1), scale2<R>(a) * (R)(int)(i / ld1));
+}
+
 // ----------------------------------------------------------------------------
 // Twiddle table generation (FP64 sincospi, rounded once)
 // ----------------------------------------------------------------------------
@@ -362,7 +381,10 @@ __device__ __forceinline__ void l2_prefetch(const void *begin, size_t bytes) {
 
 // Programmatic dependent launch: wait until the previous kernel on the
 // stream has completed and its memory is visible (a no-op when the launch is
-// an ordinary one), and let the next kernel's CTAs be scheduled.
+// an ordinary one), and let the next kernel's CTAs be scheduled once every CTA
+// of this one has said so.  Said behind the transform: said at the top, the
+// next kernel's waiting CTAs took the SMs from this one's later waves (512x1024
+// 15.4 -> 19.7 us a step).
 __device__ __forceinline__ void griddep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void griddep_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
@@ -479,7 +501,6 @@ template <class R, int LOG, bool TMA = false>
 __device__ __forceinline__ void passA_body(const FlameDesc &d, int tile, int ntiles, int pf,
                                            const CUtensorMap *tm = nullptr) {
     griddep_wait();
-    griddep_launch();
     using V = typename VecOf<R>::type;
     using C = CplxT<R>;
     constexpr int E = 16;
@@ -521,6 +542,7 @@ __device__ __forceinline__ void passA_body(const FlameDesc &d, int tile, int nti
         }
     }
     fft_line<1, LOG>(x, a.logn1, t, sm, tw1);
+    griddep_launch();
     if constexpr (TMA && std::is_same<R, float>::value && LOG > 0) {
         // Park (U, V) of this column at row n (16 bytes per row: the order of
         // a column of the interleaved uv, row pair by row pair), then the
@@ -659,7 +681,6 @@ template <class F> __device__ __forceinline__ F group_sum(F v, int T, F *scratch
 template <class R, int LOG, int E>
 __device__ __forceinline__ void passB_area_body(const FlameDesc &d, int tile) {
     griddep_wait();
-    griddep_launch();
     using V = typename VecOf<R>::type;
     using C = CplxT<R>;
     extern __shared__ __align__(16) unsigned char smraw[];
@@ -847,6 +868,7 @@ __device__ __forceinline__ void passB_area_body(const FlameDesc &d, int tile) {
         x[r] = pack2<R>(h_first[t + r * T], C{sq.x, sq.y});
     }
     fft(std::integral_constant<int, -1>{}, x);
+    griddep_launch();
     __syncthreads();
     // the post-processing of k in [0, M/2) reads H[M - k]: only H[0] and the
     // upper half (registers r >= E/2) go to shared memory
@@ -884,18 +906,6 @@ __device__ __forceinline__ double radd(double a, double b) { return __dadd_rn(a,
 __device__ __forceinline__ float rfma(float a, float b, float c) { return __fmaf_rn(a, b, c); }
 __device__ __forceinline__ double rfma(double a, double b, double c) { return __fma_rn(a, b, c); }
 
-// |kappa| = sqrt((s1 k1)^2 + (s2 k2)^2) for (k1, k2) != 0.  FP32: x times the
-// hardware reciprocal square root (within a few ulp, far inside the FP32
-// path's per-step tolerance); FP64: the correctly rounded square root.
-template <class R> __device__ __forceinline__ R kappa_norm(R s1k1, R s2k2) {
-    if constexpr (std::is_same<R, float>::value) {
-        const float x = fmaf(s1k1, s1k1, s2k2 * s2k2);
-        return x * rsqrtf(x);
-    } else {
-        return sqrt(fma(s1k1, s1k1, s2k2 * s2k2));
-    }
-}
-
 // Pass C's epilogue, shared by its kernels: the update of one box entry
 // (a8..a10), the area of the state entering the step for the record, and
 // the mean mode, time and record written by thread 0 of tile 0.
@@ -921,14 +931,18 @@ __device__ __forceinline__ void update_entry(const FlameDesc &d, const EpiArgs<R
     using C = CplxT<R>;
     const StepArgs &a = d.a;
     nw = C{0, 0};
-    [[maybe_unused]] const long long bi = (long long)k2 * (2 * a.K1 + 1) + a.K1 + k1;  // box index of (k1, k2)
+    const long long bi = (long long)k2 * (2 * a.K1 + 1) + a.K1 + k1;  // box index of (k1, k2)
     if (!FLAME_IN(d.status, bi, box_len(a), kSiteCState)) return;
     if (k1 == 0 && k2 == 0) {
         col[0] = C{0, 0};
         return;
     }
     const R rdt = e.cf.dt;
-    const R kap = kappa_norm<R>(rmul(e.s1, (R)k1), rmul(e.s2, (R)k2));
+    // FP64: from the handle's table where there is one (a correctly rounded
+    // square root is some 25 of the entry's 40 FP64 instructions)
+    R kap;
+    if (sizeof(R) == 8 && d.kap) kap = static_cast<const R *>(d.kap)[bi];
+    else kap = kappa_norm<R>(rmul(e.s1, (R)k1), rmul(e.s2, (R)k2));
     const R om = e.lin ? rmul(kap, rfma(-kap, e.cf.a, e.cf.b)) : (R)0;
     const R cn = e.nl ? e.cf.cs : (R)0;
     // the non-stiff part: c ghat (+ the forcing f_k)
@@ -1065,7 +1079,6 @@ template <class R, bool GEN, bool STEP = false> __device__ __forceinline__ void 
 template <class R, int LOG>
 __device__ __forceinline__ void passC_body(const FlameDesc &d, int tile, int ntiles, int pf) {
     griddep_wait();
-    griddep_launch();
     using V = typename VecOf<R>::type;
     using C = CplxT<R>;
     constexpr bool GEN = true;
@@ -1112,6 +1125,7 @@ __device__ __forceinline__ void passC_body(const FlameDesc &d, int tile, int nti
     // (k1 = n - N1) of columns c0 and c0 + 1
     C *sa = state + (size_t)c0 * ld1 + a.K1, *sb = sa + ld1;
     fft_line<-1, LOG>(x, a.logn1, t, sm, tw1);
+    griddep_launch();
 
     // the state entries, read after the transform (they are L2-resident in
     // the persisting window; holding them across the transform cost more)
@@ -1175,7 +1189,6 @@ template <int E> __host__ __device__ constexpr int tw_offset_e(int log) {
 // (U, V) entries of the column.
 template <class R, int LOG, int E> __device__ __forceinline__ void passA1_body(const FlameDesc &d, int k2) {
     griddep_wait();
-    griddep_launch();
     using C = CplxT<R>;
     using V1 = typename OneOf<R>::type;
     extern __shared__ __align__(16) unsigned char smraw[];
@@ -1205,6 +1218,7 @@ template <class R, int LOG, int E> __device__ __forceinline__ void passA1_body(c
         }
     }
     line_fft_ct<1, LOG, E>(x, t, sm, tw, CtaBarrier{});
+    griddep_launch();
     if (!valid) return;
     C *uv = static_cast<C *>(d.uv);
     const R s2k2 = scale2<R>(a) * (R)k2;
@@ -1220,7 +1234,6 @@ template <class R, int LOG, int E> __device__ __forceinline__ void passA1_body(c
 // transform of column k2 of gk and the update of its box entries.
 template <class R, int LOG, int E> __device__ __forceinline__ void passC1_body(const FlameDesc &d, int tile) {
     griddep_wait();
-    griddep_launch();
     using C = CplxT<R>;
     using V1 = typename OneOf<R>::type;
     constexpr bool GEN = true;
@@ -1245,6 +1258,7 @@ template <class R, int LOG, int E> __device__ __forceinline__ void passC1_body(c
         x[r] = CV<V1>{{p.x}, {p.y}};
     }
     line_fft_ct<-1, LOG, E>(x, t, sm, tw, CtaBarrier{});
+    griddep_launch();
     const bool lin = !(a.flags & kNonlinearOnly), nl = !(a.flags & kLinearOnly);
     const int stage = GEN ? d.stage : kStageEuler;
     const EpiArgs<R> ea{cfs, scale1<R>(a), scale2<R>(a), stage, lin, nl};

@@ -69,12 +69,17 @@ static int resident_ctas(const void *kernel, const Geom &g) {
 // scheduled while the previous kernel on the stream drains, and wait in
 // hardware (griddepcontrol.wait, the first statement of every step pass's
 // body) until that kernel has completed and its memory is visible.  Only
-// the step passes, whose bodies begin with that wait, are launched so.
-// Opt-in (FLAME_PDL=1): at 4096 x 8192 the graph-captured steps measured
-// 0.2026 ms per step with it against 0.1967 ms without.
-static bool pdl_on() {
+// the step passes, whose bodies begin with that wait, are launched so: in FP32,
+// and in FP64 for columns of up to 96 points (N1 <= 128).  Per step (graph):
+// FP32 256x512 9.5 -> 8.1 us, 1024x2048 18.1 -> 17.0, 4096x8192 level; FP64
+// 128x256 23.5 -> 22.1, but 512x1024 77.4 -> 83.5: the early CTAs land where
+// SMs drain first, and longer FP64 passes are bound by their fullest SM.
+// Not for ensembles (96 flames: 7.2 against 7.7 ms with it): their launches fill
+// the GPU many times over.  FLAME_PDL=0 or 1: none or all of the others.
+static bool pdl_on(bool fp64, const StepArgs &a) {
     const char *v = getenv("FLAME_PDL");
-    return v && strcmp(v, "1") == 0;
+    if (v && (strcmp(v, "0") == 0 || strcmp(v, "1") == 0)) return v[0] == '1';
+    return !fp64 || a.la <= 5;
 }
 template <class... KArgs, class... Args>
 static cudaError_t launch_x(const L2Window &w, bool pdl, void (*kernel)(KArgs...), dim3 grid, int threads,
@@ -115,11 +120,11 @@ static cudaError_t launch_w(const L2Window &w, void (*kernel)(KArgs...), dim3 gr
                             cudaStream_t s, Args... args) {
     return launch_x(w, false, kernel, grid, threads, smem, s, args...);
 }
-// a step pass of one flame: L2 window and programmatic dependent launch
+// a step pass: L2 window and programmatic dependent launch
 template <class... KArgs, class... Args>
-static cudaError_t launch_s(const L2Window &w, void (*kernel)(KArgs...), dim3 grid, int threads, size_t smem,
+static cudaError_t launch_s(const L2Window &w, bool pdl, void (*kernel)(KArgs...), dim3 grid, int threads, size_t smem,
                             cudaStream_t s, Args... args) {
-    return launch_x(w, pdl_on(), kernel, grid, threads, smem, s, args...);
+    return launch_x(w, pdl, kernel, grid, threads, smem, s, args...);
 }
 template <class... KArgs, class... Args>
 static cudaError_t launch_k(void (*kernel)(KArgs...), dim3 grid, int threads, size_t smem, cudaStream_t s,

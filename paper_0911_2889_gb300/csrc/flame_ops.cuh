@@ -171,7 +171,7 @@ cudaError_t Ops<R>::passA_full(const FlameDesc &d, cudaStream_t s, bool pairs, c
             static_for<4, 8>([&](auto lc) {
                 constexpr int L = decltype(lc)::value;
                 if (d.a.logn1 == L)
-                    err = launch_s(d.l2_state, k_passA1<R, L, E>, dim3(g.blocks), g.threads, g.smem, s, d);
+                    err = launch_w(d.l2_state, k_passA1<R, L, E>, dim3(g.blocks), g.threads, g.smem, s, d);
             });
         });
         return err;
@@ -181,7 +181,7 @@ cudaError_t Ops<R>::passA_full(const FlameDesc &d, cudaStream_t s, bool pairs, c
         static_for<8, 11>([&](auto lc) {
             constexpr int L = decltype(lc)::value;
             if (d.a.logn1 == L)
-                err = launch_s(d.l2_state, k_passA1<R, L, 16>, dim3(g.blocks), g.threads, g.smem, s, d);
+                err = launch_w(d.l2_state, k_passA1<R, L, 16>, dim3(g.blocks), g.threads, g.smem, s, d);
         });
         return err;
     }
@@ -190,11 +190,11 @@ cudaError_t Ops<R>::passA_full(const FlameDesc &d, cudaStream_t s, bool pairs, c
         constexpr int L = decltype(lc)::value;
         if constexpr (sizeof(R) == 4 && L > 0) if (uv_map) {  // tensor-store write-out
             const int pf = resident_ctas((const void *)k_passAt<R, L>, g);
-            err = launch_s(d.l2_state, k_passAt<R, L>, dim3(g.blocks), g.threads, g.smem, s, d, pf, *uv_map);
+            err = launch_w(d.l2_state, k_passAt<R, L>, dim3(g.blocks), g.threads, g.smem, s, d, pf, *uv_map);
             return;
         }
         const int pf = resident_ctas((const void *)k_passA<R, L>, g);
-        err = launch_s(d.l2_state, k_passA<R, L>, dim3(g.blocks), g.threads, g.smem, s, d, pf);
+        err = launch_w(d.l2_state, k_passA<R, L>, dim3(g.blocks), g.threads, g.smem, s, d, pf);
     });
     return err;
 }
@@ -274,7 +274,7 @@ template <class R> cudaError_t Ops<R>::passC_full(const FlameDesc &d, cudaStream
             static_for<4, 8>([&](auto lc) {
                 constexpr int L = decltype(lc)::value;
                 if (d.a.logn1 == L)
-                    err = launch_s(d.l2_state, k_passC1<R, L, E>, dim3(g.blocks + 1), g.threads, g.smem, s, d);
+                    err = launch_w(d.l2_state, k_passC1<R, L, E>, dim3(g.blocks + 1), g.threads, g.smem, s, d);
             });
         });
         return err;
@@ -284,7 +284,7 @@ template <class R> cudaError_t Ops<R>::passC_full(const FlameDesc &d, cudaStream
         static_for<8, 11>([&](auto lc) {
             constexpr int L = decltype(lc)::value;
             if (d.a.logn1 == L)
-                err = launch_s(d.l2_state, k_passC1<R, L, 16>, dim3(g.blocks + 1), g.threads, g.smem, s, d);
+                err = launch_w(d.l2_state, k_passC1<R, L, 16>, dim3(g.blocks + 1), g.threads, g.smem, s, d);
         });
         return err;
     }
@@ -292,7 +292,7 @@ template <class R> cudaError_t Ops<R>::passC_full(const FlameDesc &d, cudaStream
     with_log<R>(d.a.logn1, [&](auto lc) {
         constexpr int L = decltype(lc)::value;
         const int pf = resident_ctas((const void *)k_passC<R, L>, g);
-        err = launch_s(d.l2_state, k_passC<R, L>, dim3(g.blocks + 1), g.threads, g.smem, s, d, pf);
+        err = launch_w(d.l2_state, k_passC<R, L>, dim3(g.blocks + 1), g.threads, g.smem, s, d, pf);
     });
     return err;
 }

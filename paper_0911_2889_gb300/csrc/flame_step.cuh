@@ -64,21 +64,23 @@ __host__ __device__ __forceinline__ size_t w_index(int j1, int k2, int ldk) { re
 __host__ __device__ __forceinline__ size_t g_index(int j1, int k2, int n1) {
     return 2 * (size_t)(k2 >> 1) * n1 + 4 * (j1 >> 1) + 2 * (k2 & 1) + (j1 & 1);
 }
-// W(j1, +-k2) one at a time
-template <class R> __device__ __forceinline__ void st_w(CplxT<R> *uv, int j1, int k2, int ldk, bool minus, CplxT<R> v) {
-    CplxT<R> *e = uv + w_index(j1, k2, ldk) + 2 * w_half<R>(k2, minus);
-    if constexpr (std::is_same<R, float>::value) {
-        R *f = reinterpret_cast<R *>(e) + (j1 & 1);
-        f[0] = v.x;
-        f[2] = v.y;
-    } else e[j1 & 1] = v;
-}
+// W(j1, +-k2) of one row
 template <class R> __device__ __forceinline__ CplxT<R> ld_w(const CplxT<R> *uv, int j1, int k2, int ldk, bool minus) {
     const CplxT<R> *e = uv + w_index(j1, k2, ldk) + 2 * w_half<R>(k2, minus);
     if constexpr (std::is_same<R, float>::value) {
-        const R *f = reinterpret_cast<const R *>(e) + (j1 & 1);
-        return CplxT<R>{__ldg(f), __ldg(f + 2)};
+        const float4 q = __ldg(reinterpret_cast<const float4 *>(e));
+        return j1 & 1 ? CplxT<R>{q.y, q.w} : CplxT<R>{q.x, q.z};
     } else return __ldg(e + (j1 & 1));
+}
+// ... written by two adjacent threads, rows 2i and 2i+1 (all threads call it):
+// FP32, one shuffle, and each thread writes 8 of the 16 bytes
+template <class R> __device__ __forceinline__ void st_w(CplxT<R> *uv, int j1, int k2, int ldk, bool minus, CplxT<R> v, bool on) {
+    CplxT<R> *e = uv + w_index(j1, k2, ldk) + 2 * w_half<R>(k2, minus);
+    if constexpr (std::is_same<R, float>::value) {
+        const bool odd = j1 & 1;
+        const R got = __shfl_xor_sync(0xffffffffu, odd ? v.x : v.y, 1);
+        if (on) e[odd] = odd ? CplxT<R>{got, v.y} : CplxT<R>{v.x, got};
+    } else if (on) e[j1 & 1] = v;
 }
 // Two lines per thread: lane 0 of x is W(n, k2), lane 1 conj W(n, -k2), rows
 // 2i and 2i+1 in adjacent threads (TP is even).  One shuffle gives the even
@@ -91,13 +93,31 @@ __device__ __forceinline__ float4 w_pair(CV<float2> x, bool odd) {
     return make_float4(r0.x, r1.x, r0.y, r1.y);
 }
 
+// The tile that starts when this one ends, `by` tiles further (the CTAs
+// resident at once; 0: no prefetch), in this flame or, in an ensemble's
+// launch, a later one: its input is prefetched into L2, behind this tile's own
+// loads.
+struct Ahead {
+    int by, ntiles;
+    const FlameDesc *ds;  // ensemble: its descriptors (flame = blockIdx.y), else null
+    template <class Fn> __device__ __forceinline__ void run(const FlameDesc &d, int tile, Fn prefetch) const {
+        if (threadIdx.x != 0 || by <= 0) return;
+        const int t = tile + by;
+        if (!ds) {
+            if (t < ntiles) prefetch(d, t);
+        } else {
+            const int f = (int)blockIdx.y + t / ntiles;
+            if (f < (int)gridDim.y) prefetch(ds[f], t % ntiles);
+        }
+    }
+};
+
 // Pass A: column k2 of the box.  Two lines per thread (V = float2): lane 0 is
 // W(., k2), lane 1 conj W(., -k2); one line per thread: lines 2u and 2u+1 of
 // the CTA are the two of its column u.
 template <class R, class V, int A, int F, bool TMA>
-__device__ __forceinline__ void stepA_body(const FlameDesc &d, int tile, int ntiles, int pf, const CUtensorMap *tm) {
+__device__ __forceinline__ void stepA_body(const FlameDesc &d, int tile, const Ahead &ahead, const CUtensorMap *tm) {
     griddep_wait();
-    griddep_launch();
     using C = CplxT<R>;
     using PL = Plan3<A, F>;
     constexpr int NL = kLanes<V>, LPC = 2 / NL, SL = PL::slots(kSlotsPerWave<V>);
@@ -109,10 +129,6 @@ __device__ __forceinline__ void stepA_body(const FlameDesc &d, int tile, int nti
     const int ld1 = 2 * a.K1 + 1;
     const C *__restrict__ state = static_cast<const C *>(d.state);
     C *__restrict__ uv = static_cast<C *>(d.uv);
-    if (threadIdx.x == 0 && pf > 0 && tile + pf < ntiles) {
-        const int c = (tile + pf) * G, nc = min(G, a.K2 + 1 - c);
-        if (nc > 0) l2_prefetch(state + (size_t)c * ld1, (size_t)nc * ld1 * sizeof(C));
-    }
     CV<V> xs[PL::ES];
     {
         const int k2 = tile * G + s.line / LPC;
@@ -138,19 +154,38 @@ __device__ __forceinline__ void stepA_body(const FlameDesc &d, int tile, int nti
             }
         }
     }
+    ahead.run(d, tile, [&](const FlameDesc &q, int t) {  // that tile's columns
+        const int c = t * G, nc = min(G, q.a.K2 + 1 - c);
+        if (nc > 0) l2_prefetch(static_cast<const C *>(q.state) + (size_t)c * ld1, (size_t)nc * ld1 * sizeof(C));
+    });
     auto buf = [&](int line) { return planes3<V, R>(smstep, line, SL); };
     CV<V> xp[PL::EP];
     inverse3<PL>(xs, xp, s, p, buf, tab3<R, A, F, C>(d.tw1));
+    griddep_launch();
     const int k2 = tile * G + p.line / LPC;
     const bool valid = p.on && k2 <= a.K2;
     if constexpr (NL == 1) {
         const int f = p.line & 1;
-        if (!valid) return;
+        if constexpr (PL::TP % 2 == 0) {
 #pragma unroll
-        for (int i = 0; i < PL::EP; ++i) {
-            const int n = p.t + i * PL::TP;
-            if (FLAME_IN(d.status, w_index(n, k2, a.ldk) + 3, uv_len(a), kSiteAUv))
-                st_w<R>(uv, n, k2, a.ldk, f, C{xp[i].re.x, f ? -xp[i].im.x : xp[i].im.x});
+            for (int i = 0; i < PL::EP; ++i) {
+                const int n = p.t + i * PL::TP;
+                const bool on = valid && FLAME_IN(d.status, w_index(n, k2, a.ldk) + 3, uv_len(a), kSiteAUv);
+                st_w<R>(uv, n, k2, a.ldk, f, C{xp[i].re.x, f ? -xp[i].im.x : xp[i].im.x}, on);
+            }
+        } else if (valid) {  // lines of 12 F points: rows one by one
+#pragma unroll
+            for (int i = 0; i < PL::EP; ++i) {
+                const int n = p.t + i * PL::TP;
+                if (!FLAME_IN(d.status, w_index(n, k2, a.ldk) + 3, uv_len(a), kSiteAUv)) continue;
+                C *e = uv + w_index(n, k2, a.ldk) + 2 * w_half<R>(k2, f);
+                const C v{xp[i].re.x, f ? -xp[i].im.x : xp[i].im.x};
+                if constexpr (sizeof(R) == 4) {
+                    R *w = reinterpret_cast<R *>(e) + (n & 1);
+                    w[0] = v.x;
+                    w[2] = v.y;
+                } else e[n & 1] = v;
+            }
         }
     } else if constexpr (TMA) {
         // The column is parked in shared memory in uv's order (32 bytes a row
@@ -267,7 +302,7 @@ __device__ __forceinline__ void bulk_wait(unsigned long long *bar, int *status) 
 // Bound by shared memory: of its ~8500 wavefronts a 3072-point row pair the six
 // exchanges are 4600; two CTAs of 256 threads per SM.
 template <class R, int A, bool TMA>
-__device__ __forceinline__ void stepB2_body(const FlameDesc &d, int tile, int ntiles, int pf, const CUtensorMap *tm) {
+__device__ __forceinline__ void stepB2_body(const FlameDesc &d, int tile, const Ahead &ahead, const CUtensorMap *tm) {
     using V = float2;
     using C = CplxT<R>;
     using PL = Plan3<A, 4>;
@@ -278,10 +313,6 @@ __device__ __forceinline__ void stepB2_body(const FlameDesc &d, int tile, int nt
     C *__restrict__ gk = static_cast<C *>(d.gk);
     const int G = blockDim.x / TS;
     const Place s = place_all<TS>(), p = place<TP>(G);
-    if (threadIdx.x == 0 && pf > 0 && tile + pf < ntiles) {
-        const int p0 = (tile + pf) * G, np = min(G, (a.n1 >> 1) - p0);
-        if (np > 0) l2_prefetch(uv + w_index(2 * p0, 0, a.ldk), (size_t)np * 4 * a.ldk * sizeof(C));
-    }
     const int pair = tile * G + s.line;
     const bool valid = s.on && pair < (a.n1 >> 1);
     // The CTA's row pairs (one contiguous block) come in by one bulk copy, into
@@ -293,6 +324,10 @@ __device__ __forceinline__ void stepB2_body(const FlameDesc &d, int tile, int nt
         if (FLAME_IN(d.status, first + len - 1, uv_len(a), kSiteBUv)) bulk_load(smstep, uv + first, (unsigned)(len * sizeof(C)), &loaded);
         else bulk_load(smstep, uv, 0, &loaded);
     }
+    ahead.run(d, tile, [&](const FlameDesc &q, int t) {  // that tile's row pairs
+        const int p0 = t * G, np = min(G, (q.a.n1 >> 1) - p0);
+        if (np > 0) l2_prefetch(static_cast<const C *>(q.uv) + w_index(2 * p0, 0, q.a.ldk), (size_t)np * 4 * q.a.ldk * sizeof(C));
+    });
     auto even = [&](int line) { return planes3<V, R>(smstep, line, SL); };
     auto odd = [&](int line) { return planes3<V, R>(smstep, G + line, SL); };
     const C *tw = tab3<R, A, 4, C>(d.twm);
@@ -357,6 +392,7 @@ __device__ __forceinline__ void stepB2_body(const FlameDesc &d, int tile, int nt
         for (int i = 0; i < PL::EP; ++i) xp[i] = CV<V>{hp[i * TP], g[i]};  // the thread's own slots
     }
     forward3<PL, false>(xp, hk, p, s, odd, tw);
+    griddep_launch();
     // real-input post-processing: the pairs (k, L - k), k <= L/2
     __syncthreads();
     const Planes<V> sm = odd(s.line);
@@ -463,6 +499,7 @@ __device__ __forceinline__ void stepB1_body(const FlameDesc &d, int unit0) {
         }
     }
     forward3<PL, true>(xp, xs, fp, fs, buf, tw);
+    griddep_launch();
     __syncthreads();
     const int row = first + fs.line;
     const Planes<V> sm = buf(fs.line);
@@ -496,9 +533,8 @@ __device__ __forceinline__ void stepB1_body(const FlameDesc &d, int unit0) {
 // 2u, 2u+1 of the CTA.  FUSE_A: pass A of the next step on the updated
 // columns (two lines per thread, tensor stores).
 template <class R, class V, int A, int F, bool GEN, bool FUSE_A = false>
-__device__ __forceinline__ void stepC_body(const FlameDesc &d, int tile, int ntiles, int pf, const CUtensorMap *tm) {
+__device__ __forceinline__ void stepC_body(const FlameDesc &d, int tile, const Ahead &ahead, const CUtensorMap *tm) {
     griddep_wait();
-    griddep_launch();
     using C = CplxT<R>;
     using PL = Plan3<A, F>;
     constexpr int NL = kLanes<V>, LPC = 2 / NL, L = PL::L, TS = PL::TS, TP = PL::TP, SL = PL::slots(kSlotsPerWave<V>);
@@ -511,13 +547,6 @@ __device__ __forceinline__ void stepC_body(const FlameDesc &d, int tile, int nti
     const int G = blockDim.x / (TS * LPC);
     const Place s = NL == 2 ? place_all<TS>() : place<TS>(G * LPC), p = place<TP>(G * LPC);
     const int ld1 = 2 * a.K1 + 1;
-    if (threadIdx.x == 0 && pf > 0 && tile + pf < ntiles) {
-        const int c = 2 * (tile + pf) * G, nc = min(2 * G, a.K2 + 1 - c);
-        if (nc > 0) {
-            l2_prefetch(gk + (size_t)c * L, (size_t)nc * L * sizeof(C));
-            l2_prefetch(state + (size_t)c * ld1, (size_t)nc * ld1 * sizeof(C));
-        }
-    }
     const CoefR<R> cfs = load_coef<R>(d.coef);  // derived by pass B
     CV<V> xp[PL::EP];
     {
@@ -533,6 +562,13 @@ __device__ __forceinline__ void stepC_body(const FlameDesc &d, int tile, int nti
             else xp[i] = CV<V>{{q0.x}, {q0.y}};
         }
     }
+    ahead.run(d, tile, [&](const FlameDesc &q, int t) {  // that tile's column pairs
+        const int c = 2 * t * G, nc = min(2 * G, q.a.K2 + 1 - c);
+        if (nc > 0) {
+            l2_prefetch(static_cast<const C *>(q.gk) + (size_t)c * L, (size_t)nc * L * sizeof(C));
+            l2_prefetch(static_cast<const C *>(q.state) + (size_t)c * ld1, (size_t)nc * ld1 * sizeof(C));
+        }
+    });
     auto buf = [&](int line) { return planes3<V, R>(smstep, line, SL); };
     CV<V> xs[PL::ES];
     forward3<PL, true>(xp, xs, p, s, buf, tw);
@@ -546,14 +582,7 @@ __device__ __forceinline__ void stepC_body(const FlameDesc &d, int tile, int nti
         const int k1 = k1_of(i);
         return s.on && c0 + side <= a.K2 && (i < F ? k1 <= a.K1 : k1 >= -a.K1);
     };
-    C phi[2 * F][NL];
-#pragma unroll
-    for (int i = 0; i < 2 * F; ++i)
-#pragma unroll
-        for (int side = 0; side < NL; ++side) {
-            const bool in = in_box(i, side) && FLAME_IN(d.status, (long long)(c0 + side) * ld1 + a.K1 + k1_of(i), box_len(a), kSiteCState);
-            phi[i][side] = in ? col[(long)side * ld1 + k1_of(i)] : C{0, 0};
-        }
+    griddep_launch();  // (behind the loads, which it would hold back)
     const bool lin = !(a.flags & kNonlinearOnly), nl = !(a.flags & kLinearOnly);
     const EpiArgs<R> ea{cfs, scale1<R>(a), scale2<R>(a), GEN ? d.stage : kStageEuler, lin, nl};
     const C *fcol = GEN && d.forcing ? static_cast<const C *>(d.forcing) + (size_t)c0 * ld1 + a.K1 : nullptr;
@@ -561,9 +590,15 @@ __device__ __forceinline__ void stepC_body(const FlameDesc &d, int tile, int nti
     int bad = 0;
     C nphi[2 * F][NL];  // the updated entries (kept for the fused pass A)
 #pragma unroll
-    for (int i = 0; i < 2 * F; ++i)
+    for (int side = 0; side < NL; ++side) {
+        C phi[2 * F];
 #pragma unroll
-        for (int side = 0; side < NL; ++side) {
+        for (int i = 0; i < 2 * F; ++i) {
+            const bool in = in_box(i, side) && FLAME_IN(d.status, (long long)(c0 + side) * ld1 + a.K1 + k1_of(i), box_len(a), kSiteCState);
+            phi[i] = in ? col[(long)side * ld1 + k1_of(i)] : C{0, 0};
+        }
+#pragma unroll
+        for (int i = 0; i < 2 * F; ++i) {
             nphi[i][side] = C{0, 0};
             const int k1 = k1_of(i), k2 = c0 + side;
             if (!in_box(i, side) || (k2 == 0 && k1 < 0)) continue;  // k2 = 0, k1 < 0: the mirror of +k1
@@ -572,9 +607,10 @@ __device__ __forceinline__ void stepC_body(const FlameDesc &d, int tile, int nti
             if constexpr (NL == 2) gh = side == 0 ? lane0<R>(x) : lane1<R>(x);
             else gh = C{x.re.x, x.im.x};
             const int off = side * ld1;
-            update_entry<R, GEN>(d, ea, k1, k2, gh, phi[i][side], col + off, fcol ? fcol + off : nullptr,
+            update_entry<R, GEN>(d, ea, k1, k2, gh, phi[i], col + off, fcol ? fcol + off : nullptr,
                                  scol ? scol + off : nullptr, nphi[i][side], bad);
         }
+    }
     if (bad) atomicOr(d.status, 1 << kStatusNonfinite);
     if constexpr (FUSE_A) {
         // The k2 = 0 column's k1 < 0 half was written by other threads (the
@@ -658,7 +694,10 @@ __device__ inline void cos_sin_of(long num, long den, double &c, double &s) {  /
     if (left) c = -c;
     if (flip) s = -s;
 }
+// One entry per thread: an FP64 sine and cosine take microseconds.
 template <class R, int A> __global__ void k_twiddles3(CplxT<R> *tab) {
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    long num = -1, den = 1;
     auto table = [&](auto fc, auto ic) {
         constexpr int F = decltype(fc)::value;
         constexpr bool INV = decltype(ic)::value;
@@ -666,11 +705,10 @@ template <class R, int A> __global__ void k_twiddles3(CplxT<R> *tab) {
             using PL = Plan3<A, F>;
             static_for<1, PL::NQ + 1>([&](auto sc) {
                 constexpr int S = decltype(sc)::value, r = PL::template radix<INV>(S), Ns = PL::template stride<INV>(S);
-                CplxT<R> *t = tab + tw3_offset<A, F>() + PL::template tw_offset<INV>(S);
-                for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < (r - 1) * Ns; i += gridDim.x * blockDim.x) {
-                    double c, s;
-                    cos_sin_of((long)(i / Ns + 1) * (i % Ns), (long)r * Ns, c, s);
-                    t[i] = CplxT<R>{(R)c, (R)s};
+                const int j = i - (tw3_offset<A, F>() + PL::template tw_offset<INV>(S));
+                if (j >= 0 && j < (r - 1) * Ns) {
+                    num = (long)(j / Ns + 1) * (j % Ns);
+                    den = r * Ns;
                 }
             });
         }
@@ -680,11 +718,14 @@ template <class R, int A> __global__ void k_twiddles3(CplxT<R> *tab) {
         table(std::integral_constant<int, F>{}, std::true_type{});
         table(std::integral_constant<int, F>{}, std::false_type{});
     });
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < (3 << A); i += gridDim.x * blockDim.x) {
-        double c, s;
-        cos_sin_of(i, 6L << A, c, s);
-        tab[tw3_real_offset<A>() + i] = CplxT<R>{(R)c, (R)s};
+    if (i >= tw3_real_offset<A>() && i < tw3_alloc_len<A>()) {
+        num = i - tw3_real_offset<A>();
+        den = 6L << A;
     }
+    if (num < 0) return;
+    double c, s;
+    cos_sin_of(num, den, c, s);
+    tab[i] = CplxT<R>{(R)c, (R)s};
 }
 
 // ----------------------------------------------------------------------------
@@ -703,65 +744,70 @@ template <class R, class V, int A, int F, int LINES> constexpr int kStepBlocks =
 
 template <class R, class V, int A, int F>
 __global__ void __launch_bounds__(kStepThreads<R, V, A, F, 2>, kStepBlocks<R, V, A, F, 2>) k_stepA(FlameDesc d, int pf) {
-    stepA_body<R, V, A, F, false>(d, blockIdx.x + d.tile0, gridDim.x + d.tile0, pf, nullptr);
+    stepA_body<R, V, A, F, false>(d, blockIdx.x + d.tile0, Ahead{pf, (int)gridDim.x + d.tile0, nullptr}, nullptr);
 }
 template <class R, int A>
 __global__ void __launch_bounds__(256, 2) k_stepAt(FlameDesc d, int pf, const __grid_constant__ CUtensorMap tm) {
-    stepA_body<R, float2, A, 4, true>(d, blockIdx.x + d.tile0, gridDim.x + d.tile0, pf, &tm);
+    stepA_body<R, float2, A, 4, true>(d, blockIdx.x + d.tile0, Ahead{pf, (int)gridDim.x + d.tile0, nullptr}, &tm);
 }
 template <class R, class V, int A, int F>
-__global__ void __launch_bounds__(kStepThreads<R, V, A, F, 2>, kStepBlocks<R, V, A, F, 2>) k_stepA_n(const FlameDesc *__restrict__ ds) {
-    stepA_body<R, V, A, F, false>(ds[blockIdx.y], blockIdx.x, gridDim.x, 0, nullptr);
+__global__ void __launch_bounds__(kStepThreads<R, V, A, F, 2>, kStepBlocks<R, V, A, F, 2>) k_stepA_n(const FlameDesc *__restrict__ ds, int pf) {
+    stepA_body<R, V, A, F, false>(ds[blockIdx.y], blockIdx.x, Ahead{pf, (int)gridDim.x, ds}, nullptr);
 }
 
 template <class R, int A>
 __global__ void __launch_bounds__(256, 2) k_stepB(FlameDesc d, int pf) {
     if (blockIdx.x == 0) return coef_cta<R>(d);
     griddep_wait();
-    griddep_launch();
-    stepB2_body<R, A, false>(d, blockIdx.x - 1, gridDim.x - 1, pf, nullptr);
+    stepB2_body<R, A, false>(d, blockIdx.x - 1, Ahead{pf, (int)gridDim.x - 1, nullptr}, nullptr);
 }
 template <class R, int A>
 __global__ void __launch_bounds__(256, 2) k_stepBt(FlameDesc d, int pf, const __grid_constant__ CUtensorMap tm) {
     if (blockIdx.x == 0) return coef_cta<R>(d);
     griddep_wait();
-    griddep_launch();
-    stepB2_body<R, A, true>(d, blockIdx.x - 1, gridDim.x - 1, pf, &tm);
+    stepB2_body<R, A, true>(d, blockIdx.x - 1, Ahead{pf, (int)gridDim.x - 1, nullptr}, &tm);
 }
-template <class R, int A> __global__ void __launch_bounds__(256, 2) k_stepB_n(const FlameDesc *__restrict__ ds) {
+template <class R, int A> __global__ void __launch_bounds__(256, 2) k_stepB_n(const FlameDesc *__restrict__ ds, int pf) {
     if (blockIdx.x == 0) return coef_cta<R>(ds[blockIdx.y]);
-    stepB2_body<R, A, false>(ds[blockIdx.y], blockIdx.x - 1, gridDim.x - 1, 0, nullptr);
+    griddep_wait();
+    stepB2_body<R, A, false>(ds[blockIdx.y], blockIdx.x - 1, Ahead{pf, (int)gridDim.x - 1, ds}, nullptr);
 }
 template <class R, int A, int F, int RW>
 __global__ void __launch_bounds__(kStepThreads<R, typename OneOf<R>::type, A, F, 2 * RW>, kStepBlocks<R, typename OneOf<R>::type, A, F, 2 * RW>)
  k_stepB1(FlameDesc d) {
     if (blockIdx.x == 0) return coef_cta<R>(d);
     griddep_wait();
-    griddep_launch();
     stepB1_body<R, A, F, RW>(d, blockIdx.x - 1);
 }
 template <class R, int A, int F, int RW>
 __global__ void __launch_bounds__(kStepThreads<R, typename OneOf<R>::type, A, F, 2 * RW>, kStepBlocks<R, typename OneOf<R>::type, A, F, 2 * RW>)
  k_stepB1_n(const FlameDesc *__restrict__ ds) {
     if (blockIdx.x == 0) return coef_cta<R>(ds[blockIdx.y]);
+    griddep_wait();
     stepB1_body<R, A, F, RW>(ds[blockIdx.y], blockIdx.x - 1);
 }
 
+// Plain pass C at 80 registers a thread, three CTAs per SM, where a launch has
+// several waves of them: 3072-point columns (4096x8192 136.7 -> 133.7 us a step)
+// and ensembles (96 flames 7.37 -> 7.24 ms); elsewhere two (2048x4096 39.6
+// against 40.9 us).
+template <class R, class V, int A, int F, bool GEN, int FROM> constexpr int kStepBlocksC =
+    kLanes<V> == 2 && !GEN && A >= FROM ? 3 : kStepBlocks<R, V, A, F, 2>;
 template <class R, class V, int A, int F, bool GEN>
-__global__ void __launch_bounds__(kStepThreads<R, V, A, F, 2>, kStepBlocks<R, V, A, F, 2>) k_stepC(FlameDesc d, int pf) {
+__global__ void __launch_bounds__(kStepThreads<R, V, A, F, 2>, kStepBlocksC<R, V, A, F, GEN, 10>) k_stepC(FlameDesc d, int pf) {
     const int extra = d.tile0 == 0 ? 1 : 0;
     if (extra && blockIdx.x == 0) return finish_cta<R, GEN, true>(d);
-    stepC_body<R, V, A, F, GEN>(d, blockIdx.x - extra + d.tile0, gridDim.x - extra + d.tile0, pf, nullptr);
+    stepC_body<R, V, A, F, GEN>(d, blockIdx.x - extra + d.tile0, Ahead{pf, (int)gridDim.x - extra + d.tile0, nullptr}, nullptr);
 }
 template <class R, class V, int A, int F, bool GEN>
-__global__ void __launch_bounds__(kStepThreads<R, V, A, F, 2>, kStepBlocks<R, V, A, F, 2>) k_stepC_n(const FlameDesc *__restrict__ ds) {
+__global__ void __launch_bounds__(kStepThreads<R, V, A, F, 2>, kStepBlocksC<R, V, A, F, GEN, 6>) k_stepC_n(const FlameDesc *__restrict__ ds, int pf) {
     if (blockIdx.x == 0) return finish_cta<R, GEN, true>(ds[blockIdx.y]);
-    stepC_body<R, V, A, F, GEN>(ds[blockIdx.y], blockIdx.x - 1, gridDim.x - 1, 0, nullptr);
+    stepC_body<R, V, A, F, GEN>(ds[blockIdx.y], blockIdx.x - 1, Ahead{pf, (int)gridDim.x - 1, ds}, nullptr);
 }
 template <class R, int A, bool GEN>
 __global__ void __launch_bounds__(256, 2) k_stepCA(FlameDesc d, int pf, const __grid_constant__ CUtensorMap tm) {
     if (blockIdx.x == 0) return finish_cta<R, GEN, true>(d);
-    stepC_body<R, float2, A, 4, GEN, true>(d, blockIdx.x - 1, gridDim.x - 1, pf, &tm);
+    stepC_body<R, float2, A, 4, GEN, true>(d, blockIdx.x - 1, Ahead{pf, (int)gridDim.x - 1, nullptr}, &tm);
 }
 
 }  // namespace flame

@@ -2,6 +2,7 @@
 #include "flame_step_ops.cuh"
 
 namespace flame {
+template cudaError_t Ops<double>::init_kappa(double *, const StepArgs &, cudaStream_t);
 template cudaError_t Ops<double>::init_twiddles3(double2 *, int, cudaStream_t);
 template cudaError_t Ops<double>::passA(const FlameDesc &, cudaStream_t, int, const CUtensorMap *);
 template cudaError_t Ops<double>::passA_batch(const FlameDesc *, int, const StepArgs &, cudaStream_t, int);

@@ -4,6 +4,8 @@
 // that their kernels compile in parallel.
 #pragma once
 
+#include <algorithm>
+
 #include "flame_launch.cuh"
 #include "flame_step.cuh"
 
@@ -15,9 +17,13 @@ template <class R> constexpr bool two_line(int a) { return sizeof(R) == 4 && a >
 // One line per thread: all of FP64, and FP32 up to 1536 points (a pair of
 // 3072-point rows would not leave shared memory for a second CTA).
 template <class R> constexpr bool one_line(int a) { return sizeof(R) == 8 || a <= 9; }
-// Points per thread of the one-line kernels (4 F, spectral end 3 F).
+// Points per thread of the one-line kernels (4 F, spectral end 3 F).  FP64: a warp
+// instruction holds its SM quarter for some 68 cycles, so short lines spread
+// over more warps (256x512: 28.6 us a step with F = 1 for 192 points, 38.9 with
+// 2; 128x256 21.6 against 33.7), and long ones take the plan with the fewest
+// twiddles (1024x2048: 254 us with F = 4, 258 with 2).
 template <class R> constexpr int one_line_f(int a) {
-    if (sizeof(R) == 8) return a <= 6 ? 1 : a <= 9 ? 2 : 4;
+    if (sizeof(R) == 8) return a <= 6 ? 1 : a <= 7 ? 2 : 4;
     return a <= 5 ? 1 : a <= 8 ? 2 : 4;
 }
 // FLAME_FP64_POINTS=8: the FP64 lines of up to 96 points with 8 points per
@@ -26,9 +32,12 @@ static bool fp64_points8() {
     const char *v = getenv("FLAME_FP64_POINTS");
     return v && strcmp(v, "8") == 0;
 }
-// rows per unit of the one-line pass B: a pair where its lines fit 512
-// threads and its buffers shared memory, else one
+// rows per unit of the one-line pass B: FP32 a pair where its lines fit 512
+// threads and its buffers shared memory, else one.  FP64 one: it is bound by
+// the FP64 units of the fullest SM, and single rows spread better (512x1024:
+// 192 pairs leave 41 of 152 SMs with two).
 template <class R, int A, int F> constexpr int rows_of() {
+    if (sizeof(R) == 8) return 1;
     using V = typename OneOf<R>::type;
     const size_t pair = exchange_bytes<R, V, Plan3<A, F>>(4) + (size_t)4 * (3 << A) * sizeof(R);
     return 4 * Plan3<A, F>::TS <= 512 && pair <= kSmemBudget ? 2 : 1;
@@ -80,9 +89,14 @@ cudaError_t Ops<R>::init_twiddles3(C *tab, int a, cudaStream_t s) {
     cudaError_t e = cudaErrorInvalidValue;
     with_a(a, [&](auto ac) {
         constexpr int A = decltype(ac)::value;
-        e = launch_k(k_twiddles3<R, A>, dim3(((3 << A) + 127) / 128), 128, 0, s, tab);
+        e = launch_k(k_twiddles3<R, A>, dim3((tw3_alloc_len<A>() + 127) / 128), 128, 0, s, tab);
     });
     return e;
+}
+
+template <class R> cudaError_t Ops<R>::init_kappa(R *kap, const StepArgs &a, cudaStream_t s) {
+    const long n = (long)(2 * a.K1 + 1) * a.ldk;
+    return launch_k(k_kappa<R>, dim3((unsigned)std::min<long>((n + 255) / 256, 8L * sm_count())), 256, 0, s, kap, a);
 }
 
 // variant: kVariantTma = the tensor-store write-out through uv_map (two-line
@@ -96,7 +110,7 @@ cudaError_t Ops<R>::passA(const FlameDesc &d, cudaStream_t s, int variant, const
             constexpr int A = decltype(ac)::value, F = decltype(fc)::value;
             using V = typename OneOf<R>::type;
             const Geom g = geom_one_line<R, A, F>(ncol, 2, 0);
-            err = launch_s(d.l2_state, k_stepA<R, V, A, F>, dim3(d.tiles ? d.tiles : g.blocks), g.threads, g.smem, s, d, 0);
+            err = launch_s(d.l2_state, pdl_on(sizeof(R) == 8, d.a), k_stepA<R, V, A, F>, dim3(d.tiles ? d.tiles : g.blocks), g.threads, g.smem, s, d, 0);
         });
         return err;
     }
@@ -106,10 +120,10 @@ cudaError_t Ops<R>::passA(const FlameDesc &d, cudaStream_t s, int variant, const
         const dim3 grid(d.tiles ? d.tiles : g.blocks);
         if (variant == kVariantTma && uv_map) {
             const int pf = resident_ctas((const void *)k_stepAt<R, A>, g);
-            err = launch_s(d.l2_state, k_stepAt<R, A>, grid, g.threads, g.smem, s, d, pf, *uv_map);
+            err = launch_s(d.l2_state, pdl_on(sizeof(R) == 8, d.a), k_stepAt<R, A>, grid, g.threads, g.smem, s, d, pf, *uv_map);
         } else {
             const int pf = resident_ctas((const void *)k_stepA<R, float2, A, 4>, g);
-            err = launch_s(d.l2_state, k_stepA<R, float2, A, 4>, grid, g.threads, g.smem, s, d, pf);
+            err = launch_s(d.l2_state, pdl_on(sizeof(R) == 8, d.a), k_stepA<R, float2, A, 4>, grid, g.threads, g.smem, s, d, pf);
         }
     });
     return err;
@@ -121,7 +135,7 @@ cudaError_t Ops<R>::passA_batch(const FlameDesc *ds, int n, const StepArgs &a, c
         with_one_line<R>(a.la, [&](auto ac, auto fc) {
             constexpr int A = decltype(ac)::value, F = decltype(fc)::value;
             const Geom g = geom_one_line<R, A, F>(a.K2 + 1, 2, 0);
-            err = launch_k(k_stepA_n<R, typename OneOf<R>::type, A, F>, dim3(g.blocks, n), g.threads, g.smem, s, ds);
+            err = launch_k(k_stepA_n<R, typename OneOf<R>::type, A, F>, dim3(g.blocks, n), g.threads, g.smem, s, ds, 0);
         });
         return err;
     }
@@ -129,7 +143,8 @@ cudaError_t Ops<R>::passA_batch(const FlameDesc *ds, int n, const StepArgs &a, c
         constexpr int A = decltype(ac)::value;
         const Geom g = geom_two_line(A, n * (a.K2 + 1), pair_bytes<A>());
         const int G = g.threads >> (A - 2);
-        err = launch_k(k_stepA_n<R, float2, A, 4>, dim3((a.K2 + G) / G, n), g.threads, g.smem, s, ds);
+        const int pf = resident_ctas((const void *)k_stepA_n<R, float2, A, 4>, g);
+        err = launch_k(k_stepA_n<R, float2, A, 4>, dim3((a.K2 + G) / G, n), g.threads, g.smem, s, ds, pf);
     });
     return err;
 }
@@ -144,7 +159,7 @@ cudaError_t Ops<R>::passB(const FlameDesc &d, cudaStream_t s, int variant, const
         with_one_line<R>(d.a.lb, [&](auto ac, auto fc) {
             constexpr int A = decltype(ac)::value, F = decltype(fc)::value, RW = rows_of<R, A, F>();
             const Geom g = geom_b1<R, A, F>(d.a.n1);
-            err = launch_s(none, k_stepB1<R, A, F, RW>, dim3(g.blocks + 1), g.threads, g.smem, s, d);
+            err = launch_s(none, pdl_on(sizeof(R) == 8, d.a), k_stepB1<R, A, F, RW>, dim3(g.blocks + 1), g.threads, g.smem, s, d);
         });
         return err;
     }
@@ -153,10 +168,10 @@ cudaError_t Ops<R>::passB(const FlameDesc &d, cudaStream_t s, int variant, const
         const Geom g = geom_b2<A>(d.a.n1 / 2);
         if ((variant == kVariantTmaB || variant == kVariantTmaB4) && gk_map) {
             const int pf = resident_ctas((const void *)k_stepBt<R, A>, g);
-            err = launch_s(none, k_stepBt<R, A>, dim3(g.blocks + 1), g.threads, g.smem, s, d, pf, *gk_map);
+            err = launch_s(none, pdl_on(sizeof(R) == 8, d.a), k_stepBt<R, A>, dim3(g.blocks + 1), g.threads, g.smem, s, d, pf, *gk_map);
         } else {
             const int pf = resident_ctas((const void *)k_stepB<R, A>, g);
-            err = launch_s(none, k_stepB<R, A>, dim3(g.blocks + 1), g.threads, g.smem, s, d, pf);
+            err = launch_s(none, pdl_on(sizeof(R) == 8, d.a), k_stepB<R, A>, dim3(g.blocks + 1), g.threads, g.smem, s, d, pf);
         }
     });
     return err;
@@ -176,7 +191,8 @@ cudaError_t Ops<R>::passB_batch(const FlameDesc *ds, int n, const StepArgs &a, c
         constexpr int A = decltype(ac)::value;
         const Geom g = geom_b2<A>(n * (a.n1 / 2));
         const int G = g.threads >> (A - 2);
-        err = launch_k(k_stepB_n<R, A>, dim3((a.n1 / 2 + G - 1) / G + 1, n), g.threads, g.smem, s, ds);
+        const int pf = resident_ctas((const void *)k_stepB_n<R, A>, g);
+        err = launch_k(k_stepB_n<R, A>, dim3((a.n1 / 2 + G - 1) / G + 1, n), g.threads, g.smem, s, ds, pf);
     });
     return err;
 }
@@ -187,7 +203,7 @@ template <class R> cudaError_t Ops<R>::passC(const FlameDesc &d, cudaStream_t s)
     const bool gen = general_epilogue(d);
     auto launch = [&](auto plain, auto general, const Geom &g, bool prefetch) {
         const int pf = prefetch ? resident_ctas((const void *)(gen ? general : plain), g) : 0;
-        return launch_s(d.l2_state, gen ? general : plain, dim3((d.tiles ? d.tiles : g.blocks) + extra), g.threads, g.smem,
+        return launch_s(d.l2_state, pdl_on(sizeof(R) == 8, d.a), gen ? general : plain, dim3((d.tiles ? d.tiles : g.blocks) + extra), g.threads, g.smem,
                         s, d, pf);
     };
     if (!two_line<R>(d.a.la) || (d.onec && one_line<R>(d.a.la))) {
@@ -215,7 +231,7 @@ cudaError_t Ops<R>::passC_batch(const FlameDesc *ds, int n, const StepArgs &a, c
             using V = typename OneOf<R>::type;
             const Geom g = geom_one_line<R, A, F>(npair, 2, 0);
             err = launch_k(gen ? k_stepC_n<R, V, A, F, true> : k_stepC_n<R, V, A, F, false>, dim3(g.blocks + 1, n),
-                            g.threads, g.smem, s, ds);
+                            g.threads, g.smem, s, ds, 0);
         });
         return err;
     }
@@ -223,8 +239,8 @@ cudaError_t Ops<R>::passC_batch(const FlameDesc *ds, int n, const StepArgs &a, c
         constexpr int A = decltype(ac)::value;
         const Geom g = geom_two_line(A, n * npair, pair_bytes<A>());
         const int G = g.threads >> (A - 2);
-        err = launch_k(gen ? k_stepC_n<R, float2, A, 4, true> : k_stepC_n<R, float2, A, 4, false>,
-                        dim3((npair + G - 1) / G + 1, n), g.threads, g.smem, s, ds);
+        const auto kernel = gen ? k_stepC_n<R, float2, A, 4, true> : k_stepC_n<R, float2, A, 4, false>;
+        err = launch_k(kernel, dim3((npair + G - 1) / G + 1, n), g.threads, g.smem, s, ds, resident_ctas((const void *)kernel, g));
     });
     return err;
 }
@@ -239,7 +255,7 @@ cudaError_t Ops<R>::passCA(const FlameDesc &d, cudaStream_t s, const CUtensorMap
             const Geom g = geom_two_line(A, (d.a.K2 + 2) / 2, pair_bytes<A>());
             const auto kernel = general_epilogue(d) ? k_stepCA<R, A, true> : k_stepCA<R, A, false>;
             const int pf = resident_ctas((const void *)kernel, g);
-            err = launch_s(d.l2_state, kernel, dim3(g.blocks + 1), g.threads, g.smem, s, d, pf, *uv_map);
+            err = launch_s(d.l2_state, pdl_on(sizeof(R) == 8, d.a), kernel, dim3(g.blocks + 1), g.threads, g.smem, s, d, pf, *uv_map);
         });
     }
     return err;
