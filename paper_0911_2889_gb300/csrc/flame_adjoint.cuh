@@ -16,7 +16,7 @@
 //          lambda_0 unchanged; dL/dgamma += <lambda, dt |kappa|/(2 r0) Phi_n>.
 #pragma once
 
-#include "flame_kernels.cuh"
+#include "flame_step.cuh"
 
 namespace flame {
 
@@ -191,7 +191,6 @@ template <class R, int LOG> __global__ void __launch_bounds__(256, kMinBlocks<R>
         hb2[r] = C{b2[0], b2[1]};
     }
     if (!valid) part = 0.0;
-    red[t] = part;  // summed by thread 0 after the barriers of real_fwd
     C *aw = static_cast<C *>(d.aw);
     C *gk = static_cast<C *>(d.gk);
     real_fwd<R, LOG>(y, a, t, P, twm, base, valid, [&](int k, CV<V> Y) {
@@ -201,11 +200,8 @@ template <class R, int LOG> __global__ void __launch_bounds__(256, kMinBlocks<R>
 #pragma unroll
     for (int r = 0; r < 16; ++r) y[r] = pack2<R>(hb2[r], C{0, 0});
     real_fwd<R, LOG>(y, a, t, P, twm, base, valid, [&](int k, CV<V> Y) { gk[(size_t)k * a.n1 + row] = lane0<R>(Y); });
-    if (t == 0 && valid) {
-        double s = 0.0;
-        for (int i = 0; i < (int)blockDim.x; ++i) s += red[i];
-        d.rowsum[row] = s;
-    }
+    const double sum = cta_sum(part, red);
+    if (t == 0 && valid) d.rowsum[row] = sum;
 }
 
 // --- area, pass C: one column per group -------------------------------------
@@ -264,142 +260,206 @@ template <class R, int LOG> __global__ void __launch_bounds__(256, kMinBlocks<R>
             if (grad) grad[(size_t)k2 * ld1 + k1 + a.K1] = gr;
         }
     }
-    if (blockIdx.x == 0 && threadIdx.x == 0) {
-        double s = 0.0;
-        for (int i = 0; i < a.n1; ++i) s += d.rowsum[i];
-        *d.area = s;
+    if (blockIdx.x == 0) {  // (one thread's sum of 512 rows took 17 of the kernel's 36 us)
+        __shared__ double red[256];
+        double v = 0.0;
+        for (int i = threadIdx.x; i < a.n1; i += blockDim.x) v += d.rowsum[i];
+        const double sum = cta_sum(v, red);
+        if (threadIdx.x == 0) *d.area = sum;
     }
 }
 
-// --- adjoint: column synthesis of lambda (two columns per group) -------------
-// gk[j1][k2] (row-major) = column synthesis of lambda, lambda_0 at k = 0.
-template <class R, int LOG> __global__ void __launch_bounds__(256, kMinBlocks<R>) k_adjL(AdjDesc d) {
+// ----------------------------------------------------------------------------
+// The adjoint step, on the step's alias-free grid: its products 2 ell d_i phi
+// are quadratic too, and only their retained harmonics are wanted.  Pass A of
+// the step gives W = the row spectra of d1 phi + i d2 phi; then
+//   L (columns): lambda -> its row spectra, for all j1
+//   B (rows):    ell and d_i phi on the row, q_i = 2 ell d_i phi, forward real
+//                transforms of q_1 and q_2
+//   C (columns): forward transforms, P, the update of lambda, dL/dgamma
+// Two lines per thread throughout (two columns, even and odd points, q_1 and
+// q_2); 3 F and 4 F points a thread, F by adj_f.
+// ----------------------------------------------------------------------------
+// (512x1024: with the public grid, 16 points a thread and every CTA deriving
+// the coefficients, an adjoint step's four kernels took 38 us.)
+template <class R> __host__ __device__ constexpr int adj_f(int a) {
+    return a == 2 ? 1 : sizeof(R) == 8 ? (a <= 6 ? 1 : a <= 9 ? 2 : 4) : (a <= 8 ? 2 : 4);
+}
+// complex index of lambda's row spectrum (j1, k2): row pairs interleaved
+__host__ __device__ __forceinline__ size_t l_index(int j1, int k2, int ldk) {
+    return 2 * ((size_t)(j1 >> 1) * ldk + k2) + (j1 & 1);
+}
+
+// Columns c0, c0 + 1 of lambda (lambda_0 at k = 0); the extra CTA derives the
+// step's coefficients for pass C (and dt / (2 t_n), dL/dgamma's factor).
+template <class R, int A> __global__ void __launch_bounds__(256, kMinBlocks<R>) k_adjL(AdjDesc d) {
     using V = typename VecOf<R>::type;
     using C = CplxT<R>;
-    extern __shared__ __align__(16) unsigned char smraw[];
+    using PL = Plan3<A, adj_f<R>(A)>;
+    constexpr int F = PL::F, SL = PL::slots(kSlotsPerWave<V>);
+    extern __shared__ __align__(128) unsigned char smstep[];
     const StepArgs &a = d.a;
-    const int N1 = 1 << a.logn1, T = N1 >> 4;
-    const int G = blockDim.x / T, g = threadIdx.x / T, t = threadIdx.x % T;
-    const int ld1 = 2 * a.K1 + 1;
-    const int c0 = 2 * (blockIdx.x * G + g);
-    const bool va = c0 <= a.K2, vb = c0 + 1 <= a.K2;
-    V *base = reinterpret_cast<V *>(smraw) + (size_t)g * 2 * plane_len(N1);
-    auto sm = make_planes(base, N1);
-    const C *lam = static_cast<const C *>(d.lam);
-    const C *la = lam + (size_t)c0 * ld1 + a.K1, *lb = la + ld1;
+    griddep_wait();
+    if (blockIdx.x == 0) {
+        if (threadIdx.x == 0) {
+            store_coef<R>(d.coef, a, *d.t, false);
+            d.coef[10] = a.dt / (2.0 * d.coef[0]);
+        }
+        griddep_launch();
+        return;
+    }
+    const int G = blockDim.x / PL::TS, ld1 = 2 * a.K1 + 1;
+    const Place s = place_all<PL::TS>(), p = place<PL::TP>(G);
     const double l0 = *d.lam0;
-    CV<V> x[16];
+    CV<V> xs[PL::ES];
+    {
+        const int c0 = 2 * ((blockIdx.x - 1) * G + s.line);
+        const C *la = static_cast<const C *>(d.lam) + (size_t)c0 * ld1 + a.K1, *lb = la + ld1;
 #pragma unroll
-    for (int r = 0; r < 16; ++r) {
-        x[r] = CV<V>{vzero(V{}), vzero(V{})};
-        if (r < 4 || r >= 12) {
-            const int n = t + r * T;
-            const int k1 = (r < 4) ? n : n - N1;
-            const bool in_box = (r < 4) ? (n <= a.K1) : (k1 >= -a.K1);
-            C p = (in_box && va) ? la[k1] : C{0, 0};
-            C q = (in_box && vb) ? lb[k1] : C{0, 0};
-            if (c0 == 0 && k1 == 0) p = C{(R)l0, 0};
-            x[r] = pack2<R>(p, q);
+        for (int r = 0; r < PL::ES; ++r) {
+            xs[r] = CV<V>{vzero(V{}), vzero(V{})};
+            if (r >= F && r < 2 * F) continue;
+            const int n = s.t + r * PL::TS, k1 = r < F ? n : n - PL::L;
+            const bool in_box = r < F ? n <= a.K1 : k1 >= -a.K1;
+            C p0 = in_box && c0 <= a.K2 ? la[k1] : C{0, 0};
+            const C p1 = in_box && c0 + 1 <= a.K2 ? lb[k1] : C{0, 0};
+            if (c0 == 0 && k1 == 0) p0 = C{(R)l0, 0};
+            xs[r] = pack2<R>(p0, p1);
         }
     }
-    fft_line<1, LOG>(x, a.logn1, t, sm, static_cast<const C *>(d.tw1));
-    C *gk = static_cast<C *>(d.gk);
+    auto buf = [&](int line) { return planes3<V, R>(smstep, line, SL); };
+    CV<V> xp[PL::EP];
+    inverse3<PL>(xs, xp, s, p, buf, tab3<R, A, F, C>(d.tw1));
+    griddep_launch();
+    if (!p.on) return;
+    C *out = static_cast<C *>(d.gk);
+    const int c0 = 2 * ((blockIdx.x - 1) * G + p.line);
 #pragma unroll
-    for (int r = 0; r < 16; ++r) {
-        const size_t row = (size_t)(t + r * T) * a.ldk;
-        if (va) gk[row + c0] = lane0<R>(x[r]);
-        if (vb) gk[row + c0 + 1] = lane1<R>(x[r]);
+    for (int i = 0; i < PL::EP; ++i) {
+        C *e = out + l_index(p.t + i * PL::TP, c0, a.ldk);
+        if (c0 <= a.K2) e[0] = lane0<R>(xp[i]);
+        if (c0 + 1 <= a.K2) e[2] = lane1<R>(xp[i]);
     }
 }
 
-// --- adjoint, pass B: one row per group -------------------------------------
-// ell from the lambda row (gk), u + iv from uv; q_i = 2 ell d_i phi;
-// forward real transforms of q1 and q2 (paired); writes
-// aw[k2][j1] = (hat q1, -i s2 k2 hat q2) column-major.
-template <class R, int LOG> __global__ void __launch_bounds__(256, kMinBlocks<R>) k_adjB(AdjDesc d) {
+// The inputs of a row's two half-length inverse transforms (as in the step's
+// pass B), get(k, minus) the row spectrum at +-k, 0 <= k <= K2.
+template <class PL, class R, class V, class Get>
+__device__ __forceinline__ void half_inputs(CV<V> (&x)[PL::ES], int t, bool valid, int K2, const CplxT<R> *P, Get get) {
+    using C = CplxT<R>;
+#pragma unroll
+    for (int r = 0; r < PL::ES; ++r) {
+        const int n = t + r * PL::TS, km = PL::L - n;
+        const C up = r < 2 * PL::F && valid && n <= K2 ? get(n, false) : C{0, 0};
+        const C um = r >= PL::F && valid && km <= K2 ? get(km, true) : C{0, 0};
+        const C o{up.x - um.x, up.y - um.y}, w = __ldg(P + n);
+        x[r] = pack2<R>(C{up.x + um.x, up.y + um.y}, C{fma_rn(o.x, w.x, -(o.y * w.y)), fma_rn(o.x, w.y, o.y * w.x)});
+    }
+}
+
+// One row per group: ell and w = d1 phi + i d2 phi at the even and odd points
+// (lanes), q_i = 2 ell d_i phi, forward transforms of h_i[m] = q_i[2m] + i
+// q_i[2m+1] (lanes i = 1, 2); aw[k2][j1] = (hat q1, -i s2 k2 hat q2).
+template <class R, int A> __global__ void __launch_bounds__(256, kMinBlocks<R>) k_adjB(AdjDesc d) {
     using V = typename VecOf<R>::type;
     using C = CplxT<R>;
-    extern __shared__ __align__(16) unsigned char smraw[];
+    using PL = Plan3<A, adj_f<R>(A)>;
+    constexpr int F = PL::F, L = PL::L, TS = PL::TS, ES = PL::ES, SL = PL::slots(kSlotsPerWave<V>);
+    extern __shared__ __align__(128) unsigned char smstep[];
     const StepArgs &a = d.a;
-    const C *uv = static_cast<const C *>(d.uv);
-    const C *lrow = static_cast<const C *>(d.gk);
-    const C *twm = static_cast<const C *>(d.twm);
-    const int M = 1 << a.logm, T = M >> 4;
-    const int t = threadIdx.x;
-    const int row = blockIdx.x;
+    griddep_wait();
+    const int G = blockDim.x / TS;
+    const Place s = place_all<TS>(), p = place<PL::TP>(G);
+    const int row = blockIdx.x * G + s.line;
     const bool valid = row < a.n1;
-    V *base = reinterpret_cast<V *>(smraw);
-    C *park = reinterpret_cast<C *>(base + 2 * plane_len(M));
-    const C *P = twm + tw_real_offset(a.logm);
-    const C *src = uv + uv_index(valid ? row : 0, 0, a.ldk);  // element kk at src + 4 kk
-    const C *lsrc = lrow + (size_t)(valid ? row : 0) * a.ldk;
-    CV<V> x[16];
-    halfband_ifft<R, LOG>(x, a, t, P, twm,
-                     [&](int kk, bool pos) {
-                         C e = lsrc[kk];
-                         return pos ? e : C{e.x, -e.y};
-                     },
-                     valid, base);
+    auto buf = [&](int line) { return planes3<V, R>(smstep, line, SL); };
+    const C *tw = tab3<R, A, F, C>(d.twm);
+    const C *P = static_cast<const C *>(d.twm) + tw3_real_offset<A>();
+    const C *lrow = static_cast<const C *>(d.gk), *uv = static_cast<const C *>(d.uv);
+    V ell[PL::EP];
+    {
+        CV<V> xs[ES], xp[PL::EP];
+        half_inputs<PL, R>(xs, s.t, valid, a.K2, P, [&](int k, bool minus) {
+            const C e = __ldg(lrow + l_index(row, k, a.ldk));
+            return minus ? C{e.x, -e.y} : e;
+        });
+        inverse3<PL>(xs, xp, s, p, buf, tw);
 #pragma unroll
-    for (int r = 0; r < 16; ++r) park[t + r * T] = C{x[r].re.x, x[r].re.y};  // ell(2m), ell(2m+1)
-    halfband_ifft<R, LOG>(x, a, t, P, twm,
-                     [&](int kk, bool pos) {
-                         UV<R> e = ld_uv<R>(src + 4 * (size_t)kk);
-                         if (pos) return C{e.u.x - e.v.y, e.u.y + e.v.x};
-                         return C{e.u.x + e.v.y, e.v.x - e.u.y};
-                     },
-                     valid, base);
-#pragma unroll
-    for (int r = 0; r < 16; ++r) {
-        C l = park[t + r * T];
-        const R l0 = (R)2 * l.x, l1 = (R)2 * l.y;
-        // lanes: q1 = 2 ell u at (2m, 2m+1), q2 = 2 ell v at (2m, 2m+1)
-        C h1{l0 * x[r].re.x, l1 * x[r].re.y};
-        C h2{l0 * x[r].im.x, l1 * x[r].im.y};
-        x[r] = pack2<R>(h1, h2);
+        for (int i = 0; i < PL::EP; ++i) ell[i] = vadd(xp[i].re, xp[i].re);  // 2 ell
     }
+    CV<V> xp[PL::EP];
+    {
+        CV<V> xs[ES];
+        half_inputs<PL, R>(xs, s.t, valid, a.K2, P, [&](int k, bool minus) { return ld_w<R>(uv, row, k, a.ldk, minus); });
+        __syncthreads();  // the exchange buffers are free
+        inverse3<PL>(xs, xp, s, p, buf, tw);
+    }
+#pragma unroll
+    for (int i = 0; i < PL::EP; ++i) {
+        const V q1 = vmul(ell[i], xp[i].re), q2 = vmul(ell[i], xp[i].im);
+        xp[i] = CV<V>{V{q1.x, q2.x}, V{q1.y, q2.y}};
+    }
+    CV<V> hk[ES];
+    forward3<PL, false>(xp, hk, p, s, buf, tw);
+    griddep_launch();
+    __syncthreads();
+    const Planes<V> sm = buf(s.line);
+#pragma unroll
+    for (int r = 0; r < ES; ++r)
+        if (TS * (r + 1) > L / 2) sm.st_raw(s.t + r * TS, hk[r]);
+    if (s.t == 0) sm.st_raw(0, hk[0]);
+    __syncthreads();
+    if (!valid) return;
     C *aw = static_cast<C *>(d.aw);
     const R s2 = scale2<R>(a);
-    real_fwd<R, LOG>(x, a, t, P, twm, base, valid, [&](int k, CV<V> Y) {
-        C q1 = lane0<R>(Y), q2 = lane1<R>(Y);
+    auto emit = [&](int k, CV<V> Y) {
+        const C q2 = lane1<R>(Y);
         const R f = s2 * (R)k;
-        st_uv<R>(aw + 2 * ((size_t)k * a.n1 + row), q1, C{f * q2.y, -f * q2.x});  // -i f q2
-    });
+        st_uv<R>(aw + 2 * ((size_t)k * a.n1 + row), lane0<R>(Y), C{f * q2.y, -f * q2.x});  // -i f q2
+    };
+#pragma unroll
+    for (int r = 0; r < ES; ++r) {
+        if (TS * r > L / 2) continue;
+        const int k = s.t + r * TS, kc = L - k;
+        if (k <= L / 2 && (k <= a.K2 || kc <= a.K2)) {
+            CV<V> lo, hi;
+            real_post(hk[r], sm.ld_raw(k == 0 ? 0 : kc), __ldg(P + k), lo, hi);
+            if (k <= a.K2) emit(k, lo);
+            if (kc <= a.K2 && kc != k) emit(kc, hi);
+        }
+    }
 }
 
-// --- adjoint, pass C: one column per group ----------------------------------
-// forward column transforms of (hat q1, -i k2 hat q2), P = (-i s1 k1 Q1 + Q2)
-// / (N1 N2), lambda update on the box, k2 = 0 column from its k1 > 0 half,
-// dL/dgamma contribution (FP64, one atomic per block).
-template <class R, int LOG> __global__ void __launch_bounds__(256, kMinBlocks<R>) k_adjC(AdjDesc d) {
+// One column per group: forward column transforms of (hat q1, -i k2 hat q2),
+// P = (-i s1 k1 Q1 + Q2) / (N1 N2), lambda update on the box, k2 = 0 column
+// from its k1 > 0 half, dL/dgamma contribution (FP64, one atomic per block).
+template <class R, int A> __global__ void __launch_bounds__(256, kMinBlocks<R>) k_adjC(AdjDesc d) {
     using V = typename VecOf<R>::type;
     using C = CplxT<R>;
-    extern __shared__ __align__(16) unsigned char smraw[];
-    __shared__ double red[256];  // one per thread (blockDim <= 256)
+    using PL = Plan3<A, adj_f<R>(A)>;
+    constexpr int F = PL::F, L = PL::L, TS = PL::TS, SL = PL::slots(kSlotsPerWave<V>);
+    extern __shared__ __align__(128) unsigned char smstep[];
+    __shared__ double red[256];
     const StepArgs &a = d.a;
-    const int N1 = 1 << a.logn1, T = N1 >> 4;
-    const int G = blockDim.x / T, g = threadIdx.x / T, t = threadIdx.x % T;
-    const int ld1 = 2 * a.K1 + 1;
-    const int k2 = blockIdx.x * G + g;
-    const bool valid = k2 <= a.K2;
-    V *base = reinterpret_cast<V *>(smraw) + (size_t)g * 2 * plane_len(N1);
-    auto sm = make_planes(base, N1);
-    const C *aw = static_cast<const C *>(d.aw) + 2 * (size_t)(valid ? k2 : 0) * N1;
-    CV<V> x[16];
+    griddep_wait();
+    const int G = blockDim.x / TS, ld1 = 2 * a.K1 + 1;
+    const Place s = place_all<TS>(), p = place<PL::TP>(G);
+    const CoefR<R> cfs = load_coef<R>(d.coef);  // derived by k_adjL
+    CV<V> xp[PL::EP];
+    {
+        const int k2 = blockIdx.x * G + p.line;
+        const C *aw = static_cast<const C *>(d.aw) + 2 * (size_t)k2 * L;
 #pragma unroll
-    for (int r = 0; r < 16; ++r) {
-        const int n = t + r * T;
-        UV<R> e = valid ? ld_uv<R>(aw + 2 * n) : UV<R>{C{0, 0}, C{0, 0}};
-        x[r] = pack2<R>(e.u, e.v);
+        for (int i = 0; i < PL::EP; ++i) {
+            const UV<R> e = p.on && k2 <= a.K2 ? ld_uv<R>(aw + 2 * (p.t + i * PL::TP)) : UV<R>{C{0, 0}, C{0, 0}};
+            xp[i] = pack2<R>(e.u, e.v);
+        }
     }
-    __shared__ CoefR<R> cfs;
-    Coef cf{};  // thread 0 only
-    if (threadIdx.x == 0) {
-        cf = step_coef(a, *d.t, false);
-        cfs = coef_r<R>(cf, a);
-    }
-    fft_line<-1, LOG>(x, a.logn1, t, sm, static_cast<const C *>(d.tw1));
-    __syncthreads();  // cfs
+    auto buf = [&](int line) { return planes3<V, R>(smstep, line, SL); };
+    CV<V> xs[PL::ES];
+    forward3<PL, true>(xp, xs, p, s, buf, tab3<R, A, F, C>(d.tw1));
+    griddep_launch();
+    const int k2 = blockIdx.x * G + s.line;
     const bool lin = !(a.flags & kNonlinearOnly), nl = !(a.flags & kLinearOnly);
     const R ra = cfs.a, rb = cfs.b, rcs = cfs.cs, rdt = cfs.dt;
     const R s1 = scale1<R>(a), s2 = scale2<R>(a);
@@ -408,38 +468,33 @@ template <class R, int LOG> __global__ void __launch_bounds__(256, kMinBlocks<R>
     const C *phi = static_cast<const C *>(d.state) + (size_t)k2 * ld1 + a.K1;
     double dg = 0.0;  // sum of 2 kappa (lambda . Phi); times dt / (2 r0) at the end
 #pragma unroll
-    for (int r = 0; r < 16; ++r) {
-        if (r < 4 || r >= 12) {
-            const int n = t + r * T;
-            const int k1 = (r < 4) ? n : n - N1;
-            const bool in_box = valid && ((r < 4) ? (n <= a.K1) : (k1 >= -a.K1));
-            // k2 = 0, k1 < 0: conjugate mirror of +k1, written (and counted in
-            // the gamma gradient, with the same value) by the owner of +k1
-            if (!in_box || (k1 == 0 && k2 == 0) || (k2 == 0 && k1 < 0)) continue;
-            const R f1 = s1 * (R)k1;
-            C Q1 = lane0<R>(x[r]), Q2 = lane1<R>(x[r]);
-            C Pk{f1 * Q1.y + Q2.x, -f1 * Q1.x + Q2.y};  // -i f1 Q1 + Q2
-            C l = lam[k1];
-            const R kap = kappa_norm<R>(f1, s2 * (R)k2);
-            if (lin) {
-                C ph = phi[k1];
-                // weight 2: k2 > 0 stands for +-k; k2 = 0 here counts +k1 and -k1
-                dg += 2.0 * (double)kap * ((double)l.x * ph.x + (double)l.y * ph.y);
-            }
-            const R om = lin ? kap * (rb - kap * ra) : (R)0;
-            const R cn = nl ? rcs : (R)0;
-            C nw{l.x + rdt * (om * l.x + cn * Pk.x), l.y + rdt * (om * l.y + cn * Pk.y)};
-            lout[k1] = nw;
-            if (k2 == 0) lout[-k1] = C{nw.x, -nw.y};
+    for (int r = 0; r < PL::ES; ++r) {
+        if (r >= F && r < 2 * F) continue;
+        const int n = s.t + r * TS, k1 = r < F ? n : n - L;
+        const bool in_box = k2 <= a.K2 && (r < F ? n <= a.K1 : k1 >= -a.K1);
+        // k2 = 0, k1 < 0: conjugate mirror of +k1, written (and counted in
+        // the gamma gradient, with the same value) by the owner of +k1
+        if (!in_box || (k1 == 0 && k2 == 0) || (k2 == 0 && k1 < 0)) continue;
+        const R f1 = s1 * (R)k1;
+        const C Q1 = lane0<R>(xs[r]), Q2 = lane1<R>(xs[r]);
+        const C Pk{f1 * Q1.y + Q2.x, -f1 * Q1.x + Q2.y};  // -i f1 Q1 + Q2
+        const C l = lam[k1];
+        R kap;
+        if (sizeof(R) == 8 && d.kap) kap = static_cast<const R *>(d.kap)[(size_t)k2 * ld1 + a.K1 + k1];
+        else kap = kappa_norm<R>(f1, s2 * (R)k2);
+        if (lin) {
+            const C ph = phi[k1];
+            // weight 2: k2 > 0 stands for +-k; k2 = 0 here counts +k1 and -k1
+            dg += 2.0 * (double)kap * ((double)l.x * ph.x + (double)l.y * ph.y);
         }
+        const R om = lin ? kap * (rb - kap * ra) : (R)0;
+        const R cn = nl ? rcs : (R)0;
+        const C nw{l.x + rdt * (om * l.x + cn * Pk.x), l.y + rdt * (om * l.y + cn * Pk.y)};
+        lout[k1] = nw;
+        if (k2 == 0) lout[-k1] = C{nw.x, -nw.y};
     }
-    red[threadIdx.x] = dg;  // any block size
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        double s = 0.0;
-        for (int i = 0; i < (int)blockDim.x; ++i) s += red[i];
-        if (s != 0.0) atomicAdd(d.dgamma, s * (a.dt / (2.0 * cf.tn)));
-    }
+    const double sum = cta_sum(dg, red);
+    if (threadIdx.x == 0 && sum != 0.0) atomicAdd(d.dgamma, sum * d.coef[10]);
 }
 
 }  // namespace flame

@@ -270,7 +270,7 @@ FlameDesc make_desc(flame_ctx *h, void *state, double *mean, double *t) {
     FlameDesc d;
     memset(&d, 0, sizeof d);  // descriptors are compared bytewise
     d.a = h->ss;
-    d.state = state;
+    d.state = d.state_out = state;
     d.uv = h->uv;
     d.gk = h->gk;
     d.tw1 = h->tw1s;
@@ -278,7 +278,7 @@ FlameDesc make_desc(flame_ctx *h, void *state, double *mean, double *t) {
     d.kap = h->kap;
     d.t_in = t;
     d.coef = h->dscal + 8;
-    d.mean = mean;
+    d.mean = d.mean_out = mean;
     d.t_out = t;
     d.status = h->status;
     if (h->l2_state_bytes) d.l2_state = flame::L2Window{state, h->l2_state_bytes, h->l2_state_hit};
@@ -341,7 +341,7 @@ cudaError_t enqueue_step_area(flame_ctx *h, const FlameDesc &ds, cudaStream_t s)
     d.arow = h->rowsum;
     const bool f64 = h->p.prec == FLAME_FP64;
     const CUtensorMap *um = h->has_uv_map_full ? &h->uv_map_full : nullptr;
-    if ((e = f64 ? Ops<double>::passA_full(d, s, false, nullptr) : Ops<float>::passA_full(d, s, false, um)) != cudaSuccess)
+    if ((e = f64 ? Ops<double>::passA_full(d, s, nullptr) : Ops<float>::passA_full(d, s, um)) != cudaSuccess)
         return e;
     e = f64 ? Ops<double>::passB_area(d, s) : Ops<float>::passB_area(d, s);
     if (e == cudaErrorNotSupported) {
@@ -1442,8 +1442,12 @@ flame_status flame_adjoint(flame_t h, const void *state0, const double *mean0, c
     double *trt = trm + K;
     double *lam0 = h->dscal + 1, *dgam = h->dscal + 2;
     const bool f64 = h->p.prec == FLAME_FP64;
-    auto step1 = [&](void *st, double *m, double *t, cudaStream_t q) -> cudaError_t {
+    // one step from (st, m, t) to (so, mo, to), the same or other buffers
+    auto step1 = [&](void *st, double *m, double *t, void *so, double *mo, double *to, cudaStream_t q) -> cudaError_t {
         FlameDesc d = make_desc(h, st, m, t);
+        d.state_out = so;
+        d.mean_out = mo;
+        d.t_out = to;
         d.rec = nullptr;  // the recomputed steps are not recorded
         d.rec_cap = 0;
         return enqueue_step(h, d, q);
@@ -1460,18 +1464,16 @@ flame_status flame_adjoint(flame_t h, const void *state0, const double *mean0, c
     } while (0)
     auto enqueue = [&](cudaStream_t q) -> cudaError_t {
         // forward sweep from ckpt(0): checkpoints every K steps
-        for (int g = 1; g < nseg; ++g) {
-            ADJ_TRY(cudaMemcpyAsync(ckpt(g), ckpt(g - 1), box, cudaMemcpyDeviceToDevice, q));
-            ADJ_TRY(cudaMemcpyAsync(ckm + g, ckm + g - 1, sizeof(double), cudaMemcpyDeviceToDevice, q));
-            ADJ_TRY(cudaMemcpyAsync(ckt + g, ckt + g - 1, sizeof(double), cudaMemcpyDeviceToDevice, q));
-            for (int i = 0; i < K; ++i) ADJ_TRY(step1(ckpt(g), ckm + g, ckt + g, q));
-        }
+        for (int g = 1; g < nseg; ++g)
+            for (int i = 0; i < K; ++i)
+                ADJ_TRY(step1(i ? ckpt(g) : ckpt(g - 1), ckm + g - (i ? 0 : 1), ckt + g - (i ? 0 : 1), ckpt(g), ckm + g,
+                              ckt + g, q));
         // reverse sweep from lam, lam0 (the final adjoint)
         ADJ_TRY(cudaMemsetAsync(lam + k0, 0, h->csz, q));
         ADJ_TRY(cudaMemsetAsync(dgam, 0, sizeof(double), q));
         flame::AdjDesc d;
         memset(&d, 0, sizeof d);
-        d.a = h->sa;
+        d.a = h->ss;
         d.lam = lam;
         d.lam_out = lam;
         d.lam0 = lam0;
@@ -1479,22 +1481,23 @@ flame_status flame_adjoint(flame_t h, const void *state0, const double *mean0, c
         d.gk = h->gk;
         d.aw = h->aw;
         d.dgamma = dgam;
-        d.tw1 = h->tw1;
-        d.twm = h->twm;
+        d.tw1 = h->tw1s;
+        d.twm = h->twms;
+        d.coef = h->dscal + 8;
+        d.kap = h->kap;
         for (int g = nseg - 1; g >= 0; --g) {
             const int len = (g == nseg - 1) ? nsteps - g * K : K;
-            ADJ_TRY(cudaMemcpyAsync(traj(0), ckpt(g), box, cudaMemcpyDeviceToDevice, q));
-            ADJ_TRY(cudaMemcpyAsync(trm, ckm + g, sizeof(double), cudaMemcpyDeviceToDevice, q));
-            ADJ_TRY(cudaMemcpyAsync(trt, ckt + g, sizeof(double), cudaMemcpyDeviceToDevice, q));
-            for (int i = 1; i < len; ++i) {
-                ADJ_TRY(cudaMemcpyAsync(traj(i), traj(i - 1), box, cudaMemcpyDeviceToDevice, q));
-                ADJ_TRY(cudaMemcpyAsync(trm + i, trm + i - 1, sizeof(double), cudaMemcpyDeviceToDevice, q));
-                ADJ_TRY(cudaMemcpyAsync(trt + i, trt + i - 1, sizeof(double), cudaMemcpyDeviceToDevice, q));
-                ADJ_TRY(step1(traj(i), trm + i, trt + i, q));
-            }
+            // the segment's trajectory: state 0 is the checkpoint, state i > 0
+            // is traj(i), each step's output (copied from buffer to buffer
+            // instead, a step's three small copies took half as long as it)
+            auto state_at = [&](int i) { return i ? traj(i) : ckpt(g); };
+            auto mean_at = [&](int i) { return i ? trm + i : ckm + g; };
+            auto t_at = [&](int i) { return i ? trt + i : ckt + g; };
+            for (int i = 1; i < len; ++i)
+                ADJ_TRY(step1(state_at(i - 1), mean_at(i - 1), t_at(i - 1), state_at(i), mean_at(i), t_at(i), q));
             for (int i = len - 1; i >= 0; --i) {
-                d.state = traj(i);
-                d.t = trt + i;
+                d.state = state_at(i);
+                d.t = t_at(i);
                 if (f64) ADJ_TRY(Ops<double>::adj_step(d, q));
                 else ADJ_TRY(Ops<float>::adj_step(d, q));
             }

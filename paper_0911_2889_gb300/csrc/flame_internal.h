@@ -96,7 +96,8 @@ struct L2Window {
 
 struct FlameDesc {
     StepArgs a;
-    void *state;            // compact box (in place)
+    void *state;            // compact box read by the step
+    void *state_out;        // ... and written (the same, or another buffer: the adjoint's trajectory)
     void *uv;               // N1 x ldk pairs: the row spectra at +-k2 (public grid: (U, V))
     void *gk;               // N1 x ldk workspace
     const void *tw1;        // twiddles of length N1
@@ -108,8 +109,8 @@ struct FlameDesc {
     // CoefR (1/r0^2, gamma/(2 r0), c/(N1 N2), dt, ia, ib), [8] n,
     // [9] 1/(N1 N2); 80 bytes, 16-byte aligned (handle scratch)
     double *coef;
-    double *mean;           // caller's mean mode
-    double *t_out;          // caller's t (written by pass C)
+    double *mean;           // mean mode read by the step
+    double *mean_out, *t_out;  // mean mode and t written by pass C
     int *status;            // handle's device status word
     // two-stage schemes: the stage of this pass C launch (kStage*) and the
     // box-layout buffer and FP64 scalar that carry a term from stage 1 to
@@ -163,6 +164,8 @@ struct AdjDesc {
     double *area;        // area output
     double *dmean;       // dA/dPhi_0 output
     double *dgamma;      // dL/dgamma accumulator (atomic)
+    double *coef;        // adjoint step: the step's coefficients (k_adjL to k_adjC)
+    const void *kap;     // adjoint step: |kappa| of every box entry (FP64) or null
     const void *tw1, *twm;
 };
 
@@ -211,9 +214,8 @@ template <class R> struct Ops {
     static void tiles(const StepArgs &a, int variant, int *colsA, int *pairsC);
     // A step on the public grid that also sums the surface area of its rows
     // (arow[pair]); passB_area: cudaErrorNotSupported when its shared memory
-    // exceeds the device's limit.  pairs: two lines per thread whatever the
-    // column length (the adjoint step).
-    static cudaError_t passA_full(const FlameDesc &d, cudaStream_t s, bool pairs, const CUtensorMap *uv_map);
+    // exceeds the device's limit.
+    static cudaError_t passA_full(const FlameDesc &d, cudaStream_t s, const CUtensorMap *uv_map);
     static cudaError_t passB_area(const FlameDesc &d, cudaStream_t s);
     static cudaError_t passC_full(const FlameDesc &d, cudaStream_t s);
     // geometry used by the step passes (for the autotuner and the tests)
@@ -221,8 +223,9 @@ template <class R> struct Ops {
     static Geom geom_rows(int logm, int nlines, int groups_hint);
     // Area objective (and its gradient when d.grad / d.dmean are set): 3 kernels.
     static cudaError_t area(const AdjDesc &d, cudaStream_t s);
-    // One adjoint step at (d.state, d.t): pass A on the forward state, column
-    // synthesis of lambda, row pass, column pass with the lambda update.
+    // One adjoint step at (d.state, d.t) on the alias-free grid (d.a, d.tw1,
+    // d.twm, d.uv: the step's): pass A on the forward state, column synthesis
+    // of lambda, row pass, column pass with the lambda update.
     static cudaError_t adj_step(const AdjDesc &d, cudaStream_t s);
 };
 

@@ -920,7 +920,7 @@ template <class R> struct EpiArgs {
 // transform gh = c-free ghat and the entry ph entering the step:
 // Phi <- Phi + dt (omega Phi + c ghat + f) for the Euler stage and the
 // combinations of the two-stage schemes (see kStage*).  col, fcol and scol
-// point at k1 = 0 of column k2 of the state, the forcing (or null) and the
+// point at k1 = 0 of column k2 of the new state, the forcing (or null) and the
 // stage buffer (or null); the k2 = 0 column also gets the conjugate mirror
 // at -k1.  nw returns the new entry (0 for k = 0); bad collects non-finite
 // results.
@@ -1009,11 +1009,11 @@ __device__ __forceinline__ void finish_step(const FlameDesc &d, int stage, bool 
     if (stage == kStageEuler || stage == kStageHeun1 || stage == kStageIF1) {
         if (stage == kStageHeun1) *d.save_mean = m;
         if (stage == kStageIF1) *d.save_mean = m + 0.5 * inc;
-        *d.mean = m + inc;
+        *d.mean_out = m + inc;
         *d.t_out = a.t0 + (n + 1.0) * a.dt;
     } else {
         // second stages are evaluated at t_{n+1} and leave t there
-        *d.mean = stage == kStageHeun2 ? 0.5 * (*d.save_mean + m + inc) : *d.save_mean + 0.5 * inc;
+        *d.mean_out = stage == kStageHeun2 ? 0.5 * (*d.save_mean + m + inc) : *d.save_mean + 0.5 * inc;
         *d.t_out = a.t0 + n * a.dt;
     }
 }

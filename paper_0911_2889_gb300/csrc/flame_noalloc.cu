@@ -101,14 +101,14 @@ flame_status run_steps(const flame::StepArgs &a, unsigned char *base, size_t off
     flame::FlameDesc d;
     memset(&d, 0, sizeof d);
     d.a = a;
-    d.state = state;
+    d.state = d.state_out = state;
     d.uv = base + off_uv;
     d.gk = base + off_gk;
     d.tw1 = base + off_tw1;
     d.twm = base + off_twm;
     d.t_in = t;
     d.coef = dscal + 8;  // 80 bytes at off_sc + 64 (the arena keeps 256 bytes there)
-    d.mean = mean;
+    d.mean = d.mean_out = mean;
     d.t_out = t;
     d.status = status;
     for (int i = 0; i < nsteps; ++i) {

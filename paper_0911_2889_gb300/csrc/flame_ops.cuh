@@ -160,9 +160,9 @@ template <class F> static void with_fp64_points(F &&f) {
 }
 
 // Passes A and C on the public grid: the steps that record the surface area
-// (whose sum is over that grid's points) and the adjoint step's pass A.
+// (whose sum is over that grid's points).
 template <class R>
-cudaError_t Ops<R>::passA_full(const FlameDesc &d, cudaStream_t s, bool pairs, const CUtensorMap *uv_map) {
+cudaError_t Ops<R>::passA_full(const FlameDesc &d, cudaStream_t s, const CUtensorMap *uv_map) {
     cudaError_t err = cudaErrorInvalidValue;
     if constexpr (sizeof(R) == 8) if (small_fp64<R>(d.a.logn1)) {
         with_fp64_points([&](auto ec) {
@@ -176,7 +176,7 @@ cudaError_t Ops<R>::passA_full(const FlameDesc &d, cudaStream_t s, bool pairs, c
         });
         return err;
     }
-    if constexpr (sizeof(R) == 4) if (!pairs && one_line_fp32<R>(d.a.logn1)) {
+    if constexpr (sizeof(R) == 4) if (one_line_fp32<R>(d.a.logn1)) {
         const Geom g = geom_short1<R, 16>(d.a.logn1, d.a.K2 + 1, 2, 0);
         static_for<8, 11>([&](auto lc) {
             constexpr int L = decltype(lc)::value;
@@ -328,6 +328,15 @@ template <class R> cudaError_t Ops<R>::area(const AdjDesc &d, cudaStream_t s) {
     return e;
 }
 
+// CTA of an adjoint kernel: lines of T threads, up to 128 threads, fewer lines
+// where they would not span two CTAs per SM
+template <class R, int A> static Geom geom_adj(int nlines) {
+    using V = typename VecOf<R>::type;
+    using PL = Plan3<A, adj_f<R>(A)>;
+    int G = PL::TS >= 128 ? 1 : 128 / PL::TS;
+    while (G > 1 && (G * PL::TS > 32) && (nlines + G - 1) / G < 2 * sm_count()) G >>= 1;
+    return Geom{G * PL::TS, (nlines + G - 1) / G, exchange_bytes<R, V, PL>(G)};
+}
 template <class R> cudaError_t Ops<R>::adj_step(const AdjDesc &d, cudaStream_t s) {
     const StepArgs &a = d.a;
     FlameDesc f;
@@ -336,22 +345,22 @@ template <class R> cudaError_t Ops<R>::adj_step(const AdjDesc &d, cudaStream_t s
     f.state = const_cast<void *>(d.state);
     f.uv = d.uv;
     f.tw1 = d.tw1;
-    cudaError_t e = passA_full(f, s, true, nullptr);
+    cudaError_t e = passA(f, s, a.la <= 8 ? kVariantOneLine : kVariantDirect);
     if (e != cudaSuccess) return e;
-    Geom gl = geom_cols(a.logn1, (a.K2 + 2) / 2, 0);
-    Geom gb = geom_row1<R>(a.logm, a.n1);
-    Geom ga = geom_cols(a.logn1, a.K2 + 1, 0);
-    with_log<R>(a.logn1, [&](auto lc) {
-        constexpr int L = decltype(lc)::value;
-        e = launch_k(k_adjL<R, L>, dim3(gl.blocks), gl.threads, gl.smem, s, d);
+    with_a(a.la, [&](auto ac) {
+        constexpr int A = decltype(ac)::value;
+        const Geom g = geom_adj<R, A>((a.K2 + 2) / 2);
+        e = launch_s(L2Window{nullptr, 0, 0.f}, pdl_on(sizeof(R) == 8, a), k_adjL<R, A>, dim3(g.blocks + 1), g.threads, g.smem, s, d);
     });
-    with_log<R>(a.logm, [&](auto lc) {
-        constexpr int L = decltype(lc)::value;
-        if (e == cudaSuccess) e = launch_k(k_adjB<R, L>, dim3(gb.blocks), gb.threads, gb.smem, s, d);
+    with_a(a.lb, [&](auto ac) {
+        constexpr int A = decltype(ac)::value;
+        const Geom g = geom_adj<R, A>(a.n1);
+        if (e == cudaSuccess) e = launch_s(L2Window{nullptr, 0, 0.f}, pdl_on(sizeof(R) == 8, a), k_adjB<R, A>, dim3(g.blocks), g.threads, g.smem, s, d);
     });
-    with_log<R>(a.logn1, [&](auto lc) {
-        constexpr int L = decltype(lc)::value;
-        if (e == cudaSuccess) e = launch_k(k_adjC<R, L>, dim3(ga.blocks), ga.threads, ga.smem, s, d);
+    with_a(a.la, [&](auto ac) {
+        constexpr int A = decltype(ac)::value;
+        const Geom g = geom_adj<R, A>(a.K2 + 1);
+        if (e == cudaSuccess) e = launch_s(L2Window{nullptr, 0, 0.f}, pdl_on(sizeof(R) == 8, a), k_adjC<R, A>, dim3(g.blocks), g.threads, g.smem, s, d);
     });
     return e;
 }

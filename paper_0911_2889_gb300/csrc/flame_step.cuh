@@ -43,7 +43,8 @@ template <class R, int A, int F, class C> __device__ __forceinline__ const C *ta
 }
 // exchange buffer of line (or line pair) `line`, `slots` slots each
 template <class V, class R> __device__ __forceinline__ Planes<V> planes3(unsigned char *smem, int line, int slots) {
-    if constexpr (kLanes<V> == 2) return Planes<V>(reinterpret_cast<V *>(smem) + (size_t)line * 2 * slots);
+    if constexpr (std::is_same<V, float2>::value) return Planes<V>(reinterpret_cast<V *>(smem) + (size_t)line * 2 * slots);
+    else if constexpr (kLanes<V> == 2) return Planes<V>(reinterpret_cast<V *>(smem) + (size_t)line * 2 * slots, 0, slots);
     else return Planes<V>(reinterpret_cast<R *>(smem) + (size_t)line * 2 * slots, slots);
 }
 // bytes of a CTA's exchange buffers
@@ -542,7 +543,7 @@ __device__ __forceinline__ void stepC_body(const FlameDesc &d, int tile, const A
     extern __shared__ __align__(128) unsigned char smstep[];
     const StepArgs &a = d.a;
     const C *__restrict__ gk = static_cast<const C *>(d.gk);
-    C *__restrict__ state = static_cast<C *>(d.state);
+    const C *state = static_cast<const C *>(d.state);
     const C *tw = tab3<R, A, F, C>(d.tw1);
     const int G = blockDim.x / (TS * LPC);
     const Place s = NL == 2 ? place_all<TS>() : place<TS>(G * LPC), p = place<TP>(G * LPC);
@@ -574,7 +575,8 @@ __device__ __forceinline__ void stepC_body(const FlameDesc &d, int tile, const A
     forward3<PL, true>(xp, xs, p, s, buf, tw);
 
     const int c0 = 2 * (tile * G + s.line / LPC) + (NL == 1 ? s.line & 1 : 0);
-    C *col = state + (size_t)c0 * ld1 + a.K1;
+    const C *col = state + (size_t)c0 * ld1 + a.K1;
+    C *ocol = static_cast<C *>(d.state_out) + (size_t)c0 * ld1 + a.K1;
     // the band entries of this thread: r < F (k1 = n) and r >= 2F (k1 = n - L);
     // read after the transform, from the L2 window over the state
     auto k1_of = [&](int i) { return i < F ? s.t + i * TS : s.t + (i + F) * TS - L; };
@@ -607,7 +609,7 @@ __device__ __forceinline__ void stepC_body(const FlameDesc &d, int tile, const A
             if constexpr (NL == 2) gh = side == 0 ? lane0<R>(x) : lane1<R>(x);
             else gh = C{x.re.x, x.im.x};
             const int off = side * ld1;
-            update_entry<R, GEN>(d, ea, k1, k2, gh, phi[i], col + off, fcol ? fcol + off : nullptr,
+            update_entry<R, GEN>(d, ea, k1, k2, gh, phi[i], ocol + off, fcol ? fcol + off : nullptr,
                                  scol ? scol + off : nullptr, nphi[i][side], bad);
         }
     }
@@ -619,7 +621,7 @@ __device__ __forceinline__ void stepC_body(const FlameDesc &d, int tile, const A
         if (c0 == 0 && s.on) {
 #pragma unroll
             for (int i = F; i < 2 * F; ++i)
-                if (k1_of(i) >= -a.K1 && FLAME_IN(d.status, a.K1 + k1_of(i), box_len(a), kSiteCState)) nphi[i][0] = col[k1_of(i)];
+                if (k1_of(i) >= -a.K1 && FLAME_IN(d.status, a.K1 + k1_of(i), box_len(a), kSiteCState)) nphi[i][0] = ocol[k1_of(i)];
         }
         auto park = [&](int line) { return reinterpret_cast<float4 *>(smstep) + (size_t)line * SL; };
         const bool odd = threadIdx.x & 1;

@@ -128,9 +128,11 @@ template <int A_, int F_> struct Plan3 {
         return ((a > b ? a : b) + 7) & ~7;
     }
 };
-// slots per 128-byte wavefront of an exchange buffer: two FP32 lines take 16
-// bytes a slot, one line keeps separate planes of 4 (FP32) or 8 (FP64) bytes
-template <class V> constexpr int kSlotsPerWave = std::is_same<V, float2>::value ? 8 : std::is_same<V, F1>::value ? 32 : 16;
+// slots per 128-byte wavefront of an exchange buffer: two lines take 16 bytes a
+// slot (FP64: in each of two planes), one line keeps separate planes of 4
+// (FP32) or 8 (FP64) bytes
+template <class V> constexpr int kSlotsPerWave =
+    std::is_same<V, float2>::value || std::is_same<V, double2>::value ? 8 : std::is_same<V, F1>::value ? 32 : 16;
 
 // ----------------------------------------------------------------------------
 // Twiddle allocation of a line: the tables of F = 1, 2, 4 (where the line is
