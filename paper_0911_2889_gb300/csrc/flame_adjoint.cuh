@@ -380,7 +380,7 @@ template <class R, int A> __global__ void __launch_bounds__(256, kMinBlocks<R>) 
     {
         CV<V> xs[ES], xp[PL::EP];
         half_inputs<PL, R>(xs, s.t, valid, a.K2, P, [&](int k, bool minus) {
-            const C e = __ldg(lrow + l_index(row, k, a.ldk));
+            const C e = lrow[l_index(row, k, a.ldk)];
             return minus ? C{e.x, -e.y} : e;
         });
         inverse3<PL>(xs, xp, s, p, buf, tw);

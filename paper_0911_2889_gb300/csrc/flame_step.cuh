@@ -65,13 +65,14 @@ __host__ __device__ __forceinline__ size_t w_index(int j1, int k2, int ldk) { re
 __host__ __device__ __forceinline__ size_t g_index(int j1, int k2, int n1) {
     return 2 * (size_t)(k2 >> 1) * n1 + 4 * (j1 >> 1) + 2 * (k2 & 1) + (j1 & 1);
 }
-// W(j1, +-k2) of one row
+// W(j1, +-k2) of one row.  What the previous kernel wrote is read by plain loads,
+// never __ldg or through __restrict__: those may move ahead of griddep_wait.
 template <class R> __device__ __forceinline__ CplxT<R> ld_w(const CplxT<R> *uv, int j1, int k2, int ldk, bool minus) {
     const CplxT<R> *e = uv + w_index(j1, k2, ldk) + 2 * w_half<R>(k2, minus);
     if constexpr (std::is_same<R, float>::value) {
-        const float4 q = __ldg(reinterpret_cast<const float4 *>(e));
+        const float4 q = *reinterpret_cast<const float4 *>(e);
         return j1 & 1 ? CplxT<R>{q.y, q.w} : CplxT<R>{q.x, q.z};
-    } else return __ldg(e + (j1 & 1));
+    } else return e[j1 & 1];
 }
 // ... written by two adjacent threads, rows 2i and 2i+1 (all threads call it):
 // FP32, one shuffle, and each thread writes 8 of the 16 bytes
@@ -128,7 +129,7 @@ __device__ __forceinline__ void stepA_body(const FlameDesc &d, int tile, const A
     // (two lines per thread: CTAs are whole lines)
     const Place s = NL == 2 ? place_all<PL::TS>() : place<PL::TS>(G * LPC), p = place<PL::TP>(G * LPC);
     const int ld1 = 2 * a.K1 + 1;
-    const C *__restrict__ state = static_cast<const C *>(d.state);
+    const C *state = static_cast<const C *>(d.state);
     C *__restrict__ uv = static_cast<C *>(d.uv);
     CV<V> xs[PL::ES];
     {
@@ -142,7 +143,7 @@ __device__ __forceinline__ void stepA_body(const FlameDesc &d, int tile, const A
             const int n = s.t + r * PL::TS, k1 = r < F ? n : n - PL::L;
             const bool in_box = s.on && k2 <= a.K2 && (r < F ? n <= a.K1 : k1 >= -a.K1);
             if (in_box && FLAME_IN(d.status, (long long)k2 * ld1 + a.K1 + k1, box_len(a), kSiteAState)) {
-                C phi = __ldg(col + k1);
+                C phi = col[k1];
                 if (k1 == 0 && k2 == 0) phi = C{0, 0};
                 const R f = s1 * (R)k1;
                 const C da{-f * phi.y, f * phi.x}, db{s2k2 * phi.x, s2k2 * phi.y};
@@ -310,7 +311,7 @@ __device__ __forceinline__ void stepB2_body(const FlameDesc &d, int tile, const 
     constexpr int L = PL::L, TS = PL::TS, TP = PL::TP, ES = PL::ES, SL = PL::slots(kSlotsPerWave<V>);
     extern __shared__ __align__(128) unsigned char smstep[];
     const StepArgs &a = d.a;
-    const C *__restrict__ uv = static_cast<const C *>(d.uv);
+    const C *uv = static_cast<const C *>(d.uv);
     C *__restrict__ gk = static_cast<C *>(d.gk);
     const int G = blockDim.x / TS;
     const Place s = place_all<TS>(), p = place<TP>(G);
@@ -452,7 +453,7 @@ __device__ __forceinline__ void stepB1_body(const FlameDesc &d, int unit0) {
     constexpr int L = PL::L, TS = PL::TS, TP = PL::TP, ES = PL::ES, SL = PL::slots(kSlotsPerWave<V>);
     extern __shared__ __align__(128) unsigned char smstep[];
     const StepArgs &a = d.a;
-    const C *__restrict__ uv = static_cast<const C *>(d.uv);
+    const C *uv = static_cast<const C *>(d.uv);
     C *__restrict__ gk = static_cast<C *>(d.gk);
     const int U = blockDim.x / (2 * RW * TS), lines = 2 * RW * U;  // units of the CTA
     const Place s = place<TS>(lines), p = place<TP>(lines);
@@ -468,10 +469,18 @@ __device__ __forceinline__ void stepB1_body(const FlameDesc &d, int unit0) {
         for (int r = 0; r < ES; ++r) {
             const int n = s.t + r * TS, km = L - n;
             C up{0, 0}, um{0, 0};
-            if (r < 2 * F && valid && n <= a.K2 && FLAME_IN(d.status, w_index(row, n, a.ldk) + 3, uv_len(a), kSiteBUv))
-                up = ld_w<R>(uv, row, n, a.ldk, false);
-            if (r >= F && valid && km <= a.K2 && FLAME_IN(d.status, w_index(row, km, a.ldk) + 3, uv_len(a), kSiteBUv))
-                um = ld_w<R>(uv, row, km, a.ldk, true);
+            // loads without branches (element 0 where there is none): a forced
+            // 512x1024 run 596 -> 579 us
+            if (r < 2 * F) {
+                const bool in = valid && n <= a.K2 && FLAME_IN(d.status, w_index(row, n, a.ldk) + 3, uv_len(a), kSiteBUv);
+                const C v = ld_w<R>(uv, in ? row : 0, in ? n : 0, a.ldk, false);
+                if (in) up = v;
+            }
+            if (r >= F) {
+                const bool in = valid && km <= a.K2 && FLAME_IN(d.status, w_index(row, km, a.ldk) + 3, uv_len(a), kSiteBUv);
+                const C v = ld_w<R>(uv, in ? row : 0, in ? km : 0, a.ldk, true);
+                if (in) um = v;
+            }
             C z{up.x + um.x, up.y + um.y};
             if (odd) {
                 const C o{up.x - um.x, up.y - um.y}, w = __ldg(P + n);  // exp(2 pi i n / 2L)
@@ -542,7 +551,7 @@ __device__ __forceinline__ void stepC_body(const FlameDesc &d, int tile, const A
     static_assert(!FUSE_A || NL == 2, "the fused pass is a two-line kernel");
     extern __shared__ __align__(128) unsigned char smstep[];
     const StepArgs &a = d.a;
-    const C *__restrict__ gk = static_cast<const C *>(d.gk);
+    const C *gk = static_cast<const C *>(d.gk);
     const C *state = static_cast<const C *>(d.state);
     const C *tw = tab3<R, A, F, C>(d.tw1);
     const int G = blockDim.x / (TS * LPC);
@@ -558,8 +567,8 @@ __device__ __forceinline__ void stepC_body(const FlameDesc &d, int tile, const A
             const int n = p.t + i * TP;
             const bool in = p.on && c <= a.K2 && FLAME_IN(d.status, g_index(n, c, L) + (NL == 2 ? 2 : 0), gk_len(a), kSiteCGk);
             const C *q = gk + g_index(n, c, L);
-            const C q0 = in ? __ldg(q) : C{0, 0};
-            if constexpr (NL == 2) xp[i] = pack2<R>(q0, in && c < a.K2 ? __ldg(q + 2) : C{0, 0});
+            const C q0 = in ? *q : C{0, 0};
+            if constexpr (NL == 2) xp[i] = pack2<R>(q0, in && c < a.K2 ? q[2] : C{0, 0});
             else xp[i] = CV<V>{{q0.x}, {q0.y}};
         }
     }
