@@ -159,6 +159,8 @@ struct flame_ctx {
     size_t csz;       // bytes of one complex element
     void *tabs;       // one allocation: the tables, rowsum, dscal and status below
     void *tw1, *twm;  // twiddle tables of the public grid's lines
+    void *twc;        // of the 2-D transforms' columns: N1/split points (flame::fft_split)
+    int split;
     void *tw1s, *twms;  // ... and of the step grid's
     void *kap;        // |kappa| of every box entry (FP64), else null
     void *uv, *gk;    // step workspaces
@@ -236,6 +238,7 @@ template <class R> flame_status alloc_tables(flame_ctx *h) {
     using C = typename Ops<R>::C;
     CUDA_TRY(Ops<R>::init_twiddles(static_cast<C *>(h->tw1), h->logn1, h->cap));
     CUDA_TRY(Ops<R>::init_twiddles(static_cast<C *>(h->twm), h->logm, h->cap));
+    if (h->split > 1) CUDA_TRY(Ops<R>::init_twiddles(static_cast<C *>(h->twc), h->logn1 - 2, h->cap));
     CUDA_TRY(Ops<R>::init_twiddles3(static_cast<C *>(h->tw1s), h->ss.la, h->cap));
     CUDA_TRY(Ops<R>::init_twiddles3(static_cast<C *>(h->twms), h->ss.lb, h->cap));
     if constexpr (sizeof(R) == 8) CUDA_TRY(Ops<R>::init_kappa(static_cast<R *>(h->kap), h->ss, h->cap));
@@ -876,6 +879,7 @@ flame_status flame_create(const flame_params *params, flame_t *out) {
         return fail(FLAME_ECUDA, "cudaGetDevice: %s", cudaGetErrorString(ge));
     }
     const size_t n1 = p.n_theta, ldk = a.ldk, m1 = p.n_phi / 2 + 1;
+    h->split = flame::fft_split(p.prec == FLAME_FP64, p.n_theta, h->logm);
     size_t tabs = 0;
     auto place = [&](size_t bytes) {
         const size_t at = tabs;
@@ -883,6 +887,7 @@ flame_status flame_create(const flame_params *params, flame_t *out) {
         return at;
     };
     const size_t o_tw1 = place(flame::tw_alloc_len(h->logn1) * h->csz), o_twm = place(flame::tw_alloc_len(h->logm) * h->csz),
+                 o_twc = place(h->split > 1 ? flame::tw_alloc_len(h->logn1 - 2) * h->csz : 0),
                  o_tw1s = place(flame::tw3_len_of(h->ss.la) * h->csz), o_twms = place(flame::tw3_len_of(h->ss.lb) * h->csz),
                  o_kap = place(p.prec == FLAME_FP64 ? (2 * (size_t)p.K1 + 1) * ldk * sizeof(double) : 0), o_rowsum = place(n1 * sizeof(double)), o_dscal = place(24 * sizeof(double)),
                  o_status = place(flame::kStatusWords * sizeof(int));
@@ -897,6 +902,7 @@ flame_status flame_create(const flame_params *params, flame_t *out) {
     char *tb = static_cast<char *>(h->tabs);
     h->tw1 = tb + o_tw1;
     h->twm = tb + o_twm;
+    h->twc = h->split > 1 ? tb + o_twc : h->tw1;
     h->tw1s = tb + o_tw1s;
     h->twms = tb + o_twms;
     h->kap = p.prec == FLAME_FP64 ? tb + o_kap : nullptr;
@@ -964,26 +970,49 @@ flame_status flame_get_params(flame_t h, flame_params *out) {
 
 size_t flame_state_len(flame_t h) { return h ? (size_t)(2 * h->p.K1 + 1) * (size_t)(h->p.K2 + 1) : 0; }
 
+}  // extern "C"
+
+namespace {
+// The two passes of a 2-D transform on handle h; the column pass of r2c is in place.
+template <class R> flame_status fft_r2c(flame_ctx *h, const void *real_in, void *spec_out, cudaStream_t s) {
+    using C = typename Ops<R>::C;
+    const int M = h->p.n_phi / 2;
+    C *spec = static_cast<C *>(spec_out);
+    CUDA_TRY(Ops<R>::rows_r2c(static_cast<const R *>(real_in), spec, h->p.n_theta, h->logm, static_cast<const C *>(h->twm),
+                              static_cast<const C *>(h->tw1), s, h->status));
+    CUDA_TRY(Ops<R>::cols(spec, spec, h->split > 1 ? h->logn1 - 2 : h->logn1, h->split, M + 1, M + 1, -1,
+                          static_cast<const C *>(h->twc), s, h->status));
+    return FLAME_OK;
+}
+template <class R> flame_status fft_c2r(flame_ctx *h, const void *spec_in, void *real_out, cudaStream_t s) {
+    using C = typename Ops<R>::C;
+    const int M = h->p.n_phi / 2;
+    C *spec = static_cast<C *>(h->spec);
+    CUDA_TRY(Ops<R>::cols(static_cast<const C *>(spec_in), spec, h->split > 1 ? h->logn1 - 2 : h->logn1, h->split, M + 1, M + 1,
+                          1, static_cast<const C *>(h->twc), s, h->status));
+    CUDA_TRY(Ops<R>::rows_c2r(spec, static_cast<R *>(real_out), h->p.n_theta, h->logm, static_cast<const C *>(h->twm),
+                              static_cast<const C *>(h->tw1), s, h->status));
+    return FLAME_OK;
+}
+template <class R>
+flame_status from_field(flame_ctx *h, const void *field, void *state, double *mean_mode, cudaStream_t s) {
+    using C = typename Ops<R>::C;
+    const flame_status st = fft_r2c<R>(h, field, h->spec, s);
+    if (st != FLAME_OK) return st;
+    CUDA_TRY(Ops<R>::box_from_spec(static_cast<const C *>(h->spec), static_cast<C *>(state), mean_mode, h->p.n_theta,
+                                   h->p.n_phi, h->p.K1, h->p.K2, s, h->status));
+    return FLAME_OK;
+}
+}  // namespace
+
+extern "C" {
+
 flame_status flame_fft_r2c(flame_t h, const void *real_in, void *spec_out, void *stream) {
     FLAME_RANGE("flame_fft_r2c");
     if (!h || !real_in || !spec_out) return fail(FLAME_EINVAL, "flame_fft_r2c: null pointer");
     if (inject("launch")) return fail(FLAME_ECUDA, "flame_fft_r2c: injected launch fault");
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    const int M = h->p.n_phi / 2;
-    if (h->p.prec == FLAME_FP64) {
-        using C = double2;
-        CUDA_TRY(Ops<double>::rows_r2c(static_cast<const double *>(real_in), static_cast<C *>(spec_out),
-                                       h->p.n_theta, h->logm, static_cast<const C *>(h->twm), s, h->status));
-        CUDA_TRY(Ops<double>::cols(static_cast<C *>(spec_out), static_cast<C *>(spec_out), h->logn1, M + 1,
-                                   M + 1, -1, static_cast<const C *>(h->tw1), s, h->status));
-    } else {
-        using C = float2;
-        CUDA_TRY(Ops<float>::rows_r2c(static_cast<const float *>(real_in), static_cast<C *>(spec_out),
-                                      h->p.n_theta, h->logm, static_cast<const C *>(h->twm), s, h->status));
-        CUDA_TRY(Ops<float>::cols(static_cast<C *>(spec_out), static_cast<C *>(spec_out), h->logn1, M + 1,
-                                  M + 1, -1, static_cast<const C *>(h->tw1), s, h->status));
-    }
-    return FLAME_OK;
+    return h->p.prec == FLAME_FP64 ? fft_r2c<double>(h, real_in, spec_out, s) : fft_r2c<float>(h, real_in, spec_out, s);
 }
 
 flame_status flame_state_from_field(flame_t h, const void *field, void *state, double *mean_mode, void *stream) {
@@ -991,23 +1020,8 @@ flame_status flame_state_from_field(flame_t h, const void *field, void *state, d
     if (!h || !field || !state || !mean_mode) return fail(FLAME_EINVAL, "flame_state_from_field: null pointer");
     if (inject("launch")) return fail(FLAME_ECUDA, "flame_state_from_field: injected launch fault");
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    const int n1 = h->p.n_theta, n2 = h->p.n_phi, M = n2 / 2;
-    if (h->p.prec == FLAME_FP64) {
-        using C = double2;
-        C *spec = static_cast<C *>(h->spec);
-        CUDA_TRY(Ops<double>::rows_r2c(static_cast<const double *>(field), spec, n1, h->logm,
-                                       static_cast<const C *>(h->twm), s, h->status));
-        CUDA_TRY(Ops<double>::cols(spec, spec, h->logn1, M + 1, M + 1, -1, static_cast<const C *>(h->tw1), s, h->status));
-        CUDA_TRY(Ops<double>::box_from_spec(spec, static_cast<C *>(state), mean_mode, n1, n2, h->p.K1, h->p.K2, s, h->status));
-    } else {
-        using C = float2;
-        C *spec = static_cast<C *>(h->spec);
-        CUDA_TRY(Ops<float>::rows_r2c(static_cast<const float *>(field), spec, n1, h->logm,
-                                      static_cast<const C *>(h->twm), s, h->status));
-        CUDA_TRY(Ops<float>::cols(spec, spec, h->logn1, M + 1, M + 1, -1, static_cast<const C *>(h->tw1), s, h->status));
-        CUDA_TRY(Ops<float>::box_from_spec(spec, static_cast<C *>(state), mean_mode, n1, n2, h->p.K1, h->p.K2, s, h->status));
-    }
-    return FLAME_OK;
+    return h->p.prec == FLAME_FP64 ? from_field<double>(h, field, state, mean_mode, s)
+                                   : from_field<float>(h, field, state, mean_mode, s);
 }
 
 flame_status flame_fft_c2r(flame_t h, const void *spec_in, void *real_out, void *stream) {
@@ -1015,21 +1029,7 @@ flame_status flame_fft_c2r(flame_t h, const void *spec_in, void *real_out, void 
     if (!h || !spec_in || !real_out) return fail(FLAME_EINVAL, "flame_fft_c2r: null pointer");
     if (inject("launch")) return fail(FLAME_ECUDA, "flame_fft_c2r: injected launch fault");
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    const int M = h->p.n_phi / 2;
-    if (h->p.prec == FLAME_FP64) {
-        using C = double2;
-        CUDA_TRY(Ops<double>::cols(static_cast<const C *>(spec_in), static_cast<C *>(h->spec), h->logn1, M + 1,
-                                   M + 1, 1, static_cast<const C *>(h->tw1), s, h->status));
-        CUDA_TRY(Ops<double>::rows_c2r(static_cast<const C *>(h->spec), static_cast<double *>(real_out),
-                                       h->p.n_theta, h->logm, static_cast<const C *>(h->twm), s, h->status));
-    } else {
-        using C = float2;
-        CUDA_TRY(Ops<float>::cols(static_cast<const C *>(spec_in), static_cast<C *>(h->spec), h->logn1, M + 1,
-                                  M + 1, 1, static_cast<const C *>(h->tw1), s, h->status));
-        CUDA_TRY(Ops<float>::rows_c2r(static_cast<const C *>(h->spec), static_cast<float *>(real_out),
-                                      h->p.n_theta, h->logm, static_cast<const C *>(h->twm), s, h->status));
-    }
-    return FLAME_OK;
+    return h->p.prec == FLAME_FP64 ? fft_c2r<double>(h, spec_in, real_out, s) : fft_c2r<float>(h, spec_in, real_out, s);
 }
 
 flame_status flame_step_heun(flame_t h, void *state, double *mean_mode, double *t, int nsteps, void *stream) {

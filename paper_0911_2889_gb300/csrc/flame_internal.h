@@ -179,17 +179,28 @@ struct Geom {
 // Sets the thread-local message returned by flame_last_error().
 void set_last_error(const char *msg);
 
+// Column transforms per column of a 2-D transform: 4 of N1/4 points, behind a
+// radix-4 stage in the row pass, or the whole column.  r2c + c2r, whole -> split:
+// 4096x8192 396 -> 296 us, 4096x2048 111 -> 71, 2048x4096 95 -> 69, 1024x2048 32
+// -> 23; 512x1024 16.8 -> 19.8 (its whole columns already give a CTA 16).  FP64
+// is bound by its arithmetic, and four FP64 rows of 8192 do not fit a CTA.
+inline int fft_split(bool fp64, int n1, int logm) {
+    return !fp64 && logm >= 9 && logm <= 12 && n1 >= 1024 ? 4 : 1;
+}
+
 // Per-precision launchers (defined in flame_f32.cu / flame_f64.cu).
 template <class R> struct Ops {
     using C = typename std::conditional<sizeof(R) == 4, float2, double2>::type;
     static cudaError_t init_twiddles(C *tab, int logN, cudaStream_t s);
+    // 2-D transforms: the row pass (tw: table of N2/2 points, tw1: of N1), and
+    // fft_split column transforms of 2^logn points a column.
     // (status: the handle's status words, for the index checks of the
     // FLAME_DEBUG_BOUNDS build; unused otherwise)
-    static cudaError_t rows_r2c(const R *in, C *out, int n1, int logm, const C *tw, cudaStream_t s,
+    static cudaError_t rows_r2c(const R *in, C *out, int n1, int logm, const C *tw, const C *tw1, cudaStream_t s,
                                 int *status = nullptr);
-    static cudaError_t rows_c2r(const C *in, R *out, int n1, int logm, const C *tw, cudaStream_t s,
+    static cudaError_t rows_c2r(const C *in, R *out, int n1, int logm, const C *tw, const C *tw1, cudaStream_t s,
                                 int *status = nullptr);
-    static cudaError_t cols(const C *in, C *out, int logn, int ncols, int ld, int dir, const C *tw,
+    static cudaError_t cols(const C *in, C *out, int logn, int split, int ncols, int ld, int dir, const C *tw,
                             cudaStream_t s, int *status = nullptr);
     // retained modes of an r2c spectrum -> compact box + FP64 mean
     static cudaError_t box_from_spec(const C *spec, C *state, double *mean, int n1, int n2, int K1, int K2,

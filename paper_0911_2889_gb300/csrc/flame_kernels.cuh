@@ -222,6 +222,42 @@ template <class R> __global__ void k_twiddles(CplxT<R> *tab, int logN) {
     }
 }
 
+// Bulk prefetch of a contiguous range into L2 (no register or shared-memory
+// cost): the next wave's input streams from HBM while this wave computes.
+// The bulk prefetch needs a 16-byte aligned start and a size that is a
+// multiple of 16: the range is shrunk to [align_up(begin), align_down(end)),
+// so it never reaches outside [begin, end).
+__device__ __forceinline__ void l2_prefetch(const void *begin, size_t bytes) {
+    const size_t b = (reinterpret_cast<size_t>(begin) + 15) & ~(size_t)15;
+    const size_t e = (reinterpret_cast<size_t>(begin) + bytes) & ~(size_t)15;
+    if (e > b)
+        asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(b), "r"((unsigned)(e - b)) : "memory");
+}
+
+// Programmatic dependent launch: wait until the previous kernel on the
+// stream has completed and its memory is visible (a no-op when the launch is
+// an ordinary one), and let the next kernel's CTAs be scheduled once every CTA
+// of this one has said so.  Said behind the transform: said at the top, the
+// next kernel's waiting CTAs took the SMs from this one's later waves (512x1024
+// 15.4 -> 19.7 us a step).
+__device__ __forceinline__ void griddep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void griddep_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
+// E points per thread: 16 (runtime-length kernels, FP64) or 8 (compile-time
+// FP32 kernels: 512-thread CTAs at 64 registers, two CTAs per SM).
+template <int DIR, int LOG, int E, class V, class C>
+__device__ __forceinline__ void fft_line_e(CV<V> (&x)[E], int logn, int t, const Planes<V> &sm, const C *tw) {
+    if constexpr (E == 8) line_fft_ct<DIR, LOG, 8>(x, t, sm, tw + tw_table_len(LOG, 4), CtaBarrier{});
+    else if constexpr (E == 4)
+        line_fft_ct<DIR, LOG, 4>(x, t, sm, tw + tw_table_len(LOG, 4) + tw_table_len(LOG, 3), CtaBarrier{});
+    else fft_line<DIR, LOG>(x, logn, t, sm, tw);
+}
+
+// Bytes between the exchange buffers of a column CTA's G groups (k_cols).
+template <class R, int E = 16> __host__ __device__ constexpr size_t cols_group_bytes(int n, int G) {
+    return 2 * (size_t)plane_len_e<E>(n) * sizeof(typename VecOf<R>::type) + (G >= 8 ? 16 : G > 1 ? 128 / G : 0);
+}
+
 // ----------------------------------------------------------------------------
 // Standalone 2-D real FFT passes
 // ----------------------------------------------------------------------------
@@ -230,37 +266,39 @@ template <class R> __global__ void k_twiddles(CplxT<R> *tab, int logN) {
 // post-processing  Y[k] = E[k] + exp(-2 pi i k/N2) O[k],
 // E = (H[k] + conj H[M-k])/2, O = (H[k] - conj H[M-k])/(2i).
 // LOG > 0: half length 2^LOG fixed at compile time; LOG = 0: any length.
-template <class R, int LOG>
+// E points per thread (4: with LOG > 0 only).
+template <class R, int LOG, int E = 16>
 __global__ void __launch_bounds__(256, kMinBlocks<R>) k_rows_r2c(const R *__restrict__ in, CplxT<R> *__restrict__ out, int n1,
                                                   int logm, const CplxT<R> *__restrict__ tw, int *status) {
     using V = typename VecOf<R>::type;
     using C = CplxT<R>;
     extern __shared__ __align__(16) unsigned char smraw[];
-    const int M = LOG > 0 ? 1 << LOG : 1 << logm, T = M >> 4, ldo = M + 1;
+    const int M = LOG > 0 ? 1 << LOG : 1 << logm, T = M / E, ldo = M + 1;
     const int g = threadIdx.x / T, t = threadIdx.x % T, G = blockDim.x / T;
     const int pair = blockIdx.x * G + g;
     const bool valid = pair < (n1 >> 1);
-    V *base = reinterpret_cast<V *>(smraw) + (size_t)g * 2 * plane_len(M);
-    auto sm = make_planes(base, M);
+    V *base = reinterpret_cast<V *>(smraw) + (size_t)g * 2 * plane_len_e<E>(M);
+    auto sm = make_planes_e<E>(base, M);
     const C *ra = reinterpret_cast<const C *>(in) + (size_t)(2 * pair) * M;
     const C *rb = ra + M;
-    CV<V> x[16];
+    CV<V> x[E];
 #pragma unroll
-    for (int r = 0; r < 16; ++r) {
+    for (int r = 0; r < E; ++r) {
         const bool in = valid && FLAME_IN(status, (long long)(2 * pair + 1) * M + t + r * T, (long long)n1 * M, kSiteFftIn);
         C a = in ? __ldg(ra + t + r * T) : C{0, 0};
         C b = in ? __ldg(rb + t + r * T) : C{0, 0};
         x[r] = pack2<R>(a, b);
     }
-    fft_line<-1, LOG>(x, logm, t, sm, tw);
+    fft_line_e<-1, LOG, E>(x, logm, t, sm, tw);
+    griddep_launch();
     __syncthreads();
 #pragma unroll
-    for (int r = 0; r < 16; ++r) sm.st(t + r * T, x[r]);
+    for (int r = 0; r < E; ++r) sm.st(t + r * T, x[r]);
     __syncthreads();
     const C *P = tw + tw_real_offset(LOG > 0 ? LOG : logm);
     C *oa = out + (size_t)(2 * pair) * ldo, *ob = oa + ldo;
 #pragma unroll
-    for (int r = 0; r < 16; ++r) {
+    for (int r = 0; r < E; ++r) {
         const int k = t + r * T;
         CV<V> h = x[r], hc = sm.ld((M - k) & (M - 1));
         const R hf = (R)0.5;
@@ -283,31 +321,33 @@ __global__ void __launch_bounds__(256, kMinBlocks<R>) k_rows_r2c(const R *__rest
 
 // Row pass of c2r: pre-processing H[k] = (Y[k] + conj Y[M-k]) +
 // i exp(+2 pi i k/N2) (Y[k] - conj Y[M-k]), half-length inverse FFT, then
-// x[2m] = Re h[m], x[2m+1] = Im h[m].
-template <class R, int LOG>
-__global__ void __launch_bounds__(256, kMinBlocks<R>) k_rows_c2r(const CplxT<R> *__restrict__ in, R *__restrict__ out, int n1,
+// x[2m] = Re h[m], x[2m+1] = Im h[m].  (in is the previous kernel's output: not
+// __restrict__ or __ldg, whose loads may move ahead of the wait for it.)
+template <class R, int LOG, int E = 16>
+__global__ void __launch_bounds__(256, kMinBlocks<R>) k_rows_c2r(const CplxT<R> *in, R *out, int n1,
                                                   int logm, const CplxT<R> *__restrict__ tw, int *status) {
     using V = typename VecOf<R>::type;
     using C = CplxT<R>;
     extern __shared__ __align__(16) unsigned char smraw[];
-    const int M = LOG > 0 ? 1 << LOG : 1 << logm, T = M >> 4, ldi = M + 1;
+    const int M = LOG > 0 ? 1 << LOG : 1 << logm, T = M / E, ldi = M + 1;
     const int g = threadIdx.x / T, t = threadIdx.x % T, G = blockDim.x / T;
     const int pair = blockIdx.x * G + g;
     const bool valid = pair < (n1 >> 1);
-    V *base = reinterpret_cast<V *>(smraw) + (size_t)g * 2 * plane_len(M);
-    auto sm = make_planes(base, M);
+    V *base = reinterpret_cast<V *>(smraw) + (size_t)g * 2 * plane_len_e<E>(M);
+    auto sm = make_planes_e<E>(base, M);
     const C *ia = in + (size_t)(2 * pair) * ldi, *ib = ia + ldi;
     const C *P = tw + tw_real_offset(LOG > 0 ? LOG : logm);
-    CV<V> x[16];
+    CV<V> x[E];
+    griddep_wait();
 #pragma unroll
-    for (int r = 0; r < 16; ++r) {
+    for (int r = 0; r < E; ++r) {
         const int k = t + r * T;
         const bool in = valid && FLAME_IN(status, (long long)(2 * pair + 1) * ldi + M - k, (long long)n1 * ldi, kSiteFftIn) &&
                         FLAME_IN(status, (long long)(2 * pair + 1) * ldi + k, (long long)n1 * ldi, kSiteFftIn);
-        C a = in ? __ldg(ia + k) : C{0, 0};
-        C b = in ? __ldg(ib + k) : C{0, 0};
-        C ac = in ? __ldg(ia + M - k) : C{0, 0};
-        C bc = in ? __ldg(ib + M - k) : C{0, 0};
+        C a = in ? ia[k] : C{0, 0};
+        C b = in ? ib[k] : C{0, 0};
+        C ac = in ? ia[M - k] : C{0, 0};
+        C bc = in ? ib[M - k] : C{0, 0};
         CV<V> y = pack2<R>(a, b), yc = pack2<R>(ac, bc);
         CV<V> S{vadd(y.re, yc.re), vsub(y.im, yc.im)};
         CV<V> D{vsub(y.re, yc.re), vadd(y.im, yc.im)};
@@ -315,11 +355,12 @@ __global__ void __launch_bounds__(256, kMinBlocks<R>) k_rows_c2r(const CplxT<R> 
         CV<V> wD = cmul_s(D, w.x, w.y);
         x[r] = cadd_rot<1>(S, wD);
     }
-    fft_line<1, LOG>(x, logm, t, sm, tw);
+    fft_line_e<1, LOG, E>(x, logm, t, sm, tw);
+
     if (valid) {
         C *oa = reinterpret_cast<C *>(out) + (size_t)(2 * pair) * M, *ob = oa + M;
 #pragma unroll
-        for (int r = 0; r < 16; ++r) {
+        for (int r = 0; r < E; ++r) {
             if (!FLAME_IN(status, (long long)(2 * pair + 1) * M + t + r * T, (long long)n1 * M, kSiteFftOut)) continue;
             oa[t + r * T] = lane0<R>(x[r]);
             ob[t + r * T] = lane1<R>(x[r]);
@@ -327,67 +368,205 @@ __global__ void __launch_bounds__(256, kMinBlocks<R>) k_rows_c2r(const CplxT<R> 
     }
 }
 
-// Column FFT of length n = 2^logn over ncols columns of a row-major array
-// with row stride ld (complex units); columns 2p, 2p+1 form one thread
-// group; in may equal out.  The G groups of a CTA take adjacent column
-// pairs and interleave their threads (group = thread mod G), so that one
-// warp's access to a row covers G adjacent column pairs: NT = 512 threads
-// (FP32, 2^10 .. 2^12 points) widens that from 16 to 32 bytes and more.
-template <class R, int DIR, int LOG, int NT = 256>
-__global__ void __launch_bounds__(NT, NT == 256 ? kMinBlocks<R> : 1)
-    k_cols(const CplxT<R> *in, CplxT<R> *out, int logn, int ncols, int ld, const CplxT<R> *__restrict__ tw, int *status) {
-    using V = typename VecOf<R>::type;
-    using C = CplxT<R>;
+// Row passes with the column transform's first (r2c) or last (c2r) radix-4
+// stage (where fft_split says so).  A CTA takes the four rows
+// n + m N1/4, m = 0..3, as two thread groups of two lines each.  r2c: the rows'
+// spectra X_m become Z_q = exp(-2 pi i q n / N1) sum_m (-i)^(q m) X_m, stored
+// as row 4 n + q; what is left of the columns are four transforms of N1/4
+// points over the rows = q mod 4, in place.  c2r is the mirror image.  A
+// thread takes the bins k and M - k of all four rows, so every bin is loaded
+// once and the two bins are the lanes of the radix-4 arithmetic.
+//
+// The stage is here because of the columns: whole 4096-point columns let a CTA
+// hold four of them (32 bytes of a row at a time), quarter columns 16 (128
+// bytes, or 8 with two CTAs per SM).  4096x8192, r2c: rows 64 -> 76 us, columns
+// 126 -> 71; c2r: columns 145 -> 72, rows 60 -> 77 (79 us of bytes a transform).
+// One CTA of 512 threads per SM at 8192 points a row leaves loads, arithmetic
+// and stores in turn; the next wave's rows are therefore brought into L2
+// meanwhile (r2c 158 -> 150, c2r 167 -> 155).
+struct GroupBarrier {
+    int id, n;
+    __device__ __forceinline__ void operator()() const { asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(n) : "memory"); }
+};
+// exp(2 pi i j / N1), 0 <= j < N1, of the real-transform table (half turns)
+template <class C> __device__ __forceinline__ C root_of(const C *half, int n1, int j) {
+    const int i = 2 * j;
+    const C w = __ldg(half + (i < n1 ? i : i - n1));
+    return i < n1 ? w : C{-w.x, -w.y};
+}
+
+template <int LOG>
+__global__ void __launch_bounds__((1 << LOG) / 8, 4096 >> LOG)
+    k_rows4_r2c(const float *__restrict__ in, float2 *__restrict__ out, int n1, const float2 *__restrict__ tw,
+                const float2 *__restrict__ half1, int ahead, int *status) {
+    using V = float2;
     extern __shared__ __align__(16) unsigned char smraw[];
-    const int n = LOG > 0 ? 1 << LOG : 1 << logn, T = n >> 4;
-    const int G = blockDim.x / T, g = threadIdx.x % G, t = threadIdx.x / G;
-    const int c0 = 2 * (blockIdx.x * G + g);
-    const bool va = c0 < ncols, vb = c0 + 1 < ncols;
-    V *base = reinterpret_cast<V *>(smraw) + (size_t)g * 2 * plane_len(n);
-    auto sm = make_planes(base, n);
+    constexpr int M = 1 << LOG, T = M >> 4, ldo = M + 1;
+    const int g = threadIdx.x / T, t = threadIdx.x % T, n = blockIdx.x, nq = n1 >> 2;
+    V *base = reinterpret_cast<V *>(smraw);
+    const Planes<V> s0(base), s1(base + 2 * plane_len(M)), sm = g ? s1 : s0;
+    const GroupBarrier bar{1 + g, T};
+    const int ra = n + g * nq, rb = ra + 2 * nq;
+    const float2 *pa = reinterpret_cast<const float2 *>(in) + (size_t)ra * M + t;
+    const float2 *pb = reinterpret_cast<const float2 *>(in) + (size_t)rb * M + t;
     CV<V> x[16];
 #pragma unroll
     for (int r = 0; r < 16; ++r) {
-        const size_t row = (size_t)(t + r * T) * ld;
-        const long long len = (long long)n * ld;
-        C a = va && FLAME_IN(status, row + c0, len, kSiteFftIn) ? in[row + c0] : C{0, 0};
-        C b = vb && FLAME_IN(status, row + c0 + 1, len, kSiteFftIn) ? in[row + c0 + 1] : C{0, 0};
-        x[r] = pack2<R>(a, b);
+        const bool ok = FLAME_IN(status, (long long)rb * M + t + r * T, (long long)n1 * M, kSiteFftIn);
+        x[r] = ok ? pack2<float>(__ldg(pa + r * T), __ldg(pb + r * T)) : CV<V>{};
     }
-    fft_line<DIR, LOG>(x, logn, t, sm, tw);
+    if (t < 2 && n + ahead < nq) l2_prefetch(in + (size_t)(n + ahead + (2 * t + g) * nq) * 2 * M, 2 * M * sizeof(float));
+    line_fft_ct<-1, LOG, 16>(x, t, sm, tw, bar);
+    griddep_launch();
+    bar();
+#pragma unroll
+    for (int r = 0; r < 16; ++r) sm.st(t + r * T, x[r]);
+    const float2 w1 = root_of(half1, n1, n), w2 = root_of(half1, n1, 2 * n), w3 = root_of(half1, n1, 3 * n);
+    const float2 *P = tw + tw_real_offset(LOG);
+    float2 *o = out + (size_t)(4 * n) * ldo;
+    __syncthreads();
+    auto bins = [&](int k) {
+        const float2 w = __ldg(P + k);  // exp(+2 pi i k/N2); forward uses the conjugate
+        CV<V> lo[2], hi[2];             // sums and differences of a group's two rows, lanes = bins k, M - k
+        static_for<0, 2>([&](auto gc) {
+            constexpr int gg = decltype(gc)::value;
+            const Planes<V> &p = gg ? s1 : s0;
+            const CV<V> h = p.ld(k), hc = p.ld((M - k) & (M - 1));
+            const CV<V> E{vmul(vadd(h.re, hc.re), vbc(0.5f)), vmul(vsub(h.im, hc.im), vbc(0.5f))};
+            const CV<V> O{vmul(vadd(h.im, hc.im), vbc(0.5f)), vmul(vsub(hc.re, h.re), vbc(0.5f))};
+            const CV<V> wO = cmul_s(O, w.x, -w.y);
+            // Y[k] = E + w O, Y[M-k] = conj(E - w O)
+            const CV<V> Y = cadd(E, wO), Z{vsub(E.re, wO.re), vsub(wO.im, E.im)};
+            const CV<V> a{make_float2(Y.re.x, Z.re.x), make_float2(Y.im.x, Z.im.x)};
+            const CV<V> b{make_float2(Y.re.y, Z.re.y), make_float2(Y.im.y, Z.im.y)};
+            lo[gg] = cadd(a, b);
+            hi[gg] = csub(a, b);
+        });
+        CV<V> z[4];
+        z[0] = cadd(lo[0], lo[1]);
+        z[1] = cmul_s(cadd_rot<-1>(hi[0], hi[1]), w1.x, -w1.y);
+        z[2] = cmul_s(csub(lo[0], lo[1]), w2.x, -w2.y);
+        z[3] = cmul_s(csub_rot<-1>(hi[0], hi[1]), w3.x, -w3.y);
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            if (!FLAME_IN(status, (long long)(4 * n + q) * ldo + M - k, (long long)n1 * ldo, kSiteFftOut)) continue;
+            o[q * ldo + k] = lane0<float>(z[q]);
+            o[q * ldo + M - k] = lane1<float>(z[q]);
+        }
+    };
+#pragma unroll
+    for (int j = 0; j < 4; ++j) bins(threadIdx.x + j * 2 * T);
+    if (threadIdx.x == 0) bins(M / 2);
+}
+
+template <int LOG>
+__global__ void __launch_bounds__((1 << LOG) / 8, 4096 >> LOG)
+    k_rows4_c2r(const float2 *in, float *out, int n1, const float2 *__restrict__ tw,
+                const float2 *__restrict__ half1, int ahead, int *status) {
+    using V = float2;
+    extern __shared__ __align__(16) unsigned char smraw[];
+    constexpr int M = 1 << LOG, T = M >> 4, ldi = M + 1;
+    const int g = threadIdx.x / T, t = threadIdx.x % T, n = blockIdx.x, nq = n1 >> 2;
+    V *base = reinterpret_cast<V *>(smraw);
+    const Planes<V> s0(base), s1(base + 2 * plane_len(M)), sm = g ? s1 : s0;
+    const float2 w1 = root_of(half1, n1, n), w2 = root_of(half1, n1, 2 * n), w3 = root_of(half1, n1, 3 * n);
+    const float2 *P = tw + tw_real_offset(LOG);
+    const float2 *i = in + (size_t)(4 * n) * ldi;
+    griddep_wait();
+    auto bins = [&](int k) {
+        const float2 w = __ldg(P + k);
+        CV<V> z[4];  // lanes = bins k, M - k
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const bool ok = FLAME_IN(status, (long long)(4 * n + q) * ldi + M - k, (long long)n1 * ldi, kSiteFftIn);
+            z[q] = ok ? pack2<float>(i[q * ldi + k], i[q * ldi + M - k]) : CV<V>{};
+        }
+        z[1] = cmul_s(z[1], w1.x, w1.y);
+        z[2] = cmul_s(z[2], w2.x, w2.y);
+        z[3] = cmul_s(z[3], w3.x, w3.y);
+        const CV<V> e0 = cadd(z[0], z[2]), e1 = csub(z[0], z[2]), f0 = cadd(z[1], z[3]), f1 = csub(z[1], z[3]);
+        auto half = [&](const Planes<V> &p, CV<V> a, CV<V> b) {  // the group's rows: spectra to half-length input
+            const CV<V> y{make_float2(a.re.x, b.re.x), make_float2(a.im.x, b.im.x)};
+            const CV<V> yc{make_float2(a.re.y, b.re.y), make_float2(a.im.y, b.im.y)};
+            const CV<V> S{vadd(y.re, yc.re), vsub(y.im, yc.im)}, D{vsub(y.re, yc.re), vadd(y.im, yc.im)};
+            const CV<V> wD = cmul_s(D, w.x, w.y);
+            // H[k] = S + i w D, H[M-k] = conj(S - i w D)
+            p.st(k, cadd_rot<1>(S, wD));
+            const CV<V> m = csub_rot<1>(S, wD);
+            if (k > 0) p.st(M - k, CV<V>{m.re, vneg(m.im)});
+        };
+        half(s0, cadd(e0, f0), csub(e0, f0));
+        half(s1, cadd_rot<1>(e1, f1), csub_rot<1>(e1, f1));
+    };
+#pragma unroll
+    for (int j = 0; j < 4; ++j) bins(threadIdx.x + j * 2 * T);
+    if (threadIdx.x == 0) bins(M / 2);
+    if (threadIdx.x == 32 && n + ahead < nq) l2_prefetch(in + (size_t)(4 * (n + ahead)) * ldi, 4 * ldi * sizeof(float2));
+    __syncthreads();
+    CV<V> x[16];
+#pragma unroll
+    for (int r = 0; r < 16; ++r) x[r] = sm.ld(t + r * T);
+    line_fft_ct<1, LOG, 16>(x, t, sm, tw, GroupBarrier{1 + g, T});
+    const int ra = n + g * nq, rb = ra + 2 * nq;
+    float2 *oa = reinterpret_cast<float2 *>(out) + (size_t)ra * M + t, *ob = reinterpret_cast<float2 *>(out) + (size_t)rb * M + t;
 #pragma unroll
     for (int r = 0; r < 16; ++r) {
-        const size_t row = (size_t)(t + r * T) * ld;
-        const long long len = (long long)n * ld;
-        if (va && FLAME_IN(status, row + c0, len, kSiteFftOut)) out[row + c0] = lane0<R>(x[r]);
-        if (vb && FLAME_IN(status, row + c0 + 1, len, kSiteFftOut)) out[row + c0 + 1] = lane1<R>(x[r]);
+        if (!FLAME_IN(status, (long long)rb * M + t + r * T, (long long)n1 * M, kSiteFftOut)) continue;
+        oa[r * T] = lane0<float>(x[r]);
+        ob[r * T] = lane1<float>(x[r]);
+    }
+}
+
+// Column FFT of length n = 2^logn over ncols columns of a row-major array
+// with row stride ld (complex units); point i of blockIdx.y's transform is row
+// i * gridDim.y + blockIdx.y (gridDim.y = 1: whole columns; 4: behind the row
+// passes' radix-4 stage); in may equal out.  Columns c0 and c0 + G form one
+// thread group.  The G groups of a CTA interleave their threads (group =
+// thread mod G), so that one warp's access to a row covers G adjacent columns
+// at a time.  The groups' exchange buffers are 8/G slots of 16 bytes (one,
+// for G > 8) further apart than their length, which puts the G groups and the
+// 8/G points that a quarter warp exchanges on different banks.
+template <class R, int DIR, int LOG, int NT = 256, int E = 16>
+__global__ void __launch_bounds__(NT, NT == 256 ? kMinBlocks<R> : 1)
+    k_cols(const CplxT<R> *in, CplxT<R> *out, int logn, int ncols, int ld, const CplxT<R> *__restrict__ tw, int ahead, int *status) {
+    using V = typename VecOf<R>::type;
+    using C = CplxT<R>;
+    extern __shared__ __align__(16) unsigned char smraw[];
+    const int n = LOG > 0 ? 1 << LOG : 1 << logn, T = n / E;
+    const int G = blockDim.x / T, g = threadIdx.x % G, t = threadIdx.x / G;
+    const int ca = 2 * blockIdx.x * G + g, cb = ca + G;
+    const bool va = ca < ncols, vb = cb < ncols;
+    V *base = reinterpret_cast<V *>(smraw + (size_t)g * cols_group_bytes<R, E>(n, G));
+    auto sm = make_planes_e<E>(base, n);
+    CV<V> x[E];
+    griddep_wait();
+    const long long len = (long long)n * gridDim.y * ld;
+#pragma unroll
+    for (int r = 0; r < E; ++r) {
+        const size_t row = (size_t)((t + r * T) * gridDim.y + blockIdx.y) * ld;
+        C a = va && FLAME_IN(status, row + ca, len, kSiteFftIn) ? in[row + ca] : C{0, 0};
+        C b = vb && FLAME_IN(status, row + cb, len, kSiteFftIn) ? in[row + cb] : C{0, 0};
+        x[r] = pack2<R>(a, b);
+    }
+    if constexpr (sizeof(R) == 4 && NT == 256 && E == 16 && LOG >= 8 && LOG <= 10) if (ahead > 0) {
+        const int tile = blockIdx.y * gridDim.x + blockIdx.x + ahead, q = tile / gridDim.x, c = (tile - q * gridDim.x) * 2 * G;
+        if (q < gridDim.y)
+            for (int i = threadIdx.x; i < n; i += blockDim.x)
+                asm volatile("prefetch.global.L2 [%0];" ::"l"(in + (size_t)(i * gridDim.y + q) * ld + c));
+    }
+    fft_line_e<DIR, LOG, E>(x, logn, t, sm, tw);
+    griddep_launch();
+#pragma unroll
+    for (int r = 0; r < E; ++r) {
+        const size_t row = (size_t)((t + r * T) * gridDim.y + blockIdx.y) * ld;
+        if (va && FLAME_IN(status, row + ca, len, kSiteFftOut)) out[row + ca] = lane0<R>(x[r]);
+        if (vb && FLAME_IN(status, row + cb, len, kSiteFftOut)) out[row + cb] = lane1<R>(x[r]);
     }
 }
 
 // ----------------------------------------------------------------------------
 // Step passes
 // ----------------------------------------------------------------------------
-// Bulk prefetch of a contiguous range into L2 (no register or shared-memory
-// cost): the next wave's input streams from HBM while this wave computes.
-// The bulk prefetch needs a 16-byte aligned start and a size that is a
-// multiple of 16: the range is shrunk to [align_up(begin), align_down(end)),
-// so it never reaches outside [begin, end).
-__device__ __forceinline__ void l2_prefetch(const void *begin, size_t bytes) {
-    const size_t b = (reinterpret_cast<size_t>(begin) + 15) & ~(size_t)15;
-    const size_t e = (reinterpret_cast<size_t>(begin) + bytes) & ~(size_t)15;
-    if (e > b)
-        asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(b), "r"((unsigned)(e - b)) : "memory");
-}
-
-// Programmatic dependent launch: wait until the previous kernel on the
-// stream has completed and its memory is visible (a no-op when the launch is
-// an ordinary one), and let the next kernel's CTAs be scheduled once every CTA
-// of this one has said so.  Said behind the transform: said at the top, the
-// next kernel's waiting CTAs took the SMs from this one's later waves (512x1024
-// 15.4 -> 19.7 us a step).
-__device__ __forceinline__ void griddep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-__device__ __forceinline__ void griddep_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
-
 // Tensor stores (TMA) from shared memory.  The writing threads fence their
 // shared-memory stores towards the async proxy, the CTA synchronises, then one
 // thread issues the copies, commits them as a bulk group and waits until they
@@ -403,16 +582,6 @@ __device__ __forceinline__ void tma_store_3d(const CUtensorMap *tm, const void *
 __device__ __forceinline__ void bulk_commit_and_wait_read() {
     asm volatile("cp.async.bulk.commit_group;" ::: "memory");
     asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
-}
-
-// E points per thread: 16 (runtime-length kernels, FP64) or 8 (compile-time
-// FP32 kernels: 512-thread CTAs at 64 registers, two CTAs per SM).
-template <int DIR, int LOG, int E, class V, class C>
-__device__ __forceinline__ void fft_line_e(CV<V> (&x)[E], int logn, int t, const Planes<V> &sm, const C *tw) {
-    if constexpr (E == 8) line_fft_ct<DIR, LOG, 8>(x, t, sm, tw + tw_table_len(LOG, 4), CtaBarrier{});
-    else if constexpr (E == 4)
-        line_fft_ct<DIR, LOG, 4>(x, t, sm, tw + tw_table_len(LOG, 4) + tw_table_len(LOG, 3), CtaBarrier{});
-    else fft_line<DIR, LOG>(x, logn, t, sm, tw);
 }
 
 // Shared-memory twiddles of the compile-time FP32 pass-B kernels (E = 16,

@@ -65,56 +65,125 @@ cudaError_t Ops<R>::box_from_spec(const C *spec, C *state, double *mean, int n1,
     return launch_k(k_box_from_spec<R>, dim3(blocks), 256, 0, s, spec, state, mean, n1, n2, K1, K2, status);
 }
 
-// The standalone 2-D FFT passes take the compile-time line length where the
-// step kernels do (FP32, 2^8 .. 2^12), the runtime-length engine otherwise.
+// Lines of 2^5 .. 2^10 points where 16 points a thread would leave an SM fewer
+// than 256 threads: 4 points a thread.  Those transforms are bound by the
+// latency of one thread's chain and by launches, not by bytes.  Per transform
+// (graph), 16 -> 4 points: FP32 256x256 7.2 -> 4.7 us (with the second pass a
+// programmatic dependent launch, below), 512x512 7.2 -> 5.7, 512x2048 11.0 -> 10.0,
+// FP64 128x256 58 -> 18.5, 512x512 70 -> 23.6, 512x2048 92.5 -> 88.  Grids
+// with more lines than that stay with 16 points: fewer exchanges.
+// Programmatic dependent launch of the second pass: FP32 0.4 to 1 us a
+// transform; FP64 off (512x1024 43.6 -> 45.4 c2r, 44.6 -> 52.3 r2c with it).
+template <class R, class F> static bool with_short_lines(int logn, int npairs, bool split, F &&f) {
+    bool done = false;
+    if (((long)npairs << logn) / 16 < 256L * sm_count() && !(sizeof(R) == 4 && split))
+        static_for<5, 11>([&](auto lc) {
+            if (logn == decltype(lc)::value) {
+                f(lc);
+                done = true;
+            }
+        });
+    return done;
+}
+
+// row pairs per CTA of short lines: up to 64 threads, and a CTA for every SM
+static int short_groups(int npairs, int T) {
+    int G = 1;
+    while (2 * G * T <= 64 && npairs / (2 * G) >= sm_count()) G *= 2;
+    return G;
+}
+
 template <class R>
-cudaError_t Ops<R>::rows_r2c(const R *in, C *out, int n1, int logm, const C *tw, cudaStream_t s, int *status) {
+cudaError_t Ops<R>::rows_r2c(const R *in, C *out, int n1, int logm, const C *tw, const C *tw1, cudaStream_t s, int *status) {
     Geom g = geom_rows(logm, n1 / 2, 0);
     cudaError_t err = cudaSuccess;
+    if (with_short_lines<R>(logm, n1 / 2, fft_split(sizeof(R) == 8, n1, logm) > 1, [&](auto lc) {
+            constexpr int L = decltype(lc)::value;
+            const int G = short_groups(n1 / 2, (1 << L) / 4);
+            err = launch_k(k_rows_r2c<R, L, 4>, dim3(n1 / 2 / G), G * (1 << L) / 4, G * cols_group_bytes<R, 4>(1 << L, 1), s, in,
+                           out, n1, logm, tw, status);
+        }))
+        return err;
     with_log<R>(logm, [&](auto lc) {
-        err = launch_k(k_rows_r2c<R, decltype(lc)::value>, dim3(g.blocks), g.threads, g.smem, s, in, out, n1, logm,
-                        tw, status);
+        constexpr int L = decltype(lc)::value;
+        if constexpr (sizeof(R) == 4 && L >= 9)
+            if (fft_split(false, n1, logm) == 4) {
+                err = launch_k(k_rows4_r2c<L>, dim3(n1 / 4), (1 << L) / 8, 2 * group_smem<R>(L), s, in, out, n1, tw,
+                               tw1 + tw_real_offset(__builtin_ctz(n1)), sm_count() * (4096 >> L), status);
+                return;
+            }
+        err = launch_k(k_rows_r2c<R, L>, dim3(g.blocks), g.threads, g.smem, s, in, out, n1, logm, tw, status);
     });
     return err;
 }
 
 template <class R>
-cudaError_t Ops<R>::rows_c2r(const C *in, R *out, int n1, int logm, const C *tw, cudaStream_t s, int *status) {
+cudaError_t Ops<R>::rows_c2r(const C *in, R *out, int n1, int logm, const C *tw, const C *tw1, cudaStream_t s, int *status) {
     Geom g = geom_rows(logm, n1 / 2, 0);
     cudaError_t err = cudaSuccess;
+    if (with_short_lines<R>(logm, n1 / 2, fft_split(sizeof(R) == 8, n1, logm) > 1, [&](auto lc) {
+            constexpr int L = decltype(lc)::value;
+            const int G = short_groups(n1 / 2, (1 << L) / 4);
+            err = launch_s(L2Window{nullptr, 0, 0.f}, sizeof(R) == 4, k_rows_c2r<R, L, 4>, dim3(n1 / 2 / G), G * (1 << L) / 4,
+                           G * cols_group_bytes<R, 4>(1 << L, 1), s, in, out, n1, logm, tw, status);
+        }))
+        return err;
     with_log<R>(logm, [&](auto lc) {
-        err = launch_k(k_rows_c2r<R, decltype(lc)::value>, dim3(g.blocks), g.threads, g.smem, s, in, out, n1, logm,
-                        tw, status);
+        constexpr int L = decltype(lc)::value;
+        if constexpr (sizeof(R) == 4 && L >= 9)
+            if (fft_split(false, n1, logm) == 4) {
+                err = launch_s(L2Window{nullptr, 0, 0.f}, true, k_rows4_c2r<L>, dim3(n1 / 4), (1 << L) / 8,
+                               2 * group_smem<R>(L), s, in, out, n1, tw, tw1 + tw_real_offset(__builtin_ctz(n1)),
+                               sm_count() * (4096 >> L), status);
+                return;
+            }
+        err = launch_s(L2Window{nullptr, 0, 0.f}, sizeof(R) == 4, k_rows_c2r<R, L>, dim3(g.blocks), g.threads, g.smem, s, in, out, n1,
+                       logm, tw, status);
     });
     return err;
 }
 
 template <class R>
-cudaError_t Ops<R>::cols(const C *in, C *out, int logn, int ncols, int ld, int dir, const C *tw, cudaStream_t s,
+cudaError_t Ops<R>::cols(const C *in, C *out, int logn, int split, int ncols, int ld, int dir, const C *tw, cudaStream_t s,
                          int *status) {
-    Geom g = geom_cols(logn, (ncols + 1) / 2, 0);
+    const int npairs = (ncols + 1) / 2;
+    // the next wave's tile into L2 where the array is too large to stay there
+    // (4096x8192 -2 and -6 us; 4096x2048, which stays, +0.5)
+    const int ahead = split > 1 && ((size_t)split << logn) * ld * sizeof(C) > ((size_t)64 << 20) ? 2 * sm_count() : 0;
     cudaError_t err = cudaSuccess;
+    // r2c: behind the row pass
+    const bool pdl = dir < 0 && sizeof(R) == 4;
+    auto go = [&](auto kernel, int threads, int G, size_t smem) {
+        err = launch_s(L2Window{nullptr, 0, 0.f}, pdl, kernel, dim3((npairs + G - 1) / G, split), threads, smem, s, in,
+                       out, logn, ncols, ld, tw, ahead, status);
+    };
+    if (with_short_lines<R>(logn, npairs, split > 1, [&](auto lc) {
+            constexpr int L = decltype(lc)::value, T = (1 << L) / 4;
+            // adjacent columns in one CTA, up to 32 bytes of a row a warp
+            int G = sizeof(R) == 4 ? 4 : 2;
+            while (G > 1 && (npairs < G * sm_count() || G * T > 256)) G >>= 1;
+            const size_t smem = G * cols_group_bytes<R, 4>(1 << L, G);
+            if (dir < 0) go(k_cols<R, -1, L, 256, 4>, G * T, G, smem);
+            else go(k_cols<R, 1, L, 256, 4>, G * T, G, smem);
+        }))
+        return err;
+    const int n = 1 << logn, T = n >> 4;
+    const Geom g = geom_cols(logn, npairs * split, 0);
     with_log<R>(logn, [&](auto lc) {
         constexpr int L = decltype(lc)::value;
-        // FP32 columns of 2^10 .. 2^12 points: 512-thread CTAs of 512/T line
-        // groups (one CTA per SM), where the grid still has two CTAs per SM
+        // FP32 whole columns of 2^10 .. 2^12 points: 512-thread CTAs of 512/T
+        // line groups (one CTA per SM), where the grid still has two CTAs per SM
         if constexpr (sizeof(R) == 4 && L >= 10 && L <= 12) {
             constexpr int G = 512 / ((1 << L) >> 4);
-            const int npairs = (ncols + 1) / 2;
-            if (npairs >= 2 * G * sm_count()) {
-                const dim3 grid((npairs + G - 1) / G);
-                const size_t smem = G * group_smem<R>(L);
-                if (dir < 0) err = launch_k(k_cols<R, -1, L, 512>, grid, 512, smem, s, in, out, logn, ncols, ld, tw, status);
-                else err = launch_k(k_cols<R, 1, L, 512>, grid, 512, smem, s, in, out, logn, ncols, ld, tw, status);
+            if (split == 1 && npairs >= 2 * G * sm_count()) {
+                if (dir < 0) go(k_cols<R, -1, L, 512>, 512, G, G * cols_group_bytes<R>(n, G));
+                else go(k_cols<R, 1, L, 512>, 512, G, G * cols_group_bytes<R>(n, G));
                 return;
             }
         }
-        if (dir < 0)
-            err = launch_k(k_cols<R, -1, L>, dim3(g.blocks), g.threads, g.smem, s, in, out, logn, ncols, ld, tw,
-                            status);
-        else
-            err = launch_k(k_cols<R, 1, L>, dim3(g.blocks), g.threads, g.smem, s, in, out, logn, ncols, ld, tw,
-                            status);
+        const int G = g.threads / T;
+        if (dir < 0) go(k_cols<R, -1, L>, g.threads, G, G * cols_group_bytes<R>(n, G));
+        else go(k_cols<R, 1, L>, g.threads, G, G * cols_group_bytes<R>(n, G));
     });
     return err;
 }
