@@ -92,6 +92,8 @@ def load(build_if_missing: bool = True):
     """Loads libflame.so, or libflame_debug.so with FLAME_DEBUG_BOUNDS=1
     (building it in-tree first if it is missing)."""
     global _lib
+    if _lib is not None:  # set once, complete
+        return _lib
     with _lock:
         if _lib is None:
             path = library_path()
@@ -115,9 +117,9 @@ def _check(status: int):
 
 
 def _stream(stream=None):
-    if stream is None:
-        stream = torch.cuda.current_stream()
-    return ctypes.c_void_p(stream.cuda_stream)
+    if stream is None:  # the current stream's handle, without building a Stream object around it
+        return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
+    return stream.cuda_stream
 
 
 def _ptr(t: torch.Tensor, dtype=None, name="tensor"):
@@ -127,11 +129,11 @@ def _ptr(t: torch.Tensor, dtype=None, name="tensor"):
         raise ValueError(f"{name} must be contiguous")
     if dtype is not None and t.dtype != dtype:
         raise ValueError(f"{name} must have dtype {dtype}, got {t.dtype}")
-    return ctypes.c_void_p(t.data_ptr())
+    return t.data_ptr()
 
 
 def _optr(t, dtype=None, name="tensor"):
-    return ctypes.c_void_p(None) if t is None else _ptr(t, dtype, name)
+    return None if t is None else _ptr(t, dtype, name)
 
 
 # ----------------------------------------------------------------- raw C names
@@ -251,9 +253,9 @@ def flame_step_batch(hs, states, mean_modes, ts, nsteps=1, stream=None):
     if not (len(states) == len(mean_modes) == len(ts) == n):
         raise ValueError("flame_step_batch: list lengths differ")
     H = (ctypes.c_void_p * n)(*hs)
-    S = (ctypes.c_void_p * n)(*[_ptr(s, name="state").value for s in states])
-    M = (ctypes.c_void_p * n)(*[_ptr(m, torch.float64, "mean").value for m in mean_modes])
-    T = (ctypes.c_void_p * n)(*[_ptr(t, torch.float64, "t").value for t in ts])
+    S = (ctypes.c_void_p * n)(*[_ptr(s, name="state") for s in states])
+    M = (ctypes.c_void_p * n)(*[_ptr(m, torch.float64, "mean") for m in mean_modes])
+    T = (ctypes.c_void_p * n)(*[_ptr(t, torch.float64, "t") for t in ts])
     _check(load().flame_step_batch(ctypes.cast(H, ctypes.c_void_p), ctypes.cast(S, ctypes.c_void_p),
                                    ctypes.cast(M, ctypes.c_void_p), ctypes.cast(T, ctypes.c_void_p),
                                    n, int(nsteps), _stream(stream)))
