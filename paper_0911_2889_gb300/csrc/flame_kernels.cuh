@@ -237,7 +237,8 @@ __device__ __forceinline__ void l2_prefetch(const void *begin, size_t bytes) {
 // Programmatic dependent launch: wait until the previous kernel on the
 // stream has completed and its memory is visible (a no-op when the launch is
 // an ordinary one), and let the next kernel's CTAs be scheduled once every CTA
-// of this one has said so.  Said behind the transform: said at the top, the
+// of this one has said so.  What the previous kernel wrote is read by plain loads
+// (__ldg or __restrict__ loads may move ahead of the wait).  Said behind the transform: said at the top, the
 // next kernel's waiting CTAs took the SMs from this one's later waves (512x1024
 // 15.4 -> 19.7 us a step).
 __device__ __forceinline__ void griddep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
@@ -1223,7 +1224,7 @@ template <class R, bool GEN, bool STEP = false> __device__ __forceinline__ void 
     double v = 0.0;
     for (int n = threadIdx.x; n < a.n1; n += blockDim.x) {
         const size_t i = STEP ? 4 * (size_t)(n >> 1) + (n & 1) : gk_index(n, 0, a.n1);  // row n of column 0
-        if (FLAME_IN(d.status, i, gk_len(a), kSiteCGk)) v += (double)__ldg(&gk[i].x);
+        if (FLAME_IN(d.status, i, gk_len(a), kSiteCGk)) v += (double)gk[i].x;
     }
     const double rs = cta_sum(v, red);
     double area = __longlong_as_double(0x7ff8000000000000LL);
