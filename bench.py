@@ -649,7 +649,7 @@ def kernel_sources_sha256():
 
 
 def run_profile(args):
-    """Deterministic launch sequence for ncu: two twiddle-table launches at
+    """Deterministic launch sequence for ncu: the twiddle tables' launches at
     creation, then `--profile N` plain steps (passes A, B, C each), nothing else."""
     import torch
 

@@ -11,7 +11,9 @@
  * The quadratic term of eq. (SivCurv1c), -theta_pi^2/(2 r0^2) sum_l
  * l.(k-l) Phi_l Phi_{k-l}, is exactly c(t) times the coefficient of
  * |grad Phi|^2; it is evaluated through zero-padded FFTs (the augmented
- * array of Sec. 3, alias-free because N_i >= 4 K_i + 1).
+ * array of Sec. 3, alias-free because N_i >= 4 K_i + 1).  The step itself needs
+ * 3 K_i + 1 points a side for that and runs on the smallest 3 2^a >= 3 K_i + 1;
+ * the N1 x N2 grid is that of the transforms and of the surface area.
  *
  * Grid and coefficients: x_i = 2 pi j_i / N_i on an N1 x N2 (theta, phi) grid,
  * Phi(x) = sum_k Phi_k exp(i k.x).
@@ -103,8 +105,10 @@ typedef struct flame_ctx *flame_t;
  * hint only (results are identical either way).  Environment: FLAME_AUTOTUNE=0
  * keeps the default kernel variants, FLAME_FORCE_VARIANTS=a,b fixes them,
  * FLAME_FUSE=0 keeps the column passes of consecutive steps separate,
- * FLAME_BATCH_TMA=1 lets flame_step_batch use the tensor-store variants,
- * FLAME_TUNE_CACHE=path keeps the autotuner's choices in a JSON file. */
+ * FLAME_PDL=0 (1) launches no (every) step pass as a programmatic dependent
+ * launch, FLAME_FP64_POINTS=8 gives the FP64 public-grid short lines 8 points
+ * a thread instead of 4, FLAME_BATCH_TMA has no effect any more (ensembles take
+ * direct stores), FLAME_TUNE_CACHE=path keeps the autotuner's choices in a JSON file. */
 flame_status flame_create(const flame_params *params, flame_t *out);
 
 /* Destroys a handle (NULL is accepted).  Synchronises the device. */
@@ -113,24 +117,22 @@ flame_status flame_destroy(flame_t h);
 /* Copies the resolved parameters (K1, K2, s1, s2 filled in) into *out. */
 flame_status flame_get_params(flame_t h, flame_params *out);
 
-/* Kernel variants the autotuner chose for this handle (FP32 grids with
- * N1, N2/2 in 256..4096 are timed once per grid, precision and device at
- * creation, FLAME_AUTOTUNE=0 disables it): pass A 0 = cluster write-out
- * through distributed shared memory, 1 = direct stores, 2 = 8 points per
- * thread with the cluster write-out, 3 = write-out by tensor (TMA) stores,
- * 4 = one line per thread group (N1 <= 2048; pass C then takes the same
- * form); pass B 0 = 16 points per thread, 1 = 8 points per thread, 2 = 16
- * points per thread with the write-out by tensor stores, 3 = one line per
- * thread group (N2/2 <= 2048), 4 = as 2 with, for N2 = 8192, one exchange
- * of each row transform inside a warp (other N2: as 2).  flame_step_batch takes the fastest variants
- * other than the one-line ones (an ensemble fills the GPU without them),
- * unless FLAME_FORCE_VARIANTS fixes the variants.  EINVAL on null pointers. */
+/* Kernel variants the autotuner chose for this handle (FP32 grids whose step
+ * lines have 192 points and more are timed once per grid, K, precision and
+ * device at creation, as graphs of whole steps; FLAME_AUTOTUNE=0 disables it):
+ * pass A 1 = direct stores, 3 = write-out by tensor (TMA) stores, 4 = one line
+ * per thread group (pass C then takes the same form); pass B 0 = direct stores,
+ * 2 and 4 = write-out by tensor stores, 3 = one line per thread group.  Other
+ * numbers in 0..4, which earlier tune-cache files may hold, run the direct
+ * form.  flame_step_batch takes the two-line direct forms (an ensemble fills the
+ * GPU without the others) unless FLAME_FORCE_VARIANTS fixes the variants.
+ * EINVAL on null pointers. */
 flame_status flame_tuning(flame_t h, int *pass_a_variant, int *pass_b_variant);
 
 /* *enabled = 1 when flame_step with nsteps > 1 runs the column pass of each
  * step fused with the first column pass of the next (the same arithmetic as
  * separate steps, one HBM read of the state fewer per step).  Decided by the
- * autotuner at creation for FP32 grids with 256 <= N1 <= 4096;
+ * autotuner at creation for FP32 grids whose step columns have 192 points and more;
  * FLAME_FUSE=0 disables it.  EINVAL on null pointers. */
 flame_status flame_fused_steps(flame_t h, int *enabled);
 

@@ -244,8 +244,9 @@ __device__ __forceinline__ void l2_prefetch(const void *begin, size_t bytes) {
 __device__ __forceinline__ void griddep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void griddep_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
-// E points per thread: 16 (runtime-length kernels, FP64) or 8 (compile-time
-// FP32 kernels: 512-thread CTAs at 64 registers, two CTAs per SM).
+// E points per thread: 16, 8 (the row pass with the area: more warps where its
+// buffers leave one CTA per SM) or 4 (short lines), compile-time lengths for the
+// last two.
 template <int DIR, int LOG, int E, class V, class C>
 __device__ __forceinline__ void fft_line_e(CV<V> (&x)[E], int logn, int t, const Planes<V> &sm, const C *tw) {
     if constexpr (E == 8) line_fft_ct<DIR, LOG, 8>(x, t, sm, tw + tw_table_len(LOG, 4), CtaBarrier{});

@@ -30,13 +30,8 @@ template <class R> static Geom make_geom(int logn, int nlines, int hint, size_t 
     return g;
 }
 
-// Line lengths with compile-time step kernels: FP32 2^8 .. 2^12 (the
-// benchmark, ensemble and adjoint grids); everything else (and FP64) runs the
-// runtime-length kernels (LOG = 0).
-template <class R, class F> static void for_each_log(F &&f) {
-    f(std::integral_constant<int, 0>{});
-    if constexpr (sizeof(R) == 4) static_for<8, 13>(f);
-}
+// Line lengths with compile-time kernels: FP32 2^8 .. 2^12; everything else (and
+// FP64) runs the runtime-length kernels (LOG = 0).
 template <class R, class F> static void with_log(int logn, F &&f) {
     bool done = false;
     if constexpr (sizeof(R) == 4) {

@@ -301,8 +301,11 @@ __device__ __forceinline__ void bulk_wait(unsigned long long *bar, int *status) 
 // the row pair's W come out of shared memory; the even buffer then takes g at
 // the even points, the odd one the forward transform of g, and the even one G
 // on its way out (32 bytes of gk per column and row pair: 2/3 of a buffer).
-// Bound by shared memory: of its ~8500 wavefronts a 3072-point row pair the six
-// exchanges are 4600; two CTAs of 256 threads per SM.
+// Bound by the latency between its barriers at two CTAs of 256 threads per SM
+// (the shared-memory pipe is 42 % busy, the six exchanges most of it; issue 37 %;
+// stalls per issue: barrier 2.5, loads 1.3, shared memory 1.0).  4096x8192 (1536 pairs of 3072-point
+// rows): 123 -> 75 us, 1.99 TB/s of its 151 MB (three 4096-point transforms a
+// row pair before; on this grid, 155 -> 136 us a step by this form).
 template <class R, int A, bool TMA>
 __device__ __forceinline__ void stepB2_body(const FlameDesc &d, int tile, const Ahead &ahead, const CUtensorMap *tm) {
     using V = float2;
