@@ -106,7 +106,7 @@ typedef struct flame_ctx *flame_t;
  * keeps the default kernel variants, FLAME_FORCE_VARIANTS=a,b fixes them,
  * FLAME_FUSE=0 keeps the column passes of consecutive steps separate,
  * FLAME_PDL=0 (1) launches no (every) step pass as a programmatic dependent
- * launch, FLAME_FP64_POINTS=8 gives the FP64 public-grid short lines 8 points
+ * launch, FLAME_FP64_POINTS=8 gives short FP64 lines 8 points
  * a thread instead of 4, FLAME_BATCH_TMA has no effect any more (ensembles take
  * direct stores), FLAME_TUNE_CACHE=path keeps the autotuner's choices in a JSON file. */
 flame_status flame_create(const flame_params *params, flame_t *out);
