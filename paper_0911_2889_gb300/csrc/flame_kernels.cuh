@@ -93,10 +93,10 @@ __host__ __device__ __forceinline__ size_t uv_index(int j1, int k2, int ldk) {
 
 template <class R> __device__ __forceinline__ UV<R> ld_uv(const CplxT<R> *p) {
     if constexpr (std::is_same<R, float>::value) {
-        float4 q = __ldg(reinterpret_cast<const float4 *>(p));
+        float4 q = *reinterpret_cast<const float4 *>(p);
         return {make_float2(q.x, q.y), make_float2(q.z, q.w)};
     } else {
-        return {__ldg(p), __ldg(p + 1)};
+        return {p[0], p[1]};
     }
 }
 // (U, V) in shared memory (16-byte aligned slots)
@@ -677,7 +677,7 @@ __device__ __forceinline__ void passA_body(const FlameDesc &d, int tile, int nti
     constexpr int E = 16;
     extern __shared__ __align__(16) unsigned char smraw[];
     const StepArgs &a = d.a;
-    const C *__restrict__ state = static_cast<const C *>(d.state);
+    const C *state = static_cast<const C *>(d.state);
     C *__restrict__ uv = static_cast<C *>(d.uv);
     const C *__restrict__ tw1 = static_cast<const C *>(d.tw1);
     const int N1 = LOG > 0 ? (1 << LOG) : (1 << a.logn1), T = N1 / E;
@@ -704,7 +704,7 @@ __device__ __forceinline__ void passA_body(const FlameDesc &d, int tile, int nti
             const int k1 = (r < E / 4) ? n : n - N1;
             const bool in_box = valid && ((r < E / 4) ? (n <= a.K1) : (k1 >= -a.K1));
             if (in_box && FLAME_IN(d.status, (long long)k2 * ld1 + a.K1 + k1, box_len(a), kSiteAState)) {
-                C phi = __ldg(col + k1);
+                C phi = col[k1];
                 if (k1 == 0 && k2 == 0) phi = C{0, 0};
                 const R f = s1 * (R)k1;
                 C da{-f * phi.y, f * phi.x};  // i s1 k1 Phi
@@ -856,7 +856,7 @@ __device__ __forceinline__ void passB_area_body(const FlameDesc &d, int tile) {
     using C = CplxT<R>;
     extern __shared__ __align__(16) unsigned char smraw[];
     const StepArgs &a = d.a;
-    const C *__restrict__ uv = static_cast<const C *>(d.uv);
+    const C *uv = static_cast<const C *>(d.uv);
     C *__restrict__ gk = static_cast<C *>(d.gk);
     const C *__restrict__ twm = static_cast<const C *>(d.twm);
     const int M = LOG > 0 ? (1 << LOG) : (1 << a.logm), T = M / E;
@@ -1257,7 +1257,7 @@ __device__ __forceinline__ void passC_body(const FlameDesc &d, int tile, int nti
     constexpr int QE = E / 4;  // band registers: r < QE (k1 >= 0) and r >= E - QE (k1 < 0)
     extern __shared__ __align__(16) unsigned char smraw[];
     const StepArgs &a = d.a;
-    const C *__restrict__ gk = static_cast<const C *>(d.gk);
+    const C *gk = static_cast<const C *>(d.gk);
     C *__restrict__ state = static_cast<C *>(d.state);
     const C *__restrict__ tw1 = static_cast<const C *>(d.tw1);
     const int N1 = LOG > 0 ? (1 << LOG) : (1 << a.logn1), T = N1 / E;
@@ -1283,12 +1283,12 @@ __device__ __forceinline__ void passC_body(const FlameDesc &d, int tile, int nti
         C p, q;
         const bool in = va && FLAME_IN(d.status, gk_index(0, c0, N1) + 2 * (long long)n + 1, gk_len(a), kSiteCGk);
         if constexpr (std::is_same<R, float>::value) {
-            const float4 pq = in ? __ldg(reinterpret_cast<const float4 *>(gp) + n) : make_float4(0.f, 0.f, 0.f, 0.f);
+            const float4 pq = in ? reinterpret_cast<const float4 *>(gp)[n] : make_float4(0.f, 0.f, 0.f, 0.f);
             p = C{pq.x, pq.y};
             q = vb ? C{pq.z, pq.w} : C{0, 0};
         } else {
-            p = in ? __ldg(gp + 2 * n) : C{0, 0};
-            q = (in && vb) ? __ldg(gp + 2 * n + 1) : C{0, 0};
+            p = in ? gp[2 * n] : C{0, 0};
+            q = (in && vb) ? gp[2 * n + 1] : C{0, 0};
         }
         x[r] = pack2<R>(p, q);
     }
@@ -1381,7 +1381,7 @@ template <class R, int LOG, int E> __device__ __forceinline__ void passA1_body(c
             const int k1 = (r < E / 4) ? n : n - N1;
             const bool in_box = valid && ((r < E / 4) ? (n <= a.K1) : (k1 >= -a.K1));
             if (in_box && FLAME_IN(d.status, (long long)k2 * ld1 + a.K1 + k1, box_len(a), kSiteAState)) {
-                C phi = __ldg(col + k1);
+                C phi = col[k1];
                 if (k1 == 0 && k2 == 0) phi = C{0, 0};
                 const R fk = scale1<R>(a) * (R)k1;
                 x[r] = f == 0 ? CV<V1>{{-fk * phi.y}, {fk * phi.x}} : CV<V1>{{phi.x}, {phi.y}};
@@ -1425,7 +1425,7 @@ template <class R, int LOG, int E> __device__ __forceinline__ void passC1_body(c
     for (int r = 0; r < E; ++r) {
         const size_t i = gk_index(t + r * T, k2, N1);
         C p{0, 0};
-        if (valid && FLAME_IN(d.status, i, gk_len(a), kSiteCGk)) p = __ldg(gk + i);
+        if (valid && FLAME_IN(d.status, i, gk_len(a), kSiteCGk)) p = gk[i];
         x[r] = CV<V1>{{p.x}, {p.y}};
     }
     line_fft_ct<-1, LOG, E>(x, t, sm, tw, CtaBarrier{});

@@ -223,6 +223,15 @@ template <class F> static void with_fp64_points(F &&f) {
     else f(std::integral_constant<int, 8>{});
 }
 
+// Passes A and B of a step with the area are programmatic dependent launches in
+// FP32 (FLAME_PDL=0: not): 512x1024 25.8 -> 24.8 us a step, 1024x2048 31.9 -> 31.4,
+// 4096x8192 365 -> 364.5.  Pass C is not (1024x2048 34.5): early column CTAs take
+// SMs that the row pass, one CTA per SM, still needs.
+template <class R> static bool pdl_area() {
+    const char *v = getenv("FLAME_PDL");
+    return sizeof(R) == 4 && !(v && strcmp(v, "0") == 0);
+}
+
 // Passes A and C on the public grid: the steps that record the surface area
 // (whose sum is over that grid's points).
 template <class R>
@@ -235,7 +244,7 @@ cudaError_t Ops<R>::passA_full(const FlameDesc &d, cudaStream_t s, const CUtenso
             static_for<4, 8>([&](auto lc) {
                 constexpr int L = decltype(lc)::value;
                 if (d.a.logn1 == L)
-                    err = launch_w(d.l2_state, k_passA1<R, L, E>, dim3(g.blocks), g.threads, g.smem, s, d);
+                    err = launch_s(d.l2_state, pdl_area<R>(), k_passA1<R, L, E>, dim3(g.blocks), g.threads, g.smem, s, d);
             });
         });
         return err;
@@ -245,7 +254,7 @@ cudaError_t Ops<R>::passA_full(const FlameDesc &d, cudaStream_t s, const CUtenso
         static_for<8, 11>([&](auto lc) {
             constexpr int L = decltype(lc)::value;
             if (d.a.logn1 == L)
-                err = launch_w(d.l2_state, k_passA1<R, L, 16>, dim3(g.blocks), g.threads, g.smem, s, d);
+                err = launch_s(d.l2_state, pdl_area<R>(), k_passA1<R, L, 16>, dim3(g.blocks), g.threads, g.smem, s, d);
         });
         return err;
     }
@@ -254,11 +263,11 @@ cudaError_t Ops<R>::passA_full(const FlameDesc &d, cudaStream_t s, const CUtenso
         constexpr int L = decltype(lc)::value;
         if constexpr (sizeof(R) == 4 && L > 0) if (uv_map) {  // tensor-store write-out
             const int pf = resident_ctas((const void *)k_passAt<R, L>, g);
-            err = launch_w(d.l2_state, k_passAt<R, L>, dim3(g.blocks), g.threads, g.smem, s, d, pf, *uv_map);
+            err = launch_s(d.l2_state, pdl_area<R>(), k_passAt<R, L>, dim3(g.blocks), g.threads, g.smem, s, d, pf, *uv_map);
             return;
         }
         const int pf = resident_ctas((const void *)k_passA<R, L>, g);
-        err = launch_w(d.l2_state, k_passA<R, L>, dim3(g.blocks), g.threads, g.smem, s, d, pf);
+        err = launch_s(d.l2_state, pdl_area<R>(), k_passA<R, L>, dim3(g.blocks), g.threads, g.smem, s, d, pf);
     });
     return err;
 }
@@ -294,7 +303,7 @@ template <class R> cudaError_t Ops<R>::passB_area(const FlameDesc &d, cudaStream
             static_for<4, 8>([&](auto lc) {
                 constexpr int L = decltype(lc)::value;
                 if (d.a.logm == L)
-                    err = launch_k(k_passB_area<R, L, E, 128>, dim3(g.blocks + 1), g.threads, g.smem, s, d);
+                    err = launch_s(L2Window{nullptr, 0, 0.f}, pdl_area<R>(), k_passB_area<R, L, E, 128>, dim3(g.blocks + 1), g.threads, g.smem, s, d);
             });
         });
         return err;
@@ -309,7 +318,7 @@ template <class R> cudaError_t Ops<R>::passB_area(const FlameDesc &d, cudaStream
         if (g.smem + 4096 > (size_t)optin) return cudaErrorNotSupported;
         with_log<R>(d.a.logm, [&](auto lc) {
             constexpr int L = decltype(lc)::value;
-            if constexpr (L > 0) err = launch_k(k_passB_area<R, L, 8, 512>, dim3(g.blocks + 1), g.threads, g.smem, s, d);
+            if constexpr (L > 0) err = launch_s(L2Window{nullptr, 0, 0.f}, pdl_area<R>(), k_passB_area<R, L, 8, 512>, dim3(g.blocks + 1), g.threads, g.smem, s, d);
         });
         if (err != cudaSuccess) return err;
         return cudaGetLastError();
@@ -323,7 +332,7 @@ template <class R> cudaError_t Ops<R>::passB_area(const FlameDesc &d, cudaStream
             err = cudaErrorNotSupported;
             return;
         }
-        err = launch_k(k_passB_area<R, L, 16, 256>, dim3(ga.blocks + 1), ga.threads, ga.smem, s, d);
+        err = launch_s(L2Window{nullptr, 0, 0.f}, pdl_area<R>(), k_passB_area<R, L, 16, 256>, dim3(ga.blocks + 1), ga.threads, ga.smem, s, d);
     });
     if (err != cudaSuccess) return err;
     return cudaGetLastError();
