@@ -69,8 +69,10 @@ static int resident_ctas(const void *kernel, const Geom &g) {
 // scheduled while the previous kernel on the stream drains, and wait in
 // hardware (griddepcontrol.wait, the first statement of every step pass's
 // body) until that kernel has completed and its memory is visible.  Only
-// the step passes, whose bodies begin with that wait, are launched so: in FP32,
-// and in FP64 for columns of up to 96 points (N1 <= 128).  Per step (graph):
+// kernels whose bodies begin with that wait are launched so: the step's and the
+// adjoint's passes in FP32, and in FP64 for columns of up to 96 points (N1 <=
+// 128); in FP32 also a 2-D transform's second pass and passes A and B of a step
+// with its area.  Per step (graph):
 // FP32 256x512 9.5 -> 8.1 us, 1024x2048 18.1 -> 17.0, 4096x8192 level; FP64
 // 128x256 23.5 -> 22.1, but 512x1024 77.4 -> 83.5: the early CTAs land where
 // SMs drain first, and longer FP64 passes are bound by their fullest SM.

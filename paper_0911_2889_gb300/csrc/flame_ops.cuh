@@ -146,8 +146,10 @@ cudaError_t Ops<R>::cols(const C *in, C *out, int logn, int split, int ncols, in
     // (4096x8192 -2 and -6 us; 4096x2048, which stays, +0.5)
     const int ahead = split > 1 && ((size_t)split << logn) * ld * sizeof(C) > ((size_t)64 << 20) ? 2 * sm_count() : 0;
     cudaError_t err = cudaSuccess;
-    // r2c: behind the row pass
-    const bool pdl = dir < 0 && sizeof(R) == 4;
+    // r2c: behind the row pass; not behind the 64-thread CTAs of split rows of
+    // 1024 points, among which the early column CTAs crowd in (1024x1024 16.5 us
+    // against 9.7, 2048x1024 17.1 against 14.1; 2048x2048 18.0 against 18.9 without)
+    const bool pdl = dir < 0 && sizeof(R) == 4 && !(split > 1 && ncols < 1024);
     auto go = [&](auto kernel, int threads, int G, size_t smem) {
         err = launch_s(L2Window{nullptr, 0, 0.f}, pdl, kernel, dim3((npairs + G - 1) / G, split), threads, smem, s, in,
                        out, logn, ncols, ld, tw, ahead, status);
