@@ -50,7 +50,9 @@ flame_status fail(flame_status s, const char *fmt, ...) {
 
 // Host-side fault injection for the error-path tests:
 // FLAME_FAULT_INJECT=alloc|launch|param makes the next matching call fail
-// before it touches the device.
+// before it touches the device.  "wait" (index-checking build): steps in FP32
+// whose row pass loads by bulk copies do not issue them, so that its bounded
+// waits run out.
 bool inject(const char *what) {
     const char *v = getenv("FLAME_FAULT_INJECT");
     return v && strcmp(v, what) == 0;
@@ -285,6 +287,9 @@ FlameDesc make_desc(flame_ctx *h, void *state, double *mean, double *t) {
     d.t_out = t;
     d.status = h->status;
     if (h->l2_state_bytes) d.l2_state = flame::L2Window{state, h->l2_state_bytes, h->l2_state_hit};
+#ifdef FLAME_DEBUG_BOUNDS
+    if (inject("wait")) d.a.flags |= flame::kStallRowLoad;
+#endif
     d.stage = flame::kStageEuler;
     // the two-stage schemes carry one box between their stages in the area
     // workspace (N1 (K2+1) pairs, larger than the box) and one FP64 scalar

@@ -10,6 +10,7 @@ namespace flame {
 
 constexpr unsigned kLinearOnly = 1u;
 constexpr unsigned kNonlinearOnly = 2u;
+constexpr unsigned kStallRowLoad = 1u << 31;  // index-checking build: pass B's row copies are announced but not issued
 constexpr int kStatusNonfinite = 0;
 constexpr int kStatusTimeout = 1;
 constexpr int kStatusBounds = 2;

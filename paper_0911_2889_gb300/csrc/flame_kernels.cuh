@@ -47,8 +47,10 @@ static __device__ __noinline__ bool bounds_fail(int *status, int site, long long
 #define FLAME_IN(status, i, n, site)                                                     \
     ((unsigned long long)(long long)(i) < (unsigned long long)(long long)(n) ||          \
      ::flame::bounds_fail((status), (site), (long long)(i), (long long)(n)))
+#define FLAME_STALL(flags) ((flags) & kStallRowLoad)
 #else
 #define FLAME_IN(status, i, n, site) true
+#define FLAME_STALL(flags) false
 #endif
 // Extents (complex entries) of the step's arrays: the compact box (state,
 // forcing, stage buffer), the (U, V) workspace and the G workspace (column

@@ -274,25 +274,36 @@ template <class V, class C> __device__ __forceinline__ void real_post(CV<V> h, C
 // Bulk copy of a block (16-byte aligned, a multiple of 16 bytes) from global
 // to shared memory by one thread, and the wait of all threads for it on the
 // mbarrier `bar`, which the copying thread initialises: a CTA barrier has to
-// come between.  The wait is bounded; if it runs out, the status says so.
-__device__ __forceinline__ void bulk_load(void *dst, const void *src, unsigned bytes, unsigned long long *bar) {
+// come between.  The wait ends after a second; false: the block has not come.
+__device__ __forceinline__ void bulk_load(void *dst, const void *src, unsigned bytes, unsigned long long *bar, bool issue = true) {
     const unsigned sb = (unsigned)__cvta_generic_to_shared(bar), sd = (unsigned)__cvta_generic_to_shared(dst);
     asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(sb) : "memory");
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(sb), "r"(bytes) : "memory");
-    if (bytes)
+    if (bytes && issue)
         asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(sd),
                      "l"(reinterpret_cast<unsigned long long>(src)), "r"(bytes), "r"(sb)
                      : "memory");
 }
-__device__ __forceinline__ void bulk_wait(unsigned long long *bar, int *status) {
+__device__ __forceinline__ bool bulk_wait(unsigned long long *bar) {
     const unsigned sb = (unsigned)__cvta_generic_to_shared(bar);
+    const long long start = clock64();
     unsigned done = 0;
-#pragma unroll 1
-    for (int i = 0; i < (1 << 20) && !done; ++i)
+    do {
         asm volatile("{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], 0;\n\tselp.u32 %0, 1, 0, p;\n\t}"
                      : "=r"(done) : "r"(sb) : "memory");
-    if (!done) atomicOr(status, 1 << kStatusTimeout);
+    } while (!done && clock64() - start < 1LL << 31);
+    return done;
+}
+// All threads, at the barrier behind the reads of the block: false, and the
+// status says so, where some thread's wait ran out.  What the CTA read may not
+// be the block then: it writes nothing and returns, behind one more bounded
+// wait for the copy that may still be on its way into its shared memory.
+__device__ __forceinline__ bool bulk_read(bool came, unsigned long long *bar, int *status) {
+    if (__syncthreads_and(came)) return true;
+    if (threadIdx.x == 0) atomicOr(status, 1 << kStatusTimeout);
+    bulk_wait(bar);
+    return false;
 }
 
 // Pass B, two lines per thread (FP32): one row pair per group of TS threads,
@@ -326,7 +337,8 @@ __device__ __forceinline__ void stepB2_body(const FlameDesc &d, int tile, const 
     if (threadIdx.x == 0) {
         const int np = min(G, (a.n1 >> 1) - tile * G);
         const size_t first = w_index(2 * tile * G, 0, a.ldk), len = (size_t)np * 4 * a.ldk;
-        if (FLAME_IN(d.status, first + len - 1, uv_len(a), kSiteBUv)) bulk_load(smstep, uv + first, (unsigned)(len * sizeof(C)), &loaded);
+        if (FLAME_IN(d.status, first + len - 1, uv_len(a), kSiteBUv))
+            bulk_load(smstep, uv + first, (unsigned)(len * sizeof(C)), &loaded, !FLAME_STALL(a.flags));
         else bulk_load(smstep, uv, 0, &loaded);
     }
     ahead.run(d, tile, [&](const FlameDesc &q, int t) {  // that tile's row pairs
@@ -338,7 +350,7 @@ __device__ __forceinline__ void stepB2_body(const FlameDesc &d, int tile, const 
     const C *tw = tab3<R, A, 4, C>(d.twm);
     const C wt = __ldg(static_cast<const C *>(d.twm) + tw3_real_offset<A>() + s.t);  // exp(2 pi i t / 2L)
     __syncthreads();  // the barrier's initialisation
-    bulk_wait(&loaded, d.status);
+    const bool came = bulk_wait(&loaded);
 
     CV<V> xs[ES];
     {
@@ -354,7 +366,7 @@ __device__ __forceinline__ void stepB2_body(const FlameDesc &d, int tile, const 
             up[i] = CV<V>{make_float2(q.x, q.y), make_float2(q.z, q.w)};
             um[i] = CV<V>{make_float2(m.x, m.y), make_float2(m.z, m.w)};
         }
-        __syncthreads();  // the block has been read
+        if (!bulk_read(came, &loaded, d.status)) return;  // (a barrier: the block has been read)
         CV<V> xo[ES];
         static_for<0, ES>([&](auto rc) {
             constexpr int r = decltype(rc)::value;
