@@ -306,6 +306,15 @@ __device__ __forceinline__ bool bulk_read(bool came, unsigned long long *bar, in
     return false;
 }
 
+// Twiddles exp(2 pi i k / 2L) of the real post-processing, k = t + r TS: rows of
+// 3072 points form them from one entry per thread and compile-time roots, as
+// the inverse transforms' odd points do; shorter rows read the table, which is
+// what keeps the step's rounding error at that of the public grid's rows.  1024x2048,
+// increment (nonlinear only, flat spectrum): 3.379e-7 with roots, 3.354e-7 so,
+// 3.376e-7 on the public grid; an ensemble of 96 443.4 -> 446.1 us a step,
+// 1024x2048 level.  (Both from the table: 3.306e-7, but 460 us.)
+template <int A> constexpr bool kPostRoots = A == kMaxA;
+
 // Pass B, two lines per thread (FP32): one row pair per group of TS threads,
 // the lanes its two rows.  The even and the odd points are two inverse
 // transforms with an exchange buffer each, whose first passes run together as
@@ -321,7 +330,7 @@ template <class R, int A, bool TMA>
 __device__ __forceinline__ void stepB2_body(const FlameDesc &d, int tile, const Ahead &ahead, const CUtensorMap *tm) {
     using V = float2;
     using C = CplxT<R>;
-    using PL = Plan3<A, 4>;
+    using PL = Plan3<A, 4, A == kMaxA>;
     constexpr int L = PL::L, TS = PL::TS, TP = PL::TP, ES = PL::ES, SL = PL::slots(kSlotsPerWave<V>);
     extern __shared__ __align__(128) unsigned char smstep[];
     const StepArgs &a = d.a;
@@ -348,7 +357,8 @@ __device__ __forceinline__ void stepB2_body(const FlameDesc &d, int tile, const 
     auto even = [&](int line) { return planes3<V, R>(smstep, line, SL); };
     auto odd = [&](int line) { return planes3<V, R>(smstep, G + line, SL); };
     const C *tw = tab3<R, A, 4, C>(d.twm);
-    const C wt = __ldg(static_cast<const C *>(d.twm) + tw3_real_offset<A>() + s.t);  // exp(2 pi i t / 2L)
+    const C *P = static_cast<const C *>(d.twm) + tw3_real_offset<A>() + s.t;
+    const C wt = __ldg(P);  // exp(2 pi i t / 2L)
     __syncthreads();  // the barrier's initialisation
     const bool came = bulk_wait(&loaded);
 
@@ -411,6 +421,11 @@ __device__ __forceinline__ void stepB2_body(const FlameDesc &d, int tile, const 
     forward3<PL, false>(xp, hk, p, s, odd, tw);
     griddep_launch();
     // real-input post-processing: the pairs (k, L - k), k <= L/2
+    C post[ES / 2];  // exp(2 pi i k / 2L)
+    static_for<0, ES / 2>([&](auto rc) {
+        constexpr int r = decltype(rc)::value;
+        post[r] = kPostRoots<A> ? mul_root24<r, ES>(wt) : r == 0 ? wt : __ldg(P + r * TS);
+    });
     __syncthreads();
     const Planes<V> sm = odd(s.line);
     if (s.on) {
@@ -433,7 +448,7 @@ __device__ __forceinline__ void stepB2_body(const FlameDesc &d, int tile, const 
             const int k = s.t + r * TS, kc = L - k;
             if (k <= a.K2 || kc <= a.K2) {
                 CV<V> lo, hi;
-                real_post(hk[r], sm.ld_raw(k == 0 ? 0 : kc), mul_root24<r, ES>(wt), lo, hi);
+                real_post(hk[r], sm.ld_raw(k == 0 ? 0 : kc), post[r], lo, hi);
                 if (k <= a.K2) emit(k, lo);
                 if (kc <= a.K2) emit(kc, hi);
             }

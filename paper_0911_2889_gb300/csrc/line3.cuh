@@ -72,7 +72,9 @@ template <int F, int DIR, class V> __device__ __forceinline__ void dft_3f(CV<V> 
 // ----------------------------------------------------------------------------
 constexpr int gcd_c(int a, int b) { return b == 0 ? a : gcd_c(b, a % b); }
 
-template <int A_, int F_> struct Plan3 {
+// PRODUCTS: the last pass forms its twiddles (butterflies)
+template <int A_, int F_, bool PRODUCTS_ = false> struct Plan3 {
+    static constexpr bool PRODUCTS = PRODUCTS_;
     static constexpr int A = A_, F = F_, LF = F == 4 ? 2 : F == 2 ? 1 : 0;
     static_assert(F == 1 || F == 2 || F == 4, "F");
     static_assert(A >= LF + 2, "a line needs 12 F points");
@@ -173,11 +175,18 @@ inline int step_exponent(int K) {
 // ----------------------------------------------------------------------------
 // Passes
 // ----------------------------------------------------------------------------
-// FP32, lines of 3 * 2^8 points and more, last pass: w^q for q = 4a + b is the
-// product w^(4a) w^b of two table entries, 6 loads for radix 16 instead of 15
-// (a 3072-point line's last pass reads 9 KB of its table instead of 23).  One
-// more rounding of half an ulp; FP64, bound by its arithmetic, loads them all.
-template <class C, class PL> constexpr bool kTwiddleProducts = sizeof(C) == 8 && PL::A >= 8;
+// A plan with PRODUCTS, FP32: in the last pass w^q for q = 4a + b is the product
+// w^(4a) w^b of two table entries, 6 loads for radix 16 instead of 15 (a 3072-point
+// line's last pass reads 9 KB of its table instead of 23).  Such a twiddle is off
+// by up to about 2 * 2^-24 (the entries' errors and the product's), a table entry
+// by 0.7 * 2^-24, so only the rows of 3072 points take it, whose 4096-point
+// predecessors on the public grid had products of two entries too: 4096x8192
+// 136.1 -> 134.5 us a step, 2048x8192 74.0 -> 73.0.  Relative L2 error of the
+// step's increment (nonlinear only, flat spectrum, mean of 4): 4096x8192 3.85e-7
+// against 3.80e-7 with entries and 4.21e-7 on the public grid.  (In all passes
+// from 768 points on: 3.91e-7 for 133.7 us, and 1024x2048 3.54e-7 against
+// 3.38e-7 for 16.9 us instead of 17.0.)
+template <class C, class PL> constexpr bool kTwiddleProducts = sizeof(C) == 8 && PL::PRODUCTS;
 
 // Pass S on a thread's E points x[i] = element t + i T (T = L / E): B = E / r
 // butterflies j = t + b T, twiddles, DFTs.
