@@ -828,20 +828,18 @@ __global__ void __launch_bounds__(kStepThreads<R, typename OneOf<R>::type, A, F,
     stepB1_body<R, A, F, RW>(ds[blockIdx.y], blockIdx.x - 1);
 }
 
-// Plain pass C at 80 registers a thread, three CTAs per SM, where a launch has
-// several waves of them: 3072-point columns (4096x8192 136.7 -> 133.7 us a step)
-// and ensembles (96 flames 7.37 -> 7.24 ms); elsewhere two (2048x4096 39.6
-// against 40.9 us).
-template <class R, class V, int A, int F, bool GEN, int FROM> constexpr int kStepBlocksC =
-    kLanes<V> == 2 && !GEN && A >= FROM ? 3 : kStepBlocks<R, V, A, F, 2>;
-template <class R, class V, int A, int F, bool GEN>
-__global__ void __launch_bounds__(kStepThreads<R, V, A, F, 2>, kStepBlocksC<R, V, A, F, GEN, 10>) k_stepC(FlameDesc d, int pf) {
+// Plain pass C with THREE: 80 registers a thread, three CTAs per SM, for launches
+// of several waves (three_ctas in flame_step_ops.cuh).
+template <class R, class V, int A, int F, bool GEN, bool THREE> constexpr int kStepBlocksC =
+    THREE ? 3 : kStepBlocks<R, V, A, F, 2>;
+template <class R, class V, int A, int F, bool GEN, bool THREE = false>
+__global__ void __launch_bounds__(kStepThreads<R, V, A, F, 2>, kStepBlocksC<R, V, A, F, GEN, THREE>) k_stepC(FlameDesc d, int pf) {
     const int extra = d.tile0 == 0 ? 1 : 0;
     if (extra && blockIdx.x == 0) return finish_cta<R, GEN, true>(d);
     stepC_body<R, V, A, F, GEN>(d, blockIdx.x - extra + d.tile0, Ahead{pf, (int)gridDim.x - extra + d.tile0, nullptr}, nullptr);
 }
-template <class R, class V, int A, int F, bool GEN>
-__global__ void __launch_bounds__(kStepThreads<R, V, A, F, 2>, kStepBlocksC<R, V, A, F, GEN, 6>) k_stepC_n(const FlameDesc *__restrict__ ds, int pf) {
+template <class R, class V, int A, int F, bool GEN, bool THREE = false>
+__global__ void __launch_bounds__(kStepThreads<R, V, A, F, 2>, kStepBlocksC<R, V, A, F, GEN, THREE>) k_stepC_n(const FlameDesc *__restrict__ ds, int pf) {
     if (blockIdx.x == 0) return finish_cta<R, GEN, true>(ds[blockIdx.y]);
     stepC_body<R, V, A, F, GEN>(ds[blockIdx.y], blockIdx.x - 1, Ahead{pf, (int)gridDim.x - 1, ds}, nullptr);
 }

@@ -197,6 +197,15 @@ cudaError_t Ops<R>::passB_batch(const FlameDesc *ds, int n, const StepArgs &a, c
     return err;
 }
 
+// Plain pass C, two lines per thread, three CTAs per SM (k_stepC's THREE): columns
+// of 3072 points in more than two waves of two CTAs, which are then a wave
+// less.  us a step with two, with three: 4096x8192 137.3, 134.5; 4096x4096 72.5,
+// 72.5; 4096x2048 (under a wave) 40.9, 42.7; 4096x512 19.3, 20.7 (direct stores).
+// Shorter columns have 1.7 waves at most (2048x4096 40.5, 41.5).  Ensembles take
+// three always: of 96 uneven flames 448.8 us, by this rule 451.0 (of 8 flames of
+// 512x1024 25.7, 24.5; of 96 of 256x512 55.5, with two 64.6).
+static bool three_ctas(int tiles) { return tiles > 4 * sm_count(); }
+
 template <class R> cudaError_t Ops<R>::passC(const FlameDesc &d, cudaStream_t s) {
     cudaError_t err = cudaErrorInvalidValue;
     const int npair = (d.a.K2 + 2) / 2, extra = d.tile0 == 0 ? 1 : 0;
@@ -216,8 +225,14 @@ template <class R> cudaError_t Ops<R>::passC(const FlameDesc &d, cudaStream_t s)
     }
     if constexpr (sizeof(R) == 4) with_two_line(d.a.la, [&](auto ac) {
         constexpr int A = decltype(ac)::value;
-        err = launch(k_stepC<R, float2, A, 4, false>, k_stepC<R, float2, A, 4, true>, geom_two_line(A, npair, pair_bytes<A>()),
-                     true);
+        const Geom g = geom_two_line(A, npair, pair_bytes<A>());
+        const auto general = k_stepC<R, float2, A, 4, true>;
+        if constexpr (A == kMaxA)
+            if (three_ctas(d.tiles ? d.tiles : g.blocks)) {
+                err = launch(k_stepC<R, float2, A, 4, false, true>, general, g, true);
+                return;
+            }
+        err = launch(k_stepC<R, float2, A, 4, false>, general, g, true);
     });
     return err;
 }
@@ -239,7 +254,7 @@ cudaError_t Ops<R>::passC_batch(const FlameDesc *ds, int n, const StepArgs &a, c
         constexpr int A = decltype(ac)::value;
         const Geom g = geom_two_line(A, n * npair, pair_bytes<A>());
         const int G = g.threads >> (A - 2);
-        const auto kernel = gen ? k_stepC_n<R, float2, A, 4, true> : k_stepC_n<R, float2, A, 4, false>;
+        const auto kernel = gen ? k_stepC_n<R, float2, A, 4, true> : k_stepC_n<R, float2, A, 4, false, true>;
         err = launch_k(kernel, dim3((npair + G - 1) / G + 1, n), g.threads, g.smem, s, ds, resident_ctas((const void *)kernel, g));
     });
     return err;
