@@ -289,6 +289,8 @@ template <class R> __host__ __device__ constexpr int adj_f(int a) {
 __host__ __device__ __forceinline__ size_t l_index(int j1, int k2, int ldk) {
     return 2 * ((size_t)(j1 >> 1) * ldk + k2) + (j1 & 1);
 }
+// ... and its extent (lambda's row spectra lie in gk)
+__host__ __device__ __forceinline__ long long l_len(const StepArgs &a) { return (long long)a.n1 * a.ldk; }
 
 // Columns c0, c0 + 1 of lambda (lambda_0 at k = 0); the extra CTA derives the
 // step's coefficients for pass C (and dt / (2 t_n), dL/dgamma's factor).
@@ -321,8 +323,9 @@ template <class R, int A> __global__ void __launch_bounds__(256, kMinBlocks<R>) 
             if (r >= F && r < 2 * F) continue;
             const int n = s.t + r * PL::TS, k1 = r < F ? n : n - PL::L;
             const bool in_box = r < F ? n <= a.K1 : k1 >= -a.K1;
-            C p0 = in_box && c0 <= a.K2 ? la[k1] : C{0, 0};
-            const C p1 = in_box && c0 + 1 <= a.K2 ? lb[k1] : C{0, 0};
+            [[maybe_unused]] const long long i = (long long)c0 * ld1 + a.K1 + k1;
+            C p0 = in_box && c0 <= a.K2 && FLAME_IN(d.status, i, box_len(a), kSiteAdjLam) ? la[k1] : C{0, 0};
+            const C p1 = in_box && c0 + 1 <= a.K2 && FLAME_IN(d.status, i + ld1, box_len(a), kSiteAdjLam) ? lb[k1] : C{0, 0};
             if (c0 == 0 && k1 == 0) p0 = C{(R)l0, 0};
             xs[r] = pack2<R>(p0, p1);
         }
@@ -336,9 +339,9 @@ template <class R, int A> __global__ void __launch_bounds__(256, kMinBlocks<R>) 
     const int c0 = 2 * ((blockIdx.x - 1) * G + p.line);
 #pragma unroll
     for (int i = 0; i < PL::EP; ++i) {
-        C *e = out + l_index(p.t + i * PL::TP, c0, a.ldk);
-        if (c0 <= a.K2) e[0] = lane0<R>(xp[i]);
-        if (c0 + 1 <= a.K2) e[2] = lane1<R>(xp[i]);
+        const size_t n = l_index(p.t + i * PL::TP, c0, a.ldk);
+        if (c0 <= a.K2 && FLAME_IN(d.status, n, l_len(a), kSiteAdjRow)) out[n] = lane0<R>(xp[i]);
+        if (c0 + 1 <= a.K2 && FLAME_IN(d.status, n + 2, l_len(a), kSiteAdjRow)) out[n + 2] = lane1<R>(xp[i]);
     }
 }
 
@@ -380,7 +383,8 @@ template <class R, int A> __global__ void __launch_bounds__(256, kMinBlocks<R>) 
     {
         CV<V> xs[ES], xp[PL::EP];
         half_inputs<PL, R>(xs, s.t, valid, a.K2, P, [&](int k, bool minus) {
-            const C e = lrow[l_index(row, k, a.ldk)];
+            const size_t n = l_index(row, k, a.ldk);
+            const C e = FLAME_IN(d.status, n, l_len(a), kSiteAdjRow) ? lrow[n] : C{0, 0};
             return minus ? C{e.x, -e.y} : e;
         });
         inverse3<PL>(xs, xp, s, p, buf, tw);
@@ -390,7 +394,10 @@ template <class R, int A> __global__ void __launch_bounds__(256, kMinBlocks<R>) 
     CV<V> xp[PL::EP];
     {
         CV<V> xs[ES];
-        half_inputs<PL, R>(xs, s.t, valid, a.K2, P, [&](int k, bool minus) { return ld_w<R>(uv, row, k, a.ldk, minus); });
+        half_inputs<PL, R>(xs, s.t, valid, a.K2, P, [&](int k, bool minus) {
+            return FLAME_IN(d.status, w_index(row, k, a.ldk) + 3, uv_len(a), kSiteAdjUv) ? ld_w<R>(uv, row, k, a.ldk, minus)
+                                                                                          : C{0, 0};
+        });
         __syncthreads();  // the exchange buffers are free
         inverse3<PL>(xs, xp, s, p, buf, tw);
     }
@@ -415,7 +422,8 @@ template <class R, int A> __global__ void __launch_bounds__(256, kMinBlocks<R>) 
     auto emit = [&](int k, CV<V> Y) {
         const C q2 = lane1<R>(Y);
         const R f = s2 * (R)k;
-        st_uv<R>(aw + 2 * ((size_t)k * a.n1 + row), lane0<R>(Y), C{f * q2.y, -f * q2.x});  // -i f q2
+        if (FLAME_IN(d.status, 2 * ((long long)k * a.n1 + row) + 1, uv_len(a), kSiteAdjAw))
+            st_uv<R>(aw + 2 * ((size_t)k * a.n1 + row), lane0<R>(Y), C{f * q2.y, -f * q2.x});  // -i f q2
     };
 #pragma unroll
     for (int r = 0; r < ES; ++r) {
@@ -451,7 +459,9 @@ template <class R, int A> __global__ void __launch_bounds__(256, kMinBlocks<R>) 
         const C *aw = static_cast<const C *>(d.aw) + 2 * (size_t)k2 * L;
 #pragma unroll
         for (int i = 0; i < PL::EP; ++i) {
-            const UV<R> e = p.on && k2 <= a.K2 ? ld_uv<R>(aw + 2 * (p.t + i * PL::TP)) : UV<R>{C{0, 0}, C{0, 0}};
+            const int n = p.t + i * PL::TP;
+            const bool in = p.on && k2 <= a.K2 && FLAME_IN(d.status, 2 * ((long long)k2 * L + n) + 1, uv_len(a), kSiteAdjAw);
+            const UV<R> e = in ? ld_uv<R>(aw + 2 * n) : UV<R>{C{0, 0}, C{0, 0}};
             xp[i] = pack2<R>(e.u, e.v);
         }
     }
@@ -475,12 +485,14 @@ template <class R, int A> __global__ void __launch_bounds__(256, kMinBlocks<R>) 
         // k2 = 0, k1 < 0: conjugate mirror of +k1, written (and counted in
         // the gamma gradient, with the same value) by the owner of +k1
         if (!in_box || (k1 == 0 && k2 == 0) || (k2 == 0 && k1 < 0)) continue;
+        const long long bi = (long long)k2 * ld1 + a.K1 + k1;
+        if (!FLAME_IN(d.status, bi, box_len(a), kSiteAdjLam) || !FLAME_IN(d.status, bi, box_len(a), kSiteAdjState)) continue;
         const R f1 = s1 * (R)k1;
         const C Q1 = lane0<R>(xs[r]), Q2 = lane1<R>(xs[r]);
         const C Pk{f1 * Q1.y + Q2.x, -f1 * Q1.x + Q2.y};  // -i f1 Q1 + Q2
         const C l = lam[k1];
         R kap;
-        if (sizeof(R) == 8 && d.kap) kap = static_cast<const R *>(d.kap)[(size_t)k2 * ld1 + a.K1 + k1];
+        if (sizeof(R) == 8 && d.kap) kap = static_cast<const R *>(d.kap)[bi];
         else kap = kappa_norm<R>(f1, s2 * (R)k2);
         if (lin) {
             const C ph = phi[k1];
@@ -491,7 +503,7 @@ template <class R, int A> __global__ void __launch_bounds__(256, kMinBlocks<R>) 
         const R cn = nl ? rcs : (R)0;
         const C nw{l.x + rdt * (om * l.x + cn * Pk.x), l.y + rdt * (om * l.y + cn * Pk.y)};
         lout[k1] = nw;
-        if (k2 == 0) lout[-k1] = C{nw.x, -nw.y};
+        if (k2 == 0 && FLAME_IN(d.status, a.K1 - k1, box_len(a), kSiteAdjLam)) lout[-k1] = C{nw.x, -nw.y};
     }
     const double sum = cta_sum(dg, red);
     if (threadIdx.x == 0 && sum != 0.0) atomicAdd(d.dgamma, sum * d.coef[10]);

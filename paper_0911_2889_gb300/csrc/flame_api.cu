@@ -1490,6 +1490,7 @@ flame_status flame_adjoint(flame_t h, const void *state0, const double *mean0, c
         d.twm = h->twms;
         d.coef = h->dscal + 8;
         d.kap = h->kap;
+        d.status = h->status;
         for (int g = nseg - 1; g >= 0; --g) {
             const int len = (g == nseg - 1) ? nsteps - g * K : K;
             // the segment's trajectory: state 0 is the checkpoint, state i > 0

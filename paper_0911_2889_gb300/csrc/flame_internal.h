@@ -39,6 +39,11 @@ enum BoundsSite : int {
     kSiteFftOut = 15,   // standalone 2-D FFT passes: output entry
     kSiteBoxSpec = 16,  // state from a field: spectrum entry and state entry
     kSiteProbe = 17,    // flame_debug_bounds_probe (a check with no access)
+    kSiteAdjLam = 18,   // adjoint step: lambda load and store (incl. the k2 = 0 mirror)
+    kSiteAdjRow = 19,   // adjoint step: lambda's row spectra
+    kSiteAdjUv = 20,    // adjoint step: row spectra of the state's gradient
+    kSiteAdjAw = 21,    // adjoint step: (hat q1, hat q2) column
+    kSiteAdjState = 22, // adjoint step: state entry, |kappa| table
 };
 // One index check of (i, n) with no memory access, recorded in status
 // (index-checking build); returns cudaErrorNotSupported in the normal build.
@@ -167,6 +172,7 @@ struct AdjDesc {
     double *dgamma;      // dL/dgamma accumulator (atomic)
     double *coef;        // adjoint step: the step's coefficients (k_adjL to k_adjC)
     const void *kap;     // adjoint step: |kappa| of every box entry (FP64) or null
+    int *status;         // adjoint step: the handle's device status word
     const void *tw1, *twm;
 };
 

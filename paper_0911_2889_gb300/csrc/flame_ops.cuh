@@ -420,6 +420,7 @@ template <class R> cudaError_t Ops<R>::adj_step(const AdjDesc &d, cudaStream_t s
     f.state = const_cast<void *>(d.state);
     f.uv = d.uv;
     f.tw1 = d.tw1;
+    f.status = d.status;
     cudaError_t e = passA(f, s, a.la <= 8 ? kVariantOneLine : kVariantDirect);
     if (e != cudaSuccess) return e;
     with_a(a.la, [&](auto ac) {
