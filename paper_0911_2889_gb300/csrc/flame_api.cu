@@ -209,7 +209,7 @@ struct flame_ctx {
     int var_a_bat = 0, var_b_bat = 0;
     // tensor map of uv for the tensor-store variant of pass A (FP32)
     CUtensorMap uv_map, gk_map;  // tensor maps of uv and gk for the tensor-store variants (FP32)
-    CUtensorMap uv_map_full;  // uv of the public grid (steps that record the area)
+    CUtensorMap uv_map_full;  // uv of the public grid (steps that record the area), N1 >= 2048
     bool has_uv_map = false, has_gk_map = false, has_uv_map_full = false;
     const CUtensorMap *map() const { return has_uv_map ? &uv_map : nullptr; }
     const CUtensorMap *gmap() const { return has_gk_map ? &gk_map : nullptr; }
@@ -937,7 +937,7 @@ flame_status flame_create(const flame_params *params, flame_t *out) {
         h->has_uv_map = flame::encode_uv_map(&h->uv_map, h->uv, h->ss.n1, (int)ldk, flame::uv3_box_pairs(h->ss.n1));
     if (st == FLAME_OK && p.prec == FLAME_FP32_MIXED && h->ss.lb >= 6)
         h->has_gk_map = flame::encode_gk_map(&h->gk_map, h->gk, h->ss.n1, (int)ldk);
-    if (st == FLAME_OK && p.prec == FLAME_FP32_MIXED && h->logn1 >= 8 && h->logn1 <= 12)
+    if (st == FLAME_OK && p.prec == FLAME_FP32_MIXED && h->logn1 >= 11)
         h->has_uv_map_full = flame::encode_uv_map(&h->uv_map_full, h->uv, (int)n1, (int)ldk, flame::uv_box_pairs((int)n1));
     if (st == FLAME_OK) st = autotune(h);
     if (st != FLAME_OK) {

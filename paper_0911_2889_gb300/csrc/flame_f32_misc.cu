@@ -8,8 +8,6 @@ template cudaError_t Ops<float>::rows_r2c(const float *, float2 *, int, int, con
 template cudaError_t Ops<float>::rows_c2r(const float2 *, float *, int, int, const float2 *, const float2 *, cudaStream_t, int *);
 template cudaError_t Ops<float>::cols(const float2 *, float2 *, int, int, int, int, int, const float2 *, cudaStream_t, int *);
 template cudaError_t Ops<float>::box_from_spec(const float2 *, float2 *, double *, int, int, int, int, cudaStream_t, int *);
-template Geom Ops<float>::geom_cols(int, int, int);
-template Geom Ops<float>::geom_rows(int, int, int);
 
 #ifdef FLAME_DEBUG_BOUNDS
 static __global__ void k_bounds_probe(int *status, int i, int n) {

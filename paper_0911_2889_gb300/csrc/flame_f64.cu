@@ -8,8 +8,6 @@ template cudaError_t Ops<double>::rows_r2c(const double *, double2 *, int, int, 
 template cudaError_t Ops<double>::rows_c2r(const double2 *, double *, int, int, const double2 *, const double2 *, cudaStream_t, int *);
 template cudaError_t Ops<double>::cols(const double2 *, double2 *, int, int, int, int, int, const double2 *, cudaStream_t, int *);
 template cudaError_t Ops<double>::box_from_spec(const double2 *, double2 *, double *, int, int, int, int, cudaStream_t, int *);
-template Geom Ops<double>::geom_cols(int, int, int);
-template Geom Ops<double>::geom_rows(int, int, int);
 template cudaError_t Ops<double>::passA_full(const FlameDesc &, cudaStream_t, const CUtensorMap *);
 template cudaError_t Ops<double>::passB_area(const FlameDesc &, cudaStream_t);
 template cudaError_t Ops<double>::passC_full(const FlameDesc &, cudaStream_t);

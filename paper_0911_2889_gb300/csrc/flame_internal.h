@@ -145,8 +145,8 @@ struct FlameDesc {
     // a launch over part of the tiles (pass A and C of one flame): tiles
     // [tile0, tile0 + tiles) of the full grid; tiles = 0: all
     int tile0, tiles;
-    // pass C with one line per thread group (set with pass A's one-line
-    // variant; FP32 column lengths 2^8 .. 2^11)
+    // pass C with one line per thread (set with pass A's one-line variant; FP32
+    // columns of 192 .. 1536 points)
     int onec;
     // L2 persisting window over the state for the launches of passes A and
     // C (a launch attribute, not read by the kernels); bytes = 0: none
@@ -236,9 +236,6 @@ template <class R> struct Ops {
     static cudaError_t passA_full(const FlameDesc &d, cudaStream_t s, const CUtensorMap *uv_map);
     static cudaError_t passB_area(const FlameDesc &d, cudaStream_t s);
     static cudaError_t passC_full(const FlameDesc &d, cudaStream_t s);
-    // geometry used by the step passes (for the autotuner and the tests)
-    static Geom geom_cols(int logn, int nlines, int groups_hint);
-    static Geom geom_rows(int logm, int nlines, int groups_hint);
     // Area objective (and its gradient when d.grad / d.dmean are set): 3 kernels.
     static cudaError_t area(const AdjDesc &d, cudaStream_t s);
     // One adjoint step at (d.state, d.t) on the alias-free grid (d.a, d.tw1,

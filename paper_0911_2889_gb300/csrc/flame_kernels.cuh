@@ -1,13 +1,17 @@
 // flame_kernels.cuh -- the kernels of the spectral flame step and of the
 // standalone 2-D real FFTs, templated on the working precision R.
 //
-// Step of eq. (SivCurv1c) (Sec. 2) with the FFT evaluation of the quadratic
-// term (Sec. 3), in three passes over HBM:
+// The step's own passes, on its alias-free grid, are flame_step.cuh's.  Here are
+// what they share (epilogue, coefficients, mean mode, tensor stores, L2 and
+// dependent-launch helpers) and the passes of a step that records the surface
+// area, whose sum is over the points of the public grid.  That step of eq.
+// (SivCurv1c) (Sec. 2), with the FFT evaluation of the quadratic term (Sec. 3),
+// in three passes over HBM:
 //   pass A (columns): i kappa_1 Phi and Phi -> zero-padded inverse FFT along
 //                     k1 (the first index, Sec. 3) -> U(j1,k2), V(j1,k2)
-//   pass B (rows):    inverse FFT along k2 of U + iV -> u + iv on the grid,
-//                     g = u^2 + v^2 = |grad Phi|^2, forward real FFT of g
-//                     along j2, keep k2 <= K2 -> G(j1,k2)
+//   pass B (rows):    inverse FFT along k2 of U + iV -> u + iv on the grid, and
+//                     of Phi for the area terms, g = u^2 + v^2 = |grad Phi|^2,
+//                     forward real FFT of g along j2, keep k2 <= K2 -> G(j1,k2)
 //   pass C (columns): forward FFT along j1, keep |k1| <= K1, scale,
 //                     Euler update with the linear operator, symmetrization
 //                     of the k2 = 0 column (Sec. 3), FP64 mean mode and time.
@@ -530,8 +534,8 @@ __global__ void __launch_bounds__((1 << LOG) / 8, 4096 >> LOG)
 // at a time.  The groups' exchange buffers are 8/G slots of 16 bytes (one,
 // for G > 8) further apart than their length, which puts the G groups and the
 // 8/G points that a quarter warp exchanges on different banks.
-template <class R, int DIR, int LOG, int NT = 256, int E = 16>
-__global__ void __launch_bounds__(NT, NT == 256 ? kMinBlocks<R> : 1)
+template <class R, int DIR, int LOG, int E = 16>
+__global__ void __launch_bounds__(256, kMinBlocks<R>)
     k_cols(const CplxT<R> *in, CplxT<R> *out, int logn, int ncols, int ld, const CplxT<R> *__restrict__ tw, int ahead, int *status) {
     using V = typename VecOf<R>::type;
     using C = CplxT<R>;
@@ -552,7 +556,7 @@ __global__ void __launch_bounds__(NT, NT == 256 ? kMinBlocks<R> : 1)
         C b = vb && FLAME_IN(status, row + cb, len, kSiteFftIn) ? in[row + cb] : C{0, 0};
         x[r] = pack2<R>(a, b);
     }
-    if constexpr (sizeof(R) == 4 && NT == 256 && E == 16 && LOG >= 8 && LOG <= 10) if (ahead > 0) {
+    if constexpr (sizeof(R) == 4 && E == 16 && LOG >= 8 && LOG <= 10) if (ahead > 0) {
         const int tile = blockIdx.y * gridDim.x + blockIdx.x + ahead, q = tile / gridDim.x, c = (tile - q * gridDim.x) * 2 * G;
         if (q < gridDim.y)
             for (int i = threadIdx.x; i < n; i += blockDim.x)
@@ -588,17 +592,9 @@ __device__ __forceinline__ void bulk_commit_and_wait_read() {
     asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
 }
 
-// Shared-memory twiddles of the compile-time FP32 pass-B kernels (E = 16,
-// 2^8..2^12; pass B's ~100 KB of shared memory per CTA leaves too little L1
-// for its 64 KB of global twiddle tables):
-// the 480 factor entries of TwShared, then (pass B) the factors of the real
-// post-processing table P[k] = exp(2 pi i k / 2M): Plo[k mod 64], Phi[k / 64].
-constexpr int kTwSmemBytes = 6144;  // >= (480 + 64 + 4096/64) * 8
-template <class R, int LOG, int E> constexpr bool kSharedTw = std::is_same<R, float>::value && LOG >= 8 && E == 16;
-
 // cos and sin of k pi / 16, k = 0..15: the factors exp(i pi r / E) (E = 16,
 // or E = 8 at every second k) that relate the real-transform twiddles of
-// the E points of one thread (see passB_body).
+// the E points of one thread (see passB_area_body).
 struct Roots32 {
     static constexpr double c[16] = {1.0, 0.980785280403230449126182236134239037, 0.923879532511286756128183189396788933,
                                      0.831469612302545237078788377617905756, 0.707106781186547524400844362104849039,
@@ -637,21 +633,6 @@ template <int R_, int E, int SGN, class C> __device__ __forceinline__ C mul_root
     else if constexpr (k == 8) return C{-ci * b.y, ci * b.x};
     else return C{fma_rn(b.x, cr, -(b.y * ci)), fma_rn(b.x, ci, b.y * cr)};
 }
-
-template <class C> struct RealTw {
-    const C *lo, *hi;
-    __device__ __forceinline__ C operator()(int k) const {
-        const C a = lo[k & 63], b = hi[k >> 6];
-        return C{a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x};
-    }
-    // P = exp(2 pi i k / 2M), k < M = 2^LOGM
-    template <int LOGM> __device__ __forceinline__ static void fill(C *lo_dst, C *hi_dst, const C *P) {
-        for (int i = threadIdx.x; i < 64 + (1 << LOGM) / 64; i += blockDim.x) {
-            if (i < 64) lo_dst[i] = __ldg(P + i);
-            else hi_dst[i - 64] = __ldg(P + 64 * (i - 64));
-        }
-    }
-};
 
 // Memory layouts (the state's is also documented in include/flame.h):
 //   state  column-major compact box: element (k1, k2) at k2 * ld1 + (k1 + K1),
@@ -872,24 +853,7 @@ __device__ __forceinline__ void passB_area_body(const FlameDesc &d, int tile) {
     V *base = reinterpret_cast<V *>(smraw) + (size_t)g * gstride;
     auto sm = make_planes_e<E>(base, M);  // (E = 8 pads one slot every 8: st_raw/ld_raw)
     const C *P = twm + tw_real_offset(a.logm);  // exp(+2 pi i k/N2), k < M
-    constexpr bool STW = kSharedTw<R, LOG, E>;
-    constexpr int LS = STW ? LOG : 8;
-    C *stw = reinterpret_cast<C *>(reinterpret_cast<V *>(smraw) + (size_t)G * gstride);
-    RealTw<C> Pt{stw + 480, stw + 544};
-    if constexpr (STW) {
-        TwShared<C>::template fill<LS>(stw, twm);
-        RealTw<C>::template fill<LS>(stw + 480, stw + 544, P);
-        __syncthreads();
-    }
-    auto realtw = [&](int k) -> C {
-        if constexpr (STW) return Pt(k);
-        else return __ldg(P + k);
-    };
-    auto fft = [&](auto dirc, CV<V>(&x)[E]) {
-        constexpr int DIR = decltype(dirc)::value;
-        if constexpr (STW) fft_line_s<DIR, LS>(x, t, sm, twm, stw);
-        else fft_line_e<DIR, LOG, E>(x, a.logm, t, sm, twm);
-    };
+    auto fft = [&](auto dirc, CV<V>(&x)[E]) { fft_line_e<decltype(dirc)::value, LOG, E>(x, a.logm, t, sm, twm); };
 
     // Input staging.  Thread t loads, for k = t + r T (r < E/2: each k in
     // [0, M/2) once; K2 < M/2), the (U, V) of both rows: one 32-byte sector
@@ -930,7 +894,7 @@ __device__ __forceinline__ void passB_area_body(const FlameDesc &d, int tile) {
     // N2), for k = n = t + r T (r < E/2) and k = n - M (r >= E/2) are
     // w^t exp(i pi r / E) and -conj(w^t exp(i pi r / E)) (w^M = -1, T = M/E):
     // one table entry per thread, the rest compile-time roots.
-    const C wt = realtw(t);
+    const C wt = __ldg(P + t);
     auto build = [&](auto own, const UV<R> *stage, CV<V>(&x)[E]) {
         static_for<0, E>([&](auto rc) {
             constexpr int r = decltype(rc)::value;
@@ -1342,15 +1306,13 @@ __device__ __forceinline__ void passC_body(const FlameDesc &d, int tile, int nti
 }
 
 // ----------------------------------------------------------------------------
-// One-line step passes: each line is transformed by its own group of
+// One-line column passes: each line is transformed by its own group of
 // T = 2^LOG / E threads (one real per point and component: V = D1 or F1),
-// and a CTA holds the groups of one column (pass A: the two fields), one
-// row pair (pass B: two rows x even/odd points) or one column pair (pass
-// C).  Used for the FP64 short lines (2^4 .. 2^7 points, E = 4 or 8: the
-// FP64 parity and trajectory grids) and, as an autotuned variant, for FP32
-// lines of 2^8 .. 2^11 points (E = 16).  A small grid has too few line
-// pairs to give every SM sub-partition a warp; with one line per group its
-// work spreads over two to four times as many warps.
+// and a CTA holds the groups of one column (pass A: the two fields) or one
+// column pair (pass C).  For the FP64 short columns (2^4 .. 2^7 points, E = 4 or
+// 8) and FP32 columns of 2^8 .. 2^10 points (E = 16): too few line pairs to
+// give every SM sub-partition a warp; with one line per group the work spreads
+// over two to four times as many warps.
 // ----------------------------------------------------------------------------
 // offset of the radix-E table (E = 16, 8 or 4) in a line's twiddle allocation
 template <int E> __host__ __device__ constexpr int tw_offset_e(int log) {

@@ -14,14 +14,13 @@ template <class R> static size_t group_smem(int logn) {
 
 // G line groups of T = 2^logn / 16 threads per CTA: up to 256 threads and
 // the shared-memory budget, but no more groups than keep at least two CTAs
-// per SM busy (small grids spread over the whole GPU).  hint > 0 fixes G.
-template <class R> static Geom make_geom(int logn, int nlines, int hint, size_t extra = 0) {
+// per SM busy (small grids spread over the whole GPU).
+template <class R> static Geom make_geom(int logn, int nlines, size_t extra = 0) {
     const int T = (1 << logn) >> 4;
-    int G = hint > 0 ? hint : (T >= kThreadsTarget ? 1 : kThreadsTarget / T);
+    int G = T >= kThreadsTarget ? 1 : kThreadsTarget / T;
     const size_t per = group_smem<R>(logn) + extra;
     while (G > 1 && (G * per > kSmemBudget || G * T > kMaxThreads)) G >>= 1;
-    if (hint <= 0)
-        while (G > 1 && (nlines + G - 1) / G < 2 * sm_count()) G >>= 1;
+    while (G > 1 && (nlines + G - 1) / G < 2 * sm_count()) G >>= 1;
 
     Geom g;
     g.threads = G * T;
@@ -30,12 +29,12 @@ template <class R> static Geom make_geom(int logn, int nlines, int hint, size_t 
     return g;
 }
 
-// Line lengths with compile-time kernels: FP32 2^8 .. 2^12; everything else (and
+// Line lengths with compile-time kernels: FP32 2^LO .. 2^12; everything else (and
 // FP64) runs the runtime-length kernels (LOG = 0).
-template <class R, class F> static void with_log(int logn, F &&f) {
+template <class R, int LO = 8, class F> static void with_log(int logn, F &&f) {
     bool done = false;
     if constexpr (sizeof(R) == 4) {
-        static_for<8, 13>([&](auto lc) {
+        static_for<LO, 13>([&](auto lc) {
             if (!done && logn == decltype(lc)::value) {
                 f(lc);
                 done = true;
@@ -44,9 +43,6 @@ template <class R, class F> static void with_log(int logn, F &&f) {
     }
     if (!done) f(std::integral_constant<int, 0>{});
 }
-
-template <class R> Geom Ops<R>::geom_cols(int logn, int nlines, int hint) { return make_geom<R>(logn, nlines, hint); }
-template <class R> Geom Ops<R>::geom_rows(int logm, int nlines, int hint) { return make_geom<R>(logm, nlines, hint); }
 
 template <class R> cudaError_t Ops<R>::init_twiddles(C *tab, int logN, cudaStream_t s) {
     return launch_k(k_twiddles<R>, dim3((tw_table_len(logN, 4) + 255) / 256, 3), 256, 0, s, tab, logN);
@@ -90,7 +86,7 @@ static int short_groups(int npairs, int T) {
 
 template <class R>
 cudaError_t Ops<R>::rows_r2c(const R *in, C *out, int n1, int logm, const C *tw, const C *tw1, cudaStream_t s, int *status) {
-    Geom g = geom_rows(logm, n1 / 2, 0);
+    Geom g = make_geom<R>(logm, n1 / 2);
     cudaError_t err = cudaSuccess;
     if (with_short_lines<R>(logm, n1 / 2, fft_split(sizeof(R) == 8, n1, logm) > 1, [&](auto lc) {
             constexpr int L = decltype(lc)::value;
@@ -114,7 +110,7 @@ cudaError_t Ops<R>::rows_r2c(const R *in, C *out, int n1, int logm, const C *tw,
 
 template <class R>
 cudaError_t Ops<R>::rows_c2r(const C *in, R *out, int n1, int logm, const C *tw, const C *tw1, cudaStream_t s, int *status) {
-    Geom g = geom_rows(logm, n1 / 2, 0);
+    Geom g = make_geom<R>(logm, n1 / 2);
     cudaError_t err = cudaSuccess;
     if (with_short_lines<R>(logm, n1 / 2, fft_split(sizeof(R) == 8, n1, logm) > 1, [&](auto lc) {
             constexpr int L = decltype(lc)::value;
@@ -160,24 +156,14 @@ cudaError_t Ops<R>::cols(const C *in, C *out, int logn, int split, int ncols, in
             int G = sizeof(R) == 4 ? 4 : 2;
             while (G > 1 && (npairs < G * sm_count() || G * T > 256)) G >>= 1;
             const size_t smem = G * cols_group_bytes<R, 4>(1 << L, G);
-            if (dir < 0) go(k_cols<R, -1, L, 256, 4>, G * T, G, smem);
-            else go(k_cols<R, 1, L, 256, 4>, G * T, G, smem);
+            if (dir < 0) go(k_cols<R, -1, L, 4>, G * T, G, smem);
+            else go(k_cols<R, 1, L, 4>, G * T, G, smem);
         }))
         return err;
     const int n = 1 << logn, T = n >> 4;
-    const Geom g = geom_cols(logn, npairs * split, 0);
+    const Geom g = make_geom<R>(logn, npairs * split);
     with_log<R>(logn, [&](auto lc) {
         constexpr int L = decltype(lc)::value;
-        // FP32 whole columns of 2^10 .. 2^12 points: 512-thread CTAs of 512/T
-        // line groups (one CTA per SM), where the grid still has two CTAs per SM
-        if constexpr (sizeof(R) == 4 && L >= 10 && L <= 12) {
-            constexpr int G = 512 / ((1 << L) >> 4);
-            if (split == 1 && npairs >= 2 * G * sm_count()) {
-                if (dir < 0) go(k_cols<R, -1, L, 512>, 512, G, G * cols_group_bytes<R>(n, G));
-                else go(k_cols<R, 1, L, 512>, 512, G, G * cols_group_bytes<R>(n, G));
-                return;
-            }
-        }
         const int G = g.threads / T;
         if (dir < 0) go(k_cols<R, -1, L>, g.threads, G, G * cols_group_bytes<R>(n, G));
         else go(k_cols<R, 1, L>, g.threads, G, G * cols_group_bytes<R>(n, G));
@@ -189,11 +175,11 @@ cudaError_t Ops<R>::cols(const C *in, C *out, int logn, int split, int ncols, in
 // CTA (the runtime kernels give such lines 2^LOG/16 threads, a quarter warp
 // at 128 points, and are bound by the latency of their FP64 chains)
 template <class R> static bool small_fp64(int logn) { return sizeof(R) == 8 && logn >= 4 && logn <= 7; }
-// Points per thread of the FP64 short-line kernels: 4 (a warp per 128-point
-// line pair), or 8 with FLAME_FP64_POINTS=8 (read at every launch, so tests
-// can run both).  Measured on the 128 x 256 FP64 trajectory: 46.1 us per
-// step with 4, 78.4 us with 8: the lines' FP64 chains are latency-bound,
-// and a full warp per line pair halves each thread's chain.
+// Points per thread of those kernels, which a step with its area runs: 4 (a warp
+// per 128-point line pair), or 8 with FLAME_FP64_POINTS=8 (read at every launch,
+// so tests can run both).  The lines' FP64 chains are latency-bound, and a full
+// warp per line pair halves each thread's: when the plain step ran them too,
+// 128x256 took 46.1 us a step with 4 and 78.4 with 8.
 static int fp64_points() {
     const char *v = getenv("FLAME_FP64_POINTS");
     return (v && strcmp(v, "8") == 0) ? 8 : 4;
@@ -205,9 +191,9 @@ template <class R, int E> static Geom geom_small_fp64(int logn, int nlines, size
     g.smem = 2 * (size_t)plane_len_e<E>(1 << logn) * sizeof(typename VecOf<R>::type) + extra;
     return g;
 }
-// CTA of the one-line kernels (k_passA1/B1/C1): `groups` line
-// groups of 2^logn / E threads, each with its own exchange planes, and
-// `extra` bytes more (pass B's parked g of two rows); one CTA per unit
+// CTA of the one-line kernels (k_passA1, k_passC1): `groups` line groups of
+// 2^logn / E threads, each with its own exchange planes, and `extra` bytes more;
+// one CTA per unit
 template <class R, int E> static Geom geom_short1(int logn, int units, int groups, size_t extra) {
     Geom g;
     g.threads = groups * ((1 << logn) / E);
@@ -260,8 +246,8 @@ cudaError_t Ops<R>::passA_full(const FlameDesc &d, cudaStream_t s, const CUtenso
         });
         return err;
     }
-    const Geom g = geom_cols(d.a.logn1, d.a.K2 + 1, 0);
-    with_log<R>(d.a.logn1, [&](auto lc) {
+    const Geom g = make_geom<R>(d.a.logn1, d.a.K2 + 1);
+    with_log<R, 11>(d.a.logn1, [&](auto lc) {
         constexpr int L = decltype(lc)::value;
         if constexpr (sizeof(R) == 4 && L > 0) if (uv_map) {  // tensor-store write-out
             const int pf = resident_ctas((const void *)k_passAt<R, L>, g);
@@ -325,19 +311,10 @@ template <class R> cudaError_t Ops<R>::passB_area(const FlameDesc &d, cudaStream
         if (err != cudaSuccess) return err;
         return cudaGetLastError();
     }
-    Geom g = make_geom<R>(d.a.logm, d.a.n1 / 2, 0, (size_t)M * sizeof(typename VecOf<R>::c) + area_extra);
-    with_log<R>(d.a.logm, [&](auto lc) {
-        constexpr int L = decltype(lc)::value;
-        Geom ga = g;
-        if (kSharedTw<R, L, 16>) ga.smem += kTwSmemBytes;
-        if (ga.smem + 4096 > (size_t)optin) {
-            err = cudaErrorNotSupported;
-            return;
-        }
-        err = launch_s(L2Window{nullptr, 0, 0.f}, pdl_area<R>(), k_passB_area<R, L, 16, 256>, dim3(ga.blocks + 1), ga.threads, ga.smem, s, d);
-    });
-    if (err != cudaSuccess) return err;
-    return cudaGetLastError();
+    // other rows: the runtime-length kernel
+    const Geom g = make_geom<R>(d.a.logm, d.a.n1 / 2, (size_t)M * sizeof(typename VecOf<R>::c) + area_extra);
+    if (g.smem + 4096 > (size_t)optin) return cudaErrorNotSupported;
+    return launch_s(L2Window{nullptr, 0, 0.f}, pdl_area<R>(), k_passB_area<R, 0, 16, 256>, dim3(g.blocks + 1), g.threads, g.smem, s, d);
 }
 
 template <class R> cudaError_t Ops<R>::passC_full(const FlameDesc &d, cudaStream_t s) {
@@ -363,8 +340,8 @@ template <class R> cudaError_t Ops<R>::passC_full(const FlameDesc &d, cudaStream
         });
         return err;
     }
-    const Geom g = geom_cols(d.a.logn1, (d.a.K2 + 2) / 2, 0);
-    with_log<R>(d.a.logn1, [&](auto lc) {
+    const Geom g = make_geom<R>(d.a.logn1, (d.a.K2 + 2) / 2);
+    with_log<R, 11>(d.a.logn1, [&](auto lc) {
         constexpr int L = decltype(lc)::value;
         const int pf = resident_ctas((const void *)k_passC<R, L>, g);
         err = launch_w(d.l2_state, k_passC<R, L>, dim3(g.blocks + 1), g.threads, g.smem, s, d, pf);
@@ -385,7 +362,7 @@ template <class R> static Geom geom_row1(int logm, int nrows) {
 // half row length (log2 N2/2) as their compile-time LOG (0: any length).
 template <class R> cudaError_t Ops<R>::area(const AdjDesc &d, cudaStream_t s) {
     const StepArgs &a = d.a;
-    Geom ga = geom_cols(a.logn1, a.K2 + 1, 0);
+    Geom ga = make_geom<R>(a.logn1, a.K2 + 1);
     Geom gb = geom_row1<R>(a.logm, a.n1);
     cudaError_t e = cudaSuccess;
     with_log<R>(a.logn1, [&](auto lc) {
