@@ -363,7 +363,8 @@ flame_status flame_adjoint(flame_t h, const void *state0, const double *mean0,
  * keeps the last call's contents; each call rewrites the tables and
  * workspaces it reads and clears the status word, but calls whose work
  * overlaps on the GPU (unordered streams) race on the array.  Non-finite
- * values are not reported (there is no handle to read them from). */
+ * values are not reported (there is no handle to read them from), nor is a
+ * device-side wait that ran out, which leaves the state and the mean mode NaN. */
 flame_status flame_step_noalloc(const flame_params *params, void *state, double *mean_mode,
                                 double *t, int nsteps, void *stream);
 

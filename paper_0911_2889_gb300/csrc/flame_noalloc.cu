@@ -22,6 +22,7 @@
 #include <cmath>
 #include <cstdarg>
 #include <cstdio>
+#include <cstdlib>
 #include <cstring>
 #include <mutex>
 
@@ -101,6 +102,10 @@ flame_status run_steps(const flame::StepArgs &a, unsigned char *base, size_t off
     flame::FlameDesc d;
     memset(&d, 0, sizeof d);
     d.a = a;
+#ifdef FLAME_DEBUG_BOUNDS
+    const char *fault = getenv("FLAME_FAULT_INJECT");
+    if (fault && strcmp(fault, "wait") == 0) d.a.flags |= flame::kStallRowLoad;
+#endif
     d.state = d.state_out = state;
     d.uv = base + off_uv;
     d.gk = base + off_gk;

@@ -297,8 +297,9 @@ __device__ __forceinline__ bool bulk_wait(unsigned long long *bar) {
 }
 // All threads, at the barrier behind the reads of the block: false, and the
 // status says so, where some thread's wait ran out.  What the CTA read may not
-// be the block then: it writes nothing and returns, behind one more bounded
-// wait for the copy that may still be on its way into its shared memory.
+// be the block then: it makes its part of the output NaN, so that a caller
+// who does not ask for the status sees it too, and returns, behind one more
+// bounded wait for the copy that may still be on its way into its shared memory.
 __device__ __forceinline__ bool bulk_read(bool came, unsigned long long *bar, int *status) {
     if (__syncthreads_and(came)) return true;
     if (threadIdx.x == 0) atomicOr(status, 1 << kStatusTimeout);
@@ -376,7 +377,13 @@ __device__ __forceinline__ void stepB2_body(const FlameDesc &d, int tile, const 
             up[i] = CV<V>{make_float2(q.x, q.y), make_float2(q.z, q.w)};
             um[i] = CV<V>{make_float2(m.x, m.y), make_float2(m.z, m.w)};
         }
-        if (!bulk_read(came, &loaded, d.status)) return;  // (a barrier: the block has been read)
+        if (!bulk_read(came, &loaded, d.status)) {  // (a barrier: the block has been read)
+            const R nan = (R)__int_as_float(0x7fc00000);
+            for (int k = s.t; valid && k <= a.K2; k += TS)
+                if (FLAME_IN(d.status, g_index(2 * pair, k, a.n1) + 1, gk_len(a), kSiteBGk))
+                    *reinterpret_cast<float4 *>(gk + g_index(2 * pair, k, a.n1)) = make_float4(nan, nan, nan, nan);
+            return;
+        }
         CV<V> xo[ES];
         static_for<0, ES>([&](auto rc) {
             constexpr int r = decltype(rc)::value;
